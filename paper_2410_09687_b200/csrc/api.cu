@@ -213,16 +213,16 @@ moin_status moin_router_prepare(const void* centroids, int32_t K, int32_t D, flo
 }
 
 size_t moin_route_workspace_bytes(int32_t Q, int32_t K, int32_t D) {
-  (void)K; (void)D;
-  return align_up((size_t)(Q > 0 ? Q : 0) * sizeof(unsigned long long), 256) + 256;
+  if (Q <= 0) return 256;
+  return align_up((size_t)Q * (size_t)route_parts(Q, K, D) * sizeof(unsigned long long), 256) + 256;
 }
 
 // Kernel choice shared by moin_route and moin_route_static, so that both compute the same values for the same
-// shapes and options: 0 = cluster kernel (decode-sized batch: one launch, no scratch), 1 = tensor-core GEMM with
-// one 64-bit key of scratch per query, 2 = CUDA-core kernel (no scratch).
+// shapes and options: 0 = cluster kernel (few queries; one 64-bit key of scratch per query and part when it cuts the
+// table), 1 = tensor-core GEMM with one 64-bit key of scratch per query, 2 = CUDA-core kernel (no scratch).
 static moin_status route_choice(const HostState* hs, int Q, int K, int D, int* choice) {
   const bool tc_ok = tc_router_supported(Q, K, D);
-  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 16);
+  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 12);
   if (hs->gemm_impl == 1) use_tc = false;
   if (hs->gemm_impl == 2) {
     if (!tc_ok) return MOIN_ERR_BAD_SHAPE;
@@ -238,10 +238,10 @@ static moin_status route_launch(HostState* hs, int choice, const moin_router* ro
                                 unsigned long long* keys, cudaStream_t s) {
   const int K = router->K, D = router->D;
   if (choice == 0) {
-    ProfScope prof(MOIN_K_ROUTE_CLUSTER, 1, s);
+    ProfScope prof(MOIN_K_ROUTE_CLUSTER, route_parts(Q, K, D) > 1 ? 2 : 1, s);
     return record_cuda(launch_route_cluster((const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
                                             router->inv_norm, router->centroid_to_expert, Q, K, D, out_expert,
-                                            out_centroid, out_best_sim, s));
+                                            out_centroid, out_best_sim, keys, s));
   }
   if (choice == 1) {
     // the merge across column tiles is a max, so the keys must start from zero
@@ -283,16 +283,22 @@ moin_status moin_route(const moin_router* router, const void* queries, int32_t Q
   if ((st = host_state(&hs))) return st;
   int choice;
   if ((st = route_choice(hs, Q, router->K, router->D, &choice))) return st;
-  if (choice == 1 && (!workspace || workspace_bytes < moin_route_workspace_bytes(Q, router->K, router->D) ||
-                      !aligned16(workspace)))
-    return MOIN_ERR_WORKSPACE;
-  return route_launch(hs, choice, router, queries, Q, out_expert, out_centroid, out_best_sim,
-                      reinterpret_cast<unsigned long long*>(workspace), (cudaStream_t)stream);
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(workspace);
+  if (!workspace || workspace_bytes < moin_route_workspace_bytes(Q, router->K, router->D) || !aligned16(workspace)) {
+    // small problems run without scratch: the cluster kernel with the table in one part, or the CUDA-core kernel
+    keys = nullptr;
+    if (choice == 1 && hs->gemm_impl != 2) {
+      if (Q <= 1024 && router->K <= 1024 && router->D <= 3072) choice = 0;
+      else if ((long long)Q * router->K < (1ll << 16)) choice = 2;
+    }
+    if (choice == 1) return MOIN_ERR_WORKSPACE;
+  }
+  return route_launch(hs, choice, router, queries, Q, out_expert, out_centroid, out_best_sim, keys, (cudaStream_t)stream);
 }
 
 size_t moin_route_top2_workspace_bytes(int32_t Q, int32_t K, int32_t D) {
-  (void)K; (void)D;
-  return 2 * align_up((size_t)(Q > 0 ? Q : 0) * sizeof(unsigned long long), 256) + 256;
+  if (Q <= 0) return 256;
+  return 2 * align_up((size_t)Q * (size_t)route_parts(Q, K, D) * sizeof(unsigned long long), 256) + 256;
 }
 
 moin_status moin_route_top2(const moin_router* router, const void* queries, int32_t Q, int32_t* out_expert,
@@ -309,11 +315,23 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
   if (st) return st;
   cudaStream_t s = (cudaStream_t)stream;
   const bool tc_ok = tc_router_supported(Q, K, D);
-  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 16);
+  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 12);
   if (hs->gemm_impl == 1) use_tc = false;
   if (hs->gemm_impl == 2) {
     if (!tc_ok) return MOIN_ERR_BAD_SHAPE;
     use_tc = true;
+  }
+  const bool fits = workspace && workspace_bytes >= moin_route_top2_workspace_bytes(Q, K, D) && aligned16(workspace);
+  if (use_tc && !fits && !(hs->gemm_impl == 0 && route_cluster_supported(Q, K, D))) {
+    if (hs->gemm_impl == 2 || (long long)Q * K >= (1ll << 16)) return MOIN_ERR_WORKSPACE;
+    use_tc = false;
+  }
+  if (hs->gemm_impl == 0 && route_cluster_supported(Q, K, D)) {
+    ProfScope prof(MOIN_K_ROUTE_CLUSTER, route_parts(Q, K, D) > 1 ? 2 : 1, s);
+    return record_cuda(launch_route_top2_cluster((const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
+                                                 router->inv_norm, router->centroid_to_expert, Q, K, D, out_expert,
+                                                 out_centroid, out_second, out_best_sim, out_margin,
+                                                 fits ? reinterpret_cast<unsigned long long*>(workspace) : nullptr, s));
   }
   if (!use_tc) {
     ProfScope prof(MOIN_K_ROUTE_SIMPLE, 1, s);
@@ -321,8 +339,6 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
                                                 router->inv_norm, router->centroid_to_expert, Q, K, D, out_expert,
                                                 out_centroid, out_second, out_best_sim, out_margin, s));
   }
-  if (!workspace || workspace_bytes < moin_route_top2_workspace_bytes(Q, K, D) || !aligned16(workspace))
-    return MOIN_ERR_WORKSPACE;
   const size_t half = align_up((size_t)Q * sizeof(unsigned long long), 256);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(workspace);
   unsigned long long* keys2 = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(workspace) + half);
@@ -355,7 +371,7 @@ moin_status moin_route_static(const moin_router* router, const void* queries, in
   int choice;
   if ((st = route_choice(hs, Q, router->K, router->D, &choice))) return st;
   unsigned long long* keys = nullptr;
-  if (choice == 1) {   // only the tensor-core kernel needs scratch
+  if (choice == 1 || (choice == 0 && route_parts(Q, router->K, router->D) > 1)) {
     if (g_route_static_ptr[hs->device] == nullptr) {   // set-up: once per device, that device is current here
       void* p = nullptr;
       cudaError_t e = cudaGetSymbolAddress(&p, g_route_static_keys);

@@ -117,6 +117,27 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Programmatic dependent launch: the next kernel of the stream may start once every CTA has got here / this CTA goes
+// on once the kernels before it are complete and their writes visible (no-ops in an ordinary launch).
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch as the programmatic dependent of the kernel before it in the stream: the grid may start as soon as every CTA
+// of that kernel has called pdl_launch_dependents (or ended); what depends on it waits with pdl_wait.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*fn)(P...), int grid, int threads, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+
 // Launchers implemented in the .cu files (host side).
 int plan_launches(int T, int E);   // kernels launch_plan_build issues for this shape
 cudaError_t launch_plan_build(const int* token_expert, const PlanView& v, DeviceStatus* status, bool want_tiles,
@@ -164,7 +185,15 @@ cudaError_t launch_route_simple(const __nv_bfloat16* q, const __nv_bfloat16* c, 
 bool route_cluster_supported(int Q, int K, int D);
 cudaError_t launch_route_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                  const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
-                                 float* out_best, cudaStream_t stream);
+                                 float* out_best, unsigned long long* part_keys, cudaStream_t stream);
+// Parts the cluster kernel cuts the table into, given route_parts(Q, K, D) * Q keys of scratch (top-2: twice as many);
+// with part_keys == nullptr it takes the table in one part.
+constexpr int kRouteMaxParts = 12;
+int route_parts(int Q, int K, int D);
+cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
+                                      const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
+                                      int* out_second, float* out_best, float* out_margin,
+                                      unsigned long long* part_keys, cudaStream_t stream);
 cudaError_t launch_route_finish(const unsigned long long* keys, const __nv_bfloat16* q, const int* cmap, int Q, int D,
                                 int* out_expert, int* out_centroid, float* out_best, cudaStream_t stream);
 
@@ -190,7 +219,7 @@ moin_status record_cuda(cudaError_t e);       // MOIN_OK or MOIN_ERR_CUDA (remem
 // that attribute per device, so the "already done" note is kept per device too (slot = one id per kernel).
 enum {
   OPTIN_TC_GEMM = 0,        // + 4 * (BN index) + EPI, 12 entries; + 12 for the short-ring instantiations
-  OPTIN_ROUTE_CLUSTER = 24, OPTIN_ROUTE_SIMPLE = 25, OPTIN_ATTENTION = 29
+  OPTIN_ROUTE_CLUSTER = 24, /* .. 27 */ OPTIN_ROUTE_SIMPLE = 28, OPTIN_ATTENTION = 29
 };
 template <class Fn>
 inline cudaError_t ensure_smem_optin(int slot, Fn* fn, size_t bytes) {

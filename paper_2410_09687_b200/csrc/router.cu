@@ -2,7 +2,7 @@
 // small problems and odd shapes, and the finishing pass shared with the tensor-core router.
 #include <cooperative_groups.h>
 
-#include "common.cuh"
+#include "tc_gemm.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -153,191 +153,397 @@ route_finish_kernel(const unsigned long long* __restrict__ keys, const __nv_bflo
 }
 
 // ----------------------------------------------------------------------------------------
-// Small-batch router (decode-sized Q): one launch, no scratch memory.
+// Small-batch router.
 //
-// A cluster of kRcCluster CTAs serves kRcQ queries.  The centroids are cut into 16-row tiles,
-// dealt round-robin to the cluster's warps (two warps share a tile, half of the k range each);
-// a warp holds its tile's rows as the A operand of
-// m16n8k16 (loaded straight from global memory, 16 bytes per lane: lane t of a row group takes
-// k-elements 8t..8t+7 of every 32, and the queries, staged once in shared memory, are read with the
-// same k assignment, so the contraction is unchanged) and the kRcQ queries as kRcQ/8 B operands.
-// Every CTA merges its warps' per-query winners in its own shared memory with a 64-bit max on the
-// (similarity, index) key; after a cluster barrier CTA 0 reads the other CTAs' keys through
-// distributed shared memory and writes the result.
+// A cluster of 8 CTAs serves NQ queries against one part of the centroid table.  The part is cut into 16-row
+// tiles, dealt round-robin to the cluster's warps; a warp holds its tile's rows as the A operand of m16n8k16 (loaded
+// straight from global memory, 16 bytes per lane: lane t of a row group takes k-elements 8t..8t+7 of every 32, and the
+// queries, staged once in shared memory, are read with the same k assignment, so the contraction is unchanged) and the
+// NQ queries as NQ/8 B operands.  Every lane keeps the best candidate of its rows over all its tiles; they meet per CTA
+// in shared memory with a 64-bit max on the (similarity, index) key, and after a cluster barrier CTA 0 reads the other
+// CTAs' keys through distributed shared memory.  A table in one part (up to 512 centroids) is finished right there:
+// one launch, no scratch.  Larger tables are cut into parts, one cluster each, whose keys go to
+// scratch and meet in a small second launch.
+//
+// What bounds it: a few dependent memory round trips, and what the SMs of one cluster can pull - one cluster of 16
+// needs 15.3 us for 1 x 5000 x 768 (480 KB per SM), ten clusters and the second launch 7.4 us (the CUDA-core kernel
+// with its one CTA per eight queries: 1446 us).  The centroid loads run one batch of kRcBatch k-steps ahead of
+// the products, across tiles too (deeper register rings measured slower: 16.5 us), and the queries' rows are skewed to
+// 64 bytes past a multiple of 128, so that the eight rows of a fragment sit on distinct banks.  NQ = 8 for up to eight
+// queries: 5.8 us at 500 centroids against 9.1 us for a 32-wide query block.
 // ----------------------------------------------------------------------------------------
-constexpr int kRcCluster = 8, kRcTileWarps = 4, kRcKSplit = 2, kRcWarps = kRcTileWarps * kRcKSplit, kRcQ = 32,
-              kRcUnroll = 12;
+constexpr int kRcWarps = 8, kRcBatch = 6;
 
 __device__ __forceinline__ unsigned long long route_key(float sim, int k) {
   uint32_t u = __float_as_uint(sim);
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   return ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)k);
 }
+__device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v, int o) {
+  return __shfl_xor_sync(0xffffffffu, v, o);
+}
+// best two of two (best, second) pairs of distinct keys (0 = none)
+__device__ __forceinline__ void merge_top2(unsigned long long& b, unsigned long long& s, unsigned long long ob,
+                                           unsigned long long os) {
+  const unsigned long long hi = b > ob ? b : ob, lo = b > ob ? ob : b, se = s > os ? s : os;
+  b = hi;
+  s = lo > se ? lo : se;
+}
+__host__ __device__ inline int route_pitch(int D) {   // bytes of a query row in shared memory, 64 mod 128
+  const int row = (D + 31) / 32 * 64;
+  return (row & 127) ? row : row + 64;
+}
+__device__ __forceinline__ void add_sq8(const uint4& v, float& ss) {   // ss += the squares of eight bf16
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    ss = fmaf(bf16_lo(w[e]), bf16_lo(w[e]), ss);
+    ss = fmaf(bf16_hi(w[e]), bf16_hi(w[e]), ss);
+  }
+}
 
-// Warp w works on centroid tile (w % kRcTileWarps) of the CTA's current round and on the
-// (w / kRcTileWarps)-th part of the k range; the parts are added in shared memory in a fixed order.
-__global__ void __cluster_dims__(kRcCluster, 1, 1) __launch_bounds__(kRcWarps * 32)
+struct RouteOut { int *expert, *centroid, *second; float *best, *margin; };
+
+// keys -> outputs of query i (ss = |q_i|^2)
+template <bool TOP2>
+__device__ __forceinline__ void route_write(const RouteOut& out, const int* cmap, int i, unsigned long long k1,
+                                            unsigned long long k2, float ss) {
+  const int id = (k1 == 0ull) ? 0 : (int)(0xFFFFFFFFu - (uint32_t)(k1 & 0xFFFFFFFFull));
+  const float rq = rsqrtf(ss), s1 = key_to_float((uint32_t)(k1 >> 32)), s2 = key_to_float((uint32_t)(k2 >> 32));
+  if (out.centroid) out.centroid[i] = id;
+  if (out.expert) out.expert[i] = cmap ? cmap[id] : id;
+  if (out.best) out.best[i] = (k1 == 0ull) ? -INFINITY : s1 * rq;
+  if (TOP2) {
+    if (out.second) out.second[i] = (k2 == 0ull) ? -1 : (int)(0xFFFFFFFFu - (uint32_t)(k2 & 0xFFFFFFFFull));
+    if (out.margin) out.margin[i] = (k1 == 0ull || k2 == 0ull) ? INFINITY : (s1 - s2) * rq;
+  }
+}
+
+// part_keys (nullptr when parts == 1): [parts][Q] keys, and with TOP2 [parts][Q] runner-up keys behind them
+template <int NQ, bool TOP2>
+__global__ void __launch_bounds__(kRcWarps * 32)
 route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ c,
-                     const float* __restrict__ inv_norm, const int* __restrict__ cmap, int Q, int K, int D,
-                     int* __restrict__ out_expert, int* __restrict__ out_centroid, float* __restrict__ out_best) {
+                     const float* __restrict__ inv_norm, const int* __restrict__ cmap, int Q, int K, int D, int parts,
+                     unsigned long long* __restrict__ part_keys, const RouteOut out) {
+  constexpr int NJ = NQ / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ unsigned long long s_keys[kRcQ];
-  __shared__ float s_part[kRcTileWarps][kRcQ / 8][4][32];
+  __shared__ unsigned long long s_keys[NQ], s_keys2[NQ];
+  __shared__ float s_part[kRcWarps / 2][NJ][4][32];
+  pdl_launch_dependents();
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int tw = warp % kRcTileWarps, kpart = warp / kRcTileWarps;
-  const int rank = (int)cluster.block_rank();
-  const int q0 = (blockIdx.x / kRcCluster) * kRcQ;
-  const int pitch = D * 2 + 16;  // bytes; the 16-byte skew keeps the 8 rows of a fragment on distinct banks
-  const int nch = D / 8;
-  const int n_tiles = (K + 15) / 16, steps = D / 32;
-  const int steps_part = (steps + kRcKSplit - 1) / kRcKSplit;
+  const int rank = (int)cluster.block_rank(), csize = (int)cluster.num_blocks();
+  const int cl = blockIdx.x / csize, part = cl % parts, q0 = (cl / parts) * NQ;
+  const int pitch = route_pitch(D);
+  const int nch = D / 8, steps = (nch + 3) / 4, all_tiles = (K + 15) / 16;
+  const int tile_lo = (int)((long long)all_tiles * part / parts), tile_hi = (int)((long long)all_tiles * (part + 1) / parts);
+  // few tiles: two warps share one, half of the k range each (the parts are added in shared memory in a fixed order)
+  const int ksplit = (tile_hi - tile_lo <= csize * (kRcWarps / 2)) ? 2 : 1, tile_warps = kRcWarps / ksplit;
+  const int tw = warp % tile_warps, kpart = warp / tile_warps;
+  const int steps_part = (steps + ksplit - 1) / ksplit;
   const int s_lo = kpart * steps_part, s_hi = min(steps, s_lo + steps_part);
+  const int nb = (steps_part + kRcBatch - 1) / kRcBatch;   // batches per tile
 
-  // the first batch of centroid rows is requested before the queries are staged: one round trip for both
-  int tile = rank * kRcTileWarps + tw;
-  uint4 a0[kRcUnroll], a1[kRcUnroll];
-  auto load_a = [&](int tl, int s0) {
+  uint4 a[2][kRcBatch][2];
+  auto load = [&](uint4 (&r)[kRcBatch][2], int tl, int b) {
     const int r0 = tl * 16 + g, r1 = r0 + 8;
     // rows past K read row K-1 (in bounds) and are masked at the end
-    const __nv_bfloat16* a0p = c + (size_t)min(r0, K - 1) * D + t * 8;
-    const __nv_bfloat16* a1p = c + (size_t)min(r1, K - 1) * D + t * 8;
+    const __nv_bfloat16* p0 = c + (size_t)min(r0, K - 1) * D;
+    const __nv_bfloat16* p1 = c + (size_t)min(r1, K - 1) * D;
 #pragma unroll
-    for (int u = 0; u < kRcUnroll; ++u) {
-      const bool on = tl < n_tiles && s0 + u < s_hi;
-      a0[u] = on ? ldg_cached(a0p + (s0 + u) * 32) : make_uint4(0, 0, 0, 0);
-      a1[u] = on ? ldg_cached(a1p + (s0 + u) * 32) : make_uint4(0, 0, 0, 0);
+    for (int u = 0; u < kRcBatch; ++u) {
+      const int st = s_lo + b * kRcBatch + u, ch = st * 4 + t;
+      const bool on = tl < tile_hi && st < s_hi && ch < nch;
+      r[u][0] = on ? ldg_cached(p0 + ch * 8) : make_uint4(0, 0, 0, 0);
+      r[u][1] = on ? ldg_cached(p1 + ch * 8) : make_uint4(0, 0, 0, 0);
     }
   };
-  load_a(tile, s_lo);
-  for (int i0 = 0; i0 < kRcQ * nch; i0 += kRcWarps * 32 * 8) {
-    uint4 v[8];
+  // the first centroid rows are requested before the queries are staged: one round trip for both
+  int tile = tile_lo + rank * tile_warps + tw;
+  const int stride = csize * tile_warps;
+  load(a[0], tile, 0);
+  const int row_ch = steps * 4;   // chunks of a staged row, zero beyond the embedding
+  for (int i0 = 0; i0 < NQ * row_ch; i0 += kRcWarps * 32 * 12) {
+    uint4 v[12];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 12; ++u) {
       const int i = i0 + u * kRcWarps * 32 + tid;
-      const int qi = i / nch, ch = i - qi * nch;
-      v[u] = (i < kRcQ * nch && q0 + qi < Q) ? ldg_cached(q + (size_t)(q0 + qi) * D + ch * 8) : make_uint4(0, 0, 0, 0);
+      const int qi = i / row_ch, ch = i - qi * row_ch;
+      v[u] = (i < NQ * row_ch && q0 + qi < Q && ch < nch) ? ldg_cached(q + (size_t)(q0 + qi) * D + ch * 8) : make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 12; ++u) {
       const int i = i0 + u * kRcWarps * 32 + tid;
-      const int qi = i / nch, ch = i - qi * nch;
-      if (i < kRcQ * nch) *reinterpret_cast<uint4*>(smem_raw + (size_t)qi * pitch + ch * 16) = v[u];
+      const int qi = i / row_ch, ch = i - qi * row_ch;
+      if (i < NQ * row_ch) *reinterpret_cast<uint4*>(smem_raw + (size_t)qi * pitch + ch * 16) = v[u];
     }
   }
-  if (tid < kRcQ) s_keys[tid] = 0ull;
+  if (tid < NQ) {
+    s_keys[tid] = 0ull;
+    s_keys2[tid] = 0ull;
+  }
   __syncthreads();
 
-  for (bool first = true; tile - tw < n_tiles; tile += kRcCluster * kRcTileWarps, first = false) {   // CTA-uniform trip count
-    float acc[kRcQ / 8][4];
+  // candidates of this lane: queries j*8 + 2t + e; rows in increasing order, strict '>' keeps the lowest index
+  float best[NJ][2], second[NJ][2];
+  int best_k[NJ][2], second_k[NJ][2];
 #pragma unroll
-    for (int j = 0; j < kRcQ / 8; ++j)
+  for (int j = 0; j < NJ; ++j)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
-    for (int s0 = s_lo; s0 < s_hi; s0 += kRcUnroll) {
-      if (!first || s0 > s_lo) load_a(tile, s0);
+    for (int e = 0; e < 2; ++e) {
+      best[j][e] = second[j][e] = -INFINITY;
+      best_k[j][e] = second_k[j][e] = 0;
+    }
+  float acc[NJ][4];
 #pragma unroll
-      for (int u = 0; u < kRcUnroll; ++u) {
-        if (s0 + u >= s_hi) break;
+  for (int j = 0; j < NJ; ++j)
 #pragma unroll
-        for (int j = 0; j < kRcQ / 8; ++j) {
-          const uint4 b = *reinterpret_cast<const uint4*>(smem_raw + (size_t)(j * 8 + g) * pitch + (s0 + u) * 64 + t * 16);
-          mma_bf16_16816(acc[j], a0[u].x, a1[u].x, a0[u].y, a1[u].y, b.x, b.y);
-          mma_bf16_16816(acc[j], a0[u].z, a1[u].z, a0[u].w, a1[u].w, b.z, b.w);
-        }
+    for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+  auto multiply = [&](uint4 (&r)[kRcBatch][2], int b) {
+#pragma unroll
+    for (int u = 0; u < kRcBatch; ++u) {
+      const int st = s_lo + b * kRcBatch + u;
+      if (st >= s_hi) break;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const uint4 bv = *reinterpret_cast<const uint4*>(smem_raw + (size_t)(j * 8 + g) * pitch + st * 64 + t * 16);
+        mma_bf16_16816(acc[j], r[u][0].x, r[u][1].x, r[u][0].y, r[u][1].y, bv.x, bv.y);
+        mma_bf16_16816(acc[j], r[u][0].z, r[u][1].z, r[u][0].w, r[u][1].w, bv.z, bv.w);
       }
     }
-    // add the k parts: part 1.. hand their sums to part 0 through shared memory
-    if (kpart > 0) {
-#pragma unroll
-      for (int j = 0; j < kRcQ / 8; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s_part[tw][j][e][lane] = acc[j][e];
+  };
+  auto take = [&](float sim, int k, int j, int e) {
+    if (sim > best[j][e]) {
+      if (TOP2) { second[j][e] = best[j][e]; second_k[j][e] = best_k[j][e]; }
+      best[j][e] = sim;
+      best_k[j][e] = k;
+    } else if (TOP2 && sim > second[j][e]) {
+      second[j][e] = sim;
+      second_k[j][e] = k;
     }
-    __syncthreads();
-    if (kpart == 0 && tile < n_tiles) {
+  };
+  auto finish_tile = [&]() {   // (CTA-uniform trip count when two warps share a tile)
+    if (ksplit == 2) {
+      if (kpart > 0) {
 #pragma unroll
-      for (int j = 0; j < kRcQ / 8; ++j)
+        for (int j = 0; j < NJ; ++j)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[j][e] += s_part[tw][j][e][lane];
+          for (int e = 0; e < 4; ++e) s_part[tw][j][e][lane] = acc[j][e];
+      }
+      __syncthreads();
+      if (kpart == 0) {
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[j][e] += s_part[tw][j][e][lane];
+      }
+    }
+    if (kpart == 0 && tile < tile_hi) {
       // acc[j][0..1]: centroid r0, queries j*8 + 2t, 2t+1;  acc[j][2..3]: centroid r1
       const int r0 = tile * 16 + g, r1 = r0 + 8;
       const float inv0 = (r0 < K) ? inv_norm[r0] : 0.f, inv1 = (r1 < K) ? inv_norm[r1] : 0.f;
 #pragma unroll
-      for (int j = 0; j < kRcQ / 8; ++j)
+      for (int j = 0; j < NJ; ++j)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          const float sim0 = acc[j][e] * inv0, sim1 = acc[j][2 + e] * inv1;
-          unsigned long long key = 0ull;   // 0 = no candidate (zero-norm or padding row, NaN or -inf similarity)
-          if (inv0 > 0.f && sim0 > -INFINITY) key = route_key(sim0, r0);
-          if (inv1 > 0.f && sim1 > -INFINITY) {
-            const unsigned long long k1 = route_key(sim1, r1);
-            key = k1 > key ? k1 : key;
-          }
-#pragma unroll
-          for (int o = 4; o < 32; o <<= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
-            key = other > key ? other : key;
-          }
-          if (g == 0 && key != 0ull) atomicMax(&s_keys[j * 8 + 2 * t + e], key);
+          if (inv0 > 0.f) take(acc[j][e] * inv0, r0, j, e);
+          if (inv1 > 0.f) take(acc[j][2 + e] * inv1, r1, j, e);
         }
     }
-    __syncthreads();   // s_part is free again
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+  };
+  if (ksplit == 2) {   // at most one tile per warp: every warp walks the same number of batches
+    for (int b = 0; b < nb; b += 2) {
+      if (b + 1 < nb) load(a[1], tile, b + 1);
+      multiply(a[0], b);
+      if (b + 2 < nb) load(a[0], tile, b + 2);
+      if (b + 1 < nb) multiply(a[1], b + 1);
+    }
+    finish_tile();
+  } else {             // (tile, batch) pairs in sequence, two per turn so that the buffers are static
+    int b = 0;
+    auto advance = [&](int& tl, int& bb) {
+      if (++bb == nb) { bb = 0; tl += stride; }
+    };
+    while (tile < tile_hi) {
+      int tl = tile, bb = b;
+      advance(tl, bb);
+      load(a[1], tl, bb);
+      multiply(a[0], b);
+      if (b == nb - 1) finish_tile();
+      tile = tl; b = bb;
+      if (tile >= tile_hi) break;
+      advance(tl, bb);
+      load(a[0], tl, bb);
+      multiply(a[1], b);
+      if (b == nb - 1) finish_tile();
+      tile = tl; b = bb;
+    }
+  }
+  // the eight row groups of a warp meet by shuffles, the warps in shared memory, the CTAs below
+  if (kpart == 0) {
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        // key 0 = no candidate (zero-norm or padding row, NaN or -inf similarity)
+        unsigned long long k1 = best[j][e] > -INFINITY ? route_key(best[j][e], best_k[j][e]) : 0ull;
+        unsigned long long k2 = (TOP2 && second[j][e] > -INFINITY) ? route_key(second[j][e], second_k[j][e]) : 0ull;
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+          const unsigned long long o1 = shfl_xor_u64(k1, o);
+          if (TOP2) merge_top2(k1, k2, o1, shfl_xor_u64(k2, o));
+          else k1 = o1 > k1 ? o1 : k1;
+        }
+        if (g == 0 && k1 != 0ull) {
+          // two-slot merge: whatever loses a comparison for the first slot is offered to the second
+          unsigned long long old = atomicMax(&s_keys[j * 8 + 2 * t + e], k1);
+          if (TOP2) {
+            old = old < k1 ? old : k1;
+            if (old != 0ull) atomicMax(&s_keys2[j * 8 + 2 * t + e], old);
+            if (k2 != 0ull) atomicMax(&s_keys2[j * 8 + 2 * t + e], k2);
+          }
+        }
+      }
   }
   cluster.sync();
   if (rank == 0) {
-    // one warp per query: lanes 0..kRcCluster-1 fetch the CTAs' keys, all lanes share the norm
-    for (int qi = warp; qi < kRcQ; qi += kRcWarps) {
-      if (q0 + qi >= Q) break;
-      unsigned long long key = 0ull;
-      if (lane < kRcCluster) key = *cluster.map_shared_rank(&s_keys[qi], lane);
-#pragma unroll
-      for (int o = 1; o < kRcCluster; o <<= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
-        key = other > key ? other : key;
+    // eight lanes per query fetch the CTAs' keys and share the norm
+    const int qi = tid >> 3, sub = tid & 7;
+    const bool on = qi < NQ && q0 + qi < Q;
+    unsigned long long k1 = 0ull, k2 = 0ull;
+    if (on) {
+      for (int r = sub; r < csize; r += 8) {
+        const unsigned long long o1 = *cluster.map_shared_rank(&s_keys[qi], r);
+        if (TOP2) merge_top2(k1, k2, o1, *cluster.map_shared_rank(&s_keys2[qi], r));
+        else k1 = o1 > k1 ? o1 : k1;
       }
-      key = __shfl_sync(0xffffffffu, key, 0);
-      const int id = (key == 0ull) ? 0 : (int)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
-      if (lane == 0) {
-        if (out_centroid) out_centroid[q0 + qi] = id;
-        out_expert[q0 + qi] = cmap ? cmap[id] : id;
-      }
-      if (out_best) {
-        float ss = 0.f;
-        for (int ch = lane; ch < nch; ch += 32) {
-          const uint4 v = *reinterpret_cast<const uint4*>(smem_raw + (size_t)qi * pitch + ch * 16);
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    }
+    float ss = 0.f;
+    if (on && parts == 1 && (out.best || out.margin))
+      for (int ch = sub; ch < nch; ch += 8) add_sq8(*reinterpret_cast<const uint4*>(smem_raw + (size_t)qi * pitch + ch * 16), ss);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            ss = fmaf(bf16_lo(w[e]), bf16_lo(w[e]), ss);
-            ss = fmaf(bf16_hi(w[e]), bf16_hi(w[e]), ss);
-          }
-        }
-        ss = warp_sum(ss);
-        if (lane == 0)
-          out_best[q0 + qi] = (key == 0ull) ? -INFINITY : key_to_float((uint32_t)(key >> 32)) * rsqrtf(ss);
+    for (int o = 1; o < 8; o <<= 1) {
+      const unsigned long long o1 = shfl_xor_u64(k1, o);
+      if (TOP2) merge_top2(k1, k2, o1, shfl_xor_u64(k2, o));
+      else k1 = o1 > k1 ? o1 : k1;
+      ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    }
+    if (on && sub == 0) {
+      if (parts > 1) {
+        part_keys[(size_t)part * Q + q0 + qi] = k1;
+        if (TOP2) part_keys[(size_t)(parts + part) * Q + q0 + qi] = k2;
+      } else {
+        route_write<TOP2>(out, cmap, q0 + qi, k1, k2, ss);
       }
     }
   }
   cluster.sync();  // the other CTAs' shared memory stays alive until CTA 0 has read it
 }
 
-bool route_cluster_supported(int Q, int K, int D) {
-  // few queries and at most two rounds of centroid tiles per cluster: beyond that the tensor-core GEMM wins
-  return Q >= 1 && Q <= 1024 && K >= 1 && K <= 16 * 2 * kRcCluster * kRcTileWarps && (D % 32) == 0 &&
-         (size_t)kRcQ * (D * 2 + 16) <= 200 * 1024;
+// The parts of a table meet: eight lanes per query.
+template <bool TOP2>
+__global__ void __launch_bounds__(128)
+route_parts_kernel(const unsigned long long* __restrict__ part_keys, int parts, const __nv_bfloat16* __restrict__ q,
+                   const int* __restrict__ cmap, int Q, int D, const RouteOut out) {
+  const int i = blockIdx.x * 16 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
+  const bool on = i < Q;
+  float ss = 0.f;
+  if (on && (out.best || out.margin))
+    for (int ch = sub; ch < D / 8; ch += 8) add_sq8(ldg_cached(q + (size_t)i * D + ch * 8), ss);
+  pdl_wait();   // the parts' keys
+  unsigned long long k1 = 0ull, k2 = 0ull;
+  if (on) {
+    for (int r = sub; r < parts; r += 8) {
+      const unsigned long long o1 = __ldcg(part_keys + (size_t)r * Q + i);
+      if (TOP2) merge_top2(k1, k2, o1, __ldcg(part_keys + (size_t)(parts + r) * Q + i));
+      else k1 = o1 > k1 ? o1 : k1;
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    const unsigned long long o1 = shfl_xor_u64(k1, o);
+    if (TOP2) merge_top2(k1, k2, o1, shfl_xor_u64(k2, o));
+    else k1 = o1 > k1 ? o1 : k1;
+    ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  }
+  if (on && sub == 0) route_write<TOP2>(out, cmap, i, k1, k2, ss);
+}
+
+// How a problem is cut: queries per cluster, CTAs per cluster, parts of the table; fast = the rule picks this kernel.
+struct RouteCut { int nq, csize, parts, groups; bool fast; };
+static RouteCut route_cut(int Q, int K, int D) {
+  RouteCut r = {0, 8, 1, 0, false};
+  if (Q < 1 || K < 1 || (D % 8) != 0 || 8 * route_pitch(D) > 200 * 1024) return r;
+  const int nq = r.nq = (Q > 8 && 32 * route_pitch(D) <= 200 * 1024) ? 32 : 8;
+  r.groups = (Q + nq - 1) / nq;
+  // One tile per warp pair of a cluster of 8 = 512 centroids per part, while all clusters are resident at once: a
+  // cluster of 8 one-per-SM CTAs needs 8 free SMs of one GPC, and 16 of them take two waves (500 centroids x 768,
+  // 256 queries = 8 clusters 9.8 us, 512 queries = 16 clusters 18.4 us).
+  constexpr int kResident = 12;
+  while (r.parts < kRouteMaxParts && K > 512 * r.parts && r.groups * (r.parts + 1) <= kResident) ++r.parts;
+  const int tiles = (K + 512 * r.parts - 1) / (512 * r.parts);   // tiles per warp pair
+  // Against the tensor-core GEMM with its clearing and finishing launches (12.4 us up to 128 queries, 14.4 at 256 x
+  // 5000 x 768): 7.3 us for up to 8 queries and 9.8-10.6 us for up to 32 per cluster with one tile per warp pair,
+  // 13.3 and 18.7 with two.
+  r.fast = r.groups * r.parts <= kResident && tiles <= (nq == 8 ? 2 : 1);
+  if (!tc_router_supported(Q, K, D)) r.fast = r.fast || r.groups <= 64;   // else only the CUDA-core kernel is left
+  return r;
+}
+bool route_cluster_supported(int Q, int K, int D) { return route_cut(Q, K, D).fast; }
+int route_parts(int Q, int K, int D) {
+  const RouteCut r = route_cut(Q, K, D);
+  return r.fast ? r.parts : 1;
+}
+// without scratch the table stays in one part
+static RouteCut route_cut_scratch(int Q, int K, int D, const unsigned long long* part_keys) {
+  RouteCut r = route_cut(Q, K, D);
+  if (part_keys == nullptr) r.parts = 1;
+  return r;
+}
+
+template <int NQ, bool TOP2>
+static cudaError_t launch_rc(int optin, const RouteCut& cut, const __nv_bfloat16* q, const __nv_bfloat16* c,
+                             const float* inv_norm, const int* cmap, int Q, int K, int D, const RouteOut& out,
+                             unsigned long long* part_keys, cudaStream_t stream) {
+  const size_t smem = (size_t)NQ * route_pitch(D);
+  cudaError_t ce = ensure_smem_optin(optin, route_cluster_kernel<NQ, TOP2>, smem > 64 * 1024 ? smem : 64 * 1024);
+  if (ce != cudaSuccess) return ce;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cut.csize;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(cut.groups * cut.parts * cut.csize));
+  cfg.blockDim = dim3(kRcWarps * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  ce = cudaLaunchKernelEx(&cfg, route_cluster_kernel<NQ, TOP2>, q, c, inv_norm, cmap, Q, K, D, cut.parts, part_keys, out);
+  if (ce != cudaSuccess || cut.parts == 1) return ce;
+  return launch_dependent(route_parts_kernel<TOP2>, (Q + 15) / 16, 128, stream, part_keys, cut.parts, q, cmap, Q, D, out);
 }
 
 cudaError_t launch_route_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                  const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
-                                 float* out_best, cudaStream_t stream) {
-  const size_t smem = (size_t)kRcQ * (D * 2 + 16);
-  cudaError_t ce = ensure_smem_optin(OPTIN_ROUTE_CLUSTER, route_cluster_kernel, smem);
-  if (ce != cudaSuccess) return ce;
-  const int groups = (Q + kRcQ - 1) / kRcQ;
-  route_cluster_kernel<<<groups * kRcCluster, kRcWarps * 32, smem, stream>>>(q, c, inv_norm, cmap, Q, K, D, out_expert,
-                                                                            out_centroid, out_best);
-  return cudaGetLastError();
+                                 float* out_best, unsigned long long* part_keys, cudaStream_t stream) {
+  const RouteOut out = {out_expert, out_centroid, nullptr, out_best, nullptr};
+  const RouteCut cut = route_cut_scratch(Q, K, D, part_keys);
+  if (cut.nq == 32) return launch_rc<32, false>(OPTIN_ROUTE_CLUSTER, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
+  return launch_rc<8, false>(OPTIN_ROUTE_CLUSTER + 1, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
+}
+cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
+                                      const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
+                                      int* out_second, float* out_best, float* out_margin,
+                                      unsigned long long* part_keys, cudaStream_t stream) {
+  const RouteOut out = {out_expert, out_centroid, out_second, out_best, out_margin};
+  const RouteCut cut = route_cut_scratch(Q, K, D, part_keys);
+  if (cut.nq == 32) return launch_rc<32, true>(OPTIN_ROUTE_CLUSTER + 2, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
+  return launch_rc<8, true>(OPTIN_ROUTE_CLUSTER + 3, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
 }
 
 // ----------------------------------------------------------------------------------------

@@ -145,3 +145,22 @@ def test_router_runner_up_and_margin(impl, Q, K, D):
     assert (np.abs(cos2 - (ref["best"] - ref["margin"])) <= tol).all()
     assert (out["second"] != out["centroid"]).all()
     assert moin.device_status()["timeout_flag"] == 0
+
+
+@pytest.mark.parametrize("Q,K,D", [(1, 5000, 768), (8, 5000, 216), (9, 1025, 40), (256, 1030, 384), (33, 513, 72),
+                                   (3, 9000, 8), (12, 600, 3200), (64, 5000, 64), (2, 8200, 64), (1024, 16, 768), (700, 3, 40)])
+def test_router_cluster_large_tables(Q, K, D):
+    # the cluster kernel beyond 512 centroids: the table in parts whose keys meet in a second launch (several tiles per
+    # warp once the parts run out), the 8-query variant (Q <= 8, or rows too long for 32 of them), embeddings that are
+    # no multiple of 32, with the runner-up
+    case = mi.planted_router(K=K, Q=Q, D=D, seed=70 + Q, unit_centroid_noise=True)
+    _, cid, best = _route(case)
+    ref = _oracle(case)
+    assert_router_matches(cid, ref)
+    np.testing.assert_allclose(best, ref["best"], atol=2e-3)
+    router = moin.Router(case.centroids.to(DEV))
+    out = {k: v.cpu().numpy() for k, v in moin.route_top2(router, case.queries.to(DEV)).items()}
+    assert_router_matches(out["centroid"], ref)
+    # fp32 sums of bf16 products: the margin is off by at most a few ulps of the two cosines
+    assert (np.abs(out["margin"] - ref["margin"]) <= 2e-5 + 2e-3 * np.abs(ref["margin"])).all()
+    assert (out["second"] != out["centroid"]).all() and (out["second"] >= 0).all()
