@@ -250,22 +250,25 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    {   // the whole warp walks the loop, one elected lane issues (as in the GEMMs)
+      const bool leader = elect_one();
       uint32_t kfph = 0, kpos = 0, vq = 0, sq = 0, pq = 0, nit = 0;   // kfph: per-stage phase bits of the "full" barriers
       bool ok = true;
       const uint64_t dq = at_sdesc(sQ);
       auto issue_s = [&]() -> bool {   // S[sq & 1] = Q K^T with the next K stage of the ring
         const uint32_t b = sq & 1u, bph = (sq >> 1) & 1u, s = kpos, ph = (kfph >> s) & 1u;
-        if (!mbar_wait(sfree + 8 * b, bph ^ 1u, abort_flag, p.status, 33)) return false;
-        if (!mbar_wait(kfull + 8 * s, ph, abort_flag, p.status, 34)) return false;
+        if (!mbar_wait_warp(sfree + 8 * b, bph ^ 1u, abort_flag, p.status, 33)) return false;
+        if (!mbar_wait_warp(kfull + 8 * s, ph, abort_flag, p.status, 34)) return false;
         kfph ^= 1u << s;
         kpos = (kpos + 1) % kAtKS;
         tc_fence_after();
         const uint64_t dk = at_sdesc(sK + s * kAtKV);
+        if (leader) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem + b * 64, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), kAtIdesc, k > 0 ? 1u : 0u);
-        tc_commit(kempty + 8 * s);
-        tc_commit(sready + 8 * b);
+          for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem + b * 64, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), kAtIdesc, k > 0 ? 1u : 0u);
+          tc_commit(kempty + 8 * s);
+          tc_commit(sready + 8 * b);
+        }
         ++sq;
         return true;
       };
@@ -274,36 +277,40 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         if (!it.on) continue;
         // the accumulator columns are free once the O of the item before has been read (all of its score reads
         // come earlier); then the rotated Q tile of this item
-        if (!(ok = mbar_wait(ofree, (nit & 1u) ^ 1u, abort_flag, p.status, 36))) break;
-        if (!(ok = mbar_wait(qready, nit & 1u, abort_flag, p.status, 35))) break;
+        if (!(ok = mbar_wait_warp(ofree, (nit & 1u) ^ 1u, abort_flag, p.status, 36))) break;
+        if (!(ok = mbar_wait_warp(qready, nit & 1u, abort_flag, p.status, 35))) break;
         tc_fence_after();
         auto issue_pv = [&](uint32_t o_col, bool first) -> bool {   // O (+)= P V with the next P buffer and V stage
           const uint32_t b = pq & 1u, bph = (pq >> 1) & 1u, s = vq % kAtVS, ph = (vq / kAtVS) & 1u;
-          if (!mbar_wait(pready + 8 * b, bph, abort_flag, p.status, 37)) return false;
-          if (!mbar_wait(vfull + 8 * s, ph, abort_flag, p.status, 38)) return false;
+          if (!mbar_wait_warp(pready + 8 * b, bph, abort_flag, p.status, 37)) return false;
+          if (!mbar_wait_warp(vfull + 8 * s, ph, abort_flag, p.status, 38)) return false;
           tc_fence_after();
           const uint64_t dp = at_sdesc(sP + b * kAtTile), dv = at_sdesc(sV + s * kAtKV);
+          if (leader) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            tc_mma_bf16(tmem + o_col, dp + (uint64_t)(2 * k), dv + kAtVStep * k, kAtIdescPV, (!first || k > 0) ? 1u : 0u);
-          tc_commit(vempty + 8 * s);
-          tc_commit(pfree + 8 * b);
+            for (int k = 0; k < 4; ++k)
+              tc_mma_bf16(tmem + o_col, dp + (uint64_t)(2 * k), dv + kAtVStep * k, kAtIdescPV, (!first || k > 0) ? 1u : 0u);
+            tc_commit(vempty + 8 * s);
+            tc_commit(pfree + 8 * b);
+          }
           ++pq; ++vq;
           return true;
         };
         if (it.n_tiles <= kAtResident) {
           // resident item: the scores against all of its keys in one product per 16 dims (the key tiles lie side
           // by side in stages 0 .. n - 1), one hand-over; then the second products as the P tiles arrive
-          if (!(ok = mbar_wait(kfull, kfph & 1u, abort_flag, p.status, 34))) break;
+          if (!(ok = mbar_wait_warp(kfull, kfph & 1u, abort_flag, p.status, 34))) break;
           kfph ^= 1u;
           kpos = 0;
           tc_fence_after();
           const uint64_t dk = at_sdesc(sK);
           const uint32_t idn = at_idesc_n(it.n_tiles);
+          if (leader) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), idn, k > 0 ? 1u : 0u);
-          for (int j = 0; j < it.n_tiles; ++j) tc_commit(kempty + 8 * j);
-          tc_commit(sall);
+            for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), idn, k > 0 ? 1u : 0u);
+            for (int j = 0; j < it.n_tiles; ++j) tc_commit(kempty + 8 * j);
+            tc_commit(sall);
+          }
           for (int j = 0; j < it.n_tiles && ok; ++j) ok = issue_pv(0, j == 0);
         } else {
           // streaming item, pass 1: scores only (the softmax warps take the row maxima)
@@ -316,7 +323,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             ok = issue_pv(128, j == 0);
           }
         }
-        if (ok) tc_commit(oready);
+        if (ok && leader) tc_commit(oready);
         ++nit;
       }
     }

@@ -55,6 +55,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return true;
 }
 
+// One lane of a converged warp (the same one every time).  Code that issues MMAs or copies stays warp-uniform and
+// predicates only the issue with this.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+// mbar_wait by a whole warp: the answer is the same for every lane, and the warp is converged afterwards.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, DeviceStatus* st,
+                                               int site) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, st, site));
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
