@@ -250,8 +250,8 @@ static moin_status route_launch(HostState* hs, int choice, const moin_router* ro
     moin_status st;
     {
       ProfScope prof(MOIN_K_ROUTE_TC, 1, s);
-      st = launch_tc_router(hs, (const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
-                            router->inv_norm, Q, K, D, keys, s);
+      st = launch_pair_router(hs, (const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
+                              router->inv_norm, Q, K, D, keys, s);
     }
     if (st) return st;
     ProfScope prof(MOIN_K_ROUTE_FINISH, 1, s);
@@ -346,8 +346,8 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
   if (e != cudaSuccess) return record_cuda(e);
   {
     ProfScope prof(MOIN_K_ROUTE_TC, 1, s);
-    st = launch_tc_router(hs, (const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids, router->inv_norm,
-                          Q, K, D, keys, s, keys2);
+    st = launch_pair_router(hs, (const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids, router->inv_norm,
+                            Q, K, D, keys, s, keys2);
   }
   if (st) return st;
   ProfScope prof(MOIN_K_ROUTE_FINISH, 1, s);
@@ -587,10 +587,18 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
         if ((st = launch_tc_shrink_group(hs, pv, gp, gx, gh, n, scale, s))) return st;
         j0 += n;
       }
-      for (int j = 0; j < n_jobs; ++j) {
-        st = launch_tc_fused(hs, pv, jobs[j].pool, (const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W,
-                             (__nv_bfloat16*)jobs[j].y, reinterpret_cast<__nv_bfloat16*>(ws_job[j]), s);
-        if (st) return st;
+      for (int j0 = 0; j0 < n_jobs;) {   // projections of one reduction length and rank: one launch
+        PairJob pj[kPairJobs];
+        int n = 0;
+        while (j0 + n < n_jobs && n < kPairJobs && d_in[j0 + n] == d_in[j0] && r[j0 + n] == r[j0]) {
+          const moin_lora_job& g = jobs[j0 + n];
+          pj[n] = {(const __nv_bfloat16*)g.x, (const __nv_bfloat16*)g.W, reinterpret_cast<__nv_bfloat16*>(ws_job[j0 + n]),
+                   (__nv_bfloat16*)g.y, g.pool, d_out[j0 + n]};
+          ++n;
+        }
+        ProfScope prof(MOIN_K_FUSED_TC, 1, s);
+        if ((st = launch_pair_gemm(hs, &pv, pj, n, T, d_in[j0], s))) return st;
+        j0 += n;
       }
       return MOIN_OK;
     }
@@ -681,6 +689,10 @@ moin_status moin_lora_linear(const moin_plan* plan, const void* x, const void* W
   if ((st = pick_gemm(hs, T, d_in, d_out, &use_tc))) return st;
   cudaStream_t s = (cudaStream_t)stream;
   ProfScope prof(use_tc ? MOIN_K_GEMM_TC : MOIN_K_GEMM_WARP, 1, s);
+  if (use_tc && T >= 512) {   // (fewer rows: too few pairs of row tiles)
+    const PairJob job = {(const __nv_bfloat16*)x, (const __nv_bfloat16*)W, nullptr, (__nv_bfloat16*)y, nullptr, d_out};
+    return launch_pair_gemm(hs, nullptr, &job, 1, T, d_in, s);
+  }
   if (use_tc) return launch_tc_gemm(hs, (const __nv_bfloat16*)x, (const __nv_bfloat16*)W, (__nv_bfloat16*)y, nullptr, T, d_in, d_out, s);
   return record_cuda(launch_gemm_warp((const __nv_bfloat16*)x, (const __nv_bfloat16*)W, (__nv_bfloat16*)y, nullptr, T, d_in, d_out, s));
 }

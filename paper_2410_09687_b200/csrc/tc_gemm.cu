@@ -9,16 +9,11 @@
 //   warps 2-9  epilogue, two warps per TMEM lane quarter (half of the tile's columns each): tcgen05.ld of the
 //              accumulator (TMEM lane = tile row), then one of
 //              EPI_STORE   y = bf16(acc) (+ optional fp32 copy)
-//              EPI_ROUTER  running (max, argmax) of acc * inv_norm[col], merged across tiles with a
-//                          64-bit atomicMax on (orderable(sim) << 32 | ~col): order independent,
-//                          lowest index wins ties
 //              EPI_SHRINK  scale * acc for the LoRA rank columns, stored as bf16 hi + lo parts
 // Two accumulator buffers in TMEM let the epilogue of tile i overlap the MMAs of tile i+1.
 //
-// Row tiles come either from a regular grid over M or from a batch plan (runs of tokens with
-// one expert, <= 128 rows).  With a plan, EPI_STORE appends two extra K blocks per tile taken
-// from hi/lo[rows, r] and B_e[d_out, r] of the tile's adapter: y = [x | hi(s h) | lo(s h)] [W ; B_e ; B_e]^T,
-// so the low-rank term is added inside the accumulator (to ~fp32 accuracy) and y is written once.
+// Row tiles come either from a regular grid over M or from a batch plan (EPI_SHRINK: runs of tokens with one expert,
+// <= 128 rows).  The long-run GEMMs and the router run on CTA pairs (tc_pair.cu).
 // Every wait on an mbarrier is bounded; on expiry the kernel raises the status flag and returns.
 #include <cuda.h>
 
@@ -31,7 +26,7 @@ constexpr int kBM = 128, kBK = 64;
 constexpr int kTcThreads = 320;      // producer warp, MMA warp, eight epilogue warps
 constexpr int kTcThreadsLean = 192;  // four epilogue warps and no output staging: the launch that runs beside the
                                      // adapter streams at decode size and should leave them registers and shared memory
-enum { EPI_STORE = 0, EPI_ROUTER = 1, EPI_SHRINK = 2, EPI_ROUTER2 = 3 };   // ROUTER2: best and runner-up
+enum { EPI_STORE = 0, EPI_SHRINK = 1 };
 
 constexpr int kMaxShrinkJobs = 3;
 struct TcParams {
@@ -42,8 +37,7 @@ struct TcParams {
   const int* tile_rows;
   const int* tile_expert;
   const int* slot_of_expert;
-  int tail_r;                  // EPI_STORE with plan: LoRA rank of the appended K block (0 = none)
-  int rows_per_slot;           // rows of the B-side pool tensor per adapter slot (d_out, or r for EPI_SHRINK)
+  int rows_per_slot;           // EPI_SHRINK: rows of the B-side pool tensor per adapter slot (r)
   int b_box_rows;              // rows of the B-side TMA box when it is shorter than the tile's BN (0 = BN); the
                                // rest of the stage's B region keeps stale bytes, whose columns nobody stores
   __nv_bfloat16* y;            // EPI_STORE / EPI_SHRINK output, leading dimension ldy
@@ -66,11 +60,7 @@ struct TcParams {
   __nv_bfloat16* ys_lo[3];
   // per-slot adapter rank (nullable: the stored rank) and the function applied to x A^T (MOIN_ACT_*):
   const int* rank_tabs[3];     // EPI_SHRINK: table of job j (n_jobs = 0: rank_tabs[0])
-  const int* slot_rank;        // EPI_STORE with plan: table of the projection's pool
   int act;                     // EPI_SHRINK
-  const float* inv_norm;       // EPI_ROUTER
-  unsigned long long* keys;    // EPI_ROUTER / EPI_ROUTER2: best (similarity, index) key per row
-  unsigned long long* keys2;   // EPI_ROUTER2: runner-up key per row
   DeviceStatus* status;
 };
 
@@ -89,11 +79,6 @@ __device__ __forceinline__ uint64_t make_sdesc(uint32_t saddr) {
 // Instruction descriptor: D fp32, A/B bf16, both K-major, M = 128, N = BN.
 __host__ __device__ constexpr uint32_t make_idesc(int bn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-}
-
-__device__ __forceinline__ uint32_t orderable(float f) {
-  const uint32_t u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
 template <int BN> struct TcCfg {
@@ -153,7 +138,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int nkb_main = (p.K + kBK - 1) / kBK;
 
   int job = 0;   // projection of the current tile (EPI_SHRINK with several jobs), set by tile_info
-  int r_use = (EPI == EPI_SHRINK) ? p.N : p.tail_r;   // rank of the current tile's adapter, set by tile_info
+  int r_use = p.N;   // EPI_SHRINK: rank of the current tile's adapter, set by tile_info
   const bool stacked = (EPI == EPI_SHRINK) && p.n_stack > 1;
   int st_slot[kMaxShrinkJobs] = {-1, -1, -1}, st_ruse[kMaxShrinkJobs] = {0, 0, 0};   // stacked: per projection
   auto tile_info = [&](int tile, int& row0, int& rows, int& n0, int& slot) {
@@ -178,11 +163,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           st_ruse[j] = (st_slot[j] >= 0 && p.rank_tabs[j]) ? min(p.rank_tabs[j][st_slot[j]], p.stack_r) : p.stack_r;
         }
         slot = st_slot[0];
-      } else if (EPI == EPI_SHRINK || EPI == EPI_STORE) {
-        const int r_full = (EPI == EPI_SHRINK) ? p.N : p.tail_r;
-        const int* rt = (EPI == EPI_STORE) ? p.slot_rank
-                                           : (job == 0 ? p.rank_tabs[0] : job == 1 ? p.rank_tabs[1] : p.rank_tabs[2]);
-        r_use = (slot >= 0 && rt) ? min(rt[slot], r_full) : r_full;
+      } else {
+        const int* rt = job == 0 ? p.rank_tabs[0] : job == 1 ? p.rank_tabs[1] : p.rank_tabs[2];
+        r_use = (slot >= 0 && rt) ? min(rt[slot], p.N) : p.N;
       }
     } else {
       row0 = tm * kBM;
@@ -198,16 +181,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
         int row0, rows, n0, slot;
         tile_info(tile, row0, rows, n0, slot);
-        const bool tail = (EPI == EPI_STORE) && planned && p.tail_r > 0 && slot >= 0;
-        const int nrb = (p.tail_r + kBK - 1) / kBK;   // 64-wide blocks of the rank
-        const int nkb = nkb_main + (tail ? 2 * nrb : 0);   // tail: [hi(s h) | lo(s h)] x [B_e ; B_e], nrb blocks each
         const int brow = (EPI == EPI_SHRINK) ? (slot >= 0 ? slot : 0) * p.rows_per_slot : n0;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = 0; kb < nkb_main; ++kb, ++it) {
           const uint32_t s = it % S, ph = (it / S) & 1u;
           if (!(ok = mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 1))) break;
           const uint32_t sa = tiles_base + s * Cfg::kStageBytes, sb = sa + kBM * kBK * 2;
           const uint32_t b_rows = stacked ? (uint32_t)(p.n_stack * p.stack_r)
-                                          : (kb < nkb_main && p.b_box_rows > 0) ? (uint32_t)p.b_box_rows : (uint32_t)BN;
+                                          : p.b_box_rows > 0 ? (uint32_t)p.b_box_rows : (uint32_t)BN;
           mbar_expect_tx(full0 + 8 * s, (kBM + b_rows) * kBK * 2);
           if (stacked) {
             tma_load_2d(sa, &tmA, full0 + 8 * s, kb * kBK, row0);
@@ -216,7 +196,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               if (j < p.n_stack)   // (a projection without this adapter loads slot 0: its columns are not stored)
                 tma_load_2d(sb + (uint32_t)(j * p.stack_r) * kBK * 2, j == 0 ? &tmB : j == 1 ? &tmB2 : &tmB3, full0 + 8 * s,
                             kb * kBK, (st_slot[j] >= 0 ? st_slot[j] : 0) * p.stack_r);
-          } else if (kb < nkb_main) {
+          } else {
             const CUtensorMap* ma = &tmA;
             const CUtensorMap* mb = &tmB;
             if (EPI == EPI_SHRINK && job > 0) {
@@ -225,10 +205,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
             tma_load_2d(sa, ma, full0 + 8 * s, kb * kBK, row0);
             tma_load_2d(sb, mb, full0 + 8 * s, kb * kBK, brow);
-          } else {
-            const int j = kb - nkb_main, rb = (j >= nrb) ? j - nrb : j;   // hi blocks first, then lo blocks
-            tma_load_2d(sa, j < nrb ? &tmA2 : &tmA3, full0 + 8 * s, rb * kBK, row0);
-            tma_load_2d(sb, &tmB2, full0 + 8 * s, rb * kBK, slot * p.rows_per_slot + n0);
           }
         }
       }
@@ -243,26 +219,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t it = 0, lt = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, ++lt) {
-      int row0, rows, n0, slot;
-      tile_info(tile, row0, rows, n0, slot);
-      const bool tail = (EPI == EPI_STORE) && planned && p.tail_r > 0 && slot >= 0;
-      const int nrb = (p.tail_r + kBK - 1) / kBK;
-      const int nkb = nkb_main + (tail ? 2 * nrb : 0);
       const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
       if (!(ok = mbar_wait_warp(tempty0 + 8 * acc, aph ^ 1u, abort_flag, p.status, 2))) break;
       tc_fence_after();
       const uint32_t tmem_d = tmem_base + acc * BN;
-      for (int kb = 0; kb < nkb; ++kb, ++it) {
+      for (int kb = 0; kb < nkb_main; ++kb, ++it) {
         const uint32_t s = it % S, ph = (it / S) & 1u;
         if (!(ok = mbar_wait_warp(full0 + 8 * s, ph, abort_flag, p.status, 3))) break;
         tc_fence_after();
         const uint32_t sa = tiles_base + s * Cfg::kStageBytes, sb = sa + kBM * kBK * 2;
         const uint64_t da = make_sdesc(sa), db = make_sdesc(sb);
-        int nk16 = (min(kBK, p.K - kb * kBK) + 15) / 16;
-        if (kb >= nkb_main) {
-          const int j = kb - nkb_main, rb = (j >= nrb) ? j - nrb : j;
-          nk16 = (min(kBK, r_use - rb * kBK) + 15) / 16;   // columns beyond the adapter's rank: no MMA (<= 0 steps)
-        }
+        const int nk16 = (min(kBK, p.K - kb * kBK) + 15) / 16;
         if (leader) {
           if (nk16 == 4) {
 #pragma unroll
@@ -296,10 +263,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tc_fence_after();
       const bool row_ok = trow < rows;
       const size_t grow = (size_t)(row0 + trow);
-      float best = -INFINITY;
-      int best_k = 0;
-      float second = -INFINITY;   // EPI_ROUTER2: runner-up of this tile's columns
-      int second_k = 0;
       const int ncols = (EPI == EPI_SHRINK) ? min(BN, (p.N + 31) / 32 * 32) : BN;
       // Plain store of a warp's 32 rows when all of them belong to the tile: 64 columns at a time are laid down in
       // shared memory (128-byte swizzled rows) and leave as one tiled store of whole 128-byte lines.  Written
@@ -345,27 +308,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         uint32_t v[32];
         tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + c, v);
         tmem_ld_wait();
-        if (EPI == EPI_ROUTER || EPI == EPI_ROUTER2) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int k = n0 + c + j;
-            if (k < p.N) {
-              const float inv = __ldg(p.inv_norm + k);
-              const float sim = __uint_as_float(v[j]) * inv;
-              if (inv > 0.f && sim > best) {
-                if (EPI == EPI_ROUTER2) {
-                  second = best;
-                  second_k = best_k;
-                }
-                best = sim;
-                best_k = k;
-              } else if (EPI == EPI_ROUTER2 && inv > 0.f && sim > second) {
-                second = sim;
-                second_k = k;
-              }
-            }
-          }
-        } else if (row_ok && (EPI == EPI_STORE || stacked || slot >= 0)) {
+        if (row_ok && (EPI == EPI_STORE || stacked || slot >= 0)) {
           const float sc = (EPI == EPI_SHRINK) ? p.scale : 1.f;
           __nv_bfloat16* ybase = p.y;
           __nv_bfloat16* ylo_base = p.y_lo;
@@ -421,28 +364,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       tc_fence_before();
       mbar_arrive(tempty0 + 8 * acc);
-      if (EPI == EPI_ROUTER && row_ok && best > -INFINITY) {
-        const unsigned long long key = ((unsigned long long)orderable(best) << 32) |
-                                       (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k);
-        atomicMax(p.keys + grow, key);
-      }
-      if (EPI == EPI_ROUTER2 && row_ok) {
-        // Two-slot merge: the max goes to keys; whatever loses a comparison there (the value it displaced, or
-        // the candidate itself) is offered to keys2.  Every candidate but the overall best is a loser exactly
-        // once, keys are distinct (they carry the index), and both slots are maxima: order independent.
-        const float cand[2] = {best, second};
-        const int cand_k[2] = {best_k, second_k};
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          if (cand[i] > -INFINITY) {
-            const unsigned long long key = ((unsigned long long)orderable(cand[i]) << 32) |
-                                           (unsigned long long)(0xFFFFFFFFu - (uint32_t)cand_k[i]);
-            const unsigned long long old = atomicMax(p.keys + grow, key);
-            const unsigned long long loser = old < key ? old : key;
-            if (loser != 0ull) atomicMax(p.keys2 + grow, loser);
-          }
-        }
-      }
     }
   }
   // ------------------------------------------------------------------ teardown
@@ -501,7 +422,7 @@ static moin_status launch_cfg(HostState* hs, const CUtensorMap& a, const CUtenso
                               cudaStream_t stream, const CUtensorMap* b3 = nullptr, const CUtensorMap* ymap = nullptr,
                               bool lean = false) {
   using Cfg = TcCfg<BN>;
-  constexpr int slot = OPTIN_TC_GEMM + 4 * (BN == 256 ? 2 : BN == 128 ? 1 : 0) + EPI;
+  constexpr int slot = OPTIN_TC_GEMM + 2 * (BN == 256 ? 2 : BN == 128 ? 1 : 0) + EPI;
   cudaError_t e = ensure_smem_optin(slot, tc_gemm_kernel<BN, EPI>, Cfg::kSmemBytes);
   if (e != cudaSuccess) return record_cuda(e);
   long grid = max_tiles < hs->n_sms ? max_tiles : hs->n_sms;
@@ -571,28 +492,6 @@ moin_status launch_tc_gemm(HostState* hs, const __nv_bfloat16* x, const __nv_bfl
   return launch_cfg<64, EPI_STORE>(hs, a, b, a, a, b, p, tiles, stream, nullptr, &ym, lean);
 }
 
-moin_status launch_tc_router(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
-                             int Q, int K, int D, unsigned long long* keys, cudaStream_t stream,
-                             unsigned long long* keys2) {
-  const long tiles_m = (Q + kBM - 1) / kBM;
-  const int bn = pick_bn(tiles_m, K, hs->n_sms);
-  CUtensorMap a, b;
-  moin_status st = make_map(&a, q, Q, D, kBM);
-  if (!st) st = make_map(&b, c, K, D, bn);
-  if (st) return st;
-  TcParams p = {};
-  p.M = Q; p.N = K; p.K = D; p.inv_norm = inv_norm; p.keys = keys; p.keys2 = keys2; p.status = hs->status;
-  const long tiles = tiles_m * ((K + bn - 1) / bn);
-  if (keys2 != nullptr) {
-    if (bn == 256) return launch_cfg<256, EPI_ROUTER2>(hs, a, b, a, a, b, p, tiles, stream);
-    if (bn == 128) return launch_cfg<128, EPI_ROUTER2>(hs, a, b, a, a, b, p, tiles, stream);
-    return launch_cfg<64, EPI_ROUTER2>(hs, a, b, a, a, b, p, tiles, stream);
-  }
-  if (bn == 256) return launch_cfg<256, EPI_ROUTER>(hs, a, b, a, a, b, p, tiles, stream);
-  if (bn == 128) return launch_cfg<128, EPI_ROUTER>(hs, a, b, a, a, b, p, tiles, stream);
-  return launch_cfg<64, EPI_ROUTER>(hs, a, b, a, a, b, p, tiles, stream);
-}
-
 // Long-run mode, step 1 for up to kMaxShrinkJobs projections that share the plan, d_in and the rank:
 // hb_j[row, :r] = hi/lo bf16 parts of scale * x_j A_j,e^T in ONE launch (row tiles of all the projections in
 // one persistent grid, so set-up, first round trip and tail are paid once).
@@ -641,36 +540,6 @@ moin_status launch_tc_shrink_group(HostState* hs, const PlanView& pv, const moin
   // the grid is capped at the SM count and the kernel reads the true count
   if (r > 64) return launch_cfg<128, EPI_SHRINK>(hs, ax[0], bA[0], ax[1], ax[2], bA[1], p, (long)T * n_jobs, stream, &bA[2]);
   return launch_cfg<64, EPI_SHRINK>(hs, ax[0], bA[0], ax[1], ax[2], bA[1], p, (long)T * n_jobs, stream, &bA[2]);
-}
-
-// Long-run mode, step 2: y = [x | hi | lo] [W ; B_e ; B_e]^T with hb from step 1.
-moin_status launch_tc_fused(HostState* hs, const PlanView& pv, const moin_pool* pool, const __nv_bfloat16* x,
-                            const __nv_bfloat16* W, __nv_bfloat16* y, __nv_bfloat16* hb, cudaStream_t stream) {
-  const int T = pv.T, d_in = pool->d_in, d_out = pool->d_out, r = pool->r;
-  const long max_tiles_m = T;
-  CUtensorMap ax, bW, ah, al, bB;
-  __nv_bfloat16* hb_lo = hb + (size_t)T * r;
-  ProfScope prof(MOIN_K_FUSED_TC, 1, stream);
-  const long full_tiles_m = (T + kBM - 1) / kBM;
-  const int bn = pick_bn(full_tiles_m, d_out, hs->n_sms);
-  moin_status st = make_map(&ax, x, T, d_in, kBM);
-  if (!st) st = make_map(&ah, hb, T, r, kBM);
-  if (!st) st = make_map(&al, hb_lo, T, r, kBM);
-  if (!st) st = make_map(&bW, W, d_out, d_in, bn);
-  if (!st) st = make_map(&bB, pool->B, (uint64_t)pool->n_slots * d_out, r, bn);
-  CUtensorMap ym;
-  if (!st) st = make_map(&ym, y, T, d_out, 32);
-  if (st) return st;
-  TcParams p = {};
-  p.M = T; p.N = d_out; p.K = d_in; p.header = pv.header; p.tile_row0 = pv.tile_row0; p.tile_rows = pv.tile_rows;
-  p.tile_expert = pv.tile_expert; p.slot_of_expert = pool->slot_of_expert; p.tail_r = r; p.rows_per_slot = d_out;
-  p.slot_rank = pool->slot_rank;
-  p.y = y; p.ldy = d_out; p.scale = 1.f; p.status = hs->status;
-  p.tma_store = 1;
-  const long tiles = max_tiles_m * ((d_out + bn - 1) / bn);
-  if (bn == 256) return launch_cfg<256, EPI_STORE>(hs, ax, bW, ah, al, bB, p, tiles, stream, nullptr, &ym);
-  if (bn == 128) return launch_cfg<128, EPI_STORE>(hs, ax, bW, ah, al, bB, p, tiles, stream, nullptr, &ym);
-  return launch_cfg<64, EPI_STORE>(hs, ax, bW, ah, al, bB, p, tiles, stream, nullptr, &ym);
 }
 
 }  // namespace moin

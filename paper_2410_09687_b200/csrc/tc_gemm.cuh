@@ -19,18 +19,21 @@ bool tc_fused_supported(int r);
 // `cta_budget` > 0: widen the tiles until the launch has at most that many CTAs (when it runs beside other kernels).
 moin_status launch_tc_gemm(HostState* hs, const __nv_bfloat16* x, const __nv_bfloat16* W, __nv_bfloat16* y, float* y0,
                            int T, int d_in, int d_out, cudaStream_t stream, int cta_budget = 0);
+// Long-run GEMMs on CTA pairs (tc_pair.cu): y_j = x_j W_j^T for up to kPairJobs projections of one K; with a plan the
+// low-rank term s x A_e^T B_e^T is added from hb (hi / lo parts of s x A_e^T, [2][M][r], all jobs of the same r).
+constexpr int kPairJobs = 3;
+struct PairJob { const __nv_bfloat16 *x, *W, *hb; __nv_bfloat16* y; const moin_pool* pool; int N; };
+moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* jobs, int n_jobs, int M, int K,
+                             cudaStream_t stream);
 // keys[i] = max over k of (orderable(<q_i,c_k> * inv_norm[k]) << 32 | (0xFFFFFFFF - k)), merged with atomicMax.
-moin_status launch_tc_router(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
-                             int Q, int K, int D, unsigned long long* keys, cudaStream_t stream,
-                             unsigned long long* keys2 = nullptr);   // keys2 != nullptr: also the runner-up
-// Tile mode: hb = hi/lo bf16 parts of s * x A_e^T per row tile ([2][T][r]), then y = [x | hi | lo] [W ; B_e ; B_e]^T
-// in one GEMM.
+moin_status launch_pair_router(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm, int Q,
+                               int K, int D, unsigned long long* keys, cudaStream_t stream,
+                               unsigned long long* keys2 = nullptr);   // keys2 != nullptr: also the runner-up
+// Tile mode: hb = hi/lo bf16 parts of s * x A_e^T per row tile ([2][T][r]); launch_pair_gemm adds hb B_e^T.
 moin_status launch_tc_shrink_group(HostState* hs, const PlanView& pv, const moin_pool* const* pools,
                                    const __nv_bfloat16* const* xs, __nv_bfloat16* const* hbs, int n_jobs, float scale,
                                    cudaStream_t stream);
 constexpr int kTcMaxShrinkJobs = 3;   // projections one grouped shrink launch can take
-moin_status launch_tc_fused(HostState* hs, const PlanView& pv, const moin_pool* pool, const __nv_bfloat16* x,
-                            const __nv_bfloat16* W, __nv_bfloat16* y, __nv_bfloat16* hb, cudaStream_t stream);
 
 // Causal GQA attention on tcgen05 (attention_tc.cu).  q not rotated, k rotated.
 bool attention_tc_supported(int n_heads, int n_kv_heads, int head_dim);

@@ -1,0 +1,507 @@
+// Long-run GEMMs on CTA pairs: tcgen05 with cta_group::2, sm_100a.
+//
+// Two CTAs on neighbouring SMs work on one [256 x BN] tile of  A[M,K] B[N,K]^T : each holds 128 rows of A, HALF of the
+// B rows and 128 rows of the accumulator, and the first CTA issues the MMAs for both.  Why pairs: an SM receives about
+// 64 bytes per clock from L2.  A single-CTA 128 x 256 tile needs 48 KB per 64-wide k-block (96 bytes per clock at the
+// tensor rate, so two thirds of it at best); in a pair the same MMA work needs 32 KB per SM, which the fill rate covers.
+//
+// Roles per CTA: warp 0 TMA producer (its own A rows and its half of B; completion of both CTAs' copies is counted on
+// the FIRST CTA's barrier), warp 1 TMEM allocation and - first CTA only - MMA issue, warps 2-9 epilogue of the CTA's
+// own 128 rows.  A commit arrives on both CTAs' barriers (stage free, accumulator ready); both epilogues release an
+// accumulator on the first CTA's barrier.  Two accumulators in TMEM: the epilogue of tile i overlaps the MMAs of i + 1.
+//
+// Row tiles come from a regular grid or from a batch plan (runs of one expert, at most 128 rows); the pair takes plan
+// tiles 2i and 2i + 1.  With a plan every tile ends with extra K blocks [hi(s h) | lo(s h)] x [B_e ; B_e] that add the
+// low-rank term inside the accumulator.  Both halves of a pair multiply the same B rows, so where the two row tiles
+// have different experts the blocks run once per expert, the other CTA's rows being zero (a copy that starts past the
+// last row fills zeros).
+//
+// A launch covers up to kPairJobs projections that share the plan and the reduction length (the column tiles of all of
+// them side by side under one row tile, so an x they share comes from L2): one ramp and one partial last wave per group.
+// Every wait on an mbarrier is bounded; on expiry the kernel raises the status flag and returns.
+#include <cuda.h>
+
+#include "tc_gemm.cuh"
+#include "ptx.cuh"
+
+namespace moin {
+
+constexpr int kPairThreads = 320, kPairM = 128, kPairK = 64;
+enum { PAIR_STORE = 0, PAIR_ROUTER = 1, PAIR_ROUTER2 = 2 };
+
+struct PairMaps { CUtensorMap x[kPairJobs], w[kPairJobs], b[kPairJobs], hi[kPairJobs], lo[kPairJobs], y[kPairJobs]; };
+struct PairParams {
+  int M, K, n_jobs, bn;                  // bn: tile width, a multiple of 16 up to 256
+  int N[kPairJobs], tn_end[kPairJobs];   // columns, column tiles of jobs 0 .. j
+  const int *header, *tile_row0, *tile_rows, *tile_expert;   // plan (header == nullptr: regular grid over M)
+  int tail_r;                            // stored rank of the appended low-rank blocks (0 = none)
+  const int* slot_of_expert[kPairJobs];
+  const int* slot_rank[kPairJobs];       // nullable: the stored rank
+  __nv_bfloat16* y[kPairJobs];
+  const float* inv_norm;                 // PAIR_ROUTER*
+  unsigned long long *keys, *keys2;
+  DeviceStatus* status;
+};
+
+constexpr int kPairMaxN = 256, kPairStageBytes = (kPairM + kPairMaxN / 2) * kPairK * 2, kPairStages = 6;
+constexpr int kPairOutBytes = 8 * 32 * 128;   // epilogue staging: [32 rows x 64 columns] bf16 per warp
+constexpr size_t kPairSmem = (size_t)kPairStages * kPairStageBytes + 1024 /*align*/ + 1024 /*barriers*/ + kPairOutBytes;
+
+__device__ __forceinline__ uint32_t pair_orderable(float f) {
+  const uint32_t u = __float_as_uint(f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+// What a tile is: its job, first column, and for both CTAs of the pair the row tile and the adapter slot.
+struct PairTile { int job, n0, row0[2], rows[2], slot[2], rank[2]; };
+
+__device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int tiles_m) {
+  PairTile t;
+  const int tn_all = p.tn_end[p.n_jobs - 1];
+  const int pm = tile / tn_all;
+  int tn = tile - pm * tn_all;
+  t.job = 0;
+#pragma unroll
+  for (int j = 0; j + 1 < kPairJobs; ++j)
+    if (j + 1 < p.n_jobs && tn >= p.tn_end[j]) t.job = j + 1;
+  int first = 0;
+  const int* slots = p.slot_of_expert[0];
+  const int* ranks = p.slot_rank[0];
+#pragma unroll
+  for (int j = 1; j < kPairJobs; ++j)
+    if (t.job == j) { first = p.tn_end[j - 1]; slots = p.slot_of_expert[j]; ranks = p.slot_rank[j]; }
+  t.n0 = (tn - first) * p.bn;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int tm = 2 * pm + c;
+    t.slot[c] = -1;
+    t.rank[c] = 0;
+    t.row0[c] = p.M;      // no such row tile: the copy fills zeros, nothing is stored
+    t.rows[c] = 0;
+    if (tm < tiles_m) {
+      if (p.header != nullptr) {
+        t.row0[c] = __ldg(p.tile_row0 + tm);
+        t.rows[c] = __ldg(p.tile_rows + tm);
+        const int e = __ldg(p.tile_expert + tm);
+        if (e >= 0 && p.tail_r > 0) t.slot[c] = __ldg(slots + e);
+        if (t.slot[c] >= 0) t.rank[c] = ranks ? min(__ldg(ranks + t.slot[c]), p.tail_r) : p.tail_r;
+      } else {
+        t.row0[c] = tm * kPairM;
+        t.rows[c] = min(kPairM, p.M - t.row0[c]);
+      }
+    }
+  }
+  return t;
+}
+// Low-rank passes of a tile: pass 0 multiplies the adapter of the first CTA's rows (and of the second's where it is
+// the same one), pass 1 the second's where it differs.  live: bit c = CTA c's rows take part.
+struct PairPasses { int n, slot[2], rank[2]; uint32_t live[2]; };
+__device__ __forceinline__ PairPasses pair_passes(const PairTile& t) {
+  PairPasses q;
+  q.n = 0;
+  q.slot[0] = q.slot[1] = -1; q.rank[0] = q.rank[1] = 0; q.live[0] = q.live[1] = 0u;
+  if (t.slot[0] >= 0) {
+    q.slot[0] = t.slot[0]; q.rank[0] = t.rank[0];
+    q.live[0] = (t.slot[1] == t.slot[0]) ? 3u : 1u;
+    q.n = 1;
+  }
+  if (t.slot[1] >= 0 && t.slot[1] != t.slot[0]) {
+    if (q.n == 0) { q.slot[0] = t.slot[1]; q.rank[0] = t.rank[1]; q.live[0] = 2u; }
+    else { q.slot[1] = t.slot[1]; q.rank[1] = t.rank[1]; q.live[1] = 2u; }
+    ++q.n;
+  }
+  return q;
+}
+
+template <int EPI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
+  constexpr int S = kPairStages;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t ring = (raw + 1023u) & ~1023u;
+  const uint32_t out0 = ring + (uint32_t)S * kPairStageBytes;   // 1024-byte aligned: the swizzle is a function of the address
+  const uint32_t bars = out0 + kPairOutBytes;
+  uint8_t* bar_ptr = smem_raw + (bars - raw);
+  const uint32_t full0 = bars, empty0 = bars + 8 * S, tfull0 = bars + 16 * S, tempty0 = tfull0 + 16;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + 16 * S + 32);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 16 * S + 40);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full0 + 8 * s, 1);     // used in the first CTA: its producer's arrival plus both CTAs' bytes
+      mbar_init(empty0 + 8 * s, 1);    // each CTA's own, by commit
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(tfull0 + 8 * a, 1);    // each CTA's own, by commit
+      mbar_init(tempty0 + 8 * a, 16);  // used in the first CTA: one arrival per epilogue warp of the pair
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(tmem_slot), 512);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_arrive();   // the other CTA's barriers exist before anything is signalled there
+  cluster_wait();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  const int tiles_m = p.header != nullptr ? p.header[PH_NTILES] : (p.M + kPairM - 1) / kPairM;
+  const int total = (tiles_m + 1) / 2 * p.tn_end[p.n_jobs - 1];
+  const int nkb_main = (p.K + kPairK - 1) / kPairK;
+  const int nrb = (p.tail_r + kPairK - 1) / kPairK;   // 64-wide blocks of the rank
+  const int pair = (int)blockIdx.x >> 1, n_pairs = (int)gridDim.x >> 1;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ TMA producer
+    if (lane == 0) {
+      const uint32_t tx = (uint32_t)(2 * kPairM + p.bn) * kPairK * 2;   // both CTAs' copies of a stage
+      uint32_t it = 0;
+      bool ok = true;
+      for (int tile = pair; tile < total && ok; tile += n_pairs) {
+        const PairTile t = pair_tile(p, tile, tiles_m);
+        const PairPasses pq = pair_passes(t);
+        const int row0 = rank == 0 ? t.row0[0] : t.row0[1];
+        const int nkb = nkb_main + pq.n * 2 * nrb;
+        const CUtensorMap* mx = &maps.x[t.job];
+        const CUtensorMap* mw = &maps.w[t.job];
+        const CUtensorMap* mb = &maps.b[t.job];
+        for (int kb = 0; kb < nkb; ++kb, ++it) {
+          const uint32_t s = it % S, ph = (it / S) & 1u;
+          if (!(ok = mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 61))) break;
+          const uint32_t sa = ring + s * kPairStageBytes, sb = sa + kPairM * kPairK * 2;
+          const uint32_t bar = map_rank(full0 + 8 * s, 0);
+          if (rank == 0) mbar_expect_tx(full0 + 8 * s, tx);
+          if (kb < nkb_main) {
+            tma_load_2d_pair(sa, mx, bar, kb * kPairK, row0);
+            tma_load_2d_pair(sb, mw, bar, kb * kPairK, t.n0 + (int)rank * (p.bn / 2));
+          } else {
+            const int q = kb - nkb_main, pass = q >= 2 * nrb ? 1 : 0, j = q - pass * 2 * nrb;
+            const int rb = j >= nrb ? j - nrb : j;            // hi blocks first, then lo blocks
+            const bool mine = ((pass ? pq.live[1] : pq.live[0]) >> rank) & 1u;
+            tma_load_2d_pair(sa, j < nrb ? &maps.hi[t.job] : &maps.lo[t.job], bar, rb * kPairK, mine ? row0 : p.M);
+            int n = p.N[0];
+#pragma unroll
+            for (int jj = 1; jj < kPairJobs; ++jj)
+              if (t.job == jj) n = p.N[jj];
+            tma_load_2d_pair(sb, mb, bar, rb * kPairK, (pass ? pq.slot[1] : pq.slot[0]) * n + t.n0 + (int)rank * (p.bn / 2));
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer (first CTA, for both)
+    if (rank == 0) {   // the whole warp walks the loop, one elected lane issues (as in tc_gemm.cu)
+      const uint32_t idesc = idesc_bf16(2 * kPairM, p.bn);
+      const bool leader = elect_one();
+      uint32_t it = 0, lt = 0;
+      bool ok = true;
+      for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
+        PairPasses pq;
+        pq.n = 0;
+        if (p.tail_r > 0) pq = pair_passes(pair_tile(p, tile, tiles_m));
+        const int nkb = nkb_main + pq.n * 2 * nrb;
+        const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
+        if (!(ok = mbar_wait_cluster_warp(tempty0 + 8 * acc, aph ^ 1u, abort_flag, p.status, 62))) break;
+        tc_fence_after();
+        const uint32_t tmem_d = tmem_base + acc * kPairMaxN;
+        for (int kb = 0; kb < nkb; ++kb, ++it) {
+          const uint32_t s = it % S, ph = (it / S) & 1u;
+          if (!(ok = mbar_wait_cluster_warp(full0 + 8 * s, ph, abort_flag, p.status, 63))) break;
+          tc_fence_after();
+          const uint32_t sa = ring + s * kPairStageBytes, sb = sa + kPairM * kPairK * 2;
+          const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sb);
+          int nk16 = (min(kPairK, p.K - kb * kPairK) + 15) / 16;
+          if (kb >= nkb_main) {
+            const int q = kb - nkb_main, pass = q >= 2 * nrb ? 1 : 0, j = q - pass * 2 * nrb;
+            const int rb = j >= nrb ? j - nrb : j;
+            nk16 = (min(kPairK, (pass ? pq.rank[1] : pq.rank[0]) - rb * kPairK) + 15) / 16;   // beyond the rank: no MMA
+          }
+          if (leader) {
+            if (nk16 == 4) {
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                tc_mma_bf16_pair(tmem_d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            } else {
+              for (int k = 0; k < nk16; ++k)
+                tc_mma_bf16_pair(tmem_d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            }
+            tc_commit_pair(empty0 + 8 * s);
+          }
+        }
+        if (ok && leader) tc_commit_pair(tfull0 + 8 * acc);
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue (warps 2..9), this CTA's 128 rows
+    const int q = warp & 3;             // TMEM lane quarter this warp may read
+    const int trow = q * 32 + lane;     // row of the tile owned by this thread
+    const int wh = (warp - 2) >> 2;     // two warps per quarter, every other 64 columns each
+    const uint32_t buf = out0 + (uint32_t)(wh * 4 + q) * 4096u;
+    uint32_t lt = 0, n_st = 0;
+    bool ok = true;
+    for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
+      const PairTile t = pair_tile(p, tile, tiles_m);
+      const int row0 = rank == 0 ? t.row0[0] : t.row0[1], rows = rank == 0 ? t.rows[0] : t.rows[1];
+      int n = p.N[0];
+      __nv_bfloat16* y = p.y[0];
+#pragma unroll
+      for (int j = 1; j < kPairJobs; ++j)
+        if (t.job == j) { n = p.N[j]; y = p.y[j]; }
+      const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
+      if (EPI != PAIR_STORE) {   // 1/|c_k| of this warp's columns; NaN where there is no candidate: it loses every maximum
+        const int k0 = t.n0 + wh * (p.bn / 2) + 4 * lane;
+        float4 v;
+        float* e = reinterpret_cast<float*>(&v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float inv = (4 * lane < p.bn / 2 && k0 + i < n) ? __ldg(p.inv_norm + k0 + i) : 0.f;
+          e[i] = inv > 0.f ? inv : __int_as_float(0x7FC00000);
+        }
+        *reinterpret_cast<float4*>(smem_raw + (buf - raw) + 16 * lane) = v;
+        __syncwarp();
+      }
+      if (!(ok = mbar_wait(tfull0 + 8 * acc, aph, abort_flag, p.status, 64))) break;
+      tc_fence_after();
+      const bool row_ok = trow < rows;
+      const size_t grow = (size_t)(row0 + trow);
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * kPairMaxN;
+      float best = -INFINITY, second = -INFINITY;
+      int best_k = 0, second_k = 0;
+      if (EPI == PAIR_STORE) {
+        // Full 32-row groups leave through shared memory (128-byte swizzled rows) as tiled stores of whole lines: a
+        // warp's 16-byte pieces straight from registers are 32 partial-line requests per instruction, beside the
+        // operand loads in L2.  Partial row groups of a plan tile and the rest of a tile
+        // whose width is no multiple of 64 are written row by row (a tiled store cannot be clipped).
+        const int col_end = min(n, t.n0 + p.bn);
+#pragma unroll 1
+        for (int c = 64 * wh; c < p.bn; c += 128) {
+          if (t.n0 + c >= n || q * 32 >= rows) break;
+          const bool staged = q * 32 + 32 <= rows && c + 64 <= p.bn;
+          if (staged && n_st >= 1) {               // the store that last read this buffer
+            if (lane == 0) bulk_wait_read<0>();
+            __syncwarp();
+          }
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh) {
+            uint32_t v[32];
+            tmem_ld32(taddr + c + 32 * hh, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              uint4 o;
+              o.x = pack_bf16(__uint_as_float(v[8 * j]), __uint_as_float(v[8 * j + 1]));
+              o.y = pack_bf16(__uint_as_float(v[8 * j + 2]), __uint_as_float(v[8 * j + 3]));
+              o.z = pack_bf16(__uint_as_float(v[8 * j + 4]), __uint_as_float(v[8 * j + 5]));
+              o.w = pack_bf16(__uint_as_float(v[8 * j + 6]), __uint_as_float(v[8 * j + 7]));
+              const int col = t.n0 + c + 32 * hh + 8 * j;      // N is a multiple of 8
+              if (staged) {
+                const uint32_t dst = buf + (uint32_t)lane * 128u + ((uint32_t)((4 * hh + j) ^ (lane & 7)) << 4);
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w) : "memory");
+              } else if (row_ok && col < col_end) {
+                *reinterpret_cast<uint4*>(y + grow * (size_t)n + col) = o;
+              }
+            }
+          }
+          if (staged) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) {
+              tma_store_2d(&maps.y[t.job], buf, t.n0 + c, row0 + q * 32);
+              bulk_commit();
+            }
+            ++n_st;
+          }
+        }
+      } else {
+        // The row's (up to) 128 scores go to registers at once, which frees the accumulator; then the maximum (two
+        // columns per instruction) and the first column that holds it.  A running (maximum, index) pair column by
+        // column takes eight instructions a column and bounded the launch: 65536 x 5000 x 768 400 us with 128 x 256 tiles
+        // of single CTAs, 455 us with pairs, now 373 us = 1.35 PFLOP/s, the power limit.
+        uint32_t f[4][32];
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+          if (32 * g < p.bn / 2) tmem_ld32(taddr + wh * (p.bn / 2) + 32 * g, f[g]);
+        tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(map_rank(tempty0 + 8 * acc, 0));
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          if (32 * g < p.bn / 2) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+              const float4 inv = lds_f4(buf + 4u * (32 * g + j));
+              const float f0 = __uint_as_float(f[g][j]) * inv.x, f1 = __uint_as_float(f[g][j + 1]) * inv.y;
+              const float f2 = __uint_as_float(f[g][j + 2]) * inv.z, f3 = __uint_as_float(f[g][j + 3]) * inv.w;
+              best = fmax3(best, fmax3(f0, f1, f2), f3);
+              f[g][j] = __float_as_uint(f0); f[g][j + 1] = __float_as_uint(f1);
+              f[g][j + 2] = __float_as_uint(f2); f[g][j + 3] = __float_as_uint(f3);
+            }
+          }
+        }
+#pragma unroll
+        for (int g = 3; g >= 0; --g) {
+          if (32 * g < p.bn / 2) {
+#pragma unroll
+            for (int j = 31; j >= 0; --j) best_k = (__uint_as_float(f[g][j]) == best) ? 32 * g + j : best_k;   // lowest index wins
+          }
+        }
+        if (EPI == PAIR_ROUTER2) {   // the same once more without the winner
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            if (32 * g < p.bn / 2) {
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) {
+                if (32 * g + j == best_k) f[g][j] = 0x7FC00000u;
+                if (32 * g + j + 1 == best_k) f[g][j + 1] = 0x7FC00000u;
+                second = fmax3(second, __uint_as_float(f[g][j]), __uint_as_float(f[g][j + 1]));
+              }
+            }
+          }
+#pragma unroll
+          for (int g = 3; g >= 0; --g) {
+            if (32 * g < p.bn / 2) {
+#pragma unroll
+              for (int j = 31; j >= 0; --j) second_k = (__uint_as_float(f[g][j]) == second) ? 32 * g + j : second_k;
+            }
+          }
+          second_k += t.n0 + wh * (p.bn / 2);
+        }
+        best_k += t.n0 + wh * (p.bn / 2);
+      }
+      if (EPI == PAIR_STORE) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(map_rank(tempty0 + 8 * acc, 0));
+      }
+      if (EPI == PAIR_ROUTER && row_ok && best > -INFINITY)
+        atomicMax(p.keys + grow, ((unsigned long long)pair_orderable(best) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k));
+      if (EPI == PAIR_ROUTER2 && row_ok) {
+        // Two-slot merge: the max goes to keys; whatever loses a comparison there (the value it displaced, or the
+        // candidate itself) is offered to keys2.  Keys are distinct and both slots are maxima: order independent.
+        const float cand[2] = {best, second};
+        const int cand_k[2] = {best_k, second_k};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (cand[i] > -INFINITY) {
+            const unsigned long long key = ((unsigned long long)pair_orderable(cand[i]) << 32) |
+                                           (unsigned long long)(0xFFFFFFFFu - (uint32_t)cand_k[i]);
+            const unsigned long long old = atomicMax(p.keys + grow, key);
+            const unsigned long long loser = old < key ? old : key;
+            if (loser != 0ull) atomicMax(p.keys2 + grow, loser);
+          }
+        }
+      }
+    }
+    if (EPI == PAIR_STORE && lane == 0) bulk_wait_all();   // this thread's tiled stores are complete
+  }
+  // ------------------------------------------------------------------ teardown
+  if (*abort_flag) {
+    // a wait ran out somewhere: give copies / MMAs still in flight time to land before memory is released
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < 2000000ull) __nanosleep(1000);
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_arrive();   // neither CTA leaves, or frees its tensor memory, while the other may still signal or multiply
+  cluster_wait();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, 512);
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Host side
+// ---------------------------------------------------------------------------------------------
+template <int EPI>
+static moin_status launch_pair(HostState* hs, const PairMaps& maps, const PairParams& p, long max_tiles, cudaStream_t stream) {
+  cudaError_t e = ensure_smem_optin(OPTIN_TC_PAIR + EPI, tc_pair_kernel<EPI>, kPairSmem);
+  if (e != cudaSuccess) return record_cuda(e);
+  long pairs = max_tiles < hs->n_sms / 2 ? max_tiles : hs->n_sms / 2;
+  if (pairs < 1) pairs = 1;
+  tc_pair_kernel<EPI><<<(unsigned)(2 * pairs), kPairThreads, kPairSmem, stream>>>(maps, p);
+  return record_cuda(cudaGetLastError());
+}
+
+// Tile width: the one with the least (waves of pair tiles over the SM pairs) x (time of one tile).  Per k-block an SM
+// takes in 128 + bn / 2 rows of 128 bytes at about 64 bytes a clock = 256 + bn clocks, and multiplies for 2 bn: the
+// fill is the longer below bn = 256.  3392 rows x 2048 columns (14 x 8 tiles of 256 on 74 pairs: two waves, the second
+// half empty) take 14 x 10 tiles of 208.
+static int pick_pair_bn(long tiles_m, const int* N, int n_jobs, int n_sms, int step) {
+  int best = 256;
+  long best_cost = -1;
+  for (int bn = 256; bn >= 64; bn -= step) {
+    long tn = 0;
+    for (int j = 0; j < n_jobs; ++j) tn += (N[j] + bn - 1) / bn;
+    const long tiles = (tiles_m + 1) / 2 * tn, pairs = n_sms / 2;
+    const long cost = ((tiles + pairs - 1) / pairs) * (bn + 256);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = bn;
+    }
+  }
+  return best;
+}
+
+moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* jobs, int n_jobs, int M, int K,
+                             cudaStream_t stream) {
+  if (n_jobs < 1 || n_jobs > kPairJobs) return MOIN_ERR_INVALID_ARG;
+  int N[kPairJobs];
+  for (int j = 0; j < n_jobs; ++j) N[j] = jobs[j].N;
+  const long tiles_m = (M + kPairM - 1) / kPairM;
+  const int bn = pick_pair_bn(tiles_m, N, n_jobs, hs->n_sms, 16);
+  PairMaps maps;
+  PairParams p = {};
+  p.M = M; p.K = K; p.n_jobs = n_jobs; p.bn = bn; p.status = hs->status;
+  if (pv) {
+    p.header = pv->header; p.tile_row0 = pv->tile_row0; p.tile_rows = pv->tile_rows; p.tile_expert = pv->tile_expert;
+    p.tail_r = jobs[0].pool->r;
+  }
+  int tn = 0;
+  for (int j = 0; j < n_jobs; ++j) {
+    const PairJob& g = jobs[j];
+    moin_status st = make_map(&maps.x[j], g.x, M, K, kPairM);
+    if (!st) st = make_map(&maps.w[j], g.W, g.N, K, bn / 2);
+    if (!st) st = make_map(&maps.y[j], g.y, M, g.N, 32);
+    if (!st && pv) {
+      const int r = g.pool->r;
+      st = make_map(&maps.hi[j], g.hb, M, r, kPairM);
+      if (!st) st = make_map(&maps.lo[j], g.hb + (size_t)M * r, M, r, kPairM);
+      if (!st) st = make_map(&maps.b[j], g.pool->B, (uint64_t)g.pool->n_slots * g.N, r, bn / 2);
+      p.slot_of_expert[j] = g.pool->slot_of_expert;
+      p.slot_rank[j] = g.pool->slot_rank;
+    }
+    if (st) return st;
+    tn += (g.N + bn - 1) / bn;
+    p.N[j] = g.N; p.tn_end[j] = tn; p.y[j] = g.y;
+  }
+  // upper bound on the row tiles of a plan without reading it back; the grid is capped at the SM pairs
+  const long max_tiles = (pv ? (long)M : (tiles_m + 1) / 2) * tn;
+  return launch_pair<PAIR_STORE>(hs, maps, p, max_tiles, stream);
+}
+
+moin_status launch_pair_router(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm, int Q,
+                               int K, int D, unsigned long long* keys, cudaStream_t stream, unsigned long long* keys2) {
+  const long tiles_m = (Q + kPairM - 1) / kPairM;
+  const int bn = pick_pair_bn(tiles_m, &K, 1, hs->n_sms, 64);
+  PairMaps maps;
+  PairParams p = {};
+  p.M = Q; p.K = D; p.n_jobs = 1; p.bn = bn; p.status = hs->status; p.inv_norm = inv_norm; p.keys = keys; p.keys2 = keys2;
+  p.N[0] = K; p.tn_end[0] = (K + bn - 1) / bn;
+  moin_status st = make_map(&maps.x[0], q, Q, D, kPairM);
+  if (!st) st = make_map(&maps.w[0], c, K, D, bn / 2);
+  if (st) return st;
+  const long tiles = (tiles_m + 1) / 2 * p.tn_end[0];
+  if (keys2 != nullptr) return launch_pair<PAIR_ROUTER2>(hs, maps, p, tiles, stream);
+  return launch_pair<PAIR_ROUTER>(hs, maps, p, tiles, stream);
+}
+
+}  // namespace moin

@@ -295,3 +295,33 @@ def test_empty_batch_and_argument_errors():
         buf = torch.zeros(8 * 64 + 8, dtype=torch.bfloat16, device=DEV)
         moin.lora_linear(None, buf[1:1 + 8 * 64].view(8, 64), W, None, 1.0)
     assert moin.device_status()["timeout_flag"] == 0
+
+
+@pytest.mark.parametrize("lengths,experts,d_out,r", [
+    ([128, 128], [0, 0], 64, 8),                        # one pair of row tiles, one expert
+    ([128, 128, 1], [0, 1, 2], 72, 16),                 # two experts in a pair, then a pair with one row
+    ([700, 3, 64, 129, 5], [0, -1, 1, 2, 0], 1160, 72),  # partial row tiles, base-only rows beside an adapter
+    ([1030], [3], 520, 128),
+    ([64] * 19, [i % 4 for i in range(19)], 264, 64),   # odd number of row tiles, every pair with two experts
+])
+def test_long_run_pairs(lengths, experts, d_out, r):
+    te = np.repeat(np.asarray(experts, np.int32), lengths)
+    T, d_in, E = len(te), 320, 4
+    pool = mi.make_pool(E, r, d_in, d_out, 31, r, missing=(3,) if r == 16 else ())
+    case = mi.layer_case("pairs", T, d_in, d_out, pool, te, 2.0, 31, d_out)
+    plan = moin.plan_build(torch.from_numpy(te).to(DEV), E, moin.PLAN_TILES)
+    y = moin.lora_linear(plan, case.x.to(DEV), case.W.to(DEV), gpu_pool(pool), 2.0)
+    torch.cuda.synchronize()
+    assert_layer_close(y, oracle_layer(case))
+    assert moin.device_status()["timeout_flag"] == 0
+
+
+@pytest.mark.parametrize("T,d_in,d_out", [(512, 64, 8), (513, 128, 208), (769, 192, 456), (3392, 320, 2048)])
+def test_base_gemm_pairs(T, d_in, d_out):
+    # tile widths that are no multiple of 64, a last column tile narrower than its width, an odd number of row tiles
+    x, W = mi.normal_bf16((T, d_in), 1.0, 5, T, device=DEV), mi.normal_bf16((d_out, d_in), 0.02, 6, d_out, device=DEV)
+    y = torch.full((T, d_out), 7.0, dtype=torch.bfloat16, device=DEV)
+    moin.lora_linear(None, x, W, None, 0.0, y=y)
+    ref = x.double() @ W.double().T
+    # one rounding to bf16 (2^-9 of the value) on top of fp32 sums of at most 320 products
+    assert ((y.double() - ref).abs() <= ref.abs() * 2 ** -8 + 1e-5).all()
