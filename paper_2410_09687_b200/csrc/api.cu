@@ -35,14 +35,6 @@ moin_status host_state(HostState** out) {
     e = cudaGetSymbolAddress(&p, g_device_status);
     if (e != cudaSuccess) return record_cuda(e);
     g_state.status = reinterpret_cast<DeviceStatus*>(p);
-    if (g_state.ev_fork == nullptr) {
-      e = cudaEventCreateWithFlags(&g_state.ev_fork, cudaEventDisableTiming);
-      for (int j = 0; j < kMaxStreamJobs && e == cudaSuccess; ++j) {
-        e = cudaStreamCreateWithFlags(&g_state.side[j], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g_state.ev_join[j], cudaEventDisableTiming);
-      }
-      if (e != cudaSuccess) return record_cuda(e);
-    }
     g_state.n_sms = prop.multiProcessorCount;
     g_state.device = dev;
   }
@@ -522,13 +514,29 @@ static moin_status check_job(const moin_plan* plan, const void* x, const void* W
 
 static moin_status pick_gemm(const HostState* hs, int T, int d_in, int d_out, bool* use_tc) {
   const bool tc_ok = tc_gemm_supported(T, d_in, d_out);
-  *use_tc = tc_ok && T >= 64 && d_out >= 64;
+  *use_tc = tc_ok;
   if (hs->gemm_impl == 1) *use_tc = false;
   if (hs->gemm_impl == 2) {
     if (!tc_ok) return MOIN_ERR_BAD_SHAPE;
     *use_tc = true;
   }
   return MOIN_OK;
+}
+
+// y (and y0) = x W^T for one projection: few tokens, the token-wide kernel (W is read once); many, CTA pairs.
+static moin_status launch_base_gemm(HostState* hs, bool use_tc, const __nv_bfloat16* x, const __nv_bfloat16* W,
+                                    __nv_bfloat16* y, float* y0, int T, int d_in, int d_out, cudaStream_t s) {
+  ProfScope prof(use_tc ? MOIN_K_GEMM_TC : MOIN_K_GEMM_WARP, 1, s);
+  if (!use_tc) return record_cuda(launch_gemm_warp(x, W, y, y0, T, d_in, d_out, s));
+  if (T <= kDecodeGemmMaxT) {
+    const DecodeGemmJob job = {x, W, y, y0, d_in, d_out};
+    return launch_decode_gemm(hs, &job, 1, T, s);
+  }
+  if (y0 == nullptr) {
+    const PairJob job = {x, W, nullptr, y, nullptr, d_out};
+    return launch_pair_gemm(hs, nullptr, &job, 1, T, d_in, s);
+  }
+  return launch_tc_gemm(hs, x, W, y, y0, T, d_in, d_out, s);
 }
 
 size_t moin_lora_linear_group_workspace_bytes(int32_t T, const moin_lora_job* jobs, int32_t n_jobs) {
@@ -569,7 +577,8 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
   if (plan->mode == MOIN_PLAN_TILES) {
     // Long runs: every projection is one grouped-shrink + one fused GEMM launch on the tensor cores.
     bool all_tc = true;
-    for (int j = 0; j < n_jobs; ++j) all_tc = all_tc && use_tc[j] && tc_fused_supported(r[j]);
+    for (int j = 0; j < n_jobs; ++j)
+      all_tc = all_tc && use_tc[j] && tc_fused_supported(r[j]) && (hs->gemm_impl == 2 || (T >= 64 && d_out[j] >= 64));
     if (all_tc) {
       // shrinks first: projections with the same d_in and rank share one launch (up to kTcMaxShrinkJobs)
       for (int j0 = 0; j0 < n_jobs;) {
@@ -603,33 +612,31 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
       return MOIN_OK;
     }
   }
-  // Short segments.  Per projection: y0 = x W^T (fp32 + bf16 copy), h = x A_e^T, y = bf16(y0 + s h B_e^T).
-  // The base GEMMs do not depend on the shrink, so each runs on one of the library's side streams between
-  // a fork and a join event, concurrently with the shrink; the shrink and the expand each cover all the
-  // projections of the group in ONE launch, so their launch and ramp-up costs are paid once per group.
+  // Short segments.  Per projection: y0 = x W^T (fp32 + bf16 copy), h = x A_e^T, y = bf16(y0 + s h B_e^T), each of the
+  // three steps ONE launch for the whole group, all on the caller's stream.  The shrink does not depend on the GEMM: it
+  // is launched as its programmatic dependent and takes the SM slots the GEMM leaves free from the start
+  // (launch_lora_shrink_stream).  (Forking the GEMMs to side streams between events took 10-15 us per group in plain
+  // launches: decode step of 256 tokens 270-300 us, 244 replayed from a graph.)
   float* h[kMaxStreamJobs];
   float* y0[kMaxStreamJobs];
   for (int j = 0; j < n_jobs; ++j) {
     h[j] = reinterpret_cast<float*>(ws_job[j]);   // [T][r] shrink results
     y0[j] = reinterpret_cast<float*>(ws_job[j] + align_up((size_t)T * (size_t)r[j] * sizeof(float), 256));
   }
-  cudaError_t ce = cudaEventRecord(hs->ev_fork, s);
-  if (ce != cudaSuccess) return record_cuda(ce);
-  moin_status st_gemm = MOIN_OK;
-  for (int j = 0; j < n_jobs; ++j) {
-    ce = cudaStreamWaitEvent(hs->side[j], hs->ev_fork, 0);
-    if (ce != cudaSuccess) return record_cuda(ce);
-    ProfScope prof(use_tc[j] ? MOIN_K_GEMM_TC : MOIN_K_GEMM_WARP, 1, hs->side[j]);
-    moin_status sj;
-    if (use_tc[j])   // the group's base GEMMs together get three quarters of the SMs, the shrink beside them the rest
-      sj = launch_tc_gemm(hs, (const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W, (__nv_bfloat16*)jobs[j].y,
-                          y0[j], T, d_in[j], d_out[j], hs->side[j], hs->n_sms * 3 / 4 / n_jobs);
-    else
-      sj = record_cuda(launch_gemm_warp((const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W,
-                                        (__nv_bfloat16*)jobs[j].y, y0[j], T, d_in[j], d_out[j], hs->side[j]));
-    if (sj && !st_gemm) st_gemm = sj;
+  bool grouped = T <= kDecodeGemmMaxT;
+  for (int j = 0; j < n_jobs; ++j) grouped = grouped && use_tc[j];
+  if (grouped) {
+    ProfScope prof(MOIN_K_GEMM_TC, 1, s);
+    DecodeGemmJob gj[kMaxStreamJobs];
+    for (int j = 0; j < n_jobs; ++j)
+      gj[j] = {(const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W, (__nv_bfloat16*)jobs[j].y, y0[j], d_in[j], d_out[j]};
+    st = launch_decode_gemm(hs, gj, n_jobs, T, s);
+  } else {
+    for (int j = 0; j < n_jobs && !st; ++j)
+      st = launch_base_gemm(hs, use_tc[j], (const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W,
+                            (__nv_bfloat16*)jobs[j].y, y0[j], T, d_in[j], d_out[j], s);
   }
-  moin_status st_shrink;
+  if (st) return st;
   {
     ProfScope prof(MOIN_K_SHRINK_STREAM, 1, s);
     ShrinkJobs sj = {};
@@ -643,16 +650,9 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
       sj.r[j] = r[j];
       sj.d_in[j] = d_in[j];
     }
-    st_shrink = record_cuda(launch_lora_shrink_stream(pv, sj, hs->n_sms, s));
+    st = record_cuda(launch_lora_shrink_stream(pv, sj, hs->n_sms, s));
   }
-  // always join, even after a failed launch, so the side streams never outlive the call's ordering
-  for (int j = 0; j < n_jobs; ++j) {
-    ce = cudaEventRecord(hs->ev_join[j], hs->side[j]);
-    if (ce == cudaSuccess) ce = cudaStreamWaitEvent(s, hs->ev_join[j], 0);
-    if (ce != cudaSuccess) return record_cuda(ce);
-  }
-  if (st_gemm) return st_gemm;
-  if (st_shrink) return st_shrink;
+  if (st) return st;
   ProfScope prof(MOIN_K_EXPAND_STREAM, 1, s);
   ExpandJobs ej = {};
   ej.n = n_jobs;
@@ -688,13 +688,8 @@ moin_status moin_lora_linear(const moin_plan* plan, const void* x, const void* W
   bool use_tc;
   if ((st = pick_gemm(hs, T, d_in, d_out, &use_tc))) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  ProfScope prof(use_tc ? MOIN_K_GEMM_TC : MOIN_K_GEMM_WARP, 1, s);
-  if (use_tc && T >= 512) {   // (fewer rows: too few pairs of row tiles)
-    const PairJob job = {(const __nv_bfloat16*)x, (const __nv_bfloat16*)W, nullptr, (__nv_bfloat16*)y, nullptr, d_out};
-    return launch_pair_gemm(hs, nullptr, &job, 1, T, d_in, s);
-  }
-  if (use_tc) return launch_tc_gemm(hs, (const __nv_bfloat16*)x, (const __nv_bfloat16*)W, (__nv_bfloat16*)y, nullptr, T, d_in, d_out, s);
-  return record_cuda(launch_gemm_warp((const __nv_bfloat16*)x, (const __nv_bfloat16*)W, (__nv_bfloat16*)y, nullptr, T, d_in, d_out, s));
+  return launch_base_gemm(hs, use_tc, (const __nv_bfloat16*)x, (const __nv_bfloat16*)W, (__nv_bfloat16*)y, nullptr, T,
+                          d_in, d_out, s);
 }
 
 }  // extern "C"

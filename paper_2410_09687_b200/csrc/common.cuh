@@ -198,8 +198,8 @@ cudaError_t launch_route_finish(const unsigned long long* keys, const __nv_bfloa
                                 int* out_expert, int* out_centroid, float* out_best, cudaStream_t stream);
 
 // Host state of the entry points (api.cu): one record per device ordinal, filled on the first call made with
-// that device current.  Streams, events, the status block's address and the kernels' shared-memory opt-ins all
-// belong to one device, so nothing here is shared between devices.
+// that device current.  The status block's address and the kernels' shared-memory opt-ins belong to one device, so
+// nothing here is shared between devices.
 constexpr int kMaxDevices = 64;
 constexpr int kOptinSlots = 48;
 struct HostState {
@@ -207,9 +207,6 @@ struct HostState {
   int device = -1;
   int n_sms = 0;
   int gemm_impl = 0;               // MOIN_OPT_GEMM_IMPL (process-wide option, copied in on every call)
-  // fork/join inside one call: independent kernels of a call run on `side` between two events
-  cudaStream_t side[kMaxStreamJobs] = {nullptr, nullptr, nullptr, nullptr};
-  cudaEvent_t ev_fork = nullptr, ev_join[kMaxStreamJobs] = {nullptr, nullptr, nullptr, nullptr};
   size_t smem_optin[kOptinSlots] = {};   // dynamic shared memory already opted in, per kernel (see ensure_smem_optin)
 };
 moin_status host_state(HostState** out);      // lazily initialised for the current device

@@ -81,6 +81,7 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
   __shared__ float red[kShrinkWarps][32][4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
+  pdl_launch_dependents();
   const int nseg = header[PH_NSEG];
   int items = 0;
 #pragma unroll
@@ -156,6 +157,9 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
       }
     }
   }
+  // One CTA ends only after the base GEMM launched before this kernel: whoever waits for this grid (the expand, in
+  // stream order) has waited for the GEMM too, although the two run side by side.
+  if (blockIdx.x == gridDim.x - 1) pdl_wait();
 }
 
 // y[perm[pos]][j] = bf16( y0[perm[pos]][j] + scale * sum_rho B[slot][j][rho] * h[pos][rho] )
@@ -178,6 +182,8 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
   const int g = lane >> 2, t = lane & 3;
   const long long wid = (long long)blockIdx.x * (kExpandThreads / 32) + warp;
   const long long nw = (long long)gridDim.x * (kExpandThreads / 32);
+  pdl_launch_dependents();
+  pdl_wait();   // h (shrink) and y0 (base GEMM, which the shrink's completion covers)
   const int nseg = __ldg(header + PH_NSEG);
   const long long units = (long long)nseg * tps;
   long long u = units * wid / nw;
@@ -313,9 +319,8 @@ cudaError_t launch_lora_shrink_stream(const PlanView& pv, ShrinkJobs jobs, int n
     items += (long)pv.Smax * jobs.per_seg[j];
   }
   // one CTA per item (capped; CTAs stride over the items beyond the cap)
-  lora_shrink_stream_kernel<<<stream_grid(items, n_sms, 1024), kShrinkThreads, 0, stream>>>(pv.header, pv.perm, pv.seg_tab,
-                                                                                       jobs);
-  return cudaGetLastError();
+  return launch_dependent(lora_shrink_stream_kernel, stream_grid(items, n_sms, 1024), kShrinkThreads, stream, pv.header,
+                          pv.perm, pv.seg_tab, jobs);
 }
 
 cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float scale, int n_sms,
@@ -332,16 +337,12 @@ cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float
   const int grid = stream_grid(max_ctas, n_sms, 4);
   bool var = false;
   for (int j = 0; j < jobs.n; ++j) var = var || jobs.slot_rank[j] != nullptr || jobs.act[j] != MOIN_ACT_NONE;
-#define MOIN_EXPAND(P)                                                                                          \
-  do {                                                                                                          \
-    if (var) lora_expand_stream_kernel<P, true><<<grid, kExpandThreads, 0, stream>>>(pv.header, pv.perm, pv.seg_tab, jobs, scale, tps); \
-    else lora_expand_stream_kernel<P, false><<<grid, kExpandThreads, 0, stream>>>(pv.header, pv.perm, pv.seg_tab, jobs, scale, tps);    \
-  } while (0)
-  if (rmax <= 32) MOIN_EXPAND(1);
-  else if (rmax <= 64) MOIN_EXPAND(2);
-  else MOIN_EXPAND(4);
-#undef MOIN_EXPAND
-  return cudaGetLastError();
+  auto go = [&](auto* fn) {
+    return launch_dependent(fn, grid, kExpandThreads, stream, pv.header, pv.perm, pv.seg_tab, jobs, scale, tps);
+  };
+  if (rmax <= 32) return var ? go(lora_expand_stream_kernel<1, true>) : go(lora_expand_stream_kernel<1, false>);
+  if (rmax <= 64) return var ? go(lora_expand_stream_kernel<2, true>) : go(lora_expand_stream_kernel<2, false>);
+  return var ? go(lora_expand_stream_kernel<4, true>) : go(lora_expand_stream_kernel<4, false>);
 }
 
 }  // namespace moin

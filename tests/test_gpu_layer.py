@@ -325,3 +325,16 @@ def test_base_gemm_pairs(T, d_in, d_out):
     ref = x.double() @ W.double().T
     # one rounding to bf16 (2^-9 of the value) on top of fp32 sums of at most 320 products
     assert ((y.double() - ref).abs() <= ref.abs() * 2 ** -8 + 1e-5).all()
+
+
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 63, 65, 120, 255, 256, 257, 400, 512])
+@pytest.mark.parametrize("d_in,d_out", [(64, 8), (192, 136), (2048, 264)])
+def test_base_gemm_few_tokens(T, d_in, d_out):
+    # token tiles (one or two of up to 256), feature tiles with a remainder, reductions cut over a cluster or not
+    x, W = mi.normal_bf16((T, d_in), 1.0, 7, T, device=DEV), mi.normal_bf16((d_out, d_in), 0.02, 8, d_in, device=DEV)
+    y = torch.full((T, d_out), 7.0, dtype=torch.bfloat16, device=DEV)
+    moin.lora_linear(None, x, W, None, 0.0, y=y)
+    ref = x.double() @ W.double().T
+    # one rounding to bf16 (2^-9 of the value) on top of fp32 sums of at most 2048 products of size 0.02
+    assert ((y.double() - ref).abs() <= ref.abs() * 2 ** -8 + 2e-5).all()
+    assert moin.device_status()["timeout_flag"] == 0
