@@ -21,7 +21,8 @@ struct DeviceStatus {
 
 // Plan buffer layout (int32 words).  Header first, then the arrays.
 constexpr int kPlanHeaderWords = 16;
-enum PlanHeader { PH_NSEG = 0, PH_NTILES = 1, PH_NLORA = 2, PH_MAXSEG = 3, PH_T = 4, PH_E = 5 };
+enum PlanHeader { PH_NSEG = 0, PH_NTILES = 1, PH_NLORA = 2, PH_MAXSEG = 3, PH_T = 4, PH_E = 5, PH_NCHUNK = 6 };
+constexpr int kSegChunk = 8;      // token columns of one warp MMA: what a work item of the stream kernels covers
 constexpr int kPlanChunk = 256;   // tokens per histogram chunk
 constexpr int kTileRows = 128;    // rows per GEMM tile
 
@@ -31,14 +32,16 @@ struct PlanView {   // pointers into the plan buffer
   int* seg_expert;   // [Smax]
   int* seg_start;    // [Smax + 1]
   int4* seg_tab;     // [Smax + 1] packed (expert, start, length, 0): one 16-byte load per segment
+  int4* chunk_tab;   // [Cmax] the segments cut into pieces of at most kSegChunk tokens: (expert, start, length, 0)
   int* tile_row0;    // [T + 1]
   int* tile_rows;    // [T]
   int* tile_expert;  // [T]
   int* rank;         // [T]   scratch
   int* key;          // [T]   scratch
   int* keybase;      // [E+1] scratch
+  int* chunkbase;    // [E+1] scratch
   int* hist;         // [n_chunks * (E+1)] scratch
-  int T, E, Smax, n_chunks;
+  int T, E, Smax, Cmax, n_chunks;
 };
 
 __host__ __device__ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -47,6 +50,7 @@ inline PlanView plan_view(void* buffer, int T, int E, size_t* total_words = null
   PlanView v;
   v.T = T; v.E = E;
   v.Smax = T < E ? T : E;
+  v.Cmax = T / kSegChunk + v.Smax;
   v.n_chunks = (T + kPlanChunk - 1) / kPlanChunk;
   int* base = reinterpret_cast<int*>(buffer);
   size_t off = 0;
@@ -56,12 +60,14 @@ inline PlanView plan_view(void* buffer, int T, int E, size_t* total_words = null
   v.seg_expert = take(v.Smax + 1);
   v.seg_start = take(v.Smax + 2);
   v.seg_tab = reinterpret_cast<int4*>(take(4 * (size_t)(v.Smax + 1)));
+  v.chunk_tab = reinterpret_cast<int4*>(take(4 * (size_t)(v.Cmax + 1)));
   v.tile_row0 = take(T + 1);
   v.tile_rows = take(T + 1);
   v.tile_expert = take(T + 1);
   v.rank = take(T);
   v.key = take(T);
   v.keybase = take(E + 2);
+  v.chunkbase = take(E + 2);
   v.hist = take((size_t)v.n_chunks * (size_t)(E + 1));
   if (total_words) *total_words = off;
   return v;

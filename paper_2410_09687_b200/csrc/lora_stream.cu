@@ -19,8 +19,11 @@ constexpr int kShrinkUnroll = 4;         // 32-wide k steps in flight per warp
 constexpr int kExpandThreads = 128;      // 4 warps
 constexpr int kExpandTilesPerBatch = 2;  // 16-row tiles whose loads are in flight together, per warp
 
+// The unit both kernels work on is a CHUNK of the plan: at most 8 tokens (the columns of one MMA) of one expert.  A
+// longer segment is several chunks that run side by side and find the adapter in L2; walking them one after the other
+// in one CTA cost a round trip each (264 tokens over 8 experts, 256 -> 256: shrink 10.6 us, expand 17 us; a call of the layer 21.9 us, now 8.7).
 // Work items of a launch span up to kMaxStreamJobs projections that share one batch plan: item index ->
-// (job, segment, sub-block), jobs laid out one after the other, `per_seg[j]` items per segment in job j.
+// (job, chunk, sub-block), jobs laid out one after the other, `per_seg[j]` items per chunk in job j.
 // Kernel parameters are only ever indexed with compile-time indices (a run-time index would force a
 // local-memory copy of the parameter block): pick(arr, j) selects arr[j] with a compare chain.
 template <class V>
@@ -34,13 +37,13 @@ __device__ __forceinline__ V pick(const V (&arr)[kMaxStreamJobs], int j) {
 
 struct ItemRef { int job, seg, sub; };
 template <class Jobs>
-__device__ __forceinline__ ItemRef decode_item(int item, int nseg, const Jobs& jobs) {
+__device__ __forceinline__ ItemRef decode_item(int item, int nchunk, const Jobs& jobs) {
   ItemRef it = {0, 0, 0};
   int rem = item;
 #pragma unroll
   for (int j = 0; j + 1 < kMaxStreamJobs; ++j) {
-    if (it.job == j && j + 1 < jobs.n && rem >= nseg * jobs.per_seg[j]) {
-      rem -= nseg * jobs.per_seg[j];
+    if (it.job == j && j + 1 < jobs.n && rem >= nchunk * jobs.per_seg[j]) {
+      rem -= nchunk * jobs.per_seg[j];
       it.job = j + 1;
     }
   }
@@ -52,12 +55,12 @@ __device__ __forceinline__ ItemRef decode_item(int item, int nseg, const Jobs& j
 
 struct SegMeta { int slot, s0, n, job, sub, r_use; };   // r_use: rank of the slot's adapter (<= the stored rank)
 template <class Jobs>
-__device__ __forceinline__ SegMeta load_seg(const int4* __restrict__ seg_tab, const Jobs& jobs, int item, int items,
-                                            int nseg) {
+__device__ __forceinline__ SegMeta load_seg(const int4* __restrict__ chunk_tab, const Jobs& jobs, int item, int items,
+                                            int nchunk) {
   SegMeta m = {-1, 0, 0, 0, 0, 0};
   if (item < items) {
-    const ItemRef it = decode_item(item, nseg, jobs);
-    const int4 e = __ldg(seg_tab + it.seg);   // (expert, start, length, -)
+    const ItemRef it = decode_item(item, nchunk, jobs);
+    const int4 e = __ldg(chunk_tab + it.seg);   // (expert, start, length, -)
     m.slot = __ldg(pick(jobs.slot_of_expert, it.job) + e.x);
     const int* rank_tab = pick(jobs.slot_rank, it.job);
     m.r_use = (m.slot >= 0 && rank_tab) ? min(__ldg(rank_tab + m.slot), pick(jobs.r, it.job)) : pick(jobs.r, it.job);
@@ -70,28 +73,28 @@ __device__ __forceinline__ SegMeta load_seg(const int4* __restrict__ seg_tab, co
 }
 
 // h[pos][rho] = sum_i A[slot][rho][i] * x[perm[pos]][i]      (fp32, pos = position in sorted order)
-// Work item = (job, segment, group of 16 adapter rows); the CTA's warps interleave over k.
+// Work item = (job, chunk, group of 16 adapter rows); the CTA's warps interleave over k.
 // Small CTAs (4 warps, 80 registers: six per SM, and room beside a base-GEMM CTA) and one CTA per item:
 // the hardware's block scheduler hands the items out as slots free up, so a launch ends evenly whatever
-// the base GEMMs on the side streams occupy, and a CTA's metadata hops (segment count, table entry,
+// the base GEMM beside it occupies, and a CTA's metadata hops (segment count, table entry,
 // slot) hide behind the streams of the other CTAs on its SM.
 __global__ void __launch_bounds__(kShrinkThreads, 6)
 lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict__ perm,
-                          const int4* __restrict__ seg_tab, const ShrinkJobs jobs) {
+                          const int4* __restrict__ chunk_tab, const ShrinkJobs jobs) {
   __shared__ float red[kShrinkWarps][32][4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   pdl_launch_dependents();
-  const int nseg = header[PH_NSEG];
+  const int nchunk = header[PH_NCHUNK];
   int items = 0;
 #pragma unroll
   for (int j = 0; j < kMaxStreamJobs; ++j)
-    if (j < jobs.n) items += nseg * jobs.per_seg[j];
+    if (j < jobs.n) items += nchunk * jobs.per_seg[j];
   int item = blockIdx.x;
-  SegMeta nxt = load_seg(seg_tab, jobs, item, items, nseg);
+  SegMeta nxt = load_seg(chunk_tab, jobs, item, items, nchunk);
   for (; item < items; item += gridDim.x) {
     const SegMeta cur = nxt;
-    nxt = load_seg(seg_tab, jobs, item + gridDim.x, items, nseg);  // lookahead
+    nxt = load_seg(chunk_tab, jobs, item + gridDim.x, items, nchunk);  // lookahead
     if (cur.slot < 0 || cur.sub * 16 >= cur.r_use) continue;  // uniform per CTA: no adapter, or rows beyond its rank
     const int r = pick(jobs.r, cur.job), d_in = pick(jobs.d_in, cur.job);
     const __nv_bfloat16* __restrict__ x = pick(jobs.x, cur.job);
@@ -102,8 +105,8 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
     const bool v0 = rho0 < cur.r_use, v1 = rho1 < cur.r_use;   // rows beyond the slot's rank are not read
     const __nv_bfloat16* a_row0 = A + ((size_t)cur.slot * r + (v0 ? rho0 : 0)) * (size_t)d_in + 8 * t;
     const __nv_bfloat16* a_row1 = A + ((size_t)cur.slot * r + (v1 ? rho1 : 0)) * (size_t)d_in + 8 * t;
-    for (int tc = 0; tc < cur.n; tc += 8) {
-      const bool vx = (tc + g) < cur.n;
+    {
+      const bool vx = g < cur.n;
       float c[4] = {0.f, 0.f, 0.f, 0.f};
       const __nv_bfloat16* x_row = nullptr;
       for (int base = 0; base < steps; base += kShrinkWarps * kShrinkUnroll) {
@@ -116,7 +119,7 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
           a0[u] = (vi && v0) ? ldg_stream(a_row0 + i * 32) : z;
           a1[u] = (vi && v1) ? ldg_stream(a_row1 + i * 32) : z;
         }
-        if (x_row == nullptr) x_row = x + (size_t)(vx ? perm[cur.s0 + tc + g] : 0) * (size_t)d_in + 8 * t;
+        if (x_row == nullptr) x_row = x + (size_t)(vx ? perm[cur.s0 + g] : 0) * (size_t)d_in + 8 * t;
 #pragma unroll
         for (int u = 0; u < kShrinkUnroll; ++u) {
           const int i = base + u * kShrinkWarps + warp;
@@ -144,13 +147,13 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
         }
         // c0:(rho0, col 2t) c1:(rho0, col 2t+1) c2:(rho1, col 2t) c3:(rho1, col 2t+1)
         const int col = 2 * t;
-        if (tc + col < cur.n) {
-          float* hp = h + (size_t)(cur.s0 + tc + col) * r;
+        if (col < cur.n) {
+          float* hp = h + (size_t)(cur.s0 + col) * r;
           if (v0) hp[rho0] = s[0];
           if (v1) hp[rho1] = s[2];
         }
-        if (tc + col + 1 < cur.n) {
-          float* hp = h + (size_t)(cur.s0 + tc + col + 1) * r;
+        if (col + 1 < cur.n) {
+          float* hp = h + (size_t)(cur.s0 + col + 1) * r;
           if (v0) hp[rho0] = s[1];
           if (v1) hp[rho1] = s[3];
         }
@@ -165,18 +168,18 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
 // y[perm[pos]][j] = bf16( y0[perm[pos]][j] + scale * sum_rho B[slot][j][rho] * h[pos][rho] )
 // h is split into bf16 hi + lo parts (two MMAs) so the low-rank term keeps ~fp32 accuracy.
 //
-// The unit of work is one 16-row tile of B for one (segment, job); units are ordered (segment, job, tile)
+// The unit of work is one 16-row tile of B for one (chunk, job); units are ordered (chunk, job, tile)
 // and every warp of the grid takes one contiguous, equally long range of them (tiles need no reduction
 // across each other, so a range may start and end anywhere).  All warps therefore stream the same number
 // of adapter bytes, whatever the mix of projection widths in the launch, and a warp's range is contiguous
-// in memory inside a (segment, job).  A warp walks its range kExpandTilesPerBatch tiles at a time with
+// in memory inside a (chunk, job).  A warp walks its range kExpandTilesPerBatch tiles at a time with
 // the adapter rows and the base values y0 of a batch loaded together.  `jobs.per_seg[j]` = tiles of job j.
 // VAR: some pool of the launch has a rank per slot or an activation; without it the kernel is the plain layer's
 // (the rank is the stored rank, h is used as it is) and carries none of the variant's bookkeeping.
 template <int P, bool VAR>  // P: number of 32-wide rho groups, ceil(max r / 32)
 __global__ void __launch_bounds__(kExpandThreads, 4)
 lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict__ perm,
-                          const int4* __restrict__ seg_tab, const ExpandJobs jobs, float scale, int tps) {
+                          const int4* __restrict__ chunk_tab, const ExpandJobs jobs, float scale, int tps) {
   constexpr int TB = P > 2 ? 1 : kExpandTilesPerBatch;   // wide ranks: one tile's rows already fill the load registers
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -184,14 +187,14 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
   const long long nw = (long long)gridDim.x * (kExpandThreads / 32);
   pdl_launch_dependents();
   pdl_wait();   // h (shrink) and y0 (base GEMM, which the shrink's completion covers)
-  const int nseg = __ldg(header + PH_NSEG);
-  const long long units = (long long)nseg * tps;
+  const int nchunk = __ldg(header + PH_NCHUNK);
+  const long long units = (long long)nchunk * tps;
   long long u = units * wid / nw;
   const long long u_end = units * (wid + 1) / nw;
   while (u < u_end) {
-    // ---- segment: expert, rows, adapter slots of all jobs (one hop after the table entry)
+    // ---- chunk: expert, rows, adapter slots of all jobs (one hop after the table entry)
     const int seg = (int)(u / tps);
-    const int4 e = __ldg(seg_tab + seg);   // (expert, start, length, -)
+    const int4 e = __ldg(chunk_tab + seg);   // (expert, start, length, -)
     const int s0 = e.y, n = e.z;
     int slots[kMaxStreamJobs];
 #pragma unroll
@@ -201,7 +204,8 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
     for (int j = 0; j < kMaxStreamJobs; ++j)
       ranks[j] = (VAR && j < jobs.n && slots[j] >= 0 && jobs.slot_rank[j]) ? min(__ldg(jobs.slot_rank[j] + slots[j]), jobs.r[j])
                                                                      : (j < jobs.n ? jobs.r[j] : 0);
-    const int row_first = (g < n) ? __ldg(perm + s0 + g) : -1;
+    const bool vx = g < n;
+    const int my_row = vx ? __ldg(perm + s0 + g) : -1;
     const long long seg_end = (long long)(seg + 1) * tps;
     int rem = (int)(u - (long long)seg * tps);
     int job = 0;
@@ -212,7 +216,7 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
         job = j + 1;
       }
     }
-    // ---- (segment, job) pieces of the range
+    // ---- (chunk, job) pieces of the range
     while (u < u_end && u < seg_end) {
       const int tiles_j = pick(jobs.per_seg, job);
       const int tile0 = rem;
@@ -226,18 +230,16 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
         const float* __restrict__ y0 = pick(jobs.y0, job);
         __nv_bfloat16* __restrict__ y = pick(jobs.y, job);
         const __nv_bfloat16* Bs = pick(jobs.B, job) + (size_t)slot * (size_t)d_out * (size_t)r;
-        for (int tc = 0; tc < n; tc += 8) {
-          // token operand (MMA "B" fragment): column g = token tc+g, k slots <- rho 32p + 8t .. +7
-          const bool vx = (tc + g) < n;
-          const int my_row = (tc == 0) ? row_first : (vx ? __ldg(perm + s0 + tc + g) : -1);
+        {
+          // token operand (MMA "B" fragment): column g = token g, k slots <- rho 32p + 8t .. +7
           uint32_t hh[P][4], hl[P][4];
 #pragma unroll
           for (int p = 0; p < P; ++p) {
             const int rb = 32 * p + 8 * t;
             float v[8];
             if (vx && rb < r_use) {
-              const float4 f0 = *reinterpret_cast<const float4*>(h + (size_t)(s0 + tc + g) * r + rb);
-              const float4 f1 = *reinterpret_cast<const float4*>(h + (size_t)(s0 + tc + g) * r + rb + 4);
+              const float4 f0 = *reinterpret_cast<const float4*>(h + (size_t)(s0 + g) * r + rb);
+              const float4 f1 = *reinterpret_cast<const float4*>(h + (size_t)(s0 + g) * r + rb + 4);
               v[0] = f0.x; v[1] = f0.y; v[2] = f0.z; v[3] = f0.w; v[4] = f1.x; v[5] = f1.y; v[6] = f1.z; v[7] = f1.w;
             } else {
 #pragma unroll
@@ -316,11 +318,11 @@ cudaError_t launch_lora_shrink_stream(const PlanView& pv, ShrinkJobs jobs, int n
   long items = 0;
   for (int j = 0; j < jobs.n; ++j) {
     jobs.per_seg[j] = (jobs.r[j] + 15) / 16;
-    items += (long)pv.Smax * jobs.per_seg[j];
+    items += (long)pv.Cmax * jobs.per_seg[j];
   }
   // one CTA per item (capped; CTAs stride over the items beyond the cap)
   return launch_dependent(lora_shrink_stream_kernel, stream_grid(items, n_sms, 1024), kShrinkThreads, stream, pv.header,
-                          pv.perm, pv.seg_tab, jobs);
+                          pv.perm, pv.chunk_tab, jobs);
 }
 
 cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float scale, int n_sms,
@@ -328,17 +330,17 @@ cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float
   int tps = 0, rmax = 0;
   for (int j = 0; j < jobs.n; ++j) {
     jobs.rows_per_item[j] = 16;
-    jobs.per_seg[j] = (jobs.d_out[j] + 15) / 16;   // 16-row tiles per segment
+    jobs.per_seg[j] = (jobs.d_out[j] + 15) / 16;   // 16-row tiles per chunk
     tps += jobs.per_seg[j];
     rmax = jobs.r[j] > rmax ? jobs.r[j] : rmax;
   }
   // one warp per 2 tiles at least; at most one CTA per resident slot (4 per SM)
-  const long max_ctas = ((long)pv.Smax * tps + 2 * (kExpandThreads / 32) - 1) / (2 * (kExpandThreads / 32));
+  const long max_ctas = ((long)pv.Cmax * tps + 2 * (kExpandThreads / 32) - 1) / (2 * (kExpandThreads / 32));
   const int grid = stream_grid(max_ctas, n_sms, 4);
   bool var = false;
   for (int j = 0; j < jobs.n; ++j) var = var || jobs.slot_rank[j] != nullptr || jobs.act[j] != MOIN_ACT_NONE;
   auto go = [&](auto* fn) {
-    return launch_dependent(fn, grid, kExpandThreads, stream, pv.header, pv.perm, pv.seg_tab, jobs, scale, tps);
+    return launch_dependent(fn, grid, kExpandThreads, stream, pv.header, pv.perm, pv.chunk_tab, jobs, scale, tps);
   };
   if (rmax <= 32) return var ? go(lora_expand_stream_kernel<1, true>) : go(lora_expand_stream_kernel<1, false>);
   if (rmax <= 64) return var ? go(lora_expand_stream_kernel<2, true>) : go(lora_expand_stream_kernel<2, false>);

@@ -134,47 +134,89 @@ __global__ void __launch_bounds__(kPrefixIds * kPrefixGroups) plan_prefix_kernel
 }
 
 // Row tiles: maximal runs of equal expert id in token order, cut every kTileRows rows.  One CTA of NT
-// threads; `key[t]` is the sanitised id of token t (shared or global memory).  smem: 33 ints, s_carry: 2.
+// threads; `key[t]` is the sanitised id of token t (shared or global memory).  smem: 33 ints.
 // `row0` is where the tile starts are read back from to form the tile lengths: v.tile_row0 itself, or a
 // shared-memory copy ([T + 1] ints) when the caller has one.
+// Every thread takes one contiguous range of the tokens (a multiple of 4, read 16 bytes at a time), so the whole batch
+// needs two block-wide scans; two scans per NT tokens made the kernel 27 us long at 16 384 tokens.
 template <int NT>
-__device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, int* smem, int* s_carry, int* row0) {
+__device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, int* smem, int* row0) {
   const int tid = threadIdx.x;
   const int T = v.T, E = v.E;
-  int carry_start = 0, carry_tiles = 0;
-  for (int t0 = 0; t0 < T; t0 += NT) {
-    int t = t0 + tid;
-    int k = (t < T) ? key[t] : -3;
-    int is_start = (t < T) && (t == 0 || key[t - 1] != k);
-    int rs = block_incl_max<NT>(is_start ? t : -1, smem);
-    rs = max(rs, carry_start);
-    int flag = (t < T) && (((t - rs) % kTileRows) == 0);
-    int tot;
-    int idx = carry_tiles + block_excl_sum<NT>(flag, smem, &tot);
-    if (flag) {
-      v.tile_row0[idx] = t;
-      if (row0 != v.tile_row0) row0[idx] = t;
-      v.tile_expert[idx] = (k == E) ? -1 : k;
+  const int per = ((T + NT - 1) / NT + 3) / 4 * 4;
+  const int lo = min(T, tid * per), hi = min(T, lo + per);
+  auto load4 = [&](int t, int (&k)[4]) {   // ids of tokens t .. t + 3 (t is a multiple of 4; -3 beyond the batch)
+    if (t + 4 <= T) {
+      const int4 w = *reinterpret_cast<const int4*>(key + t);
+      k[0] = w.x; k[1] = w.y; k[2] = w.z; k[3] = w.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) k[i] = (t + i < T) ? key[t + i] : -3;
     }
-    if (tid == NT - 1) s_carry[0] = rs;
-    __syncthreads();
-    carry_start = s_carry[0];
-    carry_tiles += tot;
-    __syncthreads();
+  };
+  const int before = (lo > 0 && lo < T) ? key[lo - 1] : -4;   // id of the token in front of the range
+  // 1. last run start inside the range; its maximum over the earlier ranges is the run this range begins in
+  int last = -1, prev = before;
+  for (int t = lo; t < hi; t += 4) {
+    int k[4];
+    load4(t, k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (t + i < hi) {
+        if (k[i] != prev) last = t + i;
+        prev = k[i];
+      }
+  }
+  const int incl = block_incl_max<NT>(last, smem);
+  int run = __shfl_up_sync(0xffffffffu, incl, 1);   // exclusive: the lane before, or the last lane of the warp before
+  if ((tid & 31) == 0) run = tid > 0 ? smem[(tid >> 5) - 1] : -1;
+  // 2. tiles that start inside the range
+  int count = 0, rs = run;
+  prev = before;
+  for (int t = lo; t < hi; t += 4) {
+    int k[4];
+    load4(t, k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (t + i < hi) {
+        if (k[i] != prev) rs = t + i;
+        prev = k[i];
+        count += ((t + i - rs) % kTileRows) == 0;
+      }
+  }
+  int total;
+  int idx = block_excl_sum<NT>(count, smem, &total);
+  // 3. the list
+  rs = run;
+  prev = before;
+  for (int t = lo; t < hi; t += 4) {
+    int k[4];
+    load4(t, k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (t + i < hi) {
+        if (k[i] != prev) rs = t + i;
+        prev = k[i];
+        if (((t + i - rs) % kTileRows) == 0) {
+          v.tile_row0[idx] = t + i;
+          if (row0 != v.tile_row0) row0[idx] = t + i;
+          v.tile_expert[idx] = (k[i] == E) ? -1 : k[i];
+          ++idx;
+        }
+      }
   }
   if (tid == 0) {
-    v.tile_row0[carry_tiles] = T;
-    if (row0 != v.tile_row0) row0[carry_tiles] = T;
-    v.header[PH_NTILES] = carry_tiles;
+    v.tile_row0[total] = T;
+    if (row0 != v.tile_row0) row0[total] = T;
+    v.header[PH_NTILES] = total;
   }
   __syncthreads();
-  for (int i = tid; i < carry_tiles; i += NT) v.tile_rows[i] = row0[i + 1] - row0[i];
+  for (int i = tid; i < total; i += NT) v.tile_rows[i] = row0[i + 1] - row0[i];
 }
 
 __global__ void __launch_bounds__(1024) plan_scan_kernel(PlanView v, int do_prefix, int want_tiles) {
   constexpr int NT = 1024;
   __shared__ int smem[33];
-  __shared__ int s_carry[2];
   const int tid = threadIdx.x;
   const int T = v.T, E = v.E, nc = v.n_chunks;
   const size_t pitch = (size_t)(E + 1);
@@ -192,31 +234,40 @@ __global__ void __launch_bounds__(1024) plan_scan_kernel(PlanView v, int do_pref
   }
   __syncthreads();
 
-  // 2. prefix over expert ids -> segment list (ascending expert id), "no adapter" bucket last
-  int carry_tok = 0, carry_seg = 0, max_seg = 0;
-  for (int k0 = 0; k0 < E; k0 += 1024) {
-    int k = k0 + tid;
-    int n = (k < E) ? v.keybase[k] : 0;
-    int tot_tok, tot_seg;
-    int ex_tok = block_excl_sum<NT>(n, smem, &tot_tok);
-    int ex_seg = block_excl_sum<NT>(n > 0 ? 1 : 0, smem, &tot_seg);
-    if (k < E) {
-      v.keybase[k] = carry_tok + ex_tok;
-      if (n > 0) {
-        v.seg_expert[carry_seg + ex_seg] = k;
-        v.seg_start[carry_seg + ex_seg] = carry_tok + ex_tok;
-        v.seg_tab[carry_seg + ex_seg] = make_int4(k, carry_tok + ex_tok, n, 0);
-      }
-    }
+  // 2. prefix over expert ids -> segment list (ascending expert id), "no adapter" bucket last; a contiguous range of
+  // ids per thread, so one set of scans whatever E
+  const int per = (E + NT - 1) / NT, k_lo = min(E, tid * per), k_hi = min(E, k_lo + per);
+  int n_tok = 0, n_seg = 0, n_chunk = 0, max_seg = 0;
+  for (int k = k_lo; k < k_hi; ++k) {
+    const int n = v.keybase[k];
+    n_tok += n;
+    n_seg += n > 0;
+    n_chunk += (n + kSegChunk - 1) / kSegChunk;
     max_seg = max(max_seg, n);
-    carry_tok += tot_tok;
-    carry_seg += tot_seg;
+  }
+  int carry_tok, carry_seg, carry_chunk;
+  int tok = block_excl_sum<NT>(n_tok, smem, &carry_tok);
+  int seg = block_excl_sum<NT>(n_seg, smem, &carry_seg);
+  int chunk = block_excl_sum<NT>(n_chunk, smem, &carry_chunk);
+  for (int k = k_lo; k < k_hi; ++k) {
+    const int n = v.keybase[k];
+    v.keybase[k] = tok;
+    v.chunkbase[k] = chunk;   // (plan_scatter_kernel writes the chunks)
+    if (n > 0) {
+      v.seg_expert[seg] = k;
+      v.seg_start[seg] = tok;
+      v.seg_tab[seg] = make_int4(k, tok, n, 0);
+      ++seg;
+    }
+    tok += n;
+    chunk += (n + kSegChunk - 1) / kSegChunk;
   }
   max_seg = block_incl_max<NT>(max_seg, smem);
   if (tid == 1023) {
     v.seg_start[carry_seg] = carry_tok;
     v.keybase[E] = carry_tok;
     v.header[PH_NSEG] = carry_seg;
+    v.header[PH_NCHUNK] = carry_chunk;
     v.header[PH_NLORA] = carry_tok;
     v.header[PH_MAXSEG] = max_seg;
     v.header[PH_T] = T;
@@ -224,7 +275,7 @@ __global__ void __launch_bounds__(1024) plan_scan_kernel(PlanView v, int do_pref
   }
 
   // 3. row tiles (only the long-run kernels read them)
-  if (want_tiles) plan_tiles<NT>(v, v.key, smem, s_carry, v.tile_row0);
+  if (want_tiles) plan_tiles<NT>(v, v.key, smem, v.tile_row0);
   else if (tid == 0) v.header[PH_NTILES] = 0;
 }
 
@@ -237,11 +288,10 @@ constexpr int kPlanSmallE = 1 << 20;   // the id must fit above the 10 token bit
 template <int NT>   // threads = sort width: the power of two at or above T, at least 128
 __global__ void __launch_bounds__(NT) plan_small_kernel(const int* __restrict__ token_expert, PlanView v,
                                                         DeviceStatus* status, int want_tiles) {
-  __shared__ int s_key[NT];        // sanitised id by token
+  __shared__ __align__(16) int s_key[NT];   // sanitised id by token
   __shared__ int s_sort[NT + 1];   // sort keys, then the segment starts plus one end marker (NT segments at most)
   __shared__ int s_row0[NT + 1];   // tile starts
   __shared__ int smem[33];
-  __shared__ int s_carry[2];
   const int tid = threadIdx.x;
   const int T = v.T, E = v.E;
   int k = 0x1FFFFF;  // padding sorts last
@@ -292,15 +342,22 @@ __global__ void __launch_bounds__(NT) plan_small_kernel(const int* __restrict__ 
     v.seg_tab[seg] = make_int4(id, tid, len, 0);
   }
   if (tid == 0) v.seg_start[n_seg] = n_lora;
+  // chunks: every kSegChunk-th position of a segment starts one
+  const int my_seg = seg + is_start - 1;                     // segment of this sorted position (seg counts the starts before it)
+  const int in_seg = tid < n_lora ? tid - s_sort[my_seg] : 1;
+  int n_chunk;
+  const int chunk = block_excl_sum<NT>((in_seg % kSegChunk) == 0, smem, &n_chunk);
+  if ((in_seg % kSegChunk) == 0) v.chunk_tab[chunk] = make_int4(id, tid, min(kSegChunk, s_sort[my_seg + 1] - tid), 0);
   const int max_seg = block_incl_max<NT>(len, smem);
   if (tid == NT - 1) {
     v.header[PH_NSEG] = n_seg;
+    v.header[PH_NCHUNK] = n_chunk;
     v.header[PH_NLORA] = n_lora;
     v.header[PH_MAXSEG] = max_seg;
     v.header[PH_T] = T;
     v.header[PH_E] = E;
   }
-  if (want_tiles) plan_tiles<NT>(v, s_key, smem, s_carry, s_row0);
+  if (want_tiles) plan_tiles<NT>(v, s_key, smem, s_row0);
   else if (tid == 0) v.header[PH_NTILES] = 0;
 }
 
@@ -310,6 +367,11 @@ __global__ void __launch_bounds__(kPlanChunk) plan_scatter_kernel(PlanView v) {
   const int k = v.key[t];
   const int pos = v.keybase[k] + v.hist[(size_t)blockIdx.x * (size_t)(v.E + 1) + k] + v.rank[t];
   v.perm[pos] = t;
+  if (k < v.E) {
+    const int in_seg = pos - v.keybase[k];
+    if ((in_seg % kSegChunk) == 0)
+      v.chunk_tab[v.chunkbase[k] + in_seg / kSegChunk] = make_int4(k, pos, min(kSegChunk, v.keybase[k + 1] - pos), 0);
+  }
 }
 
 int plan_launches(int T, int E) {

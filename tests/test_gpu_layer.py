@@ -338,3 +338,17 @@ def test_base_gemm_few_tokens(T, d_in, d_out):
     # one rounding to bf16 (2^-9 of the value) on top of fp32 sums of at most 2048 products of size 0.02
     assert ((y.double() - ref).abs() <= ref.abs() * 2 ** -8 + 2e-5).all()
     assert moin.device_status()["timeout_flag"] == 0
+
+
+@pytest.mark.parametrize("counts", [[8, 9, 7, 16, 1, 17], [264], [1, 0, 1000, 8], [700, 700, 3], [0, 0, 5]])
+def test_segments_in_chunks(counts):
+    # segments around the 8-token chunk of the stream kernels, in batches of up to and of more than 1024 tokens (the two
+    # plan builders), with base-only tokens among them
+    E = len(counts)
+    te = np.repeat(np.arange(E, dtype=np.int32), counts)
+    te = np.concatenate([te, np.full(6, -1, np.int32)])
+    te = te[np.random.default_rng(len(te)).permutation(len(te))]
+    pool = mi.make_pool(E, 24, 128, 200, 41, E)
+    case = mi.layer_case("chunks", len(te), 128, 200, pool, te, 2.0, 41, len(te))
+    y, _ = run_layer(case, moin.PLAN_SEGMENTS)
+    assert_layer_close(y, oracle_layer(case))
