@@ -291,8 +291,8 @@ moin_status moin_plan_read(const moin_plan* plan, int32_t* n_segments, int32_t* 
  * document embeddings; Sec. 4: the cluster centroid is the topic embedding the router searches.
  * One Lloyd iteration over N points is moin_route (assignment: nearest centroid under the cosine
  * metric), moin_plan_build on the N assignments with E = K (grouping of the points by cluster),
- * then this call: centroid k <- arithmetic mean of its members, summed in increasing point order
- * in fp32 and rounded once to bf16.  A cluster without members keeps its previous centroid;
+ * then this call: centroid k <- arithmetic mean of its members, summed in fp32 in a fixed order (the
+ * members in increasing point order, cut into parts whose sums are added) and rounded once to bf16.  A cluster without members keeps its previous centroid;
  * points whose assignment is outside [0, K) belong to no cluster.
  *
  *   plan           built from the assignments (plan->T = N points, plan->E = K clusters), any mode

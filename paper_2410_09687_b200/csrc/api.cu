@@ -389,16 +389,16 @@ moin_status moin_kmeans_update(const moin_plan* plan, const void* x, const void*
   if (st) return st;
   cudaStream_t s = (cudaStream_t)stream;
   const int K = plan->E;
-  if (centroids_new != centroids_old) {   // clusters without members keep their centroid
-    cudaError_t e = cudaMemcpyAsync(centroids_new, centroids_old, (size_t)K * (size_t)D * sizeof(__nv_bfloat16),
-                                    cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return record_cuda(e);
-  }
   if (plan->T > 0) {
     PlanView pv = plan_view(plan->buffer, plan->T, plan->E);
     ProfScope prof(MOIN_K_KMEANS_UPDATE, 1, s);
-    st = record_cuda(launch_kmeans_mean(pv, (const __nv_bfloat16*)x, (__nv_bfloat16*)centroids_new, D, hs->n_sms, s));
-    if (st) return st;
+    return record_cuda(launch_kmeans_update(pv, (const __nv_bfloat16*)x, (const __nv_bfloat16*)centroids_old,
+                                            (__nv_bfloat16*)centroids_new, inv_norm_new, D, hs->n_sms, s));
+  }
+  if (centroids_new != centroids_old) {   // no points: every cluster keeps its centroid
+    cudaError_t e = cudaMemcpyAsync(centroids_new, centroids_old, (size_t)K * (size_t)D * sizeof(__nv_bfloat16),
+                                    cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) return record_cuda(e);
   }
   if (inv_norm_new) {
     ProfScope prof(MOIN_K_GLUE, 1, s);

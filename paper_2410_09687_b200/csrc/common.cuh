@@ -182,8 +182,8 @@ cudaError_t launch_route_finish_top2(const unsigned long long* keys, const unsig
                                      const __nv_bfloat16* q, const int* cmap, int Q, int D, int* out_expert,
                                      int* out_centroid, int* out_second, float* out_best, float* out_margin,
                                      cudaStream_t stream);
-cudaError_t launch_kmeans_mean(const PlanView& pv, const __nv_bfloat16* x, __nv_bfloat16* c_new, int D, int n_sms,
-                               cudaStream_t stream);
+cudaError_t launch_kmeans_update(const PlanView& pv, const __nv_bfloat16* x, const __nv_bfloat16* c_old,
+                                 __nv_bfloat16* c_new, float* inv_new, int D, int n_sms, cudaStream_t stream);
 cudaError_t launch_inv_norm(const __nv_bfloat16* c, int K, int D, float* inv_norm, cudaStream_t stream);
 cudaError_t launch_route_simple(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                 const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,

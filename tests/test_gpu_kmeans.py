@@ -98,3 +98,22 @@ def test_lloyd_iterations_on_planted_clusters():
     cos = (got * planted).sum(1) / (np.linalg.norm(got, axis=1) * np.linalg.norm(planted, axis=1))
     assert cos.min() > 0.99
     assert moin.device_status()["timeout_flag"] == 0
+
+
+@pytest.mark.parametrize("N,K,D", [(5000, 3, 768), (300, 290, 1096), (2000, 40, 64), (1500, 7, 120), (40, 64, 2304), (1030, 1, 8)])
+def test_update_shapes(N, K, D):
+    # few large clusters (parts of a cluster per warp), many of one or no member (empty ones before, between and behind),
+    # rows of fewer than 32 chunks (several members per warp load), rows wider than a CTA's column groups
+    rng = np.random.default_rng(N + K)
+    x = torch.from_numpy(rng.normal(size=(N, D)).astype(np.float32)).to(torch.bfloat16)
+    c_old = torch.from_numpy(rng.normal(size=(K, D)).astype(np.float32)).to(torch.bfloat16)
+    assign = rng.integers(0, K, size=N).astype(np.int32)
+    if K > 20:
+        assign[assign < 2] = 5
+        assign[assign >= K - 3] = 7
+    c_new, inv = _gpu_update(x, c_old, assign, K)
+    ref = oracle.kmeans_update(mi.bf16_bits(x), mi.bf16_bits(c_old), assign)
+    _assert_centroids_close(c_new, ref["centroids"], f"update {N}x{K}x{D}")
+    got = mi.bf16_to_f64(c_new)
+    norms = np.sqrt((got ** 2).sum(1))
+    np.testing.assert_allclose(inv.cpu().numpy(), 1.0 / norms, rtol=2e-6)
