@@ -169,6 +169,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     tmem_alloc(smem_u32(tmem_slot), kAtTmemCols);
     tmem_relinquish();
   }
+  pdl_begin();   // (the set-up above overlaps the tail of the kernel before)
   if (p.cu_smem)
     for (int i = threadIdx.x; i <= p.R; i += kAtThreads) cu_s[i] = __ldg(p.cu + i);
   tc_fence_before();
@@ -669,8 +670,7 @@ moin_status launch_attention_tc(HostState* hs, const __nv_bfloat16* q, const __n
   const long items = (long)p.n_qb * R * n_kv_heads;
   long grid = items < 2L * hs->n_sms ? items : 2L * hs->n_sms;
   if (grid < 1) grid = 1;
-  attention_tc_kernel<<<(int)grid, kAtThreads, kAtSmem, stream>>>(mk, mv, p);
-  return record_cuda(cudaGetLastError());
+  return record_cuda(launch_pdl(attention_tc_kernel, (unsigned)grid, kAtThreads, kAtSmem, stream, mk, mv, p));
 }
 
 }  // namespace moin

@@ -124,17 +124,25 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // Programmatic dependent launch: the next kernel of the stream may start once every CTA has got here / this CTA goes
-// on once the kernels before it are complete and their writes visible (no-ops in an ordinary launch).
+// on once the kernels before it are complete and their writes visible (no-ops in an ordinary launch).  The kernels of a
+// call are launched this way, so that a kernel's launch latency and set-up lie under the tail of the one before it
+// (about 2 us each).  Rule: a kernel waits before it touches global memory and lets the next one start only after that
+// - then everything before a running kernel is complete but the kernel right before it.  The adapter shrink beside the
+// decode GEMM is the one exception; lora_stream.cu says how it keeps the order.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launch as the programmatic dependent of the kernel before it in the stream: the grid may start as soon as every CTA
-// of that kernel has called pdl_launch_dependents (or ended); what depends on it waits with pdl_wait.
+__device__ __forceinline__ void pdl_begin() {
+  pdl_wait();
+  pdl_launch_dependents();
+}
+// Launch as the programmatic dependent of the kernel before it in the stream.
 template <class... P, class... A>
-inline cudaError_t launch_dependent(void (*fn)(P...), int grid, int threads, cudaStream_t stream, A... args) {
+inline cudaError_t launch_pdl(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -11,6 +11,7 @@ __global__ void __launch_bounds__(256)
 token_meta_kernel(const int* __restrict__ cu, const int* __restrict__ req_expert,
                   const int* __restrict__ token_expert_in, int R, int* __restrict__ pos,
                   int* __restrict__ token_expert, int* __restrict__ last_row) {
+  pdl_begin();
   const int r = blockIdx.x;
   if (r >= R) return;
   const int t0 = cu[r], t1 = cu[r + 1];
@@ -33,6 +34,7 @@ __device__ __forceinline__ float e4m3_to_float(uint32_t c) {
 __global__ void __launch_bounds__(256)
 dequant_fp8_kernel(const uint4* __restrict__ codes, const float* __restrict__ scale, int d_in16, long n16,
                    uint4* __restrict__ out) {
+  pdl_begin();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n16) return;
   const float sc = __ldg(scale + i / d_in16);
@@ -52,6 +54,7 @@ dequant_fp8_kernel(const uint4* __restrict__ codes, const float* __restrict__ sc
 
 // cos/sin of pos * base^(-2i/hd), computed in double once per call.
 __global__ void rope_table_kernel(float2* __restrict__ table, int n_pos, int half, double base) {
+  pdl_begin();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_pos * half) return;
   const int p = idx / half, i = idx - p * half;
@@ -62,6 +65,7 @@ __global__ void rope_table_kernel(float2* __restrict__ table, int n_pos, int hal
 __global__ void __launch_bounds__(256)
 embed_kernel(const int* __restrict__ tokens, const __nv_bfloat16* __restrict__ embed, int hidden, int vocab,
              float* __restrict__ res) {
+  pdl_begin();
   const int t = blockIdx.x;
   int tok = tokens[t];
   tok = tok < 0 ? 0 : (tok >= vocab ? vocab - 1 : tok);
@@ -82,6 +86,7 @@ add_rmsnorm_kernel(float* __restrict__ res, const __nv_bfloat16* __restrict__ ad
                    const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ out, int hidden, float eps,
                    const int* __restrict__ rows) {
   __shared__ float s_part[8];
+  pdl_begin();
   const int b = blockIdx.x;
   const int t = rows ? rows[b] : b;
   if (t < 0) return;
@@ -118,6 +123,7 @@ add_rmsnorm_kernel(float* __restrict__ res, const __nv_bfloat16* __restrict__ ad
 __global__ void __launch_bounds__(256)
 rope_kernel(__nv_bfloat16* __restrict__ v, const int* __restrict__ pos, const float2* __restrict__ table, int T,
             int n_h) {
+  pdl_begin();
   const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;  // (t, head, i)
   const long total = (long)T * n_h * 32;
   if (idx >= total) return;
@@ -133,6 +139,7 @@ rope_kernel(__nv_bfloat16* __restrict__ v, const int* __restrict__ pos, const fl
 
 __global__ void __launch_bounds__(256)
 swiglu_kernel(__nv_bfloat16* __restrict__ gate, const __nv_bfloat16* __restrict__ up, long n8) {
+  pdl_begin();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n8) return;
   const uint4 gv = *reinterpret_cast<const uint4*>(gate + i * 8);
@@ -404,8 +411,8 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
   const int qd = nh * 64, kvd = nkv * 64;
 
   { ProfScope prof(MOIN_K_GLUE, 2, s);
-  token_meta_kernel<<<R, 256, 0, s>>>(cu_seqlens, req_expert, token_expert_in, R, w.pos, w.token_expert, w.last_row);
-  rope_table_kernel<<<(max_seqlen * 32 + 255) / 256, 256, 0, s>>>(w.rope, max_seqlen, 32, (double)m->rope_base); }
+  launch_pdl(token_meta_kernel, R, 256, 0, s, cu_seqlens, req_expert, token_expert_in, R, w.pos, w.token_expert, w.last_row);
+  launch_pdl(rope_table_kernel, (max_seqlen * 32 + 255) / 256, 256, 0, s, w.rope, max_seqlen, 32, (double)m->rope_base); }
   moin_plan plan;
   memset(&plan, 0, sizeof(plan));
   const bool lora = m->pools != nullptr && (req_expert != nullptr || token_expert_in != nullptr);
@@ -422,7 +429,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     if (e != cudaSuccess) return record_cuda(e);
   } else {
     ProfScope prof(MOIN_K_GLUE, 1, s);
-    embed_kernel<<<T, 256, 0, s>>>(tokens, (const __nv_bfloat16*)m->embed, H, m->vocab, w.res);
+    launch_pdl(embed_kernel, T, 256, 0, s, tokens, (const __nv_bfloat16*)m->embed, H, m->vocab, w.res);
   }
   // weight of projection p: the caller's bf16 matrix, or - quantised base - its codes dequantised into scratch slot
   // `slot` on the call's stream (the group calls join their side streams before they return, so a slot is free again)
@@ -460,7 +467,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
   const __nv_bfloat16* pending = nullptr;
   for (int l = lb; l < le; ++l) {
     { ProfScope prof(MOIN_K_GLUE, 1, s);
-      add_rmsnorm_kernel<<<T, 256, 0, s>>>(w.res, pending, (const __nv_bfloat16*)m->attn_norm[l], w.xn, H, m->rms_eps, nullptr); }
+      launch_pdl(add_rmsnorm_kernel, T, 256, 0, s, w.res, pending, (const __nv_bfloat16*)m->attn_norm[l], w.xn, H, m->rms_eps, nullptr); }
     {
       const int din[3] = {H, H, H}, dout[3] = {qd, kvd, kvd};
       void* const outs[3] = {w.q, w.k, w.v};
@@ -469,7 +476,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     // rotary embedding: the keys are rotated in place once (every query head and every later query reads them);
     // the queries are rotated inside the attention kernel as it loads them
     { ProfScope prof(MOIN_K_GLUE, 1, s);
-      rope_kernel<<<(int)(((long)T * nkv * 32 + 255) / 256), 256, 0, s>>>(w.k, w.pos, w.rope, T, nkv); }
+      launch_pdl(rope_kernel, (int)(((long)T * nkv * 32 + 255) / 256), 256, 0, s, w.k, w.pos, w.rope, T, nkv); }
     if (hs->gemm_impl != 1 && attention_tc_supported(nh, nkv, m->head_dim)) {   // tcgen05 kernel
       ProfScope prof(MOIN_K_ATTENTION, 1, s);
       if ((st = launch_attention_tc(hs, w.q, w.k, w.v, cu_seqlens, w.att, w.rope, R, T, max_seqlen, nh, nkv,
@@ -482,33 +489,33 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     }
     if ((st = proj(l, 3, w.att, qd, H, w.o))) return st;
     { ProfScope prof(MOIN_K_GLUE, 1, s);
-      add_rmsnorm_kernel<<<T, 256, 0, s>>>(w.res, w.o, (const __nv_bfloat16*)m->mlp_norm[l], w.xn, H, m->rms_eps, nullptr); }
+      launch_pdl(add_rmsnorm_kernel, T, 256, 0, s, w.res, w.o, (const __nv_bfloat16*)m->mlp_norm[l], w.xn, H, m->rms_eps, nullptr); }
     {
       const int din[2] = {H, H}, dout[2] = {F, F};
       void* const outs[2] = {w.gate, w.up};
       if ((st = proj_group(l, 4, 2, w.xn, din, dout, outs))) return st;
     }
     { ProfScope prof(MOIN_K_GLUE, 1, s);
-      swiglu_kernel<<<(int)(((long)T * F / 8 + 255) / 256), 256, 0, s>>>(w.gate, w.up, (long)T * F / 8); }
+      launch_pdl(swiglu_kernel, (int)(((long)T * F / 8 + 255) / 256), 256, 0, s, w.gate, w.up, (long)T * F / 8); }
     if ((st = proj(l, 6, w.gate, F, H, w.o))) return st;
     pending = w.o;
   }
   if (pending) { ProfScope prof(MOIN_K_GLUE, 1, s);
-    add_rmsnorm_kernel<<<T, 256, 0, s>>>(w.res, pending, nullptr, nullptr, H, m->rms_eps, nullptr); }
+    launch_pdl(add_rmsnorm_kernel, T, 256, 0, s, w.res, pending, nullptr, nullptr, H, m->rms_eps, nullptr); }
   if (taps && taps->hidden_out) {
     cudaError_t e = cudaMemcpyAsync(taps->hidden_out, w.res, (size_t)T * H * 4, cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return record_cuda(e);
   }
   if (logits_mode == MOIN_LOGITS_ALL) {
     { ProfScope prof(MOIN_K_GLUE, 1, s);
-      add_rmsnorm_kernel<<<T, 256, 0, s>>>(w.res, nullptr, (const __nv_bfloat16*)m->final_norm, w.xn, H, m->rms_eps, nullptr); }
+      launch_pdl(add_rmsnorm_kernel, T, 256, 0, s, w.res, nullptr, (const __nv_bfloat16*)m->final_norm, w.xn, H, m->rms_eps, nullptr); }
     st = moin_lora_linear(nullptr, w.xn, m->lm_head, nullptr, 0.f, T, H, m->vocab, logits, w.lora, w.lora_bytes, stream);
     if (st) return st;
   } else if (logits_mode == MOIN_LOGITS_LAST) {
     cudaError_t e = cudaMemsetAsync(w.xlast, 0, (size_t)R * H * 2, s);
     if (e != cudaSuccess) return record_cuda(e);
     { ProfScope prof(MOIN_K_GLUE, 1, s);
-      add_rmsnorm_kernel<<<R, 256, 0, s>>>(w.res, nullptr, (const __nv_bfloat16*)m->final_norm, w.xlast, H, m->rms_eps, w.last_row); }
+      launch_pdl(add_rmsnorm_kernel, R, 256, 0, s, w.res, nullptr, (const __nv_bfloat16*)m->final_norm, w.xlast, H, m->rms_eps, w.last_row); }
     st = moin_lora_linear(nullptr, w.xlast, m->lm_head, nullptr, 0.f, R, H, m->vocab, logits, w.lora, w.lora_bytes, stream);
     if (st) return st;
   }
@@ -544,7 +551,6 @@ extern "C" moin_status moin_dequant_fp8(const void* codes, const float* scale, i
   moin_status st = host_state(&hs);
   if (st) return st;
   ProfScope prof(MOIN_K_GLUE, 1, (cudaStream_t)stream);
-  dequant_fp8_kernel<<<(unsigned)((n16 + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
-      (const uint4*)codes, scale, d_in / 16, n16, (uint4*)W);
-  return record_cuda(cudaGetLastError());
+  return record_cuda(launch_pdl(dequant_fp8_kernel, (unsigned)((n16 + 255) / 256), 256, 0, (cudaStream_t)stream,
+                                (const uint4*)codes, scale, d_in / 16, n16, (uint4*)W));
 }

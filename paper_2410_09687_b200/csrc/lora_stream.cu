@@ -321,8 +321,8 @@ cudaError_t launch_lora_shrink_stream(const PlanView& pv, ShrinkJobs jobs, int n
     items += (long)pv.Cmax * jobs.per_seg[j];
   }
   // one CTA per item (capped; CTAs stride over the items beyond the cap)
-  return launch_dependent(lora_shrink_stream_kernel, stream_grid(items, n_sms, 1024), kShrinkThreads, stream, pv.header,
-                          pv.perm, pv.chunk_tab, jobs);
+  return launch_pdl(lora_shrink_stream_kernel, stream_grid(items, n_sms, 1024), kShrinkThreads, 0, stream, pv.header,
+                    pv.perm, pv.chunk_tab, jobs);
 }
 
 cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float scale, int n_sms,
@@ -340,7 +340,7 @@ cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float
   bool var = false;
   for (int j = 0; j < jobs.n; ++j) var = var || jobs.slot_rank[j] != nullptr || jobs.act[j] != MOIN_ACT_NONE;
   auto go = [&](auto* fn) {
-    return launch_dependent(fn, grid, kExpandThreads, stream, pv.header, pv.perm, pv.chunk_tab, jobs, scale, tps);
+    return launch_pdl(fn, grid, kExpandThreads, 0, stream, pv.header, pv.perm, pv.chunk_tab, jobs, scale, tps);
   };
   if (rmax <= 32) return var ? go(lora_expand_stream_kernel<1, true>) : go(lora_expand_stream_kernel<1, false>);
   if (rmax <= 64) return var ? go(lora_expand_stream_kernel<2, true>) : go(lora_expand_stream_kernel<2, false>);

@@ -17,6 +17,9 @@ __global__ void __launch_bounds__(kPlanChunk) plan_rank_kernel(const int* __rest
                                                                int* __restrict__ hist, DeviceStatus* status) {
   __shared__ int skey[kPlanChunk];
   const int tid = threadIdx.x;
+  pdl_begin();
+  int* row = hist + (size_t)blockIdx.x * (size_t)(E + 1);   // this chunk's counts: cleared here, no separate launch
+  for (int i = tid; i <= E; i += kPlanChunk) row[i] = 0;
   const int t = blockIdx.x * kPlanChunk + tid;
   int k = -2;  // padding lanes never match
   if (t < T) {
@@ -39,7 +42,7 @@ __global__ void __launch_bounds__(kPlanChunk) plan_rank_kernel(const int* __rest
   }
   key[t] = k;
   rank[t] = before;
-  if (after == 0) hist[(size_t)blockIdx.x * (size_t)(E + 1) + k] = before + 1;
+  if (after == 0) row[k] = before + 1;
 }
 
 // Block-wide scans for NT threads (a multiple of 32, at most 1024).  `smem` must hold 33 ints.
@@ -103,6 +106,7 @@ __device__ __forceinline__ int block_incl_max(int v, int* smem) {
 constexpr int kPrefixIds = 64, kPrefixGroups = 4, kPrefixBatch = 16;
 __global__ void __launch_bounds__(kPrefixIds * kPrefixGroups) plan_prefix_kernel(PlanView v) {
   __shared__ int s_sum[kPrefixGroups][kPrefixIds];
+  pdl_begin();
   const int k = blockIdx.x * kPrefixIds + threadIdx.x, g = threadIdx.y;
   const bool on = k <= v.E;
   const size_t pitch = (size_t)(v.E + 1);
@@ -217,6 +221,7 @@ __device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, in
 __global__ void __launch_bounds__(1024) plan_scan_kernel(PlanView v, int do_prefix, int want_tiles) {
   constexpr int NT = 1024;
   __shared__ int smem[33];
+  pdl_begin();
   const int tid = threadIdx.x;
   const int T = v.T, E = v.E, nc = v.n_chunks;
   const size_t pitch = (size_t)(E + 1);
@@ -292,6 +297,7 @@ __global__ void __launch_bounds__(NT) plan_small_kernel(const int* __restrict__ 
   __shared__ int s_sort[NT + 1];   // sort keys, then the segment starts plus one end marker (NT segments at most)
   __shared__ int s_row0[NT + 1];   // tile starts
   __shared__ int smem[33];
+  pdl_begin();
   const int tid = threadIdx.x;
   const int T = v.T, E = v.E;
   int k = 0x1FFFFF;  // padding sorts last
@@ -362,6 +368,7 @@ __global__ void __launch_bounds__(NT) plan_small_kernel(const int* __restrict__ 
 }
 
 __global__ void __launch_bounds__(kPlanChunk) plan_scatter_kernel(PlanView v) {
+  pdl_begin();
   const int t = blockIdx.x * kPlanChunk + threadIdx.x;
   if (t >= v.T) return;
   const int k = v.key[t];
@@ -382,19 +389,17 @@ int plan_launches(int T, int E) {
 cudaError_t launch_plan_build(const int* token_expert, const PlanView& v, DeviceStatus* status, bool want_tiles,
                               cudaStream_t stream) {
   if (v.T <= kPlanSmallT && v.E < kPlanSmallE) {
-    if (v.T <= 128) plan_small_kernel<128><<<1, 128, 0, stream>>>(token_expert, v, status, want_tiles);
-    else if (v.T <= 256) plan_small_kernel<256><<<1, 256, 0, stream>>>(token_expert, v, status, want_tiles);
-    else if (v.T <= 512) plan_small_kernel<512><<<1, 512, 0, stream>>>(token_expert, v, status, want_tiles);
-    else plan_small_kernel<1024><<<1, 1024, 0, stream>>>(token_expert, v, status, want_tiles);
-    return cudaGetLastError();
+    const int tiles = want_tiles;
+    if (v.T <= 128) return launch_pdl(plan_small_kernel<128>, 1, 128, 0, stream, token_expert, v, status, tiles);
+    if (v.T <= 256) return launch_pdl(plan_small_kernel<256>, 1, 256, 0, stream, token_expert, v, status, tiles);
+    if (v.T <= 512) return launch_pdl(plan_small_kernel<512>, 1, 512, 0, stream, token_expert, v, status, tiles);
+    return launch_pdl(plan_small_kernel<1024>, 1, 1024, 0, stream, token_expert, v, status, tiles);
   }
-  cudaError_t e = cudaMemsetAsync(v.hist, 0, sizeof(int) * (size_t)v.n_chunks * (size_t)(v.E + 1), stream);
-  if (e != cudaSuccess) return e;
-  plan_rank_kernel<<<v.n_chunks, kPlanChunk, 0, stream>>>(token_expert, v.T, v.E, v.key, v.rank, v.hist, status);
+  launch_pdl(plan_rank_kernel, v.n_chunks, kPlanChunk, 0, stream, token_expert, v.T, v.E, v.key, v.rank, v.hist, status);
   if (v.n_chunks > 1)
-    plan_prefix_kernel<<<(v.E + 1 + kPrefixIds - 1) / kPrefixIds, dim3(kPrefixIds, kPrefixGroups), 0, stream>>>(v);
-  plan_scan_kernel<<<1, 1024, 0, stream>>>(v, v.n_chunks > 1 ? 0 : 1, want_tiles);
-  plan_scatter_kernel<<<v.n_chunks, kPlanChunk, 0, stream>>>(v);
+    launch_pdl(plan_prefix_kernel, (v.E + 1 + kPrefixIds - 1) / kPrefixIds, dim3(kPrefixIds, kPrefixGroups), 0, stream, v);
+  launch_pdl(plan_scan_kernel, 1, 1024, 0, stream, v, v.n_chunks > 1 ? 0 : 1, (int)want_tiles);
+  launch_pdl(plan_scatter_kernel, v.n_chunks, kPlanChunk, 0, stream, v);
   return cudaGetLastError();
 }
 

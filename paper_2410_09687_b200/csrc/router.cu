@@ -11,6 +11,7 @@ namespace moin {
 // inv_norm[k] = 1/|c_k| (0 for a zero row).  One warp per centroid.
 __global__ void __launch_bounds__(256)
 centroid_inv_norm_kernel(const __nv_bfloat16* __restrict__ c, int K, int D, float* __restrict__ inv_norm) {
+  pdl_begin();
   const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (k >= K) return;
   const __nv_bfloat16* row = c + (size_t)k * D;
@@ -128,6 +129,7 @@ __global__ void __launch_bounds__(256)
 route_finish_kernel(const unsigned long long* __restrict__ keys, const __nv_bfloat16* __restrict__ q,
                     const int* __restrict__ cmap, int Q, int D, int* __restrict__ out_expert,
                     int* __restrict__ out_centroid, float* __restrict__ out_best) {
+  pdl_begin();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= Q) return;
   const unsigned long long key = keys[i];
@@ -229,7 +231,7 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long s_keys[NQ], s_keys2[NQ];
   __shared__ float s_part[kRcWarps / 2][NJ][4][32];
-  pdl_launch_dependents();
+  pdl_begin();
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const int rank = (int)cluster.block_rank(), csize = (int)cluster.num_blocks();
@@ -454,7 +456,7 @@ route_parts_kernel(const unsigned long long* __restrict__ part_keys, int parts, 
   float ss = 0.f;
   if (on && (out.best || out.margin))
     for (int ch = sub; ch < D / 8; ch += 8) add_sq8(ldg_cached(q + (size_t)i * D + ch * 8), ss);
-  pdl_wait();   // the parts' keys
+  pdl_begin();   // the parts' keys (the queries above are older: the kernel before this one has waited for them)
   unsigned long long k1 = 0ull, k2 = 0ull;
   if (on) {
     for (int r = sub; r < parts; r += 8) {
@@ -512,20 +514,22 @@ static cudaError_t launch_rc(int optin, const RouteCut& cut, const __nv_bfloat16
   const size_t smem = (size_t)NQ * route_pitch(D);
   cudaError_t ce = ensure_smem_optin(optin, route_cluster_kernel<NQ, TOP2>, smem > 64 * 1024 ? smem : 64 * 1024);
   if (ce != cudaSuccess) return ce;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = cut.csize;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(cut.groups * cut.parts * cut.csize));
   cfg.blockDim = dim3(kRcWarps * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   ce = cudaLaunchKernelEx(&cfg, route_cluster_kernel<NQ, TOP2>, q, c, inv_norm, cmap, Q, K, D, cut.parts, part_keys, out);
   if (ce != cudaSuccess || cut.parts == 1) return ce;
-  return launch_dependent(route_parts_kernel<TOP2>, (Q + 15) / 16, 128, stream, part_keys, cut.parts, q, cmap, Q, D, out);
+  return launch_pdl(route_parts_kernel<TOP2>, (Q + 15) / 16, 128, 0, stream, part_keys, cut.parts, q, cmap, Q, D, out);
 }
 
 cudaError_t launch_route_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
@@ -565,6 +569,7 @@ kmeans_update_kernel(const int* __restrict__ header, const int* __restrict__ per
                      float* __restrict__ inv_new, int K, int D, int G, int P) {
   __shared__ float4 s_acc[kMeanMaxWarps][2][32];
   __shared__ float s_ss[kMeanMaxWarps];
+  pdl_begin();
   const int nseg = header[PH_NSEG];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
   const int g = warp % G, part = warp / G, nch = D / 8;
@@ -664,8 +669,8 @@ cudaError_t launch_kmeans_update(const PlanView& pv, const __nv_bfloat16* x, con
   P = P < 1 ? 1 : P > kMeanMaxWarps / G ? kMeanMaxWarps / G : P;
   long grid = pv.Smax < (long)n_sms * 16 ? pv.Smax : (long)n_sms * 16;
   if (grid < 1) grid = 1;
-  kmeans_update_kernel<<<dim3((unsigned)grid, split ? (unsigned)groups : 1u), 32 * G * P, 0, stream>>>(
-      pv.header, pv.perm, pv.seg_tab, x, c_old, c_new, split ? nullptr : inv_new, pv.E, D, G, P);
+  launch_pdl(kmeans_update_kernel, dim3((unsigned)grid, split ? (unsigned)groups : 1u), 32 * G * P, 0, stream,
+             pv.header, pv.perm, pv.seg_tab, x, c_old, c_new, split ? nullptr : inv_new, pv.E, D, G, P);
   if (split && inv_new != nullptr) return launch_inv_norm(c_new, pv.E, D, inv_new, stream);
   return cudaGetLastError();
 }
@@ -728,6 +733,7 @@ route_finish_top2_kernel(const unsigned long long* __restrict__ keys, const unsi
                          const __nv_bfloat16* __restrict__ q, const int* __restrict__ cmap, int Q, int D,
                          int* __restrict__ out_expert, int* __restrict__ out_centroid, int* __restrict__ out_second,
                          float* __restrict__ out_best, float* __restrict__ out_margin) {
+  pdl_begin();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= Q) return;
   const unsigned long long k1 = keys[i], k2 = keys2[i];
@@ -765,13 +771,13 @@ cudaError_t launch_route_finish_top2(const unsigned long long* keys, const unsig
                                      const __nv_bfloat16* q, const int* cmap, int Q, int D, int* out_expert,
                                      int* out_centroid, int* out_second, float* out_best, float* out_margin,
                                      cudaStream_t stream) {
-  route_finish_top2_kernel<<<(Q + 7) / 8, 256, 0, stream>>>(keys, keys2, q, cmap, Q, D, out_expert, out_centroid, out_second,
+  launch_pdl(route_finish_top2_kernel, (Q + 7) / 8, 256, 0, stream, keys, keys2, q, cmap, Q, D, out_expert, out_centroid, out_second,
                                                            out_best, out_margin);
   return cudaGetLastError();
 }
 
 cudaError_t launch_inv_norm(const __nv_bfloat16* c, int K, int D, float* inv_norm, cudaStream_t stream) {
-  centroid_inv_norm_kernel<<<(K + 7) / 8, 256, 0, stream>>>(c, K, D, inv_norm);
+  launch_pdl(centroid_inv_norm_kernel, (K + 7) / 8, 256, 0, stream, c, K, D, inv_norm);
   return cudaGetLastError();
 }
 
@@ -790,6 +796,7 @@ cudaError_t launch_route_simple(const __nv_bfloat16* q, const __nv_bfloat16* c, 
 __global__ void __launch_bounds__(256)
 route_finish_ids_kernel(const unsigned long long* __restrict__ keys, const int* __restrict__ cmap, int Q,
                         int* __restrict__ out_expert, int* __restrict__ out_centroid) {
+  pdl_begin();
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= Q) return;
   const unsigned long long key = keys[i];
@@ -801,9 +808,9 @@ route_finish_ids_kernel(const unsigned long long* __restrict__ keys, const int* 
 cudaError_t launch_route_finish(const unsigned long long* keys, const __nv_bfloat16* q, const int* cmap, int Q, int D,
                                 int* out_expert, int* out_centroid, float* out_best, cudaStream_t stream) {
   if (out_best == nullptr)
-    route_finish_ids_kernel<<<(Q + 255) / 256, 256, 0, stream>>>(keys, cmap, Q, out_expert, out_centroid);
+    launch_pdl(route_finish_ids_kernel, (Q + 255) / 256, 256, 0, stream, keys, cmap, Q, out_expert, out_centroid);
   else
-    route_finish_kernel<<<(Q + 7) / 8, 256, 0, stream>>>(keys, q, cmap, Q, D, out_expert, out_centroid, out_best);
+    launch_pdl(route_finish_kernel, (Q + 7) / 8, 256, 0, stream, keys, q, cmap, Q, D, out_expert, out_centroid, out_best);
   return cudaGetLastError();
 }
 

@@ -129,6 +129,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();   // (the set-up above overlaps the tail of the kernel before)
 
   const bool planned = p.header != nullptr;
   const int tiles_n = (p.N + BN - 1) / BN;
@@ -429,8 +430,8 @@ static moin_status launch_cfg(HostState* hs, const CUtensorMap& a, const CUtenso
   if (grid < 1) grid = 1;
   const int threads = lean ? kTcThreadsLean : kTcThreads;
   const size_t smem = lean ? Cfg::kSmemBytes - Cfg::kOutBytes : Cfg::kSmemBytes;   // (lean launches never stage)
-  tc_gemm_kernel<BN, EPI><<<(int)grid, threads, smem, stream>>>(a, b, a2, a3, b2, b3 ? *b3 : b2, ymap ? *ymap : a, p);
-  return record_cuda(cudaGetLastError());
+  return record_cuda(launch_pdl(tc_gemm_kernel<BN, EPI>, (unsigned)grid, threads, smem, stream, a, b, a2, a3, b2,
+                                b3 ? *b3 : b2, ymap ? *ymap : a, p));
 }
 
 // Tile width for many row tiles: the one with the least (waves of tiles over the SMs) x (time of one tile), a

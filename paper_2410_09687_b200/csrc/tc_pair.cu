@@ -151,6 +151,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
   cluster_wait();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();   // (the set-up above overlaps the tail of the kernel before)
 
   const int tiles_m = p.header != nullptr ? p.header[PH_NTILES] : (p.M + kPairM - 1) / kPairM;
   const int total = (tiles_m + 1) / 2 * p.tn_end[p.n_jobs - 1];
@@ -427,8 +428,7 @@ static moin_status launch_pair(HostState* hs, const PairMaps& maps, const PairPa
   if (e != cudaSuccess) return record_cuda(e);
   long pairs = max_tiles < hs->n_sms / 2 ? max_tiles : hs->n_sms / 2;
   if (pairs < 1) pairs = 1;
-  tc_pair_kernel<EPI><<<(unsigned)(2 * pairs), kPairThreads, kPairSmem, stream>>>(maps, p);
-  return record_cuda(cudaGetLastError());
+  return record_cuda(launch_pdl(tc_pair_kernel<EPI>, (unsigned)(2 * pairs), kPairThreads, kPairSmem, stream, maps, p));
 }
 
 // Tile width: the one with the least (waves of pair tiles over the SM pairs) x (time of one tile).  Per k-block an SM
