@@ -17,7 +17,7 @@ constexpr int kShrinkThreads = 128;      // 4 warps split the reduction dimensio
 constexpr int kShrinkWarps = kShrinkThreads / 32;
 constexpr int kShrinkUnroll = 4;         // 32-wide k steps in flight per warp
 constexpr int kExpandThreads = 128;      // 4 warps
-constexpr int kExpandTilesPerBatch = 2;  // 16-row tiles whose loads are in flight together, per warp
+constexpr int kExpandFirst = 4;          // 16-row tiles prefetched while a warp waits for the shrink
 
 // The unit both kernels work on is a CHUNK of the plan: at most 8 tokens (the columns of one MMA) of one expert.  A
 // longer segment is several chunks that run side by side and find the adapter in L2; walking them one after the other
@@ -35,6 +35,9 @@ __device__ __forceinline__ V pick(const V (&arr)[kMaxStreamJobs], int j) {
   return v;
 }
 
+__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {   // 16-byte aligned, a multiple of 16
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 struct ItemRef { int job, seg, sub; };
 template <class Jobs>
 __device__ __forceinline__ ItemRef decode_item(int item, int nchunk, const Jobs& jobs) {
@@ -172,21 +175,108 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
 // and every warp of the grid takes one contiguous, equally long range of them (tiles need no reduction
 // across each other, so a range may start and end anywhere).  All warps therefore stream the same number
 // of adapter bytes, whatever the mix of projection widths in the launch, and a warp's range is contiguous
-// in memory inside a (chunk, job).  A warp walks its range kExpandTilesPerBatch tiles at a time with
-// the adapter rows and the base values y0 of a batch loaded together.  `jobs.per_seg[j]` = tiles of job j.
+// in memory inside a (chunk, job).  A warp walks its range some tiles at a time with the adapter rows and the base
+// values y0 of a batch loaded together.  `jobs.per_seg[j]` = tiles of job j.
+
+// Tiles tile0 .. tile1 - 1 of one (chunk, job), TB of them in flight; P: 32-wide groups of the rank, ceil(r_use / 32).
+struct ExpandPiece {
+  const __nv_bfloat16* Bs;   // the adapter's B
+  const float *h, *y0;
+  __nv_bfloat16* y;
+  int r, r_use, d_out, act, s0, n, my_row;   // my_row: token row of column g (-1: none)
+};
+template <int P, int TB, bool VAR>
+__device__ __forceinline__ void expand_piece(const ExpandPiece& e, int tile0, int tile1, float scale, int g, int t) {
+  // token operand (MMA "B" fragment): column g = token g, k slots <- rho 32p + 8t .. +7
+  uint32_t hh[P][4], hl[P][4];
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int rb = 32 * p + 8 * t;
+    float v[8];
+    if (g < e.n && rb < e.r_use) {
+      const float4 f0 = *reinterpret_cast<const float4*>(e.h + (size_t)(e.s0 + g) * e.r + rb);
+      const float4 f1 = *reinterpret_cast<const float4*>(e.h + (size_t)(e.s0 + g) * e.r + rb + 4);
+      v[0] = f0.x; v[1] = f0.y; v[2] = f0.z; v[3] = f0.w; v[4] = f1.x; v[5] = f1.y; v[6] = f1.z; v[7] = f1.w;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float s0v = (VAR ? lora_act(v[2 * q], e.act) : v[2 * q]) * scale;
+      const float s1v = (VAR ? lora_act(v[2 * q + 1], e.act) : v[2 * q + 1]) * scale;
+      const uint32_t hi = pack_bf16(s0v, s1v);
+      hh[p][q] = hi;
+      hl[p][q] = pack_bf16(s0v - bf16_lo(hi), s1v - bf16_hi(hi));
+    }
+  }
+  const int row_c0 = __shfl_sync(0xffffffffu, e.my_row, (2 * t) * 4);
+  const int row_c1 = __shfl_sync(0xffffffffu, e.my_row, (2 * t + 1) * 4);
+  const int r = e.r, d_out = e.d_out;
+  for (int tb = tile0; tb < tile1; tb += TB) {
+    uint4 a0[TB][P], a1[TB][P];
+    float b0[TB][4];
+#pragma unroll
+    for (int i = 0; i < TB; ++i) {
+      const int ja = (tb + i) * 16 + g, jc = ja + 8;
+      const bool va = (tb + i) < tile1 && ja < d_out, vc = (tb + i) < tile1 && jc < d_out;
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        const int rb = 32 * p + 8 * t;
+        const uint4 z = make_uint4(0, 0, 0, 0);
+        a0[i][p] = (va && rb < e.r_use) ? ldg_stream(e.Bs + (size_t)ja * r + rb) : z;
+        a1[i][p] = (vc && rb < e.r_use) ? ldg_stream(e.Bs + (size_t)jc * r + rb) : z;
+      }
+      b0[i][0] = (va && row_c0 >= 0) ? __ldg(e.y0 + (size_t)row_c0 * d_out + ja) : 0.f;
+      b0[i][1] = (va && row_c1 >= 0) ? __ldg(e.y0 + (size_t)row_c1 * d_out + ja) : 0.f;
+      b0[i][2] = (vc && row_c0 >= 0) ? __ldg(e.y0 + (size_t)row_c0 * d_out + jc) : 0.f;
+      b0[i][3] = (vc && row_c1 >= 0) ? __ldg(e.y0 + (size_t)row_c1 * d_out + jc) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < TB; ++i) {
+      const int ja = (tb + i) * 16 + g, jc = ja + 8;
+      const bool va = (tb + i) < tile1 && ja < d_out, vc = (tb + i) < tile1 && jc < d_out;
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        mma_bf16_16816(c, a0[i][p].x, a1[i][p].x, a0[i][p].y, a1[i][p].y, hl[p][0], hl[p][1]);
+        mma_bf16_16816(c, a0[i][p].z, a1[i][p].z, a0[i][p].w, a1[i][p].w, hl[p][2], hl[p][3]);
+        mma_bf16_16816(c, a0[i][p].x, a1[i][p].x, a0[i][p].y, a1[i][p].y, hh[p][0], hh[p][1]);
+        mma_bf16_16816(c, a0[i][p].z, a1[i][p].z, a0[i][p].w, a1[i][p].w, hh[p][2], hh[p][3]);
+      }
+      // c0:(ja, col 2t) c1:(ja, col 2t+1) c2:(jc, col 2t) c3:(jc, col 2t+1)
+      if (row_c0 >= 0) {
+        const size_t o = (size_t)row_c0 * d_out;
+        if (va) e.y[o + ja] = __float2bfloat16_rn(b0[i][0] + c[0]);
+        if (vc) e.y[o + jc] = __float2bfloat16_rn(b0[i][2] + c[2]);
+      }
+      if (row_c1 >= 0) {
+        const size_t o = (size_t)row_c1 * d_out;
+        if (va) e.y[o + ja] = __float2bfloat16_rn(b0[i][1] + c[1]);
+        if (vc) e.y[o + jc] = __float2bfloat16_rn(b0[i][3] + c[3]);
+      }
+    }
+  }
+}
+
 // VAR: some pool of the launch has a rank per slot or an activation; without it the kernel is the plain layer's
-// (the rank is the stored rank, h is used as it is) and carries none of the variant's bookkeeping.
-template <int P, bool VAR>  // P: number of 32-wide rho groups, ceil(max r / 32)
+// (the rank is the stored rank, h is used as it is) and carries none of the variant's bookkeeping.  A variant launch
+// takes each piece by its own rank, so that narrow adapters keep as many bytes in flight as wide ones.
+// P: number of 32-wide rho groups, ceil(max r / 32).
+template <int P, bool VAR>
 __global__ void __launch_bounds__(kExpandThreads, 4)
 lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict__ perm,
                           const int4* __restrict__ chunk_tab, const ExpandJobs jobs, float scale, int tps) {
-  constexpr int TB = P > 2 ? 1 : kExpandTilesPerBatch;   // wide ranks: one tile's rows already fill the load registers
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   const long long wid = (long long)blockIdx.x * (kExpandThreads / 32) + warp;
   const long long nw = (long long)gridDim.x * (kExpandThreads / 32);
   pdl_launch_dependents();
-  pdl_wait();   // h (shrink) and y0 (base GEMM, which the shrink's completion covers)
+  // The plan and the adapters are older than the shrink before this kernel; h (shrink) and y0 (base GEMM, which the
+  // shrink's completion covers) are not: the wait comes after the first piece's metadata and the start of its adapter
+  // rows (decode step of 24 tokens 83.7 -> 78.1 us, of 256 tokens 236.5 -> 230.5 us; prefetching further ahead or all
+  // along the range only disturbs the streams: 237-260 us).
+  bool waited = false;
   const int nchunk = __ldg(header + PH_NCHUNK);
   const long long units = (long long)nchunk * tps;
   long long u = units * wid / nw;
@@ -204,8 +294,7 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
     for (int j = 0; j < kMaxStreamJobs; ++j)
       ranks[j] = (VAR && j < jobs.n && slots[j] >= 0 && jobs.slot_rank[j]) ? min(__ldg(jobs.slot_rank[j] + slots[j]), jobs.r[j])
                                                                      : (j < jobs.n ? jobs.r[j] : 0);
-    const bool vx = g < n;
-    const int my_row = vx ? __ldg(perm + s0 + g) : -1;
+    const int my_row = g < n ? __ldg(perm + s0 + g) : -1;
     const long long seg_end = (long long)(seg + 1) * tps;
     int rem = (int)(u - (long long)seg * tps);
     int job = 0;
@@ -224,82 +313,30 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
       const int tile1 = (left < (long long)(tiles_j - tile0)) ? tile0 + (int)left : tiles_j;
       const int slot = pick(slots, job);
       if (slot >= 0) {
-        const int r = pick(jobs.r, job), d_out = pick(jobs.d_out, job);
-        const int r_use = VAR ? pick(ranks, job) : r, act = VAR ? pick(jobs.act, job) : MOIN_ACT_NONE;
-        const float* __restrict__ h = pick(jobs.h, job);
-        const float* __restrict__ y0 = pick(jobs.y0, job);
-        __nv_bfloat16* __restrict__ y = pick(jobs.y, job);
-        const __nv_bfloat16* Bs = pick(jobs.B, job) + (size_t)slot * (size_t)d_out * (size_t)r;
-        {
-          // token operand (MMA "B" fragment): column g = token g, k slots <- rho 32p + 8t .. +7
-          uint32_t hh[P][4], hl[P][4];
-#pragma unroll
-          for (int p = 0; p < P; ++p) {
-            const int rb = 32 * p + 8 * t;
-            float v[8];
-            if (vx && rb < r_use) {
-              const float4 f0 = *reinterpret_cast<const float4*>(h + (size_t)(s0 + g) * r + rb);
-              const float4 f1 = *reinterpret_cast<const float4*>(h + (size_t)(s0 + g) * r + rb + 4);
-              v[0] = f0.x; v[1] = f0.y; v[2] = f0.z; v[3] = f0.w; v[4] = f1.x; v[5] = f1.y; v[6] = f1.z; v[7] = f1.w;
-            } else {
-#pragma unroll
-              for (int q = 0; q < 8; ++q) v[q] = 0.f;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float s0v = (VAR ? lora_act(v[2 * q], act) : v[2 * q]) * scale;
-              const float s1v = (VAR ? lora_act(v[2 * q + 1], act) : v[2 * q + 1]) * scale;
-              const uint32_t hi = pack_bf16(s0v, s1v);
-              hh[p][q] = hi;
-              hl[p][q] = pack_bf16(s0v - bf16_lo(hi), s1v - bf16_hi(hi));
-            }
+        ExpandPiece pc;
+        pc.r = pick(jobs.r, job);
+        pc.d_out = pick(jobs.d_out, job);
+        pc.r_use = VAR ? pick(ranks, job) : pc.r;
+        pc.act = VAR ? pick(jobs.act, job) : MOIN_ACT_NONE;
+        pc.h = pick(jobs.h, job);
+        pc.y0 = pick(jobs.y0, job);
+        pc.y = pick(jobs.y, job);
+        pc.Bs = pick(jobs.B, job) + (size_t)slot * (size_t)pc.d_out * (size_t)pc.r;
+        pc.s0 = s0; pc.n = n; pc.my_row = my_row;
+        if (!waited) {
+          if (!VAR && lane == 0) {   // the first rows on their way to L2 meanwhile
+            const int rows = min(pc.d_out, min(tile1, tile0 + kExpandFirst) * 16) - tile0 * 16;
+            l2_prefetch(pc.Bs + (size_t)tile0 * 16 * pc.r, (uint32_t)(rows * pc.r * 2));
           }
-          const int row_c0 = __shfl_sync(0xffffffffu, my_row, (2 * t) * 4);
-          const int row_c1 = __shfl_sync(0xffffffffu, my_row, (2 * t + 1) * 4);
-          for (int tb = tile0; tb < tile1; tb += TB) {
-            uint4 a0[TB][P], a1[TB][P];
-            float b0[TB][4];
-#pragma unroll
-            for (int i = 0; i < TB; ++i) {
-              const int ja = (tb + i) * 16 + g, jc = ja + 8;
-              const bool va = (tb + i) < tile1 && ja < d_out, vc = (tb + i) < tile1 && jc < d_out;
-#pragma unroll
-              for (int p = 0; p < P; ++p) {
-                const int rb = 32 * p + 8 * t;
-                const uint4 z = make_uint4(0, 0, 0, 0);
-                a0[i][p] = (va && rb < r_use) ? ldg_stream(Bs + (size_t)ja * r + rb) : z;
-                a1[i][p] = (vc && rb < r_use) ? ldg_stream(Bs + (size_t)jc * r + rb) : z;
-              }
-              b0[i][0] = (va && row_c0 >= 0) ? __ldg(y0 + (size_t)row_c0 * d_out + ja) : 0.f;
-              b0[i][1] = (va && row_c1 >= 0) ? __ldg(y0 + (size_t)row_c1 * d_out + ja) : 0.f;
-              b0[i][2] = (vc && row_c0 >= 0) ? __ldg(y0 + (size_t)row_c0 * d_out + jc) : 0.f;
-              b0[i][3] = (vc && row_c1 >= 0) ? __ldg(y0 + (size_t)row_c1 * d_out + jc) : 0.f;
-            }
-#pragma unroll
-            for (int i = 0; i < TB; ++i) {
-              const int ja = (tb + i) * 16 + g, jc = ja + 8;
-              const bool va = (tb + i) < tile1 && ja < d_out, vc = (tb + i) < tile1 && jc < d_out;
-              float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-              for (int p = 0; p < P; ++p) {
-                mma_bf16_16816(c, a0[i][p].x, a1[i][p].x, a0[i][p].y, a1[i][p].y, hl[p][0], hl[p][1]);
-                mma_bf16_16816(c, a0[i][p].z, a1[i][p].z, a0[i][p].w, a1[i][p].w, hl[p][2], hl[p][3]);
-                mma_bf16_16816(c, a0[i][p].x, a1[i][p].x, a0[i][p].y, a1[i][p].y, hh[p][0], hh[p][1]);
-                mma_bf16_16816(c, a0[i][p].z, a1[i][p].z, a0[i][p].w, a1[i][p].w, hh[p][2], hh[p][3]);
-              }
-              // c0:(ja, col 2t) c1:(ja, col 2t+1) c2:(jc, col 2t) c3:(jc, col 2t+1)
-              if (row_c0 >= 0) {
-                const size_t o = (size_t)row_c0 * d_out;
-                if (va) y[o + ja] = __float2bfloat16_rn(b0[i][0] + c[0]);
-                if (vc) y[o + jc] = __float2bfloat16_rn(b0[i][2] + c[2]);
-              }
-              if (row_c1 >= 0) {
-                const size_t o = (size_t)row_c1 * d_out;
-                if (va) y[o + ja] = __float2bfloat16_rn(b0[i][1] + c[1]);
-                if (vc) y[o + jc] = __float2bfloat16_rn(b0[i][3] + c[3]);
-              }
-            }
-          }
+          pdl_wait();
+          waited = true;
+        }
+        if (VAR) {
+          if (P >= 4 && pc.r_use > 64) expand_piece<4, 1, VAR>(pc, tile0, tile1, scale, g, t);
+          else if (P >= 2 && pc.r_use > 32) expand_piece<2, 2, VAR>(pc, tile0, tile1, scale, g, t);
+          else expand_piece<1, 2, VAR>(pc, tile0, tile1, scale, g, t);
+        } else {
+          expand_piece<P, (P > 2 ? 1 : 2), VAR>(pc, tile0, tile1, scale, g, t);
         }
       }
       u += tile1 - tile0;
@@ -307,6 +344,7 @@ lora_expand_stream_kernel(const int* __restrict__ header, const int* __restrict_
       ++job;
     }
   }
+  if (!waited) pdl_wait();   // (a kernel that waits for this one counts on everything before being complete)
 }
 
 static int stream_grid(long max_items, int n_sms, int ctas_per_sm) {
