@@ -532,11 +532,8 @@ static moin_status launch_base_gemm(HostState* hs, bool use_tc, const __nv_bfloa
     const DecodeGemmJob job = {x, W, y, y0, d_in, d_out};
     return launch_decode_gemm(hs, &job, 1, T, s);
   }
-  if (y0 == nullptr) {
-    const PairJob job = {x, W, nullptr, y, nullptr, d_out};
-    return launch_pair_gemm(hs, nullptr, &job, 1, T, d_in, s);
-  }
-  return launch_tc_gemm(hs, x, W, y, y0, T, d_in, d_out, s);
+  const PairJob job = {x, W, nullptr, y, y0, nullptr, d_out};
+  return launch_pair_gemm(hs, nullptr, &job, 1, T, d_in, s);
 }
 
 size_t moin_lora_linear_group_workspace_bytes(int32_t T, const moin_lora_job* jobs, int32_t n_jobs) {
@@ -602,7 +599,7 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
         while (j0 + n < n_jobs && n < kPairJobs && d_in[j0 + n] == d_in[j0] && r[j0 + n] == r[j0]) {
           const moin_lora_job& g = jobs[j0 + n];
           pj[n] = {(const __nv_bfloat16*)g.x, (const __nv_bfloat16*)g.W, reinterpret_cast<__nv_bfloat16*>(ws_job[j0 + n]),
-                   (__nv_bfloat16*)g.y, g.pool, d_out[j0 + n]};
+                   (__nv_bfloat16*)g.y, nullptr, g.pool, d_out[j0 + n]};
           ++n;
         }
         ProfScope prof(MOIN_K_FUSED_TC, 1, s);

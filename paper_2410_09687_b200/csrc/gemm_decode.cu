@@ -91,30 +91,32 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
     if (lane == 0) {
       const CUtensorMap* mw = &maps.w[job];
       const CUtensorMap* mx = &maps.x[job];
+      uint32_t s = 0, ph = 0;
       for (int kb = kb0; kb < kb1; ++kb) {
-        const uint32_t i = (uint32_t)(kb - kb0), s = i % S, ph = (i / S) & 1u;
         if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 51)) break;
-        const uint32_t sa = ring + s * stage_bytes;
-        mbar_expect_tx(full0 + 8 * s, stage_bytes);
-        tma_load_2d(sa, mw, full0 + 8 * s, kb * kDgK, f0);
-        tma_load_2d(sa + kDgM * kDgK * 2, mx, full0 + 8 * s, kb * kDgK, tok0);
+        const uint32_t sa = ring + s * stage_bytes, full = full0 + 8 * s;
+        if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
+        mbar_expect_tx(full, stage_bytes);
+        tma_load_2d(sa, mw, full, kb * kDgK, f0);
+        tma_load_2d(sa + kDgM * kDgK * 2, mx, full, kb * kDgK, tok0);
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     const uint32_t idesc = idesc_bf16(kDgM, p.nt);
     const bool leader = elect_one();
+    uint32_t s = 0, ph = 0;
     for (int kb = kb0; kb < kb1 && ok; ++kb) {
-      const uint32_t i = (uint32_t)(kb - kb0), s = i % S, ph = (i / S) & 1u;
       if (!(ok = mbar_wait_warp(full0 + 8 * s, ph, abort_flag, p.status, 52))) break;
       tc_fence_after();
-      const uint32_t sa = ring + s * stage_bytes;
+      const uint32_t sa = ring + s * stage_bytes, empty = empty0 + 8 * s;
+      if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
       const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sa + kDgM * kDgK * 2);
       if (leader) {
 #pragma unroll
         for (int k = 0; k < kDgK / 16; ++k)
-          tc_mma_bf16(tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (i > 0 || k > 0) ? 1u : 0u);
-        tc_commit(empty0 + 8 * s);
+          tc_mma_bf16(tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+        tc_commit(empty);
       }
     }
     if (ok && leader) tc_commit(done);

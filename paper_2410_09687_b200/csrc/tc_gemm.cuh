@@ -15,18 +15,15 @@ bool tc_gemm_supported(int T, int d_in, int d_out);
 bool tc_router_supported(int Q, int K, int D);
 bool tc_fused_supported(int r);
 
-// y = x W^T (bf16) and optionally y0 = x W^T (fp32).
-// `cta_budget` > 0: widen the tiles until the launch has at most that many CTAs (when it runs beside other kernels).
-moin_status launch_tc_gemm(HostState* hs, const __nv_bfloat16* x, const __nv_bfloat16* W, __nv_bfloat16* y, float* y0,
-                           int T, int d_in, int d_out, cudaStream_t stream, int cta_budget = 0);
-// The same for few tokens, up to kMaxStreamJobs projections in one launch (gemm_decode.cu).
+// y = x W^T (bf16) and optionally y0 = x W^T (fp32) for few tokens, up to kMaxStreamJobs projections in one launch
+// (gemm_decode.cu).
 struct DecodeGemmJob { const __nv_bfloat16 *x, *W; __nv_bfloat16* y; float* y0; int d_in, d_out; };
 constexpr int kDecodeGemmMaxT = 512;
 moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, cudaStream_t stream);
 // Long-run GEMMs on CTA pairs (tc_pair.cu): y_j = x_j W_j^T for up to kPairJobs projections of one K; with a plan the
 // low-rank term s x A_e^T B_e^T is added from hb (hi / lo parts of s x A_e^T, [2][M][r], all jobs of the same r).
 constexpr int kPairJobs = 3;
-struct PairJob { const __nv_bfloat16 *x, *W, *hb; __nv_bfloat16* y; const moin_pool* pool; int N; };
+struct PairJob { const __nv_bfloat16 *x, *W, *hb; __nv_bfloat16* y; float* y0; const moin_pool* pool; int N; };   // y0: fp32 copy or nullptr
 moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* jobs, int n_jobs, int M, int K,
                              cudaStream_t stream);
 // keys[i] = max over k of (orderable(<q_i,c_k> * inv_norm[k]) << 32 | (0xFFFFFFFF - k)), merged with atomicMax.

@@ -38,6 +38,7 @@ struct PairParams {
   const int* slot_of_expert[kPairJobs];
   const int* slot_rank[kPairJobs];       // nullable: the stored rank
   __nv_bfloat16* y[kPairJobs];
+  float* y0[kPairJobs];                  // fp32 copy, nullable (then the rows are written straight from registers)
   const float* inv_norm;                 // PAIR_ROUTER*
   unsigned long long *keys, *keys2;
   DeviceStatus* status;
@@ -198,7 +199,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (first CTA, for both)
-    if (rank == 0) {   // the whole warp walks the loop, one elected lane issues (as in tc_gemm.cu)
+    if (rank == 0) {   // the whole warp walks the loop, one elected lane issues (see elect_one)
       const uint32_t idesc = idesc_bf16(2 * kPairM, p.bn);
       const bool leader = elect_one();
       uint32_t it = 0, lt = 0;
@@ -252,9 +253,10 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       const int row0 = rank == 0 ? t.row0[0] : t.row0[1], rows = rank == 0 ? t.rows[0] : t.rows[1];
       int n = p.N[0];
       __nv_bfloat16* y = p.y[0];
+      float* y0 = p.y0[0];
 #pragma unroll
       for (int j = 1; j < kPairJobs; ++j)
-        if (t.job == j) { n = p.N[j]; y = p.y[j]; }
+        if (t.job == j) { n = p.N[j]; y = p.y[j]; y0 = p.y0[j]; }
       const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
       if (EPI != PAIR_STORE) {   // 1/|c_k| of this warp's columns; NaN where there is no candidate: it loses every maximum
         const int k0 = t.n0 + wh * (p.bn / 2) + 4 * lane;
@@ -284,7 +286,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
 #pragma unroll 1
         for (int c = 64 * wh; c < p.bn; c += 128) {
           if (t.n0 + c >= n || q * 32 >= rows) break;
-          const bool staged = q * 32 + 32 <= rows && c + 64 <= p.bn;
+          const bool staged = q * 32 + 32 <= rows && c + 64 <= p.bn && y0 == nullptr;
           if (staged && n_st >= 1) {               // the store that last read this buffer
             if (lane == 0) bulk_wait_read<0>();
             __syncwarp();
@@ -307,6 +309,11 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
                 asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w) : "memory");
               } else if (row_ok && col < col_end) {
                 *reinterpret_cast<uint4*>(y + grow * (size_t)n + col) = o;
+                if (y0 != nullptr) {
+                  uint4* d0 = reinterpret_cast<uint4*>(y0 + grow * (size_t)n + col);
+                  d0[0] = make_uint4(v[8 * j], v[8 * j + 1], v[8 * j + 2], v[8 * j + 3]);
+                  d0[1] = make_uint4(v[8 * j + 4], v[8 * j + 5], v[8 * j + 6], v[8 * j + 7]);
+                }
               }
             }
           }
@@ -481,7 +488,7 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
     }
     if (st) return st;
     tn += (g.N + bn - 1) / bn;
-    p.N[j] = g.N; p.tn_end[j] = tn; p.y[j] = g.y;
+    p.N[j] = g.N; p.tn_end[j] = tn; p.y[j] = g.y; p.y0[j] = g.y0;
   }
   // upper bound on the row tiles of a plan without reading it back; the grid is capped at the SM pairs
   const long max_tiles = (pv ? (long)M : (tiles_m + 1) / 2) * tn;

@@ -1,0 +1,271 @@
+// Long-run LoRA shrink  h = s act(x A_e^T)  on tcgen05 / TMEM / TMA, stored as bf16 hi + lo parts.
+//
+// A work item is one row tile of the batch plan (a run of one expert, at most 128 rows) for a SET of projections that
+// share x (a launch each): their adapters' rows stand side by side in the B operand, so x is read once.  The product is skinny (N = the
+// set's ranks together), and its time is latency: 128 rows x K of x through one SM at a time.  The reduction is
+// therefore cut over the `ks` CTAs of a cluster - as many as fill the GPU - and the parts meet in shared memory: every
+// CTA of the cluster adds its share of the rows over the parts in rank order (independent of timing), applies the
+// function, the scale and the slot's rank, and writes whole rows.
+//   warp 0     TMA producer (one thread): [128 x 64] box of x, [r x 64] box of A per projection
+//   warp 1     allocates TMEM, issues the MMAs (one elected lane)
+//   warps 2-9  TMEM -> shared memory (row pitch N + 4 floats: no bank conflicts), two warps per lane quarter
+// Against one CTA per row tile (calls of 3392 tokens in runs of 106, rank 64, to 256 columns, projection included):
+// K = 2048 26.6 -> 23.2 us, K = 5632 52 -> 42 us, three projections 46.5 -> 32.7 us; 16384 tokens fill the SMs with one
+// CTA per row tile and are bound by reading x (84 us of which 32 us at the copy bandwidth for K = 5632).
+#include <cuda.h>
+
+#include "ptx.cuh"
+#include "tc_gemm.cuh"
+
+namespace moin {
+
+constexpr int kTsThreads = 320, kTsM = 128, kTsK = 64, kTsMaxN = 256, kTsMaxStages = 8;
+
+struct TsMaps { CUtensorMap x, a[kTcMaxShrinkJobs]; };
+struct TsParams {
+  int T, K, r, n_jobs, N;                   // N: the jobs' ranks together, a multiple of 16
+  int stages, stage_bytes, tmem_cols, ks;
+  const int *header, *tile_row0, *tile_rows, *tile_expert;
+  const int* slot_of_expert[kTcMaxShrinkJobs];
+  const int* slot_rank[kTcMaxShrinkJobs];   // nullable: the stored rank
+  __nv_bfloat16* hb[kTcMaxShrinkJobs];      // [2][T][r]: hi, lo
+  int act;
+  float scale;
+  DeviceStatus* status;
+};
+
+__global__ void __launch_bounds__(kTsThreads, 1)
+tc_shrink_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__ TsParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t ring = (raw + 1023u) & ~1023u;
+  const int S = p.stages;
+  const uint32_t bars = ring + (uint32_t)S * (uint32_t)p.stage_bytes;
+  uint8_t* bar_ptr = smem_raw + (bars - raw);
+  const uint32_t full0 = bars, empty0 = bars + 8 * kTsMaxStages, done = bars + 16 * kTsMaxStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + 16 * kTsMaxStages + 8);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 16 * kTsMaxStages + 16);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = p.ks > 1 ? (int)cluster_rank() : 0;
+  const int cluster = (int)blockIdx.x / p.ks, n_clusters = (int)gridDim.x / p.ks;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    mbar_init(done, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(tmem_slot), p.tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_begin();   // (the set-up above overlaps the tail of the kernel before)
+
+  const int total = __ldg(p.header + PH_NTILES), N = p.N, pitch = N + 4;
+  const int nkb = p.K / kTsK, kb0 = nkb * rank / p.ks, kb1 = nkb * (rank + 1) / p.ks;
+  auto sync_cluster = [&]() {
+    if (p.ks > 1) {
+      cluster_arrive();
+      cluster_wait();
+    } else {
+      __syncthreads();
+    }
+  };
+  uint32_t st = 0, ph = 0, n_done = 0;   // ring position and phase (of the producer and of the MMA warp)
+  bool ok = true;
+  for (int tm = cluster; tm < total; tm += n_clusters) {
+    const int row0 = __ldg(p.tile_row0 + tm), rows = __ldg(p.tile_rows + tm), e = __ldg(p.tile_expert + tm);
+    if (e < 0) continue;
+    int slot[kTcMaxShrinkJobs];
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < kTcMaxShrinkJobs; ++j) {
+      slot[j] = j < p.n_jobs ? __ldg(p.slot_of_expert[j] + e) : -1;
+      any = any || slot[j] >= 0;
+    }
+    if (!any) continue;   // (the same for the whole cluster)
+    if (warp == 0) {
+      if (lane == 0) {
+        const uint32_t tx = (uint32_t)(kTsM + p.n_jobs * p.r) * kTsK * 2;
+        for (int kb = kb0; kb < kb1 && ok; ++kb) {
+          if (!(ok = mbar_wait(empty0 + 8 * st, ph ^ 1u, abort_flag, p.status, 71))) break;
+          const uint32_t sa = ring + st * p.stage_bytes, sb = sa + kTsM * kTsK * 2, full = full0 + 8 * st;
+          if (++st == (uint32_t)S) { st = 0; ph ^= 1u; }
+          mbar_expect_tx(full, tx);
+          tma_load_2d(sa, &maps.x, full, kb * kTsK, row0);
+#pragma unroll
+          for (int j = 0; j < kTcMaxShrinkJobs; ++j)
+            if (j < p.n_jobs)   // (a projection without this adapter loads slot 0: its columns are not stored)
+              tma_load_2d(sb + (uint32_t)(j * p.r) * (kTsK * 2), &maps.a[j], full, kb * kTsK, max(slot[j], 0) * p.r);
+        }
+      }
+      __syncwarp();
+    } else if (warp == 1) {
+      const uint32_t idesc = idesc_bf16(kTsM, N);
+      const bool leader = elect_one();
+      for (int kb = kb0; kb < kb1 && ok; ++kb) {
+        if (!(ok = mbar_wait_warp(full0 + 8 * st, ph, abort_flag, p.status, 72))) break;
+        tc_fence_after();
+        const uint32_t sa = ring + st * p.stage_bytes, empty = empty0 + 8 * st;
+        if (++st == (uint32_t)S) { st = 0; ph ^= 1u; }
+        const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sa + kTsM * kTsK * 2);
+        if (leader) {
+#pragma unroll
+          for (int k = 0; k < kTsK / 16; ++k)
+            tc_mma_bf16(tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+          tc_commit(empty);
+        }
+      }
+      if (ok && leader) tc_commit(done);
+      __syncwarp();
+    } else {
+      // this CTA's part to shared memory (the ring is free: every stage has been consumed), [row][pitch] fp32
+      if (ok && (ok = mbar_wait_warp(done, n_done & 1u, abort_flag, p.status, 73))) {
+        tc_fence_after();
+        const int q = warp & 3, wh = (warp - 2) >> 2;
+        const uint32_t dst = ring + (uint32_t)((q * 32 + lane) * pitch) * 4u;
+        for (int c = 16 * wh; c < N; c += 32) {
+          uint32_t v[16];
+          tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + c, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; i += 4)
+            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + 4u * (c + i)), "r"(v[i]), "r"(v[i + 1]), "r"(v[i + 2]),
+                         "r"(v[i + 3]) : "memory");
+        }
+        tc_fence_before();
+      }
+    }
+    ++n_done;
+    sync_cluster();
+    // this CTA's share of the rows: eight columns of a row per thread
+    const int own = kTsM / p.ks, r8 = p.r / 8, per_row = p.n_jobs * r8;
+    for (int i = threadIdx.x; i < own * per_row; i += kTsThreads) {
+      const int row = rank * own + i / per_row, c8 = i % per_row, j = c8 / r8, cj = (c8 - j * r8) * 8;
+      int sl = slot[0];
+      const int* ranks = p.slot_rank[0];
+      __nv_bfloat16* hb = p.hb[0];
+#pragma unroll
+      for (int jj = 1; jj < kTcMaxShrinkJobs; ++jj)
+        if (j == jj) { sl = slot[jj]; ranks = p.slot_rank[jj]; hb = p.hb[jj]; }
+      if (row >= rows || sl < 0 || *abort_flag) continue;
+      const int r_use = ranks ? min(__ldg(ranks + sl), p.r) : p.r;
+      const uint32_t off = (uint32_t)(row * pitch + c8 * 8) * 4u;
+      float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int k0 = 0; k0 < p.ks; k0 += 4) {
+        float4 va[4], vb[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k0 + k < p.ks) {
+            const uint32_t a = (p.ks > 1 ? map_rank(ring, (uint32_t)(k0 + k)) : ring) + off;
+            va[k] = p.ks > 1 ? ld_cluster_f4(a) : lds_f4(a);
+            vb[k] = p.ks > 1 ? ld_cluster_f4(a + 16) : lds_f4(a + 16);
+          }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k0 + k < p.ks) {
+            f[0] += va[k].x; f[1] += va[k].y; f[2] += va[k].z; f[3] += va[k].w;
+            f[4] += vb[k].x; f[5] += vb[k].y; f[6] += vb[k].z; f[7] += vb[k].w;
+          }
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) f[k] = cj + k < r_use ? lora_act(f[k], p.act) * p.scale : 0.f;   // nothing beyond the adapter's rank
+      uint4 h, l;
+      h.x = pack_bf16(f[0], f[1]); h.y = pack_bf16(f[2], f[3]); h.z = pack_bf16(f[4], f[5]); h.w = pack_bf16(f[6], f[7]);
+      l.x = pack_bf16(f[0] - bf16_lo(h.x), f[1] - bf16_hi(h.x));   // hi + lo carries the value to ~fp32 accuracy
+      l.y = pack_bf16(f[2] - bf16_lo(h.y), f[3] - bf16_hi(h.y));
+      l.z = pack_bf16(f[4] - bf16_lo(h.z), f[5] - bf16_hi(h.z));
+      l.w = pack_bf16(f[6] - bf16_lo(h.w), f[7] - bf16_hi(h.w));
+      __nv_bfloat16* dst = hb + (size_t)(row0 + row) * (size_t)p.r + cj;
+      *reinterpret_cast<uint4*>(dst) = h;
+      *reinterpret_cast<uint4*>(dst + (size_t)p.T * (size_t)p.r) = l;
+    }
+    // the parts have been read everywhere: the next item's copies may overwrite them
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    sync_cluster();
+  }
+  if (*abort_flag) {   // a wait ran out: let copies / MMAs in flight land before shared and tensor memory are released
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < 2000000ull) __nanosleep(1000);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, p.tmem_cols);
+  }
+}
+
+// One set: projections of one K, rank and activation that share x, ranks together at most 256.
+static moin_status launch_set(HostState* hs, const PlanView& pv, const moin_pool* const* pools, const __nv_bfloat16* x,
+                              __nv_bfloat16* const* hbs, int n_jobs, float scale, cudaStream_t stream) {
+  const int T = pv.T, K = pools[0]->d_in, r = pools[0]->r;
+  TsMaps maps;
+  TsParams p = {};
+  p.T = T; p.K = K; p.r = r; p.n_jobs = n_jobs; p.N = (n_jobs * r + 15) / 16 * 16;
+  p.scale = scale; p.act = pools[0]->activation; p.status = hs->status;
+  p.header = pv.header; p.tile_row0 = pv.tile_row0; p.tile_rows = pv.tile_rows; p.tile_expert = pv.tile_expert;
+  moin_status st = make_map(&maps.x, x, T, K, kTsM);
+  for (int j = 0; j < n_jobs && !st; ++j) {
+    st = make_map(&maps.a[j], pools[j]->A, (uint64_t)pools[j]->n_slots * r, K, r);   // one slot's rows
+    p.slot_of_expert[j] = pools[j]->slot_of_expert;
+    p.slot_rank[j] = pools[j]->slot_rank;
+    p.hb[j] = hbs[j];
+  }
+  if (st) return st;
+  // the ring is also the fp32 staging of the parts
+  p.stage_bytes = (kTsM + p.N) * kTsK * 2;
+  p.stages = 200 * 1024 / p.stage_bytes < kTsMaxStages ? 200 * 1024 / p.stage_bytes : kTsMaxStages;
+  while (p.stages * p.stage_bytes < kTsM * (p.N + 4) * 4) ++p.stages;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < p.N) p.tmem_cols *= 2;
+  // Cut the reduction while the row tiles leave SMs free and a CTA keeps at least four 64-wide blocks; clusters of eight
+  // only for a handful of tiles (a GPC holds few of them).
+  const long items = (T + kTsM - 1) / kTsM;
+  const int ks_max = items <= 12 ? 8 : 4;
+  p.ks = 1;
+  while (p.ks < ks_max && items * p.ks * 2 <= hs->n_sms && K / kTsK >= 4 * p.ks * 2) p.ks *= 2;
+  long clusters = hs->n_sms / p.ks;
+  if (clusters > T) clusters = T;   // (at most one row tile per token)
+  const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 /*align*/ + 256 /*barriers*/;
+  cudaError_t e = ensure_smem_optin(OPTIN_TC_SHRINK, tc_shrink_kernel, 210 * 1024);
+  if (e != cudaSuccess) return record_cuda(e);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * p.ks));
+  cfg.blockDim = dim3(kTsThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)p.ks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  ProfScope prof(MOIN_K_SHRINK_TC, 1, stream);
+  return record_cuda(cudaLaunchKernelEx(&cfg, tc_shrink_kernel, maps, p));
+}
+
+moin_status launch_tc_shrink_group(HostState* hs, const PlanView& pv, const moin_pool* const* pools,
+                                   const __nv_bfloat16* const* xs, __nv_bfloat16* const* hbs, int n_jobs, float scale,
+                                   cudaStream_t stream) {
+  if (n_jobs < 1 || n_jobs > kTcMaxShrinkJobs) return MOIN_ERR_INVALID_ARG;
+  for (int j0 = 0; j0 < n_jobs;) {
+    int n = 1;
+    while (j0 + n < n_jobs && xs[j0 + n] == xs[j0] && (n + 1) * pools[j0]->r <= kTsMaxN) ++n;
+    moin_status st = launch_set(hs, pv, pools + j0, xs[j0], hbs + j0, n, scale, stream);
+    if (st) return st;
+    j0 += n;
+  }
+  return MOIN_OK;
+}
+
+}  // namespace moin
