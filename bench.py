@@ -669,35 +669,17 @@ def kernel_timeline(fn, use_graph: bool, steps: int = 6):
 
 
 def critical_path(rows, span_us: float) -> dict:
-    """Where a step's time goes, from its kernel timeline.  Kernels on the call's own stream follow one another, so
-    their durations add up; the base GEMMs of the short-segment path run on side streams beside the shrink, and
-    only the part of a GEMM that outlasts the shrink it runs beside delays the expand ("gemm_exposed").  The
-    remainder of the step is launch gaps.  No entry can exceed the step."""
+    """Where a step's time goes, from its kernel timeline.  Kernels are launched early and overlap (a dependent kernel
+    starts under the tail of the one before it, the adapter shrink runs beside the base GEMM), so a kernel is charged
+    with the time by which it extends the step: from the end of everything that started before it to its own end.
+    The remainder of the step is launch gaps.  No entry can exceed the step."""
     def short(n):
-        n = n.split("moin::")[1].split("(")[0].split("<")[0]
-        return n.replace("_kernel", "")
-    main, side = {}, []
-    ordered = sorted(rows, key=lambda r: r[1])
-    for name, a, b in ordered:
-        k = short(name)
-        if k.startswith("tc_gemm") or k.startswith("gemm_warp"):
-            side.append((a, b))
-        else:
-            main[k] = main.get(k, 0.0) + (b - a)
-    exposed = 0.0
-    if side and any(k.startswith("lora_expand") for k in main):
-        # per expand launch: how long after the end of the shrink before it did the last GEMM before it end?
-        exp = [(a, b) for n, a, b in ordered if "lora_expand" in n]
-        shr = [(a, b) for n, a, b in ordered if "lora_shrink" in n]
-        for (ea, _), (_, sb) in zip(exp, shr):
-            g_end = max([b for a, b in side if a < ea] or [0.0])
-            exposed += max(0.0, min(g_end, ea) - sb)
-        out = dict(main)
-        out["gemm_exposed"] = exposed
-    else:   # everything on one stream
-        out = dict(main)
-        for a, b in side:
-            out["tc_gemm"] = out.get("tc_gemm", 0.0) + (b - a)
+        return n.split("moin::")[1].split("(")[0].split("<")[0].replace("_kernel", "")
+    out, t = {}, 0.0
+    for name, a, b in sorted(rows, key=lambda r: r[1]):
+        if b > t:
+            out[short(name)] = out.get(short(name), 0.0) + (b - max(a, t))
+            t = b
     out = {k: round(v, 2) for k, v in out.items()}
     out["gaps"] = round(max(0.0, span_us - sum(out.values())), 2)
     out["step_us"] = round(span_us, 2)
