@@ -69,7 +69,6 @@ ProfScope::~ProfScope() {
 
 __global__ void set_int_kernel(int* p, int v) { *p = v; }
 
-static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace moin
 

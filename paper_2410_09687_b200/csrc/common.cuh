@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <limits.h>
 #include <stdint.h>
 
@@ -86,6 +87,18 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+// Four 8-bit float codes (e4m3) -> bf16(fp32(value * scale)), in order: two to a word.
+__device__ __forceinline__ void fp8x4_to_bf16(uint32_t codes, float scale, uint32_t& lo, uint32_t& hi) {
+  uint32_t h0, h1;   // the values as fp16 (exact)
+  asm("{\n .reg .b16 a, b;\n mov.b32 {a, b}, %2;\n cvt.rn.f16x2.e4m3x2 %0, a;\n cvt.rn.f16x2.e4m3x2 %1, b;\n}\n"
+      : "=r"(h0), "=r"(h1) : "r"(codes));
+  const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&h0)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&h1));
+  lo = pack_bf16(f0.x * scale, f0.y * scale);
+  hi = pack_bf16(f1.x * scale, f1.y * scale);
 }
 
 // Streaming 16-byte load that does not allocate in L1 (adapter weights are read once).

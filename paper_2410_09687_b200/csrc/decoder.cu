@@ -24,32 +24,53 @@ token_meta_kernel(const int* __restrict__ cu, const int* __restrict__ req_expert
 }
 
 // W[j][i] = bf16(fp32(value(code[j][i]) * scale[j])): 8-bit float codes (4 exponent bits, bias 7, 3 mantissa bits,
-// no infinities, 0x7F / 0xFF = NaN) -> the bf16 weight the GEMMs read.  One thread converts 16 codes.
-__device__ __forceinline__ float e4m3_to_float(uint32_t c) {
-  const uint32_t sign = (c & 0x80u) << 24, ex = (c >> 3) & 15u, man = c & 7u;
-  if (ex == 15u && man == 7u) return __uint_as_float(0x7FC00000u);
-  if (ex == 0u) return __uint_as_float(sign | __float_as_uint((float)man * 0.001953125f));   // man * 2^-9
-  return __uint_as_float(sign | ((ex + 120u) << 23) | (man << 20));
-}
+// no infinities, 0x7F / 0xFF = NaN) -> the bf16 weight the GEMMs read, for the matrices of one projection group.  A warp
+// converts a row: eight codes a lane and load, so that loads and stores are whole lines, four loads in flight.  Bound by
+// the traffic (one byte in, two out).  One launch per matrix, a thread per 16 codes with a 64-bit division for its row
+// and the fields put together bit by bit: forward of 112 tokens on the 8-bit base 2.98 ms, with this 2.50.
+struct DequantJobs {
+  const uint2* codes[MOIN_MAX_GROUP];
+  const float* scale[MOIN_MAX_GROUP];
+  uint4* out[MOIN_MAX_GROUP];
+  int row_end[MOIN_MAX_GROUP];   // rows of jobs 0 .. j
+  int n;
+};
 __global__ void __launch_bounds__(256)
-dequant_fp8_kernel(const uint4* __restrict__ codes, const float* __restrict__ scale, int d_in16, long n16,
-                   uint4* __restrict__ out) {
+dequant_fp8_kernel(const DequantJobs jobs, int d_in8) {
   pdl_begin();
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n16) return;
-  const float sc = __ldg(scale + i / d_in16);
-  const uint4 c = ldg_stream(codes + i);
-  const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-  uint32_t o[8];
+  int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row >= jobs.row_end[jobs.n - 1]) return;
+  const uint2* codes = jobs.codes[0];
+  const float* scale = jobs.scale[0];
+  uint4* out = jobs.out[0];
+  int first = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float f0 = e4m3_to_float(w[k] & 0xFFu) * sc, f1 = e4m3_to_float((w[k] >> 8) & 0xFFu) * sc;
-    const float f2 = e4m3_to_float((w[k] >> 16) & 0xFFu) * sc, f3 = e4m3_to_float(w[k] >> 24) * sc;
-    o[2 * k] = pack_bf16(f0, f1);
-    o[2 * k + 1] = pack_bf16(f2, f3);
+  for (int j = 1; j < MOIN_MAX_GROUP; ++j)
+    if (j < jobs.n && row >= jobs.row_end[j - 1]) {
+      codes = jobs.codes[j]; scale = jobs.scale[j]; out = jobs.out[j]; first = jobs.row_end[j - 1];
+    }
+  row -= first;
+  const float sc = __ldg(scale + row);
+  codes += (size_t)row * d_in8;
+  out += (size_t)row * d_in8;
+  for (int c0 = threadIdx.x & 31; c0 < d_in8; c0 += 4 * 32) {
+    uint2 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c0 + 32 * u < d_in8) v[u] = __ldg(codes + c0 + 32 * u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c0 + 32 * u < d_in8) {
+        uint4 o;
+        fp8x4_to_bf16(v[u].x, sc, o.x, o.y);
+        fp8x4_to_bf16(v[u].y, sc, o.z, o.w);
+        out[c0 + 32 * u] = o;
+      }
   }
-  out[2 * i] = make_uint4(o[0], o[1], o[2], o[3]);
-  out[2 * i + 1] = make_uint4(o[4], o[5], o[6], o[7]);
+}
+static moin_status launch_dequant(const DequantJobs& jobs, int d_in, cudaStream_t stream) {
+  ProfScope prof(MOIN_K_GLUE, 1, stream);
+  return record_cuda(launch_pdl(dequant_fp8_kernel, (unsigned)((jobs.row_end[jobs.n - 1] + 7) / 8), 256, 0, stream, jobs, d_in / 8));
 }
 
 // cos/sin of pos * base^(-2i/hd), computed in double once per call.
@@ -431,37 +452,41 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     ProfScope prof(MOIN_K_GLUE, 1, s);
     launch_pdl(embed_kernel, T, 256, 0, s, tokens, (const __nv_bfloat16*)m->embed, H, m->vocab, w.res);
   }
-  // weight of projection p: the caller's bf16 matrix, or - quantised base - its codes dequantised into scratch slot
-  // `slot` on the call's stream (the group calls join their side streams before they return, so a slot is free again)
-  moin_status wst = MOIN_OK;
-  auto weight = [&](int layer, int p, int d_in, int d_out, int slot) -> const void* {
-    const int i = layer * 7 + p;
-    if (!m->W8 || !m->W8[i]) return m->W[i];
-    if (!m->W_scale || !m->W_scale[i]) { wst = MOIN_ERR_INVALID_ARG; return nullptr; }
-    moin_status e = moin_dequant_fp8(m->W8[i], m->W_scale[i], d_out, d_in, w.wq[slot], stream);
-    if (e) wst = e;
-    return w.wq[slot];
-  };
-  auto proj = [&](int layer, int p, const void* in, int d_in, int d_out, void* out) -> moin_status {
-    const void* W = weight(layer, p, d_in, d_out, 0);
-    if (wst) return wst;
-    return moin_lora_linear(lora ? &plan : nullptr, in, W, lora ? &m->pools[layer * 7 + p] : nullptr,
-                            m->lora_scale, T, d_in, d_out, out, w.lora, w.lora_bytes, stream);
+  // weights of the projections p0 .. p0 + n - 1, which share d_in: the caller's bf16 matrices, or - quantised base - their
+  // codes dequantised into the scratch slots by one launch on the call's stream (the group before has read its slots
+  // by then)
+  auto weights = [&](int layer, int p0, int n, int d_in, const int* d_out, const void** W) -> moin_status {
+    DequantJobs dq = {};
+    for (int j = 0; j < n; ++j) {
+      const int i = layer * 7 + p0 + j;
+      W[j] = m->W[i];
+      if (!m->W8 || !m->W8[i]) continue;
+      if (!m->W_scale || !m->W_scale[i]) return MOIN_ERR_INVALID_ARG;
+      if (!aligned16(m->W8[i])) return MOIN_ERR_MISALIGNED;
+      dq.codes[dq.n] = (const uint2*)m->W8[i];
+      dq.scale[dq.n] = m->W_scale[i];
+      dq.out[dq.n] = (uint4*)w.wq[j];
+      dq.row_end[dq.n] = (dq.n ? dq.row_end[dq.n - 1] : 0) + d_out[j];
+      W[j] = w.wq[j];
+      ++dq.n;
+    }
+    return dq.n ? launch_dequant(dq, d_in, s) : MOIN_OK;
   };
   // projections of a block that read the same input and do not depend on one another go out as one group
-  auto proj_group = [&](int layer, int p0, int n, const void* in, const int* d_in, const int* d_out,
-                        void* const* outs) -> moin_status {
-    if (!lora) {
-      for (int i = 0; i < n; ++i) {
-        moin_status e = proj(layer, p0 + i, in, d_in[i], d_out[i], outs[i]);
-        if (e) return e;
-      }
-      return MOIN_OK;
-    }
+  auto proj_group = [&](int layer, int p0, int n, const void* in, int d_in, const int* d_out, void* const* outs) -> moin_status {
+    const void* W[MOIN_MAX_GROUP];
+    moin_status e = weights(layer, p0, n, d_in, d_out, W);
+    if (e) return e;
     moin_lora_job jobs[MOIN_MAX_GROUP];
-    for (int i = 0; i < n; ++i) jobs[i] = {in, weight(layer, p0 + i, d_in[i], d_out[i], i), &m->pools[layer * 7 + p0 + i], outs[i]};
-    if (wst) return wst;
-    return moin_lora_linear_group(&plan, jobs, n, m->lora_scale, w.lora, w.lora_bytes, stream);
+    for (int i = 0; i < n; ++i) {
+      if (!lora) {
+        e = moin_lora_linear(nullptr, in, W[i], nullptr, 0.f, T, d_in, d_out[i], outs[i], w.lora, w.lora_bytes, stream);
+        if (e) return e;
+      } else {
+        jobs[i] = {in, W[i], &m->pools[layer * 7 + p0 + i], outs[i]};
+      }
+    }
+    return lora ? moin_lora_linear_group(&plan, jobs, n, m->lora_scale, w.lora, w.lora_bytes, stream) : MOIN_OK;
   };
   const float scale_log2 = 1.4426950408889634f / sqrtf(64.f);
   const __nv_bfloat16* pending = nullptr;
@@ -469,9 +494,9 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     { ProfScope prof(MOIN_K_GLUE, 1, s);
       launch_pdl(add_rmsnorm_kernel, T, 256, 0, s, w.res, pending, (const __nv_bfloat16*)m->attn_norm[l], w.xn, H, m->rms_eps, nullptr); }
     {
-      const int din[3] = {H, H, H}, dout[3] = {qd, kvd, kvd};
+      const int dout[3] = {qd, kvd, kvd};
       void* const outs[3] = {w.q, w.k, w.v};
-      if ((st = proj_group(l, 0, 3, w.xn, din, dout, outs))) return st;
+      if ((st = proj_group(l, 0, 3, w.xn, H, dout, outs))) return st;
     }
     // rotary embedding: the keys are rotated in place once (every query head and every later query reads them);
     // the queries are rotated inside the attention kernel as it loads them
@@ -487,17 +512,18 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
       attention_kernel<<<dim3((max_seqlen + 63) / 64, nh, R), 128, 0, s>>>(w.q, w.k, w.v, cu_seqlens, w.att, nh, nkv, scale_log2,
                                                                          w.rope);
     }
-    if ((st = proj(l, 3, w.att, qd, H, w.o))) return st;
+    void* const o_out[1] = {w.o};   // (also the down projection's)
+    if ((st = proj_group(l, 3, 1, w.att, qd, &H, o_out))) return st;
     { ProfScope prof(MOIN_K_GLUE, 1, s);
       launch_pdl(add_rmsnorm_kernel, T, 256, 0, s, w.res, w.o, (const __nv_bfloat16*)m->mlp_norm[l], w.xn, H, m->rms_eps, nullptr); }
     {
-      const int din[2] = {H, H}, dout[2] = {F, F};
+      const int dout[2] = {F, F};
       void* const outs[2] = {w.gate, w.up};
-      if ((st = proj_group(l, 4, 2, w.xn, din, dout, outs))) return st;
+      if ((st = proj_group(l, 4, 2, w.xn, H, dout, outs))) return st;
     }
     { ProfScope prof(MOIN_K_GLUE, 1, s);
       launch_pdl(swiglu_kernel, (int)(((long)T * F / 8 + 255) / 256), 256, 0, s, w.gate, w.up, (long)T * F / 8); }
-    if ((st = proj(l, 6, w.gate, F, H, w.o))) return st;
+    if ((st = proj_group(l, 6, 1, w.gate, F, &H, o_out))) return st;
     pending = w.o;
   }
   if (pending) { ProfScope prof(MOIN_K_GLUE, 1, s);
@@ -544,13 +570,13 @@ extern "C" moin_status moin_dequant_fp8(const void* codes, const float* scale, i
                                         moin_stream stream) {
   if (!codes || !scale || !W || d_out < 0 || d_in < 0) return MOIN_ERR_INVALID_ARG;
   if ((d_in % 16) != 0) return MOIN_ERR_BAD_SHAPE;
-  if ((reinterpret_cast<uintptr_t>(codes) & 15u) || (reinterpret_cast<uintptr_t>(W) & 15u)) return MOIN_ERR_MISALIGNED;
-  const long n16 = (long)d_out * d_in / 16;
-  if (n16 == 0) return MOIN_OK;
+  if (!aligned16(codes) || !aligned16(W)) return MOIN_ERR_MISALIGNED;
+  if (d_out == 0 || d_in == 0) return MOIN_OK;
   HostState* hs;
   moin_status st = host_state(&hs);
   if (st) return st;
-  ProfScope prof(MOIN_K_GLUE, 1, (cudaStream_t)stream);
-  return record_cuda(launch_pdl(dequant_fp8_kernel, (unsigned)((n16 + 255) / 256), 256, 0, (cudaStream_t)stream,
-                                (const uint4*)codes, scale, d_in / 16, n16, (uint4*)W));
+  DequantJobs jobs = {};
+  jobs.n = 1;
+  jobs.codes[0] = (const uint2*)codes; jobs.scale[0] = scale; jobs.out[0] = (uint4*)W; jobs.row_end[0] = d_out;
+  return launch_dequant(jobs, d_in, (cudaStream_t)stream);
 }
