@@ -409,7 +409,8 @@ moin_status moin_pool_set_adapter(const moin_pool* pool, int32_t expert, int32_t
  * scale per output row.  The weight the layer uses is W[j][i] = bf16(fp32(value(codes[j][i]) * scale[j])): this call
  * writes it, and the ordinary entry points then run on it, so the adapters, the accumulation and the tolerance are
  * those of the bf16 layer.  The base model is then stored in half of its bf16 size; a decoder forward with
- * moin_model.W8 set dequantises one projection group at a time into its workspace (at most three matrices live).
+ * moin_model.W8 set dequantises one projection group at a time into its workspace (at most three matrices live), or,
+ * with few tokens in short segments, to the same values inside the GEMM.
  *   codes  device, [d_out, d_in] bytes, 16-byte aligned; d_in a multiple of 16
  *   scale  device, [d_out] fp32
  *   W      device, [d_out, d_in] bf16, 16-byte aligned (output)

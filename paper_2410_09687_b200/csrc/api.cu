@@ -528,7 +528,7 @@ static moin_status launch_base_gemm(HostState* hs, bool use_tc, const __nv_bfloa
   ProfScope prof(use_tc ? MOIN_K_GEMM_TC : MOIN_K_GEMM_WARP, 1, s);
   if (!use_tc) return record_cuda(launch_gemm_warp(x, W, y, y0, T, d_in, d_out, s));
   if (T <= kDecodeGemmMaxT) {
-    const DecodeGemmJob job = {x, W, y, y0, d_in, d_out};
+    const DecodeGemmJob job = {x, W, y, y0, d_in, d_out, nullptr};
     return launch_decode_gemm(hs, &job, 1, T, s);
   }
   const PairJob job = {x, W, nullptr, y, y0, nullptr, d_out};
@@ -545,6 +545,13 @@ size_t moin_lora_linear_group_workspace_bytes(int32_t T, const moin_lora_job* jo
 
 moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, int32_t n_jobs, float scale,
                                    void* workspace, size_t workspace_bytes, moin_stream stream) {
+  return lora_linear_group(plan, jobs, nullptr, n_jobs, scale, workspace, workspace_bytes, stream);
+}
+
+}  // extern "C"
+
+moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, const float* const* w_scale,
+                                    int n_jobs, float scale, void* workspace, size_t workspace_bytes, moin_stream stream) {
   if (!plan || !jobs || n_jobs < 1 || n_jobs > MOIN_MAX_GROUP) return MOIN_ERR_INVALID_ARG;
   int T = 0, d_in[kMaxStreamJobs], d_out[kMaxStreamJobs], r[kMaxStreamJobs];
   for (int j = 0; j < n_jobs; ++j) {
@@ -570,7 +577,7 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
     if ((st = pick_gemm(hs, T, d_in[j], d_out[j], &use_tc[j]))) return st;
   }
 
-  if (plan->mode == MOIN_PLAN_TILES) {
+  if (plan->mode == MOIN_PLAN_TILES && !w_scale) {
     // Long runs: every projection is one grouped-shrink + one fused GEMM launch on the tensor cores.
     bool all_tc = true;
     for (int j = 0; j < n_jobs; ++j)
@@ -619,13 +626,15 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
     h[j] = reinterpret_cast<float*>(ws_job[j]);   // [T][r] shrink results
     y0[j] = reinterpret_cast<float*>(ws_job[j] + align_up((size_t)T * (size_t)r[j] * sizeof(float), 256));
   }
-  bool grouped = T <= kDecodeGemmMaxT;
+  bool grouped = T <= (w_scale ? kDecodeFp8MaxT : kDecodeGemmMaxT);
   for (int j = 0; j < n_jobs; ++j) grouped = grouped && use_tc[j];
+  if (w_scale && !grouped) return MOIN_ERR_BAD_SHAPE;   // (decode_fp8_supported says so before)
   if (grouped) {
     ProfScope prof(MOIN_K_GEMM_TC, 1, s);
     DecodeGemmJob gj[kMaxStreamJobs];
     for (int j = 0; j < n_jobs; ++j)
-      gj[j] = {(const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W, (__nv_bfloat16*)jobs[j].y, y0[j], d_in[j], d_out[j]};
+      gj[j] = {(const __nv_bfloat16*)jobs[j].x, jobs[j].W, (__nv_bfloat16*)jobs[j].y, y0[j], d_in[j], d_out[j],
+               w_scale ? w_scale[j] : nullptr};
     st = launch_decode_gemm(hs, gj, n_jobs, T, s);
   } else {
     for (int j = 0; j < n_jobs && !st; ++j)
@@ -665,6 +674,8 @@ moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* j
   }
   return record_cuda(launch_lora_expand_stream(pv, ej, scale, hs->n_sms, s));
 }
+
+extern "C" {
 
 moin_status moin_lora_linear(const moin_plan* plan, const void* x, const void* W, const moin_pool* pool,
                              float scale, int32_t base_T, int32_t base_d_in, int32_t base_d_out, void* y,

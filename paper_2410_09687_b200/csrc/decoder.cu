@@ -474,6 +474,22 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
   };
   // projections of a block that read the same input and do not depend on one another go out as one group
   auto proj_group = [&](int layer, int p0, int n, const void* in, int d_in, const int* d_out, void* const* outs) -> moin_status {
+    // few tokens in short segments: the GEMM converts the codes itself (gemm_decode.cu has both sides' times)
+    bool coded = m->W8 && decode_fp8_supported(hs, T) && (!lora || plan.mode == MOIN_PLAN_SEGMENTS);
+    for (int j = 0; j < n && coded; ++j) coded = m->W8[layer * 7 + p0 + j] && m->W_scale && m->W_scale[layer * 7 + p0 + j];
+    if (coded) {
+      moin_lora_job jobs[MOIN_MAX_GROUP];
+      DecodeGemmJob gemm[MOIN_MAX_GROUP];
+      for (int j = 0; j < n; ++j) {
+        const int i = layer * 7 + p0 + j;
+        if (!aligned16(m->W8[i])) return MOIN_ERR_MISALIGNED;
+        if (lora) jobs[j] = {in, m->W8[i], &m->pools[i], outs[j]};
+        else gemm[j] = {(const __nv_bfloat16*)in, m->W8[i], (__nv_bfloat16*)outs[j], nullptr, d_in, d_out[j], m->W_scale[i]};
+      }
+      if (lora) return lora_linear_group(&plan, jobs, m->W_scale + layer * 7 + p0, n, m->lora_scale, w.lora, w.lora_bytes, stream);
+      ProfScope prof(MOIN_K_GEMM_TC, 1, s);
+      return launch_decode_gemm(hs, gemm, n, T, s);
+    }
     const void* W[MOIN_MAX_GROUP];
     moin_status e = weights(layer, p0, n, d_in, d_out, W);
     if (e) return e;

@@ -12,6 +12,13 @@
 //   warps 2-5  read the accumulator (TMEM lane = feature, column = token); all warps store
 // What bounds it: at small T the HBM stream of W plus ~4 us of set-up and first round trip; at T = 256 the 32 KB of x
 // that every 16 KB block of W brings along (an SM takes about 64 bytes per clock from L2).
+//
+// 8-bit weights (FP8): warps 2-5, idle until the epilogue otherwise, turn each stage's codes into the bf16 weights that
+// the stand-alone conversion makes - a thread has one row of the tile, so one scale - and put them into tensor memory as
+// the A operand (32 columns a stage).  HBM reads one byte a weight and nothing is written; a tile takes at most 128
+// tokens, so that tensor memory holds the accumulator and four stages or more with two CTAs on an SM, and more tokens
+// convert a tile again from L2.  Bound by the conversion, 128 threads at about six instructions for two codes.  Forward on
+// the 8-bit base with a converted copy per group / this: 112 tokens 2499 / 1871 us, 303 3746 / 2665, 495 4525 / 3525.
 #include <cuda.h>
 
 #include "ptx.cuh"
@@ -20,6 +27,7 @@
 namespace moin {
 
 constexpr int kDgThreads = 192, kDgM = 128, kDgK = 64, kDgMaxN = 256, kDgMaxStages = 8, kDgMaxSplit = 8;
+constexpr int kDgFp8MaxN = 128, kDgFp8Cols = 256, kDgFp8Smem = 104 * 1024;
 
 struct DgMaps { CUtensorMap w[kMaxStreamJobs], x[kMaxStreamJobs]; };
 struct DgParams {
@@ -28,19 +36,23 @@ struct DgParams {
   int ks[kMaxStreamJobs], tiles[kMaxStreamJobs], K[kMaxStreamJobs], d_out[kMaxStreamJobs];
   __nv_bfloat16* y[kMaxStreamJobs];
   float* y0[kMaxStreamJobs];     // fp32 copy, nullable
+  const float* w_scale[kMaxStreamJobs];   // FP8: scale per row of W
   DeviceStatus* status;
 };
 
+template <bool FP8>
 __global__ void __launch_bounds__(kDgThreads)
 decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t ring = (raw + 1023u) & ~1023u;
   const int S = p.stages;
-  const uint32_t stage_bytes = (uint32_t)(kDgM + p.nt) * kDgK * 2;
+  constexpr uint32_t kWBytes = kDgM * kDgK * (FP8 ? 1 : 2);
+  const uint32_t stage_bytes = kWBytes + (uint32_t)p.nt * kDgK * 2;
   const uint32_t bars = ring + (uint32_t)S * stage_bytes;
   uint8_t* bar_ptr = smem_raw + (bars - raw);
   const uint32_t full0 = bars, empty0 = bars + 8 * kDgMaxStages, done = bars + 16 * kDgMaxStages;
+  const uint32_t conv0 = bars + 16 * kDgMaxStages + 32;   // FP8: the stage's weights are in tensor memory
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + 16 * kDgMaxStages + 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 16 * kDgMaxStages + 16);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -52,10 +64,12 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   int K = p.K[0], d_out = p.d_out[0], ks = p.ks[0], n_tiles = p.tiles[0], first = 0;
   __nv_bfloat16* y = p.y[0];
   float* y0 = p.y0[0];
+  const float* w_scale = p.w_scale[0];
 #pragma unroll
   for (int j = 1; j < kMaxStreamJobs; ++j)
     if (job == j) {
       K = p.K[j]; d_out = p.d_out[j]; ks = p.ks[j]; n_tiles = p.tiles[j]; y = p.y[j]; y0 = p.y0[j];
+      w_scale = p.w_scale[j];
       first = p.cta_end[j - 1];
     }
   // ks consecutive CTAs of a cluster share an item = (feature tile, token chunk)
@@ -70,6 +84,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
+      if (FP8) mbar_init(conv0 + 8 * s, 4);
     }
     mbar_init(done, 1);
     *abort_flag = 0;
@@ -87,6 +102,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   pdl_launch_dependents();   // the adapter shrink does not read this kernel's results: it may take the free SM slots
 
   bool ok = true;
+  const uint32_t a_col = ((uint32_t)p.nt + 31u) & ~31u;   // FP8: first tensor-memory column of the converted weights
   if (warp == 0) {
     if (lane == 0) {
       const CUtensorMap* mw = &maps.w[job];
@@ -98,7 +114,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
         if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
         mbar_expect_tx(full, stage_bytes);
         tma_load_2d(sa, mw, full, kb * kDgK, f0);
-        tma_load_2d(sa + kDgM * kDgK * 2, mx, full, kb * kDgK, tok0);
+        tma_load_2d(sa + kWBytes, mx, full, kb * kDgK, tok0);
       }
     }
     __syncwarp();
@@ -108,21 +124,55 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
     uint32_t s = 0, ph = 0;
     for (int kb = kb0; kb < kb1 && ok; ++kb) {
       if (!(ok = mbar_wait_warp(full0 + 8 * s, ph, abort_flag, p.status, 52))) break;
+      if (FP8 && !(ok = mbar_wait_warp(conv0 + 8 * s, ph, abort_flag, p.status, 54))) break;
       tc_fence_after();
-      const uint32_t sa = ring + s * stage_bytes, empty = empty0 + 8 * s;
+      const uint32_t sa = ring + s * stage_bytes, empty = empty0 + 8 * s, ta = tmem + a_col + s * (kDgK / 2);
       if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
-      const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sa + kDgM * kDgK * 2);
+      const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sa + kWBytes);
       if (leader) {
 #pragma unroll
-        for (int k = 0; k < kDgK / 16; ++k)
-          tc_mma_bf16(tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+        for (int k = 0; k < kDgK / 16; ++k) {
+          const uint32_t acc = (kb > kb0 || k > 0) ? 1u : 0u;
+          if (FP8) tc_mma_bf16_ta(tmem, ta + 8 * k, db + (uint64_t)(2 * k), idesc, acc);
+          else tc_mma_bf16(tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc);
+        }
         tc_commit(empty);
       }
     }
     if (ok && leader) tc_commit(done);
     __syncwarp();
   } else {
-    ok = mbar_wait(done, 0, abort_flag, p.status, 53);
+    if (FP8) {   // a thread converts one row (TMEM lane) of the stage's codes; its scale stays in a register
+      const int row = (warp & 3) * 32 + lane;
+      const float sc = on && f0 + row < d_out ? __ldg(w_scale + f0 + row) : 0.f;
+      const uint32_t swz = (uint32_t)(row >> 1) & 3u;   // 64-byte swizzle: 16-byte piece c of a row lies at c ^ swz
+      uint32_t s = 0, ph = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!(ok = mbar_wait_warp(full0 + 8 * s, ph, abort_flag, p.status, 55))) break;
+        tc_fence_after();
+        const uint32_t sa = ring + s * stage_bytes + (uint32_t)row * kDgK;
+        const uint32_t ta = tmem + ((uint32_t)((warp & 3) * 32) << 16) + a_col + s * (kDgK / 2);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t v[16];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const uint4 w = lds_u4(sa + (((uint32_t)(2 * h + c) ^ swz) << 4));
+            fp8x4_to_bf16(w.x, sc, v[8 * c], v[8 * c + 1]);
+            fp8x4_to_bf16(w.y, sc, v[8 * c + 2], v[8 * c + 3]);
+            fp8x4_to_bf16(w.z, sc, v[8 * c + 4], v[8 * c + 5]);
+            fp8x4_to_bf16(w.w, sc, v[8 * c + 6], v[8 * c + 7]);
+          }
+          tmem_st16(ta + 16 * h, v);
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(conv0 + 8 * s);
+        if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
+      }
+    }
+    ok = ok && mbar_wait(done, 0, abort_flag, p.status, 53);
     tc_fence_after();
   }
   // ---------------------------------------------------------------- epilogue
@@ -194,10 +244,14 @@ moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_j
   // Split a projection's reduction until its own CTAs fill their share of the SM slots or a CTA is down to four 64-wide
   // blocks (from the shape alone: the same bits in any group).  Beside many tokens' adapters the share is half of the
   // SMs (decode step of 256 tokens with half / all / a quarter: 237 / 264 / 248 us); up to 64 tokens two CTAs fit an SM
-  // and there is little to stream beside them (step of 24 tokens with half / all: 88 / 87 us).
-  const int chunks0 = (T + kDgMaxN - 1) / kDgMaxN;
+  // and there is little to stream beside them (step of 24 tokens with half / all: 88 / 87 us).  8-bit codes: once all
+  // SMs, whatever the tokens (forwards of 112 / 303 / 495 tokens with half 1933 / 3263 / 4020 us, all 1871 / 2665 /
+  // 3525, twice 1992 / 2795 / 3516).
+  const bool fp8 = jobs[0].w_scale != nullptr;
+  const int max_n = fp8 ? kDgFp8MaxN : kDgMaxN;
+  const int chunks0 = (T + max_n - 1) / max_n;
   const bool small = (T + chunks0 - 1) / chunks0 <= 64;
-  const int limit = small ? 2 * hs->n_sms : hs->n_sms / 2;
+  const int limit = fp8 ? hs->n_sms : small ? 2 * hs->n_sms : hs->n_sms / 2;
   int items = 0;   // CTAs with one token tile per 256 tokens
   p.cluster = 1;
   for (int j = 0; j < n_jobs; ++j) {
@@ -217,11 +271,13 @@ moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_j
     p.nt = ((T + p.n_chunks - 1) / p.n_chunks + 15) / 16 * 16;
   }
   for (int j = 0; j < n_jobs; ++j) {
-    moin_status st = make_map(&maps.w[j], jobs[j].W, jobs[j].d_out, jobs[j].d_in, kDgM);
+    moin_status st = fp8 ? make_map_u8(&maps.w[j], jobs[j].W, jobs[j].d_out, jobs[j].d_in, kDgM)
+                         : make_map(&maps.w[j], jobs[j].W, jobs[j].d_out, jobs[j].d_in, kDgM);
     if (!st) st = make_map(&maps.x[j], jobs[j].x, T, jobs[j].d_in, p.nt);
     if (st) return st;
     p.K[j] = jobs[j].d_in; p.d_out[j] = jobs[j].d_out;
     p.y[j] = jobs[j].y; p.y0[j] = jobs[j].y0;
+    p.w_scale[j] = jobs[j].w_scale;
   }
   int ctas = 0;
   for (int j = 0; j < n_jobs; ++j) {
@@ -230,15 +286,25 @@ moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_j
   }
   // Shared memory: the stream kernels beside this one feed on L1, which gets what shared memory leaves (228 KB in all):
   // 150 KB an SM against 192: decode step of 256 tokens 237 / 254 us.
-  const int stage = (kDgM + p.nt) * kDgK * 2, budget = 150 * 1024 / (p.nt <= 64 ? 2 : 1);
+  const int stage = kDgM * kDgK * (fp8 ? 1 : 2) + p.nt * kDgK * 2;
+  const int budget = fp8 ? kDgFp8Smem : 150 * 1024 / (p.nt <= 64 ? 2 : 1);
   p.stages = budget / stage < kDgMaxStages ? budget / stage : kDgMaxStages;
   p.tmem_cols = 32;
   while (p.tmem_cols < p.nt) p.tmem_cols *= 2;
+  if (fp8) {
+    const int slots = (kDgFp8Cols - (p.nt + 31) / 32 * 32) / (kDgK / 2);   // tensor-memory buffers of converted weights
+    if (p.stages > slots) p.stages = slots;
+    p.tmem_cols = kDgFp8Cols;
+  }
   // the ring is also the fp32 staging of the epilogue
   const size_t out = (size_t)p.nt * kDgM * sizeof(float);
   while ((size_t)p.stages * stage < out) ++p.stages;
-  const size_t smem = (size_t)p.stages * stage + 1024 /*align*/ + 256 /*barriers*/;
-  cudaError_t e = ensure_smem_optin(OPTIN_DECODE_GEMM, decode_gemm_kernel, 160 * 1024);
+  size_t smem = (size_t)p.stages * stage + 1024 /*align*/ + 256 /*barriers*/;
+  auto* kernel = fp8 ? decode_gemm_kernel<true> : decode_gemm_kernel<false>;
+  // Half of the tensor memory for less than half of the shared memory would let a third CTA in, which then waits in the
+  // allocation for CTAs that may wait for its own cluster: two at most.
+  if (fp8 && smem < kDgFp8Smem) smem = kDgFp8Smem;
+  cudaError_t e = ensure_smem_optin(fp8 ? OPTIN_DECODE_GEMM_FP8 : OPTIN_DECODE_GEMM, kernel, 160 * 1024);
   if (e != cudaSuccess) return record_cuda(e);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ctas);
@@ -253,7 +319,7 @@ moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_j
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  return record_cuda(cudaLaunchKernelEx(&cfg, decode_gemm_kernel, maps, p));
+  return record_cuda(cudaLaunchKernelEx(&cfg, kernel, maps, p));
 }
 
 }  // namespace moin

@@ -10,6 +10,9 @@ namespace moin {
 // (columns of the box beyond `cols` read as zero).
 moin_status make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 
+// The same for bytes: a [box_rows x 64] box, 64-byte swizzle.
+moin_status make_map_u8(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
+
 // Shape predicates (host): can the tcgen05 kernels take this problem?
 bool tc_gemm_supported(int T, int d_in, int d_out);
 bool tc_router_supported(int Q, int K, int D);
@@ -17,9 +20,15 @@ bool tc_fused_supported(int r);
 
 // y = x W^T (bf16) and optionally y0 = x W^T (fp32) for few tokens, up to kMaxStreamJobs projections in one launch
 // (gemm_decode.cu).
-struct DecodeGemmJob { const __nv_bfloat16 *x, *W; __nv_bfloat16* y; float* y0; int d_in, d_out; };
-constexpr int kDecodeGemmMaxT = 512;
+// w_scale != nullptr: W is 8-bit float codes with a scale per row (all jobs of a launch alike), T <= kDecodeFp8MaxT.
+struct DecodeGemmJob { const __nv_bfloat16* x; const void* W; __nv_bfloat16* y; float* y0; int d_in, d_out; const float* w_scale; };
+constexpr int kDecodeGemmMaxT = 512, kDecodeFp8MaxT = 512;
 moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, cudaStream_t stream);
+// moin_lora_linear_group on a base of 8-bit codes: jobs[j].W points to them and w_scale[j] to their row scales (nullptr:
+// bf16 weights).  Short segments and few tokens only.
+inline bool decode_fp8_supported(const HostState* hs, int T) { return hs->gemm_impl != 1 && T <= kDecodeFp8MaxT; }
+moin_status lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, const float* const* w_scale, int n_jobs,
+                              float scale, void* workspace, size_t workspace_bytes, moin_stream stream);
 // Long-run GEMMs on CTA pairs (tc_pair.cu): y_j = x_j W_j^T for up to kPairJobs projections of one K; with a plan the
 // low-rank term s x A_e^T B_e^T is added from hb (hi / lo parts of s x A_e^T, [2][M][r], all jobs of the same r).
 constexpr int kPairJobs = 3;

@@ -7,7 +7,7 @@ import torch
 import moin_inputs as mi
 import oracle
 import paper_2410_09687_b200 as moin
-from gpu_util import DEV
+from gpu_util import DEV, REL_FRO
 from test_gpu_quant import quantise
 
 pytestmark = pytest.mark.gpu
@@ -38,3 +38,24 @@ def test_some_projections_coded(coded):
         args = (batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths))
         # the same bf16 weights through the same kernels
         assert torch.equal(moin.decoder_forward(mixed, *args), moin.decoder_forward(ref, *args))
+
+
+@pytest.mark.parametrize("T", [1, 16, 17, 33, 64, 65, 128, 129, 300, 512, 513])
+@pytest.mark.parametrize("adapters", [True, False])
+def test_few_tokens(T, adapters):
+    """Short segments: the GEMM converts the codes itself; edges of its token tile and of the rule that takes it."""
+    cfg = mi.DecoderConfig(n_layers=1, hidden=320, n_heads=5, n_kv_heads=1, head_dim=64, ffn=1088, vocab=512, E=4, r=16, scale=2.0)
+    model = mi.decoder_model(cfg, seed=4)
+    q = {p: quantise(model.W[0][p]) for p in oracle.PROJ_ORDER}
+    same = {p: torch.from_numpy(oracle.dequant_fp8(c.numpy(), s.numpy()).view(np.int16)).view(torch.bfloat16).to(DEV)
+            for p, (c, s) in q.items()}
+    coded = _decoder(cfg, model, [{}], [{p: c.to(DEV) for p, (c, s) in q.items()}], [{p: s.to(DEV) for p, (c, s) in q.items()}])
+    ref = _decoder(cfg, model, [same])
+    lengths = [min(37, T - i) for i in range(0, T, 37)]
+    batch = mi.decoder_batch(cfg, lengths, seed=6, req_expert=[i % 4 for i in range(len(lengths))])
+    args = [batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV) if adapters else None, max(lengths)]
+    got, want = (moin.decoder_forward(m, *args).double() for m in (coded, ref))
+    # the same bf16 weights, sums of 32-bit products in another order: two bf16 roundings of a chain of four projections
+    assert torch.isfinite(got).all()
+    assert ((got - want).norm() / want.norm()).item() <= REL_FRO * 2 ** 0.5
+    assert moin.device_status()["timeout_flag"] == 0
