@@ -675,6 +675,41 @@ moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* 
   return record_cuda(launch_lora_expand_stream(pv, ej, scale, hs->n_sms, s));
 }
 
+bool moin::swiglu_supported(const HostState* hs, const moin_plan* plan, const moin_pool* pools, int T, int d_in, int d_out) {
+  if (hs->gemm_impl == 1 || !tc_gemm_supported(T, d_in, d_out) || d_out < 64) return false;
+  if (!plan) return T > kDecodeGemmMaxT;
+  return plan->mode == MOIN_PLAN_TILES && T >= 64 && pools[0].r == pools[1].r && tc_fused_supported(pools[0].r) &&
+         pools[0].activation == pools[1].activation;
+}
+
+moin_status moin::lora_swiglu(HostState* hs, const moin_plan* plan, const moin_lora_job* jobs, float scale, int T, int d_in,
+                              int d_out, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
+  int t, di, dO, r;
+  moin_status st;
+  for (int j = 0; j < 2; ++j)
+    if ((st = check_job(plan, jobs[j].x, jobs[j].W, jobs[j].pool, jobs[j].y, plan != nullptr, T, d_in, d_out, &t, &di, &dO, &r)))
+      return st;
+  if (plan && workspace_bytes < moin_lora_linear_group_workspace_bytes(T, jobs, 2)) return MOIN_ERR_WORKSPACE;
+  PairJob pj[2];
+  const moin_pool* pools[2] = {jobs[0].pool, jobs[1].pool};
+  const __nv_bfloat16* xs[2];
+  __nv_bfloat16* hbs[2];
+  char* ws = reinterpret_cast<char*>(workspace);
+  for (int j = 0; j < 2; ++j) {
+    xs[j] = (const __nv_bfloat16*)jobs[j].x;
+    hbs[j] = reinterpret_cast<__nv_bfloat16*>(ws);
+    if (plan) ws += align_up(moin_lora_linear_workspace_bytes(T, d_in, d_out, r), 256);
+    pj[j] = {xs[j], (const __nv_bfloat16*)jobs[j].W, hbs[j], (__nv_bfloat16*)jobs[0].y, nullptr, pools[j], d_out};
+  }
+  PlanView pv;
+  if (plan) {
+    pv = plan_view(plan->buffer, plan->T, plan->E);
+    if ((st = launch_tc_shrink_group(hs, pv, pools, xs, hbs, 2, scale, stream))) return st;
+  }
+  ProfScope prof(plan ? MOIN_K_FUSED_TC : MOIN_K_GEMM_TC, 1, stream);
+  return launch_pair_swiglu(hs, plan ? &pv : nullptr, pj, T, d_in, stream);
+}
+
 extern "C" {
 
 moin_status moin_lora_linear(const moin_plan* plan, const void* x, const void* W, const moin_pool* pool,

@@ -243,7 +243,7 @@ moin_status record_cuda(cudaError_t e);       // MOIN_OK or MOIN_ERR_CUDA (remem
 // that attribute per device, so the "already done" note is kept per device too (slot = one id per kernel).
 enum {
   OPTIN_ROUTE_CLUSTER = 24, /* .. 27 */ OPTIN_ROUTE_SIMPLE = 28, OPTIN_ATTENTION = 29,
-  OPTIN_DECODE_GEMM = 30, OPTIN_TC_PAIR = 31 /* .. 33 */, OPTIN_TC_SHRINK = 34, OPTIN_DECODE_GEMM_FP8 = 35
+  OPTIN_DECODE_GEMM = 30, OPTIN_TC_PAIR = 31 /* .. 34 */, OPTIN_TC_SHRINK = 35, OPTIN_DECODE_GEMM_FP8 = 36
 };
 template <class Fn>
 inline cudaError_t ensure_smem_optin(int slot, Fn* fn, size_t bytes) {

@@ -532,13 +532,20 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     if ((st = proj_group(l, 3, 1, w.att, qd, &H, o_out))) return st;
     { ProfScope prof(MOIN_K_GLUE, 1, s);
       launch_pdl(add_rmsnorm_kernel, T, 256, 0, s, w.res, w.o, (const __nv_bfloat16*)m->mlp_norm[l], w.xn, H, m->rms_eps, nullptr); }
-    {
-      const int dout[2] = {F, F};
+    const int dout_f[2] = {F, F};
+    const moin_pool* mlp_pools = lora ? &m->pools[l * 7 + 4] : nullptr;
+    if (swiglu_supported(hs, lora ? &plan : nullptr, mlp_pools, T, H, F)) {   // long runs: the product in the GEMM's epilogue
+      const void* W[2];
+      if ((st = weights(l, 4, 2, H, dout_f, W))) return st;
+      const moin_lora_job jobs[2] = {{w.xn, W[0], mlp_pools, w.gate}, {w.xn, W[1], lora ? mlp_pools + 1 : nullptr, w.up}};
+      if ((st = lora_swiglu(hs, lora ? &plan : nullptr, jobs, m->lora_scale, T, H, F, w.lora, w.lora_bytes, s)))
+        return st;
+    } else {
       void* const outs[2] = {w.gate, w.up};
-      if ((st = proj_group(l, 4, 2, w.xn, H, dout, outs))) return st;
+      if ((st = proj_group(l, 4, 2, w.xn, H, dout_f, outs))) return st;
+      ProfScope prof(MOIN_K_GLUE, 1, s);
+      launch_pdl(swiglu_kernel, (int)(((long)T * F / 8 + 255) / 256), 256, 0, s, w.gate, w.up, (long)T * F / 8);
     }
-    { ProfScope prof(MOIN_K_GLUE, 1, s);
-      launch_pdl(swiglu_kernel, (int)(((long)T * F / 8 + 255) / 256), 256, 0, s, w.gate, w.up, (long)T * F / 8); }
     if ((st = proj_group(l, 6, 1, w.gate, F, &H, o_out))) return st;
     pending = w.o;
   }

@@ -35,6 +35,13 @@ constexpr int kPairJobs = 3;
 struct PairJob { const __nv_bfloat16 *x, *W, *hb; __nv_bfloat16* y; float* y0; const moin_pool* pool; int N; };   // y0: fp32 copy or nullptr
 moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* jobs, int n_jobs, int M, int K,
                              cudaStream_t stream);
+// jobs[0].y = silu(x Wg^T + ..) * (x Wu^T + ..): gate and up projection (of one x, N and rank) in one launch.
+moin_status launch_pair_swiglu(HostState* hs, const PlanView* pv, const PairJob* jobs, int M, int K, cudaStream_t stream);
+// Can a block's gate and up projections take that path (pools: both, or nullptr without adapters)?
+bool swiglu_supported(const HostState* hs, const moin_plan* plan, const moin_pool* pools, int T, int d_in, int d_out);
+// ... and the path: the shrinks, then launch_pair_swiglu.  jobs[0].y is the result, jobs[1].y is not written.
+moin_status lora_swiglu(HostState* hs, const moin_plan* plan, const moin_lora_job* jobs, float scale, int T, int d_in,
+                        int d_out, void* workspace, size_t workspace_bytes, cudaStream_t stream);
 // keys[i] = max over k of (orderable(<q_i,c_k> * inv_norm[k]) << 32 | (0xFFFFFFFF - k)), merged with atomicMax.
 moin_status launch_pair_router(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm, int Q,
                                int K, int D, unsigned long long* keys, cudaStream_t stream,

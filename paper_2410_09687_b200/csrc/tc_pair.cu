@@ -27,11 +27,11 @@
 namespace moin {
 
 constexpr int kPairThreads = 320, kPairM = 128, kPairK = 64;
-enum { PAIR_STORE = 0, PAIR_ROUTER = 1, PAIR_ROUTER2 = 2 };
+enum { PAIR_STORE = 0, PAIR_ROUTER = 1, PAIR_ROUTER2 = 2, PAIR_SWIGLU = 3 };
 
 struct PairMaps { CUtensorMap x[kPairJobs], w[kPairJobs], b[kPairJobs], hi[kPairJobs], lo[kPairJobs], y[kPairJobs]; };
 struct PairParams {
-  int M, K, n_jobs, bn;                  // bn: tile width, a multiple of 16 up to 256
+  int M, K, n_jobs, bn, cols;            // bn: tile width, a multiple of 16 up to 256; cols: output columns of it
   int N[kPairJobs], tn_end[kPairJobs];   // columns, column tiles of jobs 0 .. j
   const int *header, *tile_row0, *tile_rows, *tile_expert;   // plan (header == nullptr: regular grid over M)
   int tail_r;                            // stored rank of the appended low-rank blocks (0 = none)
@@ -53,8 +53,8 @@ __device__ __forceinline__ uint32_t pair_orderable(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// What a tile is: its job, first column, and for both CTAs of the pair the row tile and the adapter slot.
-struct PairTile { int job, n0, row0[2], rows[2], slot[2], rank[2]; };
+// What a tile is: its job, first column, and for both CTAs of the pair the row tile and its expert.
+struct PairTile { int job, n0, row0[2], rows[2], expert[2]; };
 
 __device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int tiles_m) {
   PairTile t;
@@ -66,26 +66,21 @@ __device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int
   for (int j = 0; j + 1 < kPairJobs; ++j)
     if (j + 1 < p.n_jobs && tn >= p.tn_end[j]) t.job = j + 1;
   int first = 0;
-  const int* slots = p.slot_of_expert[0];
-  const int* ranks = p.slot_rank[0];
 #pragma unroll
   for (int j = 1; j < kPairJobs; ++j)
-    if (t.job == j) { first = p.tn_end[j - 1]; slots = p.slot_of_expert[j]; ranks = p.slot_rank[j]; }
-  t.n0 = (tn - first) * p.bn;
+    if (t.job == j) first = p.tn_end[j - 1];
+  t.n0 = (tn - first) * p.cols;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const int tm = 2 * pm + c;
-    t.slot[c] = -1;
-    t.rank[c] = 0;
+    t.expert[c] = -1;
     t.row0[c] = p.M;      // no such row tile: the copy fills zeros, nothing is stored
     t.rows[c] = 0;
     if (tm < tiles_m) {
       if (p.header != nullptr) {
         t.row0[c] = __ldg(p.tile_row0 + tm);
         t.rows[c] = __ldg(p.tile_rows + tm);
-        const int e = __ldg(p.tile_expert + tm);
-        if (e >= 0 && p.tail_r > 0) t.slot[c] = __ldg(slots + e);
-        if (t.slot[c] >= 0) t.rank[c] = ranks ? min(__ldg(ranks + t.slot[c]), p.tail_r) : p.tail_r;
+        t.expert[c] = __ldg(p.tile_expert + tm);
       } else {
         t.row0[c] = tm * kPairM;
         t.rows[c] = min(kPairM, p.M - t.row0[c]);
@@ -94,21 +89,32 @@ __device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int
   }
   return t;
 }
-// Low-rank passes of a tile: pass 0 multiplies the adapter of the first CTA's rows (and of the second's where it is
-// the same one), pass 1 the second's where it differs.  live: bit c = CTA c's rows take part.
+// Low-rank passes of a tile for a projection: pass 0 multiplies the adapter of the first CTA's rows (and of the second's
+// where it is the same one), pass 1 the second's where it differs.  live: bit c = CTA c's rows take part.
 struct PairPasses { int n, slot[2], rank[2]; uint32_t live[2]; };
-__device__ __forceinline__ PairPasses pair_passes(const PairTile& t) {
+__device__ __forceinline__ PairPasses pair_passes(const PairParams& p, const PairTile& t, int job) {
+  const int* slots = p.slot_of_expert[0];
+  const int* ranks = p.slot_rank[0];
+#pragma unroll
+  for (int j = 1; j < kPairJobs; ++j)
+    if (job == j) { slots = p.slot_of_expert[j]; ranks = p.slot_rank[j]; }
+  int slot[2], rank[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    slot[c] = t.expert[c] >= 0 && p.tail_r > 0 ? __ldg(slots + t.expert[c]) : -1;
+    rank[c] = slot[c] < 0 ? 0 : ranks ? min(__ldg(ranks + slot[c]), p.tail_r) : p.tail_r;
+  }
   PairPasses q;
   q.n = 0;
   q.slot[0] = q.slot[1] = -1; q.rank[0] = q.rank[1] = 0; q.live[0] = q.live[1] = 0u;
-  if (t.slot[0] >= 0) {
-    q.slot[0] = t.slot[0]; q.rank[0] = t.rank[0];
-    q.live[0] = (t.slot[1] == t.slot[0]) ? 3u : 1u;
+  if (slot[0] >= 0) {
+    q.slot[0] = slot[0]; q.rank[0] = rank[0];
+    q.live[0] = (slot[1] == slot[0]) ? 3u : 1u;
     q.n = 1;
   }
-  if (t.slot[1] >= 0 && t.slot[1] != t.slot[0]) {
-    if (q.n == 0) { q.slot[0] = t.slot[1]; q.rank[0] = t.rank[1]; q.live[0] = 2u; }
-    else { q.slot[1] = t.slot[1]; q.rank[1] = t.rank[1]; q.live[1] = 2u; }
+  if (slot[1] >= 0 && slot[1] != slot[0]) {
+    if (q.n == 0) { q.slot[0] = slot[1]; q.rank[0] = rank[1]; q.live[0] = 2u; }
+    else { q.slot[1] = slot[1]; q.rank[1] = rank[1]; q.live[1] = 2u; }
     ++q.n;
   }
   return q;
@@ -163,36 +169,47 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      const uint32_t tx = (uint32_t)(2 * kPairM + p.bn) * kPairK * 2;   // both CTAs' copies of a stage
+      // both CTAs' copies of a stage: the operands, the low-rank blocks (SWIGLU: of half the columns at a time)
+      const uint32_t tx = (uint32_t)(2 * kPairM + p.bn) * kPairK * 2;
+      const uint32_t tx_tail = EPI == PAIR_SWIGLU ? (uint32_t)(2 * kPairM + p.bn / 2) * kPairK * 2 : tx;
       uint32_t it = 0;
       bool ok = true;
       for (int tile = pair; tile < total && ok; tile += n_pairs) {
         const PairTile t = pair_tile(p, tile, tiles_m);
-        const PairPasses pq = pair_passes(t);
         const int row0 = rank == 0 ? t.row0[0] : t.row0[1];
-        const int nkb = nkb_main + pq.n * 2 * nrb;
         const CUtensorMap* mx = &maps.x[t.job];
-        const CUtensorMap* mw = &maps.w[t.job];
-        const CUtensorMap* mb = &maps.b[t.job];
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        const CUtensorMap* mw = &maps.w[EPI == PAIR_SWIGLU ? (int)rank : t.job];
+        const int w0 = EPI == PAIR_SWIGLU ? t.n0 : t.n0 + (int)rank * (p.bn / 2);
+        for (int kb = 0; kb < nkb_main; ++kb, ++it) {
           const uint32_t s = it % S, ph = (it / S) & 1u;
           if (!(ok = mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 61))) break;
           const uint32_t sa = ring + s * kPairStageBytes, sb = sa + kPairM * kPairK * 2;
           const uint32_t bar = map_rank(full0 + 8 * s, 0);
           if (rank == 0) mbar_expect_tx(full0 + 8 * s, tx);
-          if (kb < nkb_main) {
-            tma_load_2d_pair(sa, mx, bar, kb * kPairK, row0);
-            tma_load_2d_pair(sb, mw, bar, kb * kPairK, t.n0 + (int)rank * (p.bn / 2));
-          } else {
-            const int q = kb - nkb_main, pass = q >= 2 * nrb ? 1 : 0, j = q - pass * 2 * nrb;
-            const int rb = j >= nrb ? j - nrb : j;            // hi blocks first, then lo blocks
-            const bool mine = ((pass ? pq.live[1] : pq.live[0]) >> rank) & 1u;
-            tma_load_2d_pair(sa, j < nrb ? &maps.hi[t.job] : &maps.lo[t.job], bar, rb * kPairK, mine ? row0 : p.M);
-            int n = p.N[0];
+          tma_load_2d_pair(sa, mx, bar, kb * kPairK, row0);
+          tma_load_2d_pair(sb, mw, bar, kb * kPairK, w0);
+        }
+        if (p.tail_r == 0) continue;
+        for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g) {
+          const int job = EPI == PAIR_SWIGLU ? g : t.job;
+          const PairPasses pq = pair_passes(p, t, job);
+          int n = p.N[0];
 #pragma unroll
-            for (int jj = 1; jj < kPairJobs; ++jj)
-              if (t.job == jj) n = p.N[jj];
-            tma_load_2d_pair(sb, mb, bar, rb * kPairK, (pass ? pq.slot[1] : pq.slot[0]) * n + t.n0 + (int)rank * (p.bn / 2));
+          for (int jj = 1; jj < kPairJobs; ++jj)
+            if (job == jj) n = p.N[jj];
+          for (int pass = 0; pass < pq.n && ok; ++pass) {
+            const bool mine = ((pass ? pq.live[1] : pq.live[0]) >> rank) & 1u;
+            const int b0 = (pass ? pq.slot[1] : pq.slot[0]) * n + t.n0 + (int)rank * (p.cols / 2);
+            for (int j = 0; j < 2 * nrb; ++j, ++it) {
+              const uint32_t s = it % S, ph = (it / S) & 1u;
+              if (!(ok = mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 61))) break;
+              const uint32_t sa = ring + s * kPairStageBytes, sb = sa + kPairM * kPairK * 2;
+              const uint32_t bar = map_rank(full0 + 8 * s, 0);
+              if (rank == 0) mbar_expect_tx(full0 + 8 * s, tx_tail);
+              const int rb = j >= nrb ? j - nrb : j;            // hi blocks first, then lo blocks
+              tma_load_2d_pair(sa, j < nrb ? &maps.hi[job] : &maps.lo[job], bar, rb * kPairK, mine ? row0 : p.M);
+              tma_load_2d_pair(sb, &maps.b[job], bar, rb * kPairK, b0);
+            }
           }
         }
       }
@@ -201,30 +218,22 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
     // ------------------------------------------------------------------ MMA issuer (first CTA, for both)
     if (rank == 0) {   // the whole warp walks the loop, one elected lane issues (see elect_one)
       const uint32_t idesc = idesc_bf16(2 * kPairM, p.bn);
+      const uint32_t idesc_tail = EPI == PAIR_SWIGLU ? idesc_bf16(2 * kPairM, p.bn / 2) : idesc;
       const bool leader = elect_one();
       uint32_t it = 0, lt = 0;
       bool ok = true;
       for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
-        PairPasses pq;
-        pq.n = 0;
-        if (p.tail_r > 0) pq = pair_passes(pair_tile(p, tile, tiles_m));
-        const int nkb = nkb_main + pq.n * 2 * nrb;
         const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
         if (!(ok = mbar_wait_cluster_warp(tempty0 + 8 * acc, aph ^ 1u, abort_flag, p.status, 62))) break;
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + acc * kPairMaxN;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = 0; kb < nkb_main; ++kb, ++it) {
           const uint32_t s = it % S, ph = (it / S) & 1u;
           if (!(ok = mbar_wait_cluster_warp(full0 + 8 * s, ph, abort_flag, p.status, 63))) break;
           tc_fence_after();
           const uint32_t sa = ring + s * kPairStageBytes, sb = sa + kPairM * kPairK * 2;
           const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sb);
-          int nk16 = (min(kPairK, p.K - kb * kPairK) + 15) / 16;
-          if (kb >= nkb_main) {
-            const int q = kb - nkb_main, pass = q >= 2 * nrb ? 1 : 0, j = q - pass * 2 * nrb;
-            const int rb = j >= nrb ? j - nrb : j;
-            nk16 = (min(kPairK, (pass ? pq.rank[1] : pq.rank[0]) - rb * kPairK) + 15) / 16;   // beyond the rank: no MMA
-          }
+          const int nk16 = (min(kPairK, p.K - kb * kPairK) + 15) / 16;
           if (leader) {
             if (nk16 == 4) {
 #pragma unroll
@@ -235,6 +244,30 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
                 tc_mma_bf16_pair(tmem_d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > 0 || k > 0) ? 1u : 0u);
             }
             tc_commit_pair(empty0 + 8 * s);
+          }
+        }
+        if (p.tail_r > 0) {
+          const PairTile t = pair_tile(p, tile, tiles_m);
+          for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g) {
+            const PairPasses pq = pair_passes(p, t, EPI == PAIR_SWIGLU ? g : t.job);
+            const uint32_t tmem_g = tmem_d + g * (p.bn / 2);
+            for (int pass = 0; pass < pq.n && ok; ++pass) {
+              const int rk = pass ? pq.rank[1] : pq.rank[0];
+              for (int j = 0; j < 2 * nrb; ++j, ++it) {
+                const uint32_t s = it % S, ph = (it / S) & 1u;
+                if (!(ok = mbar_wait_cluster_warp(full0 + 8 * s, ph, abort_flag, p.status, 63))) break;
+                tc_fence_after();
+                const uint32_t sa = ring + s * kPairStageBytes, sb = sa + kPairM * kPairK * 2;
+                const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sb);
+                const int rb = j >= nrb ? j - nrb : j;
+                const int nk16 = (min(kPairK, rk - rb * kPairK) + 15) / 16;   // beyond the rank: no MMA
+                if (leader) {
+                  for (int k = 0; k < nk16; ++k)
+                    tc_mma_bf16_pair(tmem_g, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc_tail, 1u);
+                  tc_commit_pair(empty0 + 8 * s);
+                }
+              }
+            }
           }
         }
         if (ok && leader) tc_commit_pair(tfull0 + 8 * acc);
@@ -258,7 +291,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       for (int j = 1; j < kPairJobs; ++j)
         if (t.job == j) { n = p.N[j]; y = p.y[j]; y0 = p.y0[j]; }
       const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
-      if (EPI != PAIR_STORE) {   // 1/|c_k| of this warp's columns; NaN where there is no candidate: it loses every maximum
+      if (EPI == PAIR_ROUTER || EPI == PAIR_ROUTER2) {   // 1/|c_k| of this warp's columns; NaN where there is no candidate: it loses every maximum
         const int k0 = t.n0 + wh * (p.bn / 2) + 4 * lane;
         float4 v;
         float* e = reinterpret_cast<float*>(&v);
@@ -277,16 +310,16 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * kPairMaxN;
       float best = -INFINITY, second = -INFINITY;
       int best_k = 0, second_k = 0;
-      if (EPI == PAIR_STORE) {
+      if (EPI == PAIR_STORE || EPI == PAIR_SWIGLU) {
         // Full 32-row groups leave through shared memory (128-byte swizzled rows) as tiled stores of whole lines: a
         // warp's 16-byte pieces straight from registers are 32 partial-line requests per instruction, beside the
         // operand loads in L2.  Partial row groups of a plan tile and the rest of a tile
         // whose width is no multiple of 64 are written row by row (a tiled store cannot be clipped).
-        const int col_end = min(n, t.n0 + p.bn);
+        const int col_end = min(n, t.n0 + p.cols);
 #pragma unroll 1
-        for (int c = 64 * wh; c < p.bn; c += 128) {
+        for (int c = 64 * wh; c < p.cols; c += 128) {
           if (t.n0 + c >= n || q * 32 >= rows) break;
-          const bool staged = q * 32 + 32 <= rows && c + 64 <= p.bn && y0 == nullptr;
+          const bool staged = q * 32 + 32 <= rows && c + 64 <= p.cols && y0 == nullptr;
           if (staged && n_st >= 1) {               // the store that last read this buffer
             if (lane == 0) bulk_wait_read<0>();
             __syncwarp();
@@ -295,7 +328,21 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
           for (int hh = 0; hh < 2; ++hh) {
             uint32_t v[32];
             tmem_ld32(taddr + c + 32 * hh, v);
-            tmem_ld_wait();
+            if (EPI == PAIR_SWIGLU) {   // silu(gate) * up, both rounded to bf16 first as the separate projections are
+              uint32_t u[32];
+              tmem_ld32(taddr + p.cols + c + 32 * hh, u);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) {
+                const uint32_t gw = pack_bf16(__uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+                const uint32_t uw = pack_bf16(__uint_as_float(u[j]), __uint_as_float(u[j + 1]));
+                const float g0 = bf16_lo(gw), g1 = bf16_hi(gw);
+                v[j] = __float_as_uint(__fdividef(g0, 1.f + __expf(-g0)) * bf16_lo(uw));
+                v[j + 1] = __float_as_uint(__fdividef(g1, 1.f + __expf(-g1)) * bf16_hi(uw));
+              }
+            } else {
+              tmem_ld_wait();
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               uint4 o;
@@ -384,7 +431,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
         }
         best_k += t.n0 + wh * (p.bn / 2);
       }
-      if (EPI == PAIR_STORE) {
+      if (EPI == PAIR_STORE || EPI == PAIR_SWIGLU) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(map_rank(tempty0 + 8 * acc, 0));
@@ -408,7 +455,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
         }
       }
     }
-    if (EPI == PAIR_STORE && lane == 0) bulk_wait_all();   // this thread's tiled stores are complete
+    if ((EPI == PAIR_STORE || EPI == PAIR_SWIGLU) && lane == 0) bulk_wait_all();   // this thread's tiled stores are complete
   }
   // ------------------------------------------------------------------ teardown
   if (*abort_flag) {
@@ -467,7 +514,7 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
   const int bn = pick_pair_bn(tiles_m, N, n_jobs, hs->n_sms, 16);
   PairMaps maps;
   PairParams p = {};
-  p.M = M; p.K = K; p.n_jobs = n_jobs; p.bn = bn; p.status = hs->status;
+  p.M = M; p.K = K; p.n_jobs = n_jobs; p.bn = p.cols = bn; p.status = hs->status;
   if (pv) {
     p.header = pv->header; p.tile_row0 = pv->tile_row0; p.tile_rows = pv->tile_rows; p.tile_expert = pv->tile_expert;
     p.tail_r = jobs[0].pool->r;
@@ -495,13 +542,50 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
   return launch_pair<PAIR_STORE>(hs, maps, p, max_tiles, stream);
 }
 
+// The gate and up projections of a block with the product of the two: one launch, act[M][F] instead of two matrices.
+// The first CTA holds cols rows of the gate weight and the second the same rows of the up weight, so one MMA gives both
+// (accumulator columns 0 .. cols - 1 and cols .. 2 cols - 1); the low-rank blocks multiply the gate's and the up
+// projection's halves of the columns one after the other.  16384 x 2048 -> 2 x 5632: the two projections 510 us and the
+// product's own pass 94 us (553 MB), now 540 us together.
+moin_status launch_pair_swiglu(HostState* hs, const PlanView* pv, const PairJob* jobs, int M, int K, cudaStream_t stream) {
+  const int F = jobs[0].N, N2 = 2 * F;
+  const long tiles_m = (M + kPairM - 1) / kPairM;
+  const int bn = pick_pair_bn(tiles_m, &N2, 1, hs->n_sms, 64);   // (the halves start at multiples of 32 columns)
+  PairMaps maps;
+  PairParams p = {};
+  p.M = M; p.K = K; p.n_jobs = 1; p.bn = bn; p.cols = bn / 2; p.status = hs->status;
+  p.N[0] = p.N[1] = F;
+  p.tn_end[0] = (F + p.cols - 1) / p.cols;
+  p.y[0] = jobs[0].y;
+  moin_status st = make_map(&maps.x[0], jobs[0].x, M, K, kPairM);
+  if (!st) st = make_map(&maps.y[0], jobs[0].y, M, F, 32);
+  if (pv) {
+    p.header = pv->header; p.tile_row0 = pv->tile_row0; p.tile_rows = pv->tile_rows; p.tile_expert = pv->tile_expert;
+    p.tail_r = jobs[0].pool->r;
+  }
+  for (int j = 0; j < 2 && !st; ++j) {
+    const PairJob& g = jobs[j];
+    st = make_map(&maps.w[j], g.W, F, K, p.cols);
+    if (!st && pv) {
+      const int r = g.pool->r;
+      st = make_map(&maps.hi[j], g.hb, M, r, kPairM);
+      if (!st) st = make_map(&maps.lo[j], g.hb + (size_t)M * r, M, r, kPairM);
+      if (!st) st = make_map(&maps.b[j], g.pool->B, (uint64_t)g.pool->n_slots * F, r, p.cols / 2);
+      p.slot_of_expert[j] = g.pool->slot_of_expert;
+      p.slot_rank[j] = g.pool->slot_rank;
+    }
+  }
+  if (st) return st;
+  return launch_pair<PAIR_SWIGLU>(hs, maps, p, (pv ? (long)M : (tiles_m + 1) / 2) * p.tn_end[0], stream);
+}
+
 moin_status launch_pair_router(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm, int Q,
                                int K, int D, unsigned long long* keys, cudaStream_t stream, unsigned long long* keys2) {
   const long tiles_m = (Q + kPairM - 1) / kPairM;
   const int bn = pick_pair_bn(tiles_m, &K, 1, hs->n_sms, 64);
   PairMaps maps;
   PairParams p = {};
-  p.M = Q; p.K = D; p.n_jobs = 1; p.bn = bn; p.status = hs->status; p.inv_norm = inv_norm; p.keys = keys; p.keys2 = keys2;
+  p.M = Q; p.K = D; p.n_jobs = 1; p.bn = p.cols = bn; p.status = hs->status; p.inv_norm = inv_norm; p.keys = keys; p.keys2 = keys2;
   p.N[0] = K; p.tn_end[0] = (K + bn - 1) / bn;
   moin_status st = make_map(&maps.x[0], q, Q, D, kPairM);
   if (!st) st = make_map(&maps.w[0], c, K, D, bn / 2);
