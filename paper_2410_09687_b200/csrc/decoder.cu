@@ -102,7 +102,10 @@ embed_kernel(const int* __restrict__ tokens, const __nv_bfloat16* __restrict__ e
 
 // res[t] += add[t] (bf16, optional);  out[t] = bf16(res[t] / sqrt(mean(res[t]^2) + eps) * gain)  (optional)
 // rows (nullable): gather list - CTA b normalises row rows[b] into out row b (used for last-token logits).
-__global__ void __launch_bounds__(256)
+// Bound by the traffic of the row (res in and out, add, out).  A thread's pieces of rows up to 2048 wide stay in
+// registers, all loads issued before the first use; the rest of a wider row is read again for the second pass.
+constexpr int kNormKeep = 2;   // 16-byte pieces a thread keeps (more of them would cost rows in flight on an SM)
+__global__ void __launch_bounds__(256, 6)
 add_rmsnorm_kernel(float* __restrict__ res, const __nv_bfloat16* __restrict__ add,
                    const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ out, int hidden, float eps,
                    const int* __restrict__ rows) {
@@ -112,15 +115,39 @@ add_rmsnorm_kernel(float* __restrict__ res, const __nv_bfloat16* __restrict__ ad
   const int t = rows ? rows[b] : b;
   if (t < 0) return;
   float* rrow = res + (size_t)t * hidden;
-  float ss = 0.f;
-  for (int i = threadIdx.x * 4; i < hidden; i += blockDim.x * 4) {
-    float4 v = *reinterpret_cast<const float4*>(rrow + i);
-    if (add) {
-      const uint2 a = *reinterpret_cast<const uint2*>(add + (size_t)t * hidden + i);
-      v.x += bf16_lo(a.x); v.y += bf16_hi(a.x); v.z += bf16_lo(a.y); v.w += bf16_hi(a.y);
-      *reinterpret_cast<float4*>(rrow + i) = v;
+  const __nv_bfloat16* arow = add ? add + (size_t)t * hidden : nullptr;
+  const int i0 = threadIdx.x * 4, step = 256 * 4;
+  float4 v[kNormKeep];
+  uint2 a[kNormKeep], gv[kNormKeep];
+#pragma unroll
+  for (int k = 0; k < kNormKeep; ++k) {
+    const int i = i0 + k * step;
+    v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    a[k] = gv[k] = make_uint2(0u, 0u);
+    if (i < hidden) {
+      v[k] = *reinterpret_cast<const float4*>(rrow + i);
+      if (arow) a[k] = *reinterpret_cast<const uint2*>(arow + i);
+      if (out) gv[k] = __ldg(reinterpret_cast<const uint2*>(gain + i));
     }
-    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int k = 0; k < kNormKeep; ++k) {
+    const int i = i0 + k * step;
+    if (arow && i < hidden) {
+      v[k].x += bf16_lo(a[k].x); v[k].y += bf16_hi(a[k].x); v[k].z += bf16_lo(a[k].y); v[k].w += bf16_hi(a[k].y);
+      *reinterpret_cast<float4*>(rrow + i) = v[k];
+    }
+    ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
+  }
+  for (int i = i0 + kNormKeep * step; i < hidden; i += step) {
+    float4 w = *reinterpret_cast<const float4*>(rrow + i);
+    if (arow) {
+      const uint2 aw = *reinterpret_cast<const uint2*>(arow + i);
+      w.x += bf16_lo(aw.x); w.y += bf16_hi(aw.x); w.z += bf16_lo(aw.y); w.w += bf16_hi(aw.y);
+      *reinterpret_cast<float4*>(rrow + i) = w;
+    }
+    ss += w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
   }
   if (!out) return;
   ss = warp_sum(ss);
@@ -130,14 +157,18 @@ add_rmsnorm_kernel(float* __restrict__ res, const __nv_bfloat16* __restrict__ ad
 #pragma unroll
   for (int w = 0; w < 8; ++w) tot += s_part[w];
   const float inv = rsqrtf(tot / (float)hidden + eps);
-  for (int i = threadIdx.x * 4; i < hidden; i += blockDim.x * 4) {
-    const float4 v = *reinterpret_cast<const float4*>(rrow + i);
-    const uint2 gv = *reinterpret_cast<const uint2*>(gain + i);
+  auto norm = [&](const float4& w, const uint2& g) {
     uint2 o;
-    o.x = pack_bf16(v.x * inv * bf16_lo(gv.x), v.y * inv * bf16_hi(gv.x));
-    o.y = pack_bf16(v.z * inv * bf16_lo(gv.y), v.w * inv * bf16_hi(gv.y));
-    *reinterpret_cast<uint2*>(out + (size_t)b * hidden + i) = o;
-  }
+    o.x = pack_bf16(w.x * inv * bf16_lo(g.x), w.y * inv * bf16_hi(g.x));
+    o.y = pack_bf16(w.z * inv * bf16_lo(g.y), w.w * inv * bf16_hi(g.y));
+    return o;
+  };
+  __nv_bfloat16* orow = out + (size_t)b * hidden;
+#pragma unroll
+  for (int k = 0; k < kNormKeep; ++k)
+    if (i0 + k * step < hidden) *reinterpret_cast<uint2*>(orow + i0 + k * step) = norm(v[k], gv[k]);
+  for (int i = i0 + kNormKeep * step; i < hidden; i += step)
+    *reinterpret_cast<uint2*>(orow + i) = norm(*reinterpret_cast<const float4*>(rrow + i), *reinterpret_cast<const uint2*>(gain + i));
 }
 
 // In-place rotary embedding on v[T][n_h * 64], pairing (i, i + 32).
