@@ -254,7 +254,8 @@ moin_status moin_cache_slot_of(const moin_cache* cache, int32_t expert, int32_t*
  *   - a stable permutation of token indices ordered by expert id, with one segment
  *     (expert, start, length) per distinct expert - used when segments are short (decode);
  *   - the list of row tiles: maximal runs of consecutive tokens with one expert, cut into
- *     pieces of at most 128 rows - used when runs are long (prefill).  A build with mode
+ *     pieces of at most 128 rows - used when runs are long (prefill), beside a second list that cuts
+ *     the tokens every 128 rows and says which runs lie in each piece.  A build with mode
  *     MOIN_PLAN_SEGMENTS leaves this list empty (nothing in that mode reads it): such a plan
  *     must be rebuilt, not relabelled, before it is used as MOIN_PLAN_TILES.
  * Token expert ids: -1 = no expert (base model only); ids outside [-1, E) are treated as -1

@@ -22,10 +22,11 @@ struct DeviceStatus {
 
 // Plan buffer layout (int32 words).  Header first, then the arrays.
 constexpr int kPlanHeaderWords = 16;
-enum PlanHeader { PH_NSEG = 0, PH_NTILES = 1, PH_NLORA = 2, PH_MAXSEG = 3, PH_T = 4, PH_E = 5, PH_NCHUNK = 6 };
+enum PlanHeader { PH_NSEG = 0, PH_NTILES = 1, PH_NLORA = 2, PH_MAXSEG = 3, PH_T = 4, PH_E = 5, PH_NCHUNK = 6, PH_NGEMM = 7 };
 constexpr int kSegChunk = 8;      // token columns of one warp MMA: what a work item of the stream kernels covers
 constexpr int kPlanChunk = 256;   // tokens per histogram chunk
-constexpr int kTileRows = 128;    // rows per GEMM tile
+constexpr int kTileRows = 128;    // rows per tile
+constexpr int kTileRuns = 4;      // runs a row tile of the long-run GEMM covers at most
 
 struct PlanView {   // pointers into the plan buffer
   int* header;
@@ -37,6 +38,14 @@ struct PlanView {   // pointers into the plan buffer
   int* tile_row0;    // [T + 1]
   int* tile_rows;    // [T]
   int* tile_expert;  // [T]
+  // Row tiles of the long-run GEMM: the regular grid of kTileRows rows, whatever runs of one expert it cuts (a grid tile
+  // of more than kTileRuns runs is cut at run boundaries): (first row, rows, first run, runs).
+  int4* gemm_tab;    // [T]
+  int* run_expert;   // [T]   runs in token order: expert or -1
+  int* run_row0;     // [T + 1] their first rows
+  int* grid_run;     // [grid tiles] run of the grid tile's first row
+  int* grid_nrun;    // [grid tiles] runs in it
+  int* tile_run;     // [T]   run of row tile i
   int* rank;         // [T]   scratch
   int* key;          // [T]   scratch
   int* keybase;      // [E+1] scratch
@@ -65,6 +74,12 @@ inline PlanView plan_view(void* buffer, int T, int E, size_t* total_words = null
   v.tile_row0 = take(T + 1);
   v.tile_rows = take(T + 1);
   v.tile_expert = take(T + 1);
+  v.gemm_tab = reinterpret_cast<int4*>(take(4 * (size_t)(T + 1)));
+  v.run_expert = take(T + 1);
+  v.run_row0 = take(T + 2);
+  v.grid_run = take(T / kTileRows + 2);
+  v.grid_nrun = take(T / kTileRows + 2);
+  v.tile_run = take(T + 1);
   v.rank = take(T);
   v.key = take(T);
   v.keybase = take(E + 2);

@@ -137,6 +137,36 @@ __global__ void __launch_bounds__(kPrefixIds * kPrefixGroups) plan_prefix_kernel
   if (on && g == kPrefixGroups - 1) v.keybase[k] = run;
 }
 
+// Row tiles of the long-run GEMM (see PlanView) from the runs that plan_tiles has numbered: a thread per grid tile.
+template <int NT>
+__device__ __forceinline__ void plan_gemm_tiles(const PlanView& v, int* smem, int n_runs) {
+  const int tid = threadIdx.x, T = v.T;
+  const int G = (T + kTileRows - 1) / kTileRows, per = (G + NT - 1) / NT;
+  const int g_lo = min(G, tid * per), g_hi = min(G, g_lo + per);
+  int count = 0;
+  for (int g = g_lo; g < g_hi; ++g) {
+    int last = n_runs - 1;
+    if (g + 1 < G) {
+      last = v.grid_run[g + 1];
+      if (v.run_row0[last] == (g + 1) * kTileRows) --last;   // that run begins with the next tile
+    }
+    const int nr = last - v.grid_run[g] + 1;
+    v.grid_nrun[g] = nr;
+    count += (nr + kTileRuns - 1) / kTileRuns;
+  }
+  int total;
+  int idx = block_excl_sum<NT>(count, smem, &total);
+  for (int g = g_lo; g < g_hi; ++g) {
+    const int f = v.grid_run[g], nr = v.grid_nrun[g];
+    for (int r = 0; r < nr; r += kTileRuns) {
+      const int row0 = r == 0 ? g * kTileRows : v.run_row0[f + r];
+      const int end = r + kTileRuns < nr ? v.run_row0[f + r + kTileRuns] : min(T, (g + 1) * kTileRows);
+      v.gemm_tab[idx++] = make_int4(row0, end - row0, f + r, min(kTileRuns, nr - r));
+    }
+  }
+  if (tid == 0) v.header[PH_NGEMM] = total;
+}
+
 // Row tiles: maximal runs of equal expert id in token order, cut every kTileRows rows.  One CTA of NT
 // threads; `key[t]` is the sanitised id of token t (shared or global memory).  smem: 33 ints.
 // `row0` is where the tile starts are read back from to form the tile lengths: v.tile_row0 itself, or a
@@ -174,8 +204,8 @@ __device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, in
   const int incl = block_incl_max<NT>(last, smem);
   int run = __shfl_up_sync(0xffffffffu, incl, 1);   // exclusive: the lane before, or the last lane of the warp before
   if ((tid & 31) == 0) run = tid > 0 ? smem[(tid >> 5) - 1] : -1;
-  // 2. tiles that start inside the range
-  int count = 0, rs = run;
+  // 2. tiles and runs that start inside the range
+  int count = 0, n_run = 0, rs = run;
   prev = before;
   for (int t = lo; t < hi; t += 4) {
     int k[4];
@@ -183,14 +213,18 @@ __device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, in
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (t + i < hi) {
-        if (k[i] != prev) rs = t + i;
+        if (k[i] != prev) {
+          rs = t + i;
+          ++n_run;
+        }
         prev = k[i];
         count += ((t + i - rs) % kTileRows) == 0;
       }
   }
-  int total;
+  int total, n_runs;
   int idx = block_excl_sum<NT>(count, smem, &total);
-  // 3. the list
+  int ord = block_excl_sum<NT>(n_run, smem, &n_runs);
+  // 3. the lists
   rs = run;
   prev = before;
   for (int t = lo; t < hi; t += 4) {
@@ -199,9 +233,16 @@ __device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, in
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (t + i < hi) {
-        if (k[i] != prev) rs = t + i;
+        if (k[i] != prev) {
+          rs = t + i;
+          v.run_expert[ord] = (k[i] == E) ? -1 : k[i];
+          v.run_row0[ord] = rs;
+          ++ord;
+        }
         prev = k[i];
+        if ((t + i) % kTileRows == 0) v.grid_run[(t + i) / kTileRows] = ord - 1;
         if (((t + i - rs) % kTileRows) == 0) {
+          v.tile_run[idx] = ord - 1;
           v.tile_row0[idx] = t + i;
           if (row0 != v.tile_row0) row0[idx] = t + i;
           v.tile_expert[idx] = (k[i] == E) ? -1 : k[i];
@@ -211,11 +252,13 @@ __device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, in
   }
   if (tid == 0) {
     v.tile_row0[total] = T;
+    v.run_row0[n_runs] = T;
     if (row0 != v.tile_row0) row0[total] = T;
     v.header[PH_NTILES] = total;
   }
   __syncthreads();
   for (int i = tid; i < total; i += NT) v.tile_rows[i] = row0[i + 1] - row0[i];
+  plan_gemm_tiles<NT>(v, smem, n_runs);
 }
 
 __global__ void __launch_bounds__(1024) plan_scan_kernel(PlanView v, int do_prefix, int want_tiles) {
@@ -280,8 +323,11 @@ __global__ void __launch_bounds__(1024) plan_scan_kernel(PlanView v, int do_pref
   }
 
   // 3. row tiles (only the long-run kernels read them)
-  if (want_tiles) plan_tiles<NT>(v, v.key, smem, v.tile_row0);
-  else if (tid == 0) v.header[PH_NTILES] = 0;
+  if (want_tiles) {
+    plan_tiles<NT>(v, v.key, smem, v.tile_row0);
+  } else if (tid == 0) {
+    v.header[PH_NTILES] = v.header[PH_NGEMM] = 0;
+  }
 }
 
 // Whole plan of a batch of at most 1024 tokens in one CTA.  The tokens are sorted by the key
@@ -363,8 +409,11 @@ __global__ void __launch_bounds__(NT) plan_small_kernel(const int* __restrict__ 
     v.header[PH_T] = T;
     v.header[PH_E] = E;
   }
-  if (want_tiles) plan_tiles<NT>(v, s_key, smem, s_row0);
-  else if (tid == 0) v.header[PH_NTILES] = 0;
+  if (want_tiles) {
+    plan_tiles<NT>(v, s_key, smem, s_row0);
+  } else if (tid == 0) {
+    v.header[PH_NTILES] = v.header[PH_NGEMM] = 0;
+  }
 }
 
 __global__ void __launch_bounds__(kPlanChunk) plan_scatter_kernel(PlanView v) {

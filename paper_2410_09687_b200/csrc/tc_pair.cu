@@ -10,11 +10,13 @@
 // own 128 rows.  A commit arrives on both CTAs' barriers (stage free, accumulator ready); both epilogues release an
 // accumulator on the first CTA's barrier.  Two accumulators in TMEM: the epilogue of tile i overlaps the MMAs of i + 1.
 //
-// Row tiles come from a regular grid or from a batch plan (runs of one expert, at most 128 rows); the pair takes plan
-// tiles 2i and 2i + 1.  With a plan every tile ends with extra K blocks [hi(s h) | lo(s h)] x [B_e ; B_e] that add the
-// low-rank term inside the accumulator.  Both halves of a pair multiply the same B rows, so where the two row tiles
-// have different experts the blocks run once per expert, the other CTA's rows being zero (a copy that starts past the
-// last row fills zeros).
+// Row tiles are the regular grid of 128 rows, also with a batch plan: a tile may hold up to kTileRuns runs of one expert
+// (the plan cuts a grid tile of more).  With adapters every tile ends with extra K blocks [hi(s h) | lo(s h)] x
+// [B_e ; B_e], one pass per run, that add the low-rank term inside the accumulator; the rows of the other runs are zero in
+// a pass (the shrink writes h under the number of a row's run in its tile and zeros under the others), and so are those of
+// a CTA that has no row of the run (a copy that starts past the last row fills zeros).  Tiles that began anew with each
+// run instead multiplied up to a fifth of padding: 11 prompts of 65 to 600 tokens, forward 10.34 -> 8.98 ms; nine, a
+// block's projections 464 -> 400 us.
 //
 // A launch covers up to kPairJobs projections that share the plan and the reduction length (the column tiles of all of
 // them side by side under one row tile, so an x they share comes from L2): one ramp and one partial last wave per group.
@@ -29,11 +31,12 @@ namespace moin {
 constexpr int kPairThreads = 320, kPairM = 128, kPairK = 64;
 enum { PAIR_STORE = 0, PAIR_ROUTER = 1, PAIR_ROUTER2 = 2, PAIR_SWIGLU = 3 };
 
-struct PairMaps { CUtensorMap x[kPairJobs], w[kPairJobs], b[kPairJobs], hi[kPairJobs], lo[kPairJobs], y[kPairJobs]; };
+struct PairMaps { CUtensorMap x[kPairJobs], w[kPairJobs], b[kPairJobs], h[kPairJobs], y[kPairJobs]; };
 struct PairParams {
   int M, K, n_jobs, bn, cols;            // bn: tile width, a multiple of 16 up to 256; cols: output columns of it
   int N[kPairJobs], tn_end[kPairJobs];   // columns, column tiles of jobs 0 .. j
-  const int *header, *tile_row0, *tile_rows, *tile_expert;   // plan (header == nullptr: regular grid over M)
+  const int *header, *run_expert;        // plan (header == nullptr: regular grid over M, no runs)
+  const int4* gemm_tab;
   int tail_r;                            // stored rank of the appended low-rank blocks (0 = none)
   const int* slot_of_expert[kPairJobs];
   const int* slot_rank[kPairJobs];       // nullable: the stored rank
@@ -53,8 +56,8 @@ __device__ __forceinline__ uint32_t pair_orderable(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// What a tile is: its job, first column, and for both CTAs of the pair the row tile and its expert.
-struct PairTile { int job, n0, row0[2], rows[2], expert[2]; };
+// What a tile is: its job, first column, and for both CTAs of the pair the rows and the runs in them.
+struct PairTile { int job, n0, row0[2], rows[2], run0[2], n_run[2]; };
 
 __device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int tiles_m) {
   PairTile t;
@@ -73,51 +76,40 @@ __device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const int tm = 2 * pm + c;
-    t.expert[c] = -1;
-    t.row0[c] = p.M;      // no such row tile: the copy fills zeros, nothing is stored
-    t.rows[c] = 0;
+    int4 g = make_int4(p.M, 0, 0, 0);   // no such row tile: the copy fills zeros, nothing is stored
     if (tm < tiles_m) {
-      if (p.header != nullptr) {
-        t.row0[c] = __ldg(p.tile_row0 + tm);
-        t.rows[c] = __ldg(p.tile_rows + tm);
-        t.expert[c] = __ldg(p.tile_expert + tm);
-      } else {
-        t.row0[c] = tm * kPairM;
-        t.rows[c] = min(kPairM, p.M - t.row0[c]);
-      }
+      if (p.header != nullptr) g = __ldg(p.gemm_tab + tm);
+      else g = make_int4(tm * kPairM, min(kPairM, p.M - tm * kPairM), 0, 0);
     }
+    t.row0[c] = g.x; t.rows[c] = g.y; t.run0[c] = g.z; t.n_run[c] = g.w;
   }
   return t;
 }
-// Low-rank passes of a tile for a projection: pass 0 multiplies the adapter of the first CTA's rows (and of the second's
-// where it is the same one), pass 1 the second's where it differs.  live: bit c = CTA c's rows take part.
-struct PairPasses { int n, slot[2], rank[2]; uint32_t live[2]; };
-__device__ __forceinline__ PairPasses pair_passes(const PairParams& p, const PairTile& t, int job) {
-  const int* slots = p.slot_of_expert[0];
-  const int* ranks = p.slot_rank[0];
+// Low-rank passes of a tile: one per run of the first CTA's rows, then the second's; the run in which both meet takes one
+// pass for both.  Finding a pass's adapter is a chain of three loads: an epilogue warp does it a tile ahead, lane i for
+// pass i (SWIGLU: lanes 8 .. 15 for the up projection), and leaves the result in shared memory.  (In the producer and the
+// MMA warp themselves, at the start of a tile or in steps between the quarters of its main loop, it cost 2 to 5 percent.)
+constexpr int kPairPasses = 2 * kTileRuns;
+struct PairPass { int slot, rank, run[2]; };   // adapter or -1; per CTA the number under which hb has the run's rows or -1
+constexpr uint32_t kPairTabBytes = 2 * kPairPasses * sizeof(PairPass) + 16;   // passes, then their number
+__device__ __forceinline__ void pair_passes(const PairParams& p, const PairTile& t, bool two_jobs, int lane, uint8_t* tab) {
+  const int shared = t.n_run[0] > 0 && t.n_run[1] > 0 && t.run0[0] + t.n_run[0] - 1 == t.run0[1];
+  const int n = t.n_run[0] + t.n_run[1] - shared;
+  const int i = lane % kPairPasses, job = two_jobs ? lane / kPairPasses : t.job;
+  if (lane < (two_jobs ? 2 : 1) * kPairPasses && i < n) {
+    const int k1 = i - t.n_run[0] + shared;   // run of the second CTA's rows
+    PairPass q = {-1, p.tail_r, {i < t.n_run[0] ? i : -1, k1 >= 0 ? k1 : -1}};
+    const int* slots = p.slot_of_expert[0];
+    const int* ranks = p.slot_rank[0];
 #pragma unroll
-  for (int j = 1; j < kPairJobs; ++j)
-    if (job == j) { slots = p.slot_of_expert[j]; ranks = p.slot_rank[j]; }
-  int slot[2], rank[2];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    slot[c] = t.expert[c] >= 0 && p.tail_r > 0 ? __ldg(slots + t.expert[c]) : -1;
-    rank[c] = slot[c] < 0 ? 0 : ranks ? min(__ldg(ranks + slot[c]), p.tail_r) : p.tail_r;
+    for (int j = 1; j < kPairJobs; ++j)
+      if (job == j) { slots = p.slot_of_expert[j]; ranks = p.slot_rank[j]; }
+    const int e = __ldg(p.run_expert + (i < t.n_run[0] ? t.run0[0] + i : t.run0[1] + k1));
+    if (e >= 0) q.slot = __ldg(slots + e);
+    if (q.slot >= 0 && ranks) q.rank = min(__ldg(ranks + q.slot), p.tail_r);
+    reinterpret_cast<PairPass*>(tab)[lane] = q;
   }
-  PairPasses q;
-  q.n = 0;
-  q.slot[0] = q.slot[1] = -1; q.rank[0] = q.rank[1] = 0; q.live[0] = q.live[1] = 0u;
-  if (slot[0] >= 0) {
-    q.slot[0] = slot[0]; q.rank[0] = rank[0];
-    q.live[0] = (slot[1] == slot[0]) ? 3u : 1u;
-    q.n = 1;
-  }
-  if (slot[1] >= 0 && slot[1] != slot[0]) {
-    if (q.n == 0) { q.slot[0] = slot[1]; q.rank[0] = rank[1]; q.live[0] = 2u; }
-    else { q.slot[1] = slot[1]; q.rank[1] = rank[1]; q.live[1] = 2u; }
-    ++q.n;
-  }
-  return q;
+  if (lane == 0) *reinterpret_cast<int*>(tab + 2 * kPairPasses * sizeof(PairPass)) = n;
 }
 
 template <int EPI>
@@ -133,6 +125,10 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
   const uint32_t full0 = bars, empty0 = bars + 8 * S, tfull0 = bars + 16 * S, tempty0 = tfull0 + 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + 16 * S + 32);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 16 * S + 40);
+  constexpr bool kTail = EPI == PAIR_STORE || EPI == PAIR_SWIGLU;   // low-rank blocks at the end of a tile
+  const uint32_t tab0 = bars + 16 * S + 48;   // pass tables of this and the next tile, and their barriers
+  uint8_t* tab_ptr = bar_ptr + 256;
+  static_assert(256 + 2 * kPairTabBytes <= 1024, "barrier block");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
 
@@ -144,6 +140,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull0 + 8 * a, 1);    // each CTA's own, by commit
       mbar_init(tempty0 + 8 * a, 16);  // used in the first CTA: one arrival per epilogue warp of the pair
+      mbar_init(tab0 + 8 * a, 1);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -160,7 +157,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();   // (the set-up above overlaps the tail of the kernel before)
 
-  const int tiles_m = p.header != nullptr ? p.header[PH_NTILES] : (p.M + kPairM - 1) / kPairM;
+  const int tiles_m = p.header != nullptr ? p.header[PH_NGEMM] : (p.M + kPairM - 1) / kPairM;
   const int total = (tiles_m + 1) / 2 * p.tn_end[p.n_jobs - 1];
   const int nkb_main = (p.K + kPairK - 1) / kPairK;
   const int nrb = (p.tail_r + kPairK - 1) / kPairK;   // 64-wide blocks of the rank
@@ -172,9 +169,9 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       // both CTAs' copies of a stage: the operands, the low-rank blocks (SWIGLU: of half the columns at a time)
       const uint32_t tx = (uint32_t)(2 * kPairM + p.bn) * kPairK * 2;
       const uint32_t tx_tail = EPI == PAIR_SWIGLU ? (uint32_t)(2 * kPairM + p.bn / 2) * kPairK * 2 : tx;
-      uint32_t it = 0;
+      uint32_t it = 0, lt = 0;
       bool ok = true;
-      for (int tile = pair; tile < total && ok; tile += n_pairs) {
+      for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
         const PairTile t = pair_tile(p, tile, tiles_m);
         const int row0 = rank == 0 ? t.row0[0] : t.row0[1];
         const CUtensorMap* mx = &maps.x[t.job];
@@ -189,25 +186,30 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
           tma_load_2d_pair(sa, mx, bar, kb * kPairK, row0);
           tma_load_2d_pair(sb, mw, bar, kb * kPairK, w0);
         }
-        if (p.tail_r == 0) continue;
-        for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g) {
+        if (!kTail || p.tail_r == 0 || !ok) continue;
+        if (!(ok = mbar_wait(tab0 + 8 * (lt & 1u), (lt >> 1) & 1u, abort_flag, p.status, 65))) break;
+        const volatile PairPass* pass = reinterpret_cast<const volatile PairPass*>(tab_ptr + (lt & 1u) * kPairTabBytes);
+        const int n_pass = *reinterpret_cast<const volatile int*>(pass + 2 * kPairPasses);
+        for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g, pass += kPairPasses) {
           const int job = EPI == PAIR_SWIGLU ? g : t.job;
-          const PairPasses pq = pair_passes(p, t, job);
           int n = p.N[0];
 #pragma unroll
           for (int jj = 1; jj < kPairJobs; ++jj)
             if (job == jj) n = p.N[jj];
-          for (int pass = 0; pass < pq.n && ok; ++pass) {
-            const bool mine = ((pass ? pq.live[1] : pq.live[0]) >> rank) & 1u;
-            const int b0 = (pass ? pq.slot[1] : pq.slot[0]) * n + t.n0 + (int)rank * (p.cols / 2);
+          for (int i = 0; i < n_pass && ok; ++i) {
+            const int slot = pass[i].slot, run = pass[i].run[rank];
+            if (slot < 0) continue;
+            const int b0 = slot * n + t.n0 + (int)rank * (p.cols / 2);
             for (int j = 0; j < 2 * nrb; ++j, ++it) {
               const uint32_t s = it % S, ph = (it / S) & 1u;
               if (!(ok = mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 61))) break;
               const uint32_t sa = ring + s * kPairStageBytes, sb = sa + kPairM * kPairK * 2;
               const uint32_t bar = map_rank(full0 + 8 * s, 0);
               if (rank == 0) mbar_expect_tx(full0 + 8 * s, tx_tail);
-              const int rb = j >= nrb ? j - nrb : j;            // hi blocks first, then lo blocks
-              tma_load_2d_pair(sa, j < nrb ? &maps.hi[job] : &maps.lo[job], bar, rb * kPairK, mine ? row0 : p.M);
+              const int lo = j >= nrb ? 1 : 0, rb = j - lo * nrb;   // hi blocks first, then lo blocks
+              // rows of the run under its number; a CTA without rows of it starts past the last row: zeros
+              const int h0 = run >= 0 ? (2 * run + lo) * p.M + row0 : 2 * kTileRuns * p.M;
+              tma_load_2d_pair(sa, &maps.h[job], bar, rb * kPairK, h0);
               tma_load_2d_pair(sb, &maps.b[job], bar, rb * kPairK, b0);
             }
           }
@@ -246,13 +248,15 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
             tc_commit_pair(empty0 + 8 * s);
           }
         }
-        if (p.tail_r > 0) {
-          const PairTile t = pair_tile(p, tile, tiles_m);
-          for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g) {
-            const PairPasses pq = pair_passes(p, t, EPI == PAIR_SWIGLU ? g : t.job);
+        if (kTail && p.tail_r > 0 && ok) {
+          if (!(ok = mbar_wait_warp(tab0 + 8 * (lt & 1u), (lt >> 1) & 1u, abort_flag, p.status, 66))) break;
+          const volatile PairPass* pass = reinterpret_cast<const volatile PairPass*>(tab_ptr + (lt & 1u) * kPairTabBytes);
+          const int n_pass = *reinterpret_cast<const volatile int*>(pass + 2 * kPairPasses);
+          for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g, pass += kPairPasses) {
             const uint32_t tmem_g = tmem_d + g * (p.bn / 2);
-            for (int pass = 0; pass < pq.n && ok; ++pass) {
-              const int rk = pass ? pq.rank[1] : pq.rank[0];
+            for (int i = 0; i < n_pass && ok; ++i) {
+              const int slot = pass[i].slot, rk = pass[i].rank;
+              if (slot < 0) continue;
               for (int j = 0; j < 2 * nrb; ++j, ++it) {
                 const uint32_t s = it % S, ph = (it / S) & 1u;
                 if (!(ok = mbar_wait_cluster_warp(full0 + 8 * s, ph, abort_flag, p.status, 63))) break;
@@ -281,8 +285,17 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
     const uint32_t buf = out0 + (uint32_t)(wh * 4 + q) * 4096u;
     uint32_t lt = 0, n_st = 0;
     bool ok = true;
+    // Passes of tile i into table i & 1.  Written when the epilogue of tile i - 2 is over at the earliest: its
+    // accumulator was complete, so nobody reads that tile's table any more.
+    auto scout = [&](const PairTile& n, uint32_t i) {
+      pair_passes(p, n, EPI == PAIR_SWIGLU, lane, tab_ptr + (i & 1u) * kPairTabBytes);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tab0 + 8 * (i & 1u));
+    };
+    if (kTail && warp == 2 && p.tail_r > 0 && pair < total) scout(pair_tile(p, pair, tiles_m), 0);
     for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
       const PairTile t = pair_tile(p, tile, tiles_m);
+      if (kTail && warp == 2 && p.tail_r > 0 && tile + n_pairs < total) scout(pair_tile(p, tile + n_pairs, tiles_m), lt + 1);
       const int row0 = rank == 0 ? t.row0[0] : t.row0[1], rows = rank == 0 ? t.rows[0] : t.rows[1];
       int n = p.N[0];
       __nv_bfloat16* y = p.y[0];
@@ -516,7 +529,7 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
   PairParams p = {};
   p.M = M; p.K = K; p.n_jobs = n_jobs; p.bn = p.cols = bn; p.status = hs->status;
   if (pv) {
-    p.header = pv->header; p.tile_row0 = pv->tile_row0; p.tile_rows = pv->tile_rows; p.tile_expert = pv->tile_expert;
+    p.header = pv->header; p.gemm_tab = pv->gemm_tab; p.run_expert = pv->run_expert;
     p.tail_r = jobs[0].pool->r;
   }
   int tn = 0;
@@ -527,8 +540,7 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
     if (!st) st = make_map(&maps.y[j], g.y, M, g.N, 32);
     if (!st && pv) {
       const int r = g.pool->r;
-      st = make_map(&maps.hi[j], g.hb, M, r, kPairM);
-      if (!st) st = make_map(&maps.lo[j], g.hb + (size_t)M * r, M, r, kPairM);
+      st = make_map(&maps.h[j], g.hb, 2ull * kTileRuns * M, r, kPairM);
       if (!st) st = make_map(&maps.b[j], g.pool->B, (uint64_t)g.pool->n_slots * g.N, r, bn / 2);
       p.slot_of_expert[j] = g.pool->slot_of_expert;
       p.slot_rank[j] = g.pool->slot_rank;
@@ -560,7 +572,7 @@ moin_status launch_pair_swiglu(HostState* hs, const PlanView* pv, const PairJob*
   moin_status st = make_map(&maps.x[0], jobs[0].x, M, K, kPairM);
   if (!st) st = make_map(&maps.y[0], jobs[0].y, M, F, 32);
   if (pv) {
-    p.header = pv->header; p.tile_row0 = pv->tile_row0; p.tile_rows = pv->tile_rows; p.tile_expert = pv->tile_expert;
+    p.header = pv->header; p.gemm_tab = pv->gemm_tab; p.run_expert = pv->run_expert;
     p.tail_r = jobs[0].pool->r;
   }
   for (int j = 0; j < 2 && !st; ++j) {
@@ -568,8 +580,7 @@ moin_status launch_pair_swiglu(HostState* hs, const PlanView* pv, const PairJob*
     st = make_map(&maps.w[j], g.W, F, K, p.cols);
     if (!st && pv) {
       const int r = g.pool->r;
-      st = make_map(&maps.hi[j], g.hb, M, r, kPairM);
-      if (!st) st = make_map(&maps.lo[j], g.hb + (size_t)M * r, M, r, kPairM);
+      st = make_map(&maps.h[j], g.hb, 2ull * kTileRuns * M, r, kPairM);
       if (!st) st = make_map(&maps.b[j], g.pool->B, (uint64_t)g.pool->n_slots * F, r, p.cols / 2);
       p.slot_of_expert[j] = g.pool->slot_of_expert;
       p.slot_rank[j] = g.pool->slot_rank;
