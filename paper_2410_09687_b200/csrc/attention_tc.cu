@@ -3,23 +3,30 @@
 // One work item = (request, kv head, block of query positions).  The g = n_heads / n_kv_heads query heads
 // that share a kv head are stacked into one 128-row tile: row r holds position q0 + r / g of head kvh * g + r % g,
 // so a block covers 128 / g positions and every staged K / V tile serves all g heads.  Persistent CTAs (two per
-// SM) walk the items, longest first.  Warp roles:
-//   warp 0      TMA producer: K and V tiles [64 keys x 64 dims] into small rings.  K is a K-major operand of the
+// SM) walk the items, longest first.
+//
+// The time of an item is a chain of hand-overs (scores, softmax, product), not any unit's throughput, so a CTA keeps two
+// chains going: the even key tiles are one STREAM, the odd ones another, each with its own four softmax warps, scores,
+// running maximum, row sum and accumulator; the two meet once at the end of the item.  A stream takes a thread per row and
+// one pass over its keys: p = 2^(s - m) against a maximum m that may lag behind by a factor of up to 2^8 (p is bf16 and
+// its sum fp32: the relative accuracy is the same), so the accumulator is rescaled only when a row outgrows that.  P goes
+// back into tensor memory over the scores it came from, as the A operand of the second product: nothing of it passes
+// through shared memory.  Warp roles:
+//   warp 0      TMA producer: K and V tiles [64 keys x 64 dims] into rings of four.  K is a K-major operand of the
 //               form the GEMMs use; V, whose rows run along the output dimension of the second product, is read
 //               as an MN-major operand (same staged bytes, the other operand layout), so no transposed copy exists
-//   warp 1      MMA issuer: S = Q K^T into one of two TMEM buffers, O += P V into a third
-//   warps 2-9   two threads per tile row (32 of a tile's 64 columns each): rotate and stage Q (128-byte swizzled
-//               rows, written by hand), softmax, P as the bf16 A operand of the second product (swizzled rows
-//               again), normalise and store O
-// The softmax takes two passes over the keys: the first only finds each row's maximum, the second forms
-// p = 2^(s - max) once per element, sums it in fp32 and multiplies by V - so the O accumulator in TMEM never
-// needs rescaling.  An item that sees at most 256 keys (four tiles: every item of a request of up to 256 tokens)
-// keeps all of its scores in TMEM: S is computed once, both passes read it there, and O accumulates over the
-// columns of the first score tile once that tile has been turned into P - one hand-over MMA -> softmax per item
-// instead of two per tile.  Longer items stream: two score buffers, S recomputed in the second pass (the MMAs
-// are a small part of the time; the exponentials are not).  Key tiles start at the request's first token (only the innermost coordinate of a TMA
-// copy has an alignment rule, and that is the head's first dimension); the mask is key <= query position.
+//   warp 1      MMA issuer: polls both streams and issues whatever is ready, S_h = Q K^T or O_h += P_h V
+//   warps 2-5   stream 0, warps 6-9 stream 1; between two items they rotate and stage the next Q (128-byte swizzled rows,
+//               written by hand, two buffers: its first scores are computed while this item's O is merged and stored)
+// Tensor memory: S_h / P_h at columns 64 h, O_h at 128 + 64 h; two CTAs fill an SM's 512 columns.
+// Key tiles start at the request's first token (only the innermost coordinate of a TMA copy has an alignment rule, and
+// that is the head's first dimension); the mask is key <= query position.
 // Every mbarrier wait is bounded; on expiry the CTA raises the status flag, drains and returns.
+// A tile takes a stream about 3 us (at 16 such warps an SM a warp issues an instruction every eight cycles or so; the
+// exponentials alone would take a quarter of it), an item's end another 3: four chains an SM are what tensor memory holds.
+// Per block of 64 requests of 256 tokens 99 -> 80 us, of 11 requests of 65 to 600 tokens 42.5 -> 34.8 us, against one chain
+// per CTA (two threads a row, two passes over the keys: a tile's maximum first, scores computed twice beyond 256 keys).
+// One barrier arrival per warp instead of per thread: 82 / 35.5 us.
 #include <cuda.h>
 
 #include "ptx.cuh"
@@ -29,18 +36,18 @@ namespace moin {
 
 constexpr int kAtThreads = 320;                  // producer warp, MMA warp, 8 softmax warps
 constexpr int kAtKeys = 64;                      // keys per tile
-constexpr int kAtTile = 128 * 64 * 2;            // Q and P tiles: 128 rows x 128 bytes
+constexpr int kAtTile = 128 * 64 * 2;            // Q tile: 128 rows x 128 bytes
 constexpr int kAtKV = kAtKeys * 64 * 2;          // K and V tiles: 64 keys x 128 bytes
-constexpr int kAtKS = 4, kAtVS = 2;              // K: four stages (a resident item's whole key range, contiguous); V ring
+constexpr int kAtRing = 4;                       // stages of K and of V
 constexpr int kAtCuMax = 1024;                   // request offsets kept in shared memory when there are at most this many
 constexpr int kAtRopeBytes = 4096;               // (cos, sin) rows of an item's positions, when they fit (<= 16 positions)
-constexpr int kAtSmem = kAtTile /*Q*/ + 2 * kAtTile /*P*/ + kAtKS * kAtKV + kAtVS * kAtKV + 1024 /*align*/ +
-                        256 /*barriers*/ + 2048 /*row maxima and sums of the two half rows*/ + kAtCuMax * 4 + kAtRopeBytes;
-constexpr int kAtTmemCols = 256;                 // streaming items: S0 [0,64)  S1 [64,128)  O [128,192)
-constexpr int kAtResident = 4;                   // resident items: S_j [64 j, 64 j + 64), j < 4; O over S_0
+constexpr int kAtMerge = 4096;                   // (maximum, sum) of every row by stream, for two items
+constexpr int kAtSmem = 2 * kAtTile /*Q*/ + 2 * kAtRing * kAtKV + 1024 /*align*/ + 256 /*barriers*/ + kAtMerge +
+                        kAtCuMax * 4 + kAtRopeBytes;
+constexpr int kAtTmemCols = 256;
+constexpr float kAtLag = 8.f;                    // powers of two by which a running maximum may lag behind
 
 struct AttParams {
-  const __nv_bfloat16* q;      // [T, n_heads * 64], not rotated
   __nv_bfloat16* out;          // [T, n_heads * 64]
   const int* cu;               // [R + 1]
   const float2* rope;          // [max_seqlen, 32] (cos, sin)
@@ -63,10 +70,6 @@ __device__ __forceinline__ uint64_t at_sdesc(uint32_t saddr) {
 }
 // D fp32, A / B bf16 K-major, M = 128, N = 64
 constexpr uint32_t kAtIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-// the same with N = 64 n (n key tiles side by side in one product)
-__device__ __forceinline__ uint32_t at_idesc_n(int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((64 * n) >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-}
 // the same with B MN-major (V tile: one 128-byte row per key, the 64 output dims contiguous); a 16-key step of
 // such a tile is two 8-key groups = 2048 bytes further on
 constexpr uint32_t kAtIdescPV = kAtIdesc | (1u << 16);
@@ -128,20 +131,20 @@ __device__ __forceinline__ AttItem at_item(const AttParams& p, const int* cu, in
 }
 
 __global__ void __launch_bounds__(kAtThreads, 2)
-attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttParams p) {
+attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - raw);
-  const uint32_t sQ = base, sP = base + kAtTile, sK = sP + 2 * kAtTile, sV = sK + kAtKS * kAtKV;
-  const uint32_t bars = sV + kAtVS * kAtKV;
+  const uint32_t sQ = base, sK = base + 2 * kAtTile, sV = sK + kAtRing * kAtKV;
+  const uint32_t bars = sV + kAtRing * kAtKV;
   uint8_t* bar_ptr = base_ptr + (bars - base);
   // barriers (8 bytes each)
   const uint32_t kfull = bars, kempty = bars + 32, vfull = bars + 64, vempty = bars + 96, sready = bars + 128,
-                 sfree = bars + 144, pready = bars + 160, pfree = bars + 176, oready = bars + 192, ofree = bars + 200,
-                 qready = bars + 208, sall = bars + 232, rfull = bars + 240, rempty = bars + 248;
-  int* cu_s = reinterpret_cast<int*>(bar_ptr + 256 + 2048);
-  const uint32_t sRope = bars + 256 + 2048 + kAtCuMax * 4;
+                 pready = bars + 144, pvdone = bars + 160, oready = bars + 176, ofree = bars + 184, qready = bars + 192,
+                 rfull = bars + 200, rempty = bars + 208, qraw = bars + 240;
+  int* cu_s = reinterpret_cast<int*>(bar_ptr + 256 + kAtMerge);
+  const uint32_t sRope = bars + 256 + kAtMerge + kAtCuMax * 4;
   const int* cu = p.cu_smem ? cu_s : p.cu;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + 216);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 224);
@@ -149,20 +152,21 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kAtKS; ++i) { mbar_init(kfull + 8 * i, 1); mbar_init(kempty + 8 * i, 1); }
-    for (int i = 0; i < kAtVS; ++i) { mbar_init(vfull + 8 * i, 1); mbar_init(vempty + 8 * i, 1); }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(sready + 8 * i, 1); mbar_init(sfree + 8 * i, 256);
-      mbar_init(pready + 8 * i, 256); mbar_init(pfree + 8 * i, 1);
+    for (int i = 0; i < kAtRing; ++i) {
+      mbar_init(kfull + 8 * i, 1); mbar_init(kempty + 8 * i, 1);
+      mbar_init(vfull + 8 * i, 1); mbar_init(vempty + 8 * i, 1);
+    }
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(sready + 8 * h, 1); mbar_init(pready + 8 * h, 128); mbar_init(pvdone + 8 * h, 1);
     }
     mbar_init(oready, 1);
     mbar_init(ofree, 256);
     mbar_init(qready, 256);
-    mbar_init(sall, 1);
+    mbar_init(qraw, 1);
     mbar_init(rfull, 1);
     mbar_init(rempty, 256);
     *abort_flag = 0;
-    *sm_fail = 0;
+    sm_fail[0] = sm_fail[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -187,11 +191,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
-    // K stages and their barriers are addressed by stage, each with its own phase bit (keph: next "empty" phase to
-    // wait for), because the two kinds of item use them differently: a resident item puts its tiles into stages
-    // 0 .. n - 1 (one contiguous operand, one "full" barrier), a streaming item goes round the ring from kpos.
     if (lane == 0) {
-      uint32_t keph = 0, kpos = 0, vq = 0, rq = 0;
+      uint32_t tq = 0, rq = 0;   // tiles, rope blocks so far
       bool ok = true;
       int idx = (int)blockIdx.x - (int)gridDim.x;
       AttItem it;
@@ -210,39 +211,15 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         AttItem nx;
         int nidx = idx;
         const bool have_nx = next_item(nidx, nx);
-        auto k_free = [&](uint32_t s) -> bool {
-          const bool r = mbar_wait(kempty + 8 * s, ((keph >> s) & 1u) ^ 1u, abort_flag, p.status, 31);
-          keph ^= 1u << s;
-          return r;
-        };
-        auto load_k = [&](int j) -> bool {               // streaming: next stage of the ring
-          const uint32_t s = kpos;
-          if (!k_free(s)) return false;
+        if (have_nx) ok = load_rope(nx);   // wanted after this item's first tiles (the buffer: since the item before's)
+        for (int j = 0; j < it.n_tiles && ok; ++j, ++tq) {
+          const uint32_t s = tq % kAtRing, ph = (tq / kAtRing) & 1u;
+          if (!(ok = mbar_wait(kempty + 8 * s, ph ^ 1u, abort_flag, p.status, 31))) break;
           mbar_expect_tx(kfull + 8 * s, kAtKV);
           tma_load_2d(sK + s * kAtKV, &tmK, kfull + 8 * s, it.kvh * 64, it.a0 + j * kAtKeys);
-          kpos = (kpos + 1) % kAtKS;
-          return true;
-        };
-        auto load_v = [&](int j) -> bool {
-          const uint32_t s = vq % kAtVS, ph = (vq / kAtVS) & 1u;
-          if (!mbar_wait(vempty + 8 * s, ph ^ 1u, abort_flag, p.status, 32)) return false;
+          if (!(ok = mbar_wait(vempty + 8 * s, ph ^ 1u, abort_flag, p.status, 32))) break;
           mbar_expect_tx(vfull + 8 * s, kAtKV);
           tma_load_2d(sV + s * kAtKV, &tmV, vfull + 8 * s, it.kvh * 64, it.a0 + j * kAtKeys);
-          ++vq;
-          return true;
-        };
-        if (it.n_tiles <= kAtResident) {   // resident item: its K tiles side by side, completion on the first barrier
-          for (int j = 0; j < it.n_tiles && ok; ++j) ok = k_free((uint32_t)j);
-          if (!ok) break;
-          mbar_expect_tx(kfull, (uint32_t)it.n_tiles * kAtKV);
-          for (int j = 0; j < it.n_tiles; ++j) tma_load_2d(sK + j * kAtKV, &tmK, kfull, it.kvh * 64, it.a0 + j * kAtKeys);
-          kpos = 0;
-          if (have_nx) ok = load_rope(nx);   // wanted while this item's scores are being turned into P
-          for (int j = 0; j < it.n_tiles && ok; ++j) ok = load_v(j);
-        } else {                           // streaming item: K for the maxima, then K and V side by side
-          for (int j = 0; j < it.n_tiles && ok; ++j) ok = load_k(j);
-          if (have_nx && ok) ok = load_rope(nx);
-          for (int j = 0; j < it.n_tiles && ok; ++j) ok = load_k(j) && load_v(j);
         }
         it = nx;
         idx = nidx;
@@ -253,117 +230,120 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     // ------------------------------------------------------------------ MMA issuer
     {   // the whole warp walks the loop, one elected lane issues (as in the GEMMs)
       const bool leader = elect_one();
-      uint32_t kfph = 0, kpos = 0, vq = 0, sq = 0, pq = 0, nit = 0;   // kfph: per-stage phase bits of the "full" barriers
+      uint32_t tq = 0, nit = 0;
+      uint32_t n_p[2] = {0, 0};   // products issued per stream: phases of sready / pready / pvdone
       bool ok = true;
-      const uint64_t dq = at_sdesc(sQ);
-      auto issue_s = [&]() -> bool {   // S[sq & 1] = Q K^T with the next K stage of the ring
-        const uint32_t b = sq & 1u, bph = (sq >> 1) & 1u, s = kpos, ph = (kfph >> s) & 1u;
-        if (!mbar_wait_warp(sfree + 8 * b, bph ^ 1u, abort_flag, p.status, 33)) return false;
-        if (!mbar_wait_warp(kfull + 8 * s, ph, abort_flag, p.status, 34)) return false;
-        kfph ^= 1u << s;
-        kpos = (kpos + 1) % kAtKS;
-        tc_fence_after();
-        const uint64_t dk = at_sdesc(sK + s * kAtKV);
-        if (leader) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem + b * 64, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), kAtIdesc, k > 0 ? 1u : 0u);
-          tc_commit(kempty + 8 * s);
-          tc_commit(sready + 8 * b);
-        }
-        ++sq;
-        return true;
-      };
       for (int idx = blockIdx.x; idx < n_items && ok; idx += gridDim.x) {
         const AttItem it = at_item(p, cu, idx);
         if (!it.on) continue;
-        // the accumulator columns are free once the O of the item before has been read (all of its score reads
-        // come earlier); then the rotated Q tile of this item
-        if (!(ok = mbar_wait_warp(ofree, (nit & 1u) ^ 1u, abort_flag, p.status, 36))) break;
         if (!(ok = mbar_wait_warp(qready, nit & 1u, abort_flag, p.status, 35))) break;
         tc_fence_after();
-        auto issue_pv = [&](uint32_t o_col, bool first) -> bool {   // O (+)= P V with the next P buffer and V stage
-          const uint32_t b = pq & 1u, bph = (pq >> 1) & 1u, s = vq % kAtVS, ph = (vq / kAtVS) & 1u;
-          if (!mbar_wait_warp(pready + 8 * b, bph, abort_flag, p.status, 37)) return false;
-          if (!mbar_wait_warp(vfull + 8 * s, ph, abort_flag, p.status, 38)) return false;
-          tc_fence_after();
-          const uint64_t dp = at_sdesc(sP + b * kAtTile), dv = at_sdesc(sV + s * kAtKV);
-          if (leader) {
+        const uint64_t dq = at_sdesc(sQ + (nit & 1u) * kAtTile);
+        int tile[2] = {0, 1}, left = it.n_tiles;   // next tile of each stream; products to go
+        bool scores[2] = {false, false};           // its scores have been issued
+        bool o_free = false;
+        unsigned long long t0 = 0;
+        uint32_t spins = 0;
+        while (left > 0) {
+          bool moved = false;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              tc_mma_bf16(tmem + o_col, dp + (uint64_t)(2 * k), dv + kAtVStep * k, kAtIdescPV, (!first || k > 0) ? 1u : 0u);
-            tc_commit(vempty + 8 * s);
-            tc_commit(pfree + 8 * b);
-          }
-          ++pq; ++vq;
-          return true;
-        };
-        if (it.n_tiles <= kAtResident) {
-          // resident item: the scores against all of its keys in one product per 16 dims (the key tiles lie side
-          // by side in stages 0 .. n - 1), one hand-over; then the second products as the P tiles arrive
-          if (!(ok = mbar_wait_warp(kfull, kfph & 1u, abort_flag, p.status, 34))) break;
-          kfph ^= 1u;
-          kpos = 0;
-          tc_fence_after();
-          const uint64_t dk = at_sdesc(sK);
-          const uint32_t idn = at_idesc_n(it.n_tiles);
-          if (leader) {
+          for (int h = 0; h < 2; ++h) {
+            if (tile[h] >= it.n_tiles) continue;
+            const uint32_t g = tq + (uint32_t)tile[h], s = g % kAtRing, ph = (g / kAtRing) & 1u;
+            if (!scores[h]) {
+              // P of the product before lies where these scores go
+              if (!__all_sync(0xffffffffu, (n_p[h] == 0 || mbar_test_wait(pvdone + 8 * h, (n_p[h] - 1) & 1u)) &&
+                                               mbar_test_wait(kfull + 8 * s, ph))) continue;
+              tc_fence_after();
+              const uint64_t dk = at_sdesc(sK + s * kAtKV);
+              if (leader) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), idn, k > 0 ? 1u : 0u);
-            for (int j = 0; j < it.n_tiles; ++j) tc_commit(kempty + 8 * j);
-            tc_commit(sall);
+                for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem + h * 64, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), kAtIdesc, k > 0 ? 1u : 0u);
+                tc_commit(kempty + 8 * s);
+                tc_commit(sready + 8 * h);
+              }
+              scores[h] = true;
+              moved = true;
+            } else {
+              // the accumulators are free once the O of the item before has been read
+              if (!o_free && !(o_free = __all_sync(0xffffffffu, mbar_test_wait(ofree, (nit & 1u) ^ 1u)))) continue;
+              if (!__all_sync(0xffffffffu, mbar_test_wait(pready + 8 * h, n_p[h] & 1u) && mbar_test_wait(vfull + 8 * s, ph))) continue;
+              tc_fence_after();
+              const uint64_t dv = at_sdesc(sV + s * kAtKV);
+              const uint32_t first = tile[h] == h ? 0u : 1u;
+              if (leader) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  tc_mma_bf16_ta(tmem + 128 + h * 64, tmem + h * 64 + 8 * k, dv + kAtVStep * k, kAtIdescPV, k > 0 ? 1u : first);
+                tc_commit(vempty + 8 * s);
+                tc_commit(pvdone + 8 * h);
+              }
+              ++n_p[h];
+              scores[h] = false;
+              tile[h] += 2;
+              --left;
+              moved = true;
+            }
           }
-          for (int j = 0; j < it.n_tiles && ok; ++j) ok = issue_pv(0, j == 0);
-        } else {
-          // streaming item, pass 1: scores only (the softmax warps take the row maxima)
-          for (int j = 0; j < it.n_tiles && ok; ++j) ok = issue_s();
-          if (!ok) break;
-          // pass 2: scores again, then O += P V; the scores of tile j + 1 are issued before the product of tile j
-          ok = issue_s();
-          for (int j = 0; j < it.n_tiles && ok; ++j) {
-            if (j + 1 < it.n_tiles && !(ok = issue_s())) break;
-            ok = issue_pv(128, j == 0);
+          if (moved) {
+            spins = 0;
+            t0 = 0;
+          } else if ((++spins & 0x3FFu) == 0) {   // bounded, as every wait
+            int stop = *abort_flag;
+            const unsigned long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kWaitLimitNs) {
+              stop = *abort_flag = 1;
+              atomicExch(&p.status->timeout_flag, 1);
+              atomicExch(&p.status->timeout_site, 33);
+            }
+            if (__any_sync(0xffffffffu, stop != 0)) {
+              ok = false;
+              break;
+            }
           }
         }
         if (ok && leader) tc_commit(oready);
+        tq += (uint32_t)it.n_tiles;
         ++nit;
       }
     }
   } else {
-    // ------------------------------------------------------------------ softmax / epilogue: two threads per tile row
-    // warps 2..5 take columns 0..31 of a tile, warps 6..9 columns 32..63 (a warp may only read the TMEM lanes of its
-    // quarter, warp index mod 4).  The two halves of a row meet twice per item through shared memory: for the row
-    // maximum after pass 1 and for the row sum after pass 2; those two named barriers are reached by all 256
-    // threads whatever happened before (a thread whose wait ran out skips the work, not the barriers), and the
-    // decision to give up is taken from a flag that is only written between the item's two barriers.
+    // ------------------------------------------------------------------ softmax / epilogue: a thread per row and stream
+    // The streams of an item meet through shared memory at a named barrier that all 256 threads reach whatever happened
+    // before (a thread whose wait ran out skips the work, not the barrier); the decision to give up is taken from the
+    // item's flag, which is only written before it (two flags in turn: the next item may fail before all have read).
     const int quarter = warp & 3, half = (warp - 2) >> 2;
     const int row = quarter * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const int qd = p.n_heads * 64;
-    float* xm = reinterpret_cast<float*>(bar_ptr + 256);      // [2][128] row maxima of the two halves
-    float* xl = xm + 256;                                     // [2][128] row sums
-    uint32_t sq = 0, pq = 0, nit = 0, nres = 0;
-    // Q rows: load, rotate (pairs (d, d + 32), position inside the request), lay down swizzled.  This thread takes
-    // 16-byte chunks 2 half, 2 half + 1 of its row and their rotation partners 4 further on.  The loads of the
-    // NEXT item's rows are issued while this item's scores are on their way and staged as soon as the Q tile is free
-    // (all score MMAs of this item complete), so that the MMA warp finds the tile ready when the accumulators are.
+    float2* xml = reinterpret_cast<float2*>(bar_ptr + 256);   // [item parity][stream][row]: (maximum, sum)
+    uint32_t n_s = 0, nit = 0, rq = 0;                        // score tiles of this stream, items, rope blocks
+    bool ok = true;
+    // Q rows: the raw tile comes by TMA (in the swizzled layout); a thread rotates 16-byte chunks 2 half, 2 half + 1 of its
+    // row and their partners 4 further on in place (pairs (d, d + 32), position inside the request).  Rows past the
+    // request are whatever lies there: nothing of a row reaches another.
     const int i0c = 2 * half;
     const int row_pos = row / p.g, row_head = row % p.g;   // position inside the block and head inside the group
-    auto q_load = [&](const AttItem& n, uint4 (&c)[4]) {
-      const int npos = n.q0 + row_pos, nhead = n.kvh * p.g + row_head;
-      const bool nlive = npos < n.L;
-      const uint4* src = reinterpret_cast<const uint4*>(p.q + (size_t)(n.t0 + (nlive ? npos : 0)) * qd + nhead * 64);
-      c[0] = nlive ? __ldg(src + i0c) : make_uint4(0, 0, 0, 0);
-      c[1] = nlive ? __ldg(src + i0c + 1) : make_uint4(0, 0, 0, 0);
-      c[2] = nlive ? __ldg(src + i0c + 4) : make_uint4(0, 0, 0, 0);
-      c[3] = nlive ? __ldg(src + i0c + 5) : make_uint4(0, 0, 0, 0);
+    auto q_load = [&](const AttItem& n, uint32_t buf) {    // one thread
+      mbar_expect_tx(qraw, kAtTile);
+      tma_load_3d(sQ + buf * kAtTile, &tmQ, qraw, 0, n.kvh * p.g, n.t0 + n.q0);
     };
-    uint32_t rq = 0;
-    bool ok = true;
-    auto q_stage = [&](const AttItem& n, uint4 (&c)[4]) {
+    uint32_t nq = 0;   // Q tiles staged
+    auto q_stage = [&](const AttItem& n) {
+      uint8_t* qrow = base_ptr + (sQ - base) + (nq & 1u) * kAtTile;
+      ok = mbar_wait(qraw, nq & 1u, abort_flag, p.status, 46) && ok;
+      ++nq;
       const int npos = n.q0 + row_pos;
+      const bool nlive = npos < n.L;
+      uint4 c[4];
+      c[0] = *reinterpret_cast<const uint4*>(qrow + at_swz(row, i0c));
+      c[1] = *reinterpret_cast<const uint4*>(qrow + at_swz(row, i0c + 1));
+      c[2] = *reinterpret_cast<const uint4*>(qrow + at_swz(row, i0c + 4));
+      c[3] = *reinterpret_cast<const uint4*>(qrow + at_swz(row, i0c + 5));
       // the (cos, sin) rows of the item's positions: staged by the producer when they fit, else from the table
       if (p.rope_smem) ok = mbar_wait(rfull, rq & 1u, abort_flag, p.status, 45) && ok;
-      if (npos < n.L) {
+      if (nlive) {
         const float4* rt = p.rope_smem ? reinterpret_cast<const float4*>(base_ptr + (sRope - base) + row_pos * 256)
                                        : reinterpret_cast<const float4*>(p.rope + (size_t)npos * 32);
 #pragma unroll
@@ -379,7 +359,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           }
         }
       }
-      uint8_t* qrow = base_ptr + (sQ - base);
       *reinterpret_cast<uint4*>(qrow + at_swz(row, i0c)) = c[0];
       *reinterpret_cast<uint4*>(qrow + at_swz(row, i0c + 1)) = c[1];
       *reinterpret_cast<uint4*>(qrow + at_swz(row, i0c + 4)) = c[2];
@@ -395,238 +374,163 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     AttItem it;
     bool have = next_item(idx, it);
     if (have) {
-      uint4 c[4];
-      q_load(it, c);
-      q_stage(it, c);
+      if (threadIdx.x == 64) q_load(it, 0);
+      q_stage(it);
     }
+    const uint32_t s_addr = tmem + lane_addr + half * 64;
     while (have) {
+      const int pos = it.q0 + row_pos;
+      // The next item's Q buffer is free: O of the item before this one was waited for, so all its products are complete.
       AttItem nx;
-      int nidx = idx;
-      const bool have_nx = next_item(nidx, nx);
-      const int pos = it.q0 + row_pos, head = it.kvh * p.g + row_head;
-      const bool live = pos < it.L;
-      uint4 cn[4];
-      if (have_nx && it.n_tiles <= kAtResident) q_load(nx, cn);
-      const bool resident = it.n_tiles <= kAtResident;
-      // Scores come in half tiles of 32 keys, taken as two groups of 16.  Keys are counted from the request's first
-      // token (kr); row `pos` sees kr <= pos.  A group is visible to every row of the item when it ends before the
-      // item's first position, to none when it starts after the item's last one (both the same for all threads:
-      // no exponentials are spent there), and is masked key by key otherwise.
+      const bool have_nx = next_item(idx, nx);
+      if (have_nx && threadIdx.x == 64) q_load(nx, (nit + 1) & 1u);
+      if (have_nx && half >= it.n_tiles) q_stage(nx);
+      // Keys are counted from the request's first token; row `pos` sees key <= pos.  A group of 16 is visible to every
+      // row of the item when it ends before the item's first position, to none when it starts after the item's last one
+      // (both the same for all threads), and is masked key by key otherwise.
       const int q_last = it.q0 + p.ppt - 1;
-      auto tile_max = [&](const uint32_t (&v)[32], int kr0, float m) -> float {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int kr = kr0 + 16 * q;
+      float m = -INFINITY, l = 0.f;   // running maximum of the raw scores (the scale is positive), sum of p
+      for (int j = half; j < it.n_tiles && ok; j += 2, ++n_s) {
+        if (!(ok = mbar_wait_warp(sready + 8 * half, n_s & 1u, abort_flag, p.status, 39))) break;
+        tc_fence_after();
+        // twice over the scores in groups of 16 keys, the next group's read in flight (a thread that keeps all 64 spills)
+        const int kr0 = j * kAtKeys;
+        uint32_t va[16], vb[16];
+        float ma = -INFINITY, mc = -INFINITY;
+        auto group_max = [&](const uint32_t (&v)[16], int kr) {
           if (kr + 15 <= it.q0) {
 #pragma unroll
-            for (int c = 16 * q; c < 16 * q + 16; c += 2) m = max3(m, __uint_as_float(v[c]), __uint_as_float(v[c + 1]));
+            for (int c = 0; c < 16; c += 4) {
+              ma = max3(ma, __uint_as_float(v[c]), __uint_as_float(v[c + 1]));
+              mc = max3(mc, __uint_as_float(v[c + 2]), __uint_as_float(v[c + 3]));
+            }
           } else if (kr <= q_last) {
 #pragma unroll
-            for (int c = 16 * q; c < 16 * q + 16; ++c)
-              if (kr0 + c <= pos) m = fmaxf(m, __uint_as_float(v[c]));
+            for (int c = 0; c < 16; ++c)
+              if (kr + c <= pos) ma = fmaxf(ma, __uint_as_float(v[c]));
+          }
+        };
+        tmem_ld16(s_addr, va);
+        tmem_ld16(s_addr + 16, vb);
+        tmem_ld_wait();
+        group_max(va, kr0);
+        group_max(vb, kr0 + 16);
+        tmem_ld16(s_addr + 32, va);
+        tmem_ld16(s_addr + 48, vb);
+        tmem_ld_wait();
+        group_max(va, kr0 + 32);
+        group_max(vb, kr0 + 48);
+        tmem_ld16(s_addr, va);
+        const float mx = fmaxf(ma, mc);
+        if (j == half) {
+          m = mx;
+        } else {
+          const bool grow = (mx - m) * p.scale_log2 > kAtLag;
+          if (__any_sync(0xffffffffu, grow)) {   // (these scores exist only because the product before is complete)
+            const float m_new = grow ? mx : m;
+            const float corr = grow ? fast_exp2((m - m_new) * p.scale_log2) : 1.f;
+            m = m_new;
+            l *= corr;
+#pragma unroll
+            for (int c = 0; c < 64; c += 16) {
+              uint32_t o[16];
+              tmem_ld16(s_addr + 128 + c, o);
+              tmem_ld_wait();
+#pragma unroll
+              for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * corr);
+              tmem_st16(s_addr + 128 + c, o);
+            }
           }
         }
-        return m;
-      };
-      auto tile_p = [&](const uint32_t (&v)[32], int kr0, float mb, uint8_t* prow, float l) -> float {
-        uint32_t w[16];
-        const uint64_t scale2 = pair_f32(p.scale_log2, p.scale_log2), nmb2 = pair_f32(-mb, -mb);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int kr = kr0 + 16 * q;
+        const float mb = (m == -INFINITY) ? 0.f : m * p.scale_log2;
+        const uint64_t nmb2 = pair_f32(-mb, -mb), scale2 = pair_f32(p.scale_log2, p.scale_log2);
+        uint64_t l2 = pair_f32(l, 0.f);
+        auto group_p = [&](const uint32_t (&v)[16], int kr, uint32_t* w) {
           if (kr + 15 <= it.q0) {
-            uint64_t l2 = pair_f32(l, 0.f);
 #pragma unroll
-            for (int c = 16 * q; c < 16 * q + 16; c += 2) {
+            for (int c = 0; c < 16; c += 2) {
               float x0, x1;
               unpair_f32(fma2(pair_f32(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), scale2, nmb2), x0, x1);
               const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
               l2 = add2(l2, pair_f32(p0, p1));
               w[c >> 1] = pack_bf16(p0, p1);
             }
-            float la, lb;
-            unpair_f32(l2, la, lb);
-            l = la + lb;
           } else if (kr <= q_last) {
 #pragma unroll
-            for (int c = 16 * q; c < 16 * q + 16; c += 2) {
-              const int k0 = kr0 + c;
-              const float p0 = k0 <= pos ? fast_exp2(fmaf(__uint_as_float(v[c]), p.scale_log2, -mb)) : 0.f;
-              const float p1 = k0 + 1 <= pos ? fast_exp2(fmaf(__uint_as_float(v[c + 1]), p.scale_log2, -mb)) : 0.f;
-              l += p0 + p1;
+            for (int c = 0; c < 16; c += 2) {
+              const float p0 = kr + c <= pos ? fast_exp2(fmaf(__uint_as_float(v[c]), p.scale_log2, -mb)) : 0.f;
+              const float p1 = kr + c + 1 <= pos ? fast_exp2(fmaf(__uint_as_float(v[c + 1]), p.scale_log2, -mb)) : 0.f;
+              l2 = add2(l2, pair_f32(p0, p1));
               w[c >> 1] = pack_bf16(p0, p1);
             }
           } else {
 #pragma unroll
-            for (int c = 16 * q; c < 16 * q + 16; c += 2) w[c >> 1] = 0u;
+            for (int c = 0; c < 8; ++c) w[c] = 0u;
           }
-        }
+        };
 #pragma unroll
-        for (int i = 0; i < 4; ++i)               // chunks 4 half .. 4 half + 3 of this row
-          *reinterpret_cast<uint4*>(prow + at_swz(row, 4 * half + i)) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
-        return l;
-      };
-      // the same for one group of 16 keys at a time (resident items: the TMEM read of the next group is in flight
-      // while this one is worked on); two running maxima keep the dependent chain short
-      auto group_max = [&](const uint32_t (&v)[16], int kr, float& m0, float& m1) {
-        if (kr + 15 <= it.q0) {
-#pragma unroll
-          for (int c = 0; c < 16; c += 4) {
-            m0 = max3(m0, __uint_as_float(v[c]), __uint_as_float(v[c + 1]));
-            m1 = max3(m1, __uint_as_float(v[c + 2]), __uint_as_float(v[c + 3]));
-          }
-        } else if (kr <= q_last) {
-#pragma unroll
-          for (int c = 0; c < 16; ++c)
-            if (kr + c <= pos) m0 = fmaxf(m0, __uint_as_float(v[c]));
-        }
-      };
-      auto group_p = [&](const uint32_t (&v)[16], int kr, uint64_t scale2, uint64_t nmb2, float mb, uint32_t* w, float& l) {
-        if (kr + 15 <= it.q0) {
-          uint64_t l2 = pair_f32(l, 0.f);
-#pragma unroll
-          for (int c = 0; c < 16; c += 2) {
-            float x0, x1;
-            unpair_f32(fma2(pair_f32(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), scale2, nmb2), x0, x1);
-            const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-            l2 = add2(l2, pair_f32(p0, p1));
-            w[c >> 1] = pack_bf16(p0, p1);
-          }
-          float la, lb;
-          unpair_f32(l2, la, lb);
-          l = la + lb;
-        } else if (kr <= q_last) {
-#pragma unroll
-          for (int c = 0; c < 16; c += 2) {
-            const float p0 = kr + c <= pos ? fast_exp2(fmaf(__uint_as_float(v[c]), p.scale_log2, -mb)) : 0.f;
-            const float p1 = kr + c + 1 <= pos ? fast_exp2(fmaf(__uint_as_float(v[c + 1]), p.scale_log2, -mb)) : 0.f;
-            l += p0 + p1;
-            w[c >> 1] = pack_bf16(p0, p1);
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) w[c] = 0u;
-        }
-      };
-      // group g of this thread: tile g / 2, columns half * 32 + 16 (g % 2) of it
-      const uint32_t tcol = tmem + lane_addr + half * 32;
-      auto g_col = [&](int g) -> uint32_t { return tcol + (uint32_t)((g >> 1) * 64 + (g & 1) * 16); };
-      auto g_kr = [&](int g) -> int { return (g >> 1) * kAtKeys + half * 32 + (g & 1) * 16; };
-      // ---- pass 1: row maximum of the raw scores (the scale is positive: it commutes with the maximum)
-      float m = -INFINITY;
-      if (resident) {
-        if ((ok = ok && mbar_wait(sall, nres & 1u, abort_flag, p.status, 43))) {
-          tc_fence_after();
-          float m1 = -INFINITY;
-          uint32_t va[16], vb[16];
-          const int G = 2 * it.n_tiles;
-          tmem_ld16(g_col(0), va);
-          for (int g = 0; g < G; g += 2) {
-            tmem_ld_wait();
-            tmem_ld16(g_col(g + 1), vb);
-            group_max(va, g_kr(g), m, m1);
-            tmem_ld_wait();
-            if (g + 2 < G) tmem_ld16(g_col(g + 2), va);
-            group_max(vb, g_kr(g + 1), m, m1);
-          }
-          m = fmaxf(m, m1);
-        }
-        ++nres;
-      } else {
-        for (int j = 0; j < it.n_tiles && ok; ++j) {
-          const uint32_t b = sq & 1u, bph = (sq >> 1) & 1u;
-          if (!(ok = mbar_wait(sready + 8 * b, bph, abort_flag, p.status, 39))) break;
-          tc_fence_after();
-          uint32_t v[32];
-          tmem_ld32(tmem + lane_addr + b * 64 + half * 32, v);
-          tmem_ld_wait();
-          m = tile_max(v, j * kAtKeys + half * 32, m);
-          tc_fence_before();
-          mbar_arrive(sfree + 8 * b);
-          ++sq;
-        }
-      }
-      xm[half * 128 + row] = m;
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      m = fmaxf(m, xm[(half ^ 1) * 128 + row]);
-      const float mb = (m == -INFINITY) ? 0.f : m * p.scale_log2;
-      if (have_nx && resident) q_stage(nx, cn);   // every score MMA of this item is complete: the Q tile is free
-      // ---- pass 2: p = 2^(s - max), row sum in fp32, P tile as bf16 operand
-      float l = 0.f;
-      if (resident && ok) {
-        const uint64_t scale2 = pair_f32(p.scale_log2, p.scale_log2), nmb2 = pair_f32(-mb, -mb);
-        uint32_t va[16], vb[16];
-        tmem_ld16(g_col(0), va);
-        for (int j = 0; j < it.n_tiles; ++j) {
-          const uint32_t pb = pq & 1u, pph = (pq >> 1) & 1u;
+        for (int hq = 0; hq < 2; ++hq) {   // P of 32 keys into columns whose scores have been read
           uint32_t w[16];
           tmem_ld_wait();
-          tmem_ld16(g_col(2 * j + 1), vb);
-          group_p(va, g_kr(2 * j), scale2, nmb2, mb, w, l);
+          tmem_ld16(s_addr + 32 * hq + 16, vb);
+          group_p(va, kr0 + 32 * hq, w);
           tmem_ld_wait();
-          if (j + 1 < it.n_tiles) tmem_ld16(g_col(2 * j + 2), va);
-          group_p(vb, g_kr(2 * j + 1), scale2, nmb2, mb, w + 8, l);
-          if (!(ok = mbar_wait(pfree + 8 * pb, pph ^ 1u, abort_flag, p.status, 41))) break;
-          uint8_t* prow = base_ptr + (sP - base) + pb * kAtTile;
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<uint4*>(prow + at_swz(row, 4 * half + i)) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
-          tc_fence_before();                      // this tile's scores are read: the O columns over them may be written
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          mbar_arrive(pready + 8 * pb);
-          ++pq;
+          if (hq == 0) tmem_ld16(s_addr + 32, va);
+          group_p(vb, kr0 + 32 * hq + 16, w + 8);
+          tmem_st16(s_addr + 16 * hq, w);
         }
-        if (!ok) tmem_ld_wait();
+        float la, lb;
+        unpair_f32(l2, la, lb);
+        l = la + lb;
+        tmem_st_wait();
+        tc_fence_before();
+        mbar_arrive(pready + 8 * half);
+        if (have_nx && j == half) q_stage(nx);   // under this tile's product and the next one's scores
       }
-      for (int j = 0; j < it.n_tiles && ok && !resident; ++j) {
-        const uint32_t b = sq & 1u, bph = (sq >> 1) & 1u, pb = pq & 1u, pph = (pq >> 1) & 1u;
-        if (!resident && !(ok = mbar_wait(sready + 8 * b, bph, abort_flag, p.status, 40))) break;
-        if (!(ok = mbar_wait(pfree + 8 * pb, pph ^ 1u, abort_flag, p.status, 41))) break;
-        tc_fence_after();
-        uint32_t v[32];
-        tmem_ld32(tmem + lane_addr + (resident ? j : (int)b) * 64 + half * 32, v);
-        tmem_ld_wait();
-        l = tile_p(v, j * kAtKeys + half * 32, mb, base_ptr + (sP - base) + pb * kAtTile, l);
-        tc_fence_before();                        // the scores are read: the buffer (resident: the O columns) may be written
-        if (!resident) { mbar_arrive(sfree + 8 * b); ++sq; }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(pready + 8 * pb);
-        ++pq;
-      }
-      if (have_nx && !resident) {                 // streaming item: Q was an operand up to the last score tile
-        q_load(nx, cn);
-        q_stage(nx, cn);
-      }
-      xl[half * 128 + row] = l;
-      if (!ok) *sm_fail = 1;
+      float2* mine = xml + (nit & 1u) * 256;
+      mine[half * 128 + row] = make_float2(m, l);
+      if (!ok) sm_fail[nit & 1u] = 1;
       asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (*sm_fail) break;                       // the same for all 256 threads
-      l += xl[(half ^ 1) * 128 + row];
-      // ---- O / l -> out: this thread's 32 of the row's 64 dims
-      if ((ok = mbar_wait(oready, nit & 1u, abort_flag, p.status, 42))) {
+      if (sm_fail[nit & 1u]) break;              // the same for all 256 threads
+      const float2 other = mine[(half ^ 1) * 128 + row];
+      const float top = fmaxf(m, other.x);
+      const float a_me = fast_exp2((m - top) * p.scale_log2), a_ot = fast_exp2((other.x - top) * p.scale_log2);
+      const float sum = l * a_me + other.y * a_ot;
+      const float inv = sum > 0.f ? 1.f / sum : 0.f;
+      const float f0 = (half == 0 ? a_me : a_ot) * inv, f1 = (half == 0 ? a_ot : a_me) * inv;
+      // ---- (O_0 f_0 + O_1 f_1) -> out: this thread's 32 of the row's 64 dims
+      if ((ok = mbar_wait_warp(oready, nit & 1u, abort_flag, p.status, 42))) {
         tc_fence_after();
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-        __nv_bfloat16* dst = p.out + (size_t)(it.t0 + (live ? pos : 0)) * qd + head * 64 + half * 32;
-        uint32_t v[32];
-        tmem_ld32(tmem + lane_addr + (resident ? 0 : 128) + half * 32, v);
-        tmem_ld_wait();
-        tc_fence_before();                        // O is in registers: the accumulator columns may be written again
-        mbar_arrive(ofree);
-        if (live) {
+        const bool live = it.q0 + row_pos < it.L;
+        __nv_bfloat16* dst = p.out + (size_t)(it.t0 + (live ? it.q0 + row_pos : 0)) * qd + (it.kvh * p.g + row_head) * 64 + half * 32;
+        uint32_t v[16], u[16];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint4 o;
-            o.x = pack_bf16(__uint_as_float(v[8 * i]) * inv, __uint_as_float(v[8 * i + 1]) * inv);
-            o.y = pack_bf16(__uint_as_float(v[8 * i + 2]) * inv, __uint_as_float(v[8 * i + 3]) * inv);
-            o.z = pack_bf16(__uint_as_float(v[8 * i + 4]) * inv, __uint_as_float(v[8 * i + 5]) * inv);
-            o.w = pack_bf16(__uint_as_float(v[8 * i + 6]) * inv, __uint_as_float(v[8 * i + 7]) * inv);
-            *reinterpret_cast<uint4*>(dst + 8 * i) = o;
+        for (int c = 0; c < 32; c += 16) {
+          tmem_ld16(tmem + lane_addr + 128 + half * 32 + c, v);
+          if (it.n_tiles > 1) {
+            tmem_ld16(tmem + lane_addr + 192 + half * 32 + c, u);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) u[i] = 0u;   // (nothing was ever accumulated there)
+          }
+          tmem_ld_wait();
+          if (c == 16) {                          // O is in registers: the accumulators may be written again
+            tc_fence_before();
+            mbar_arrive(ofree);
+          }
+          uint32_t o[8];
+#pragma unroll
+          for (int i = 0; i < 16; i += 2)
+            o[i >> 1] = pack_bf16(fmaf(__uint_as_float(u[i]), f1, __uint_as_float(v[i]) * f0),
+                                  fmaf(__uint_as_float(u[i + 1]), f1, __uint_as_float(v[i + 1]) * f0));
+          if (live) {
+            *reinterpret_cast<uint4*>(dst + c) = make_uint4(o[0], o[1], o[2], o[3]);
+            *reinterpret_cast<uint4*>(dst + c + 8) = make_uint4(o[4], o[5], o[6], o[7]);
           }
         }
       }
       ++nit;
       it = nx;
-      idx = nidx;
       have = have_nx;
     }
   }
@@ -655,12 +559,13 @@ moin_status launch_attention_tc(HostState* hs, const __nv_bfloat16* q, const __n
                                 int T, int max_seqlen, int n_heads, int n_kv_heads, float scale_log2,
                                 cudaStream_t stream) {
   const int kvd = n_kv_heads * 64, g = n_heads / n_kv_heads;
-  CUtensorMap mk, mv;
-  moin_status st = make_map(&mk, k, (uint64_t)T, (uint64_t)kvd, kAtKeys);
+  CUtensorMap mq, mk, mv;
+  moin_status st = make_map_heads(&mq, q, (uint64_t)T, (uint32_t)n_heads, (uint32_t)g, (uint32_t)(128 / g));
+  if (!st) st = make_map(&mk, k, (uint64_t)T, (uint64_t)kvd, kAtKeys);
   if (!st) st = make_map(&mv, v, (uint64_t)T, (uint64_t)kvd, kAtKeys);
   if (st) return st;
   AttParams p = {};
-  p.q = q; p.out = out; p.cu = cu; p.rope = rope; p.R = R; p.n_heads = n_heads; p.n_kv = n_kv_heads; p.g = g;
+  p.out = out; p.cu = cu; p.rope = rope; p.R = R; p.n_heads = n_heads; p.n_kv = n_kv_heads; p.g = g;
   p.ppt = 128 / g; p.n_qb = (max_seqlen + p.ppt - 1) / p.ppt; p.scale_log2 = scale_log2; p.status = hs->status;
   p.max_pos = max_seqlen;
   p.rope_smem = p.ppt * 256 <= kAtRopeBytes;
@@ -670,7 +575,7 @@ moin_status launch_attention_tc(HostState* hs, const __nv_bfloat16* q, const __n
   const long items = (long)p.n_qb * R * n_kv_heads;
   long grid = items < 2L * hs->n_sms ? items : 2L * hs->n_sms;
   if (grid < 1) grid = 1;
-  return record_cuda(launch_pdl(attention_tc_kernel, (unsigned)grid, kAtThreads, kAtSmem, stream, mk, mv, p));
+  return record_cuda(launch_pdl(attention_tc_kernel, (unsigned)grid, kAtThreads, kAtSmem, stream, mq, mk, mv, p));
 }
 
 }  // namespace moin

@@ -13,6 +13,9 @@ moin_status make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t
 // The same for bytes: a [box_rows x 64] box, 64-byte swizzle.
 moin_status make_map_u8(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 
+// bf16 [T][n_heads][64]: a box of box_t tokens x box_heads heads.
+moin_status make_map_heads(CUtensorMap* map, const void* base, uint64_t T, uint32_t n_heads, uint32_t box_heads, uint32_t box_t);
+
 // Shape predicates (host): can the tcgen05 kernels take this problem?
 bool tc_gemm_supported(int T, int d_in, int d_out);
 bool tc_router_supported(int Q, int K, int D);

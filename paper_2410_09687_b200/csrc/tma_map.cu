@@ -53,6 +53,21 @@ moin_status make_map_u8(CUtensorMap* map, const void* base, uint64_t rows, uint6
   return MOIN_OK;
 }
 
+// bf16 [T][n_heads][64] -> map with a box of box_t tokens x box_heads heads x 64, 128-byte swizzle, zero fill.
+moin_status make_map_heads(CUtensorMap* map, const void* base, uint64_t T, uint32_t n_heads, uint32_t box_heads, uint32_t box_t) {
+  moin_status st = get_encoder();
+  if (st) return st;
+  cuuint64_t dims[3] = {(cuuint64_t)kMapBox, n_heads, T};
+  cuuint64_t strides[2] = {kMapBox * 2, (cuuint64_t)n_heads * kMapBox * 2};
+  cuuint32_t box[3] = {(cuuint32_t)kMapBox, box_heads, box_t};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return record_cuda(cudaErrorInvalidValue);
+  return MOIN_OK;
+}
+
 bool tc_gemm_supported(int T, int d_in, int d_out) { return T >= 1 && d_in >= 64 && (d_in % 8) == 0 && (d_out % 8) == 0; }
 bool tc_router_supported(int Q, int K, int D) { return Q >= 1 && K >= 1 && D >= 64 && (D % 8) == 0; }
 bool tc_fused_supported(int r) { return r >= 8 && r <= 128 && (r % 8) == 0; }
