@@ -558,7 +558,7 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
 // The first CTA holds cols rows of the gate weight and the second the same rows of the up weight, so one MMA gives both
 // (accumulator columns 0 .. cols - 1 and cols .. 2 cols - 1); the low-rank blocks multiply the gate's and the up
 // projection's halves of the columns one after the other.  16384 x 2048 -> 2 x 5632: the two projections 510 us and the
-// product's own pass 94 us (553 MB), now 540 us together.
+// product's own pass 94 us (553 MB), now 507 us together.
 moin_status launch_pair_swiglu(HostState* hs, const PlanView* pv, const PairJob* jobs, int M, int K, cudaStream_t stream) {
   const int F = jobs[0].N, N2 = 2 * F;
   const long tiles_m = (M + kPairM - 1) / kPairM;

@@ -11,7 +11,7 @@
 //   warps 2-9  TMEM -> shared memory (row pitch N + 4 floats: no bank conflicts), two warps per lane quarter
 // Against one CTA per row tile (calls of 3392 tokens in runs of 106, rank 64, to 256 columns, projection included):
 // K = 2048 26.6 -> 23.2 us, K = 5632 52 -> 42 us, three projections 46.5 -> 32.7 us; 16384 tokens fill the SMs with one
-// CTA per row tile and are bound by reading x (84 us of which 32 us at the copy bandwidth for K = 5632).
+// CTA per row tile and are bound by reading x (rank 16, K = 5632: 41 us, 28 us of them at the copy bandwidth).
 #include <cuda.h>
 
 #include "ptx.cuh"
