@@ -236,7 +236,7 @@ static moin_status route_launch(HostState* hs, int choice, const moin_router* ro
   }
   if (choice == 1) {
     // the merge across column tiles is a max, so the keys must start from zero
-    cudaError_t e = cudaMemsetAsync(keys, 0, (size_t)Q * sizeof(unsigned long long), s);
+    cudaError_t e = launch_clear_keys(keys, (size_t)Q, s);
     if (e != cudaSuccess) return record_cuda(e);
     moin_status st;
     {
@@ -333,7 +333,7 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
   const size_t half = align_up((size_t)Q * sizeof(unsigned long long), 256);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(workspace);
   unsigned long long* keys2 = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(workspace) + half);
-  cudaError_t e = cudaMemsetAsync(workspace, 0, 2 * half, s);
+  cudaError_t e = launch_clear_keys(keys, 2 * half / sizeof(unsigned long long), s);
   if (e != cudaSuccess) return record_cuda(e);
   {
     ProfScope prof(MOIN_K_ROUTE_TC, 1, s);

@@ -475,6 +475,17 @@ route_parts_kernel(const unsigned long long* __restrict__ part_keys, int parts, 
   if (on && sub == 0) route_write<TOP2>(out, cmap, i, k1, k2, ss);
 }
 
+__global__ void __launch_bounds__(256)
+clear_keys_kernel(unsigned long long* __restrict__ keys, size_t n) {   // keys is 16-byte aligned
+  pdl_begin();
+  const size_t i = 2 * ((size_t)blockIdx.x * 256 + threadIdx.x);
+  if (i + 1 < n) *reinterpret_cast<ulonglong2*>(keys + i) = make_ulonglong2(0ull, 0ull);
+  else if (i < n) keys[i] = 0ull;
+}
+cudaError_t launch_clear_keys(unsigned long long* keys, size_t n, cudaStream_t stream) {
+  return launch_pdl(clear_keys_kernel, (unsigned)((n + 511) / 512), 256, 0, stream, keys, n);
+}
+
 // How a problem is cut: queries per cluster, CTAs per cluster, parts of the table; fast = the rule picks this kernel.
 struct RouteCut { int nq, csize, parts, groups; bool fast; };
 static RouteCut route_cut(int Q, int K, int D) {
