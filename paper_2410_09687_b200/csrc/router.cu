@@ -499,7 +499,7 @@ static RouteCut route_cut(int Q, int K, int D) {
   constexpr int kResident = 12;
   while (r.parts < kRouteMaxParts && K > 512 * r.parts && r.groups * (r.parts + 1) <= kResident) ++r.parts;
   const int tiles = (K + 512 * r.parts - 1) / (512 * r.parts);   // tiles per warp pair
-  // Against the tensor-core GEMM with its clearing and finishing launches (12.4 us up to 128 queries, 14.4 at 256 x
+  // Against the tensor-core GEMM with its clearing and finishing launches (11.8 us up to 128 queries, 14.4 at 256 x
   // 5000 x 768): 7.3 us for up to 8 queries and 9.8-10.6 us for up to 32 per cluster with one tile per warp pair,
   // 13.3 and 18.7 with two.
   r.fast = r.groups * r.parts <= kResident && tiles <= (nq == 8 ? 2 : 1);
