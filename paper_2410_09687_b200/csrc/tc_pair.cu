@@ -126,7 +126,8 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + 16 * S + 32);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 16 * S + 40);
   constexpr bool kTail = EPI == PAIR_STORE || EPI == PAIR_SWIGLU;   // low-rank blocks at the end of a tile
-  const uint32_t tab0 = bars + 16 * S + 48;   // pass tables of this and the next tile, and their barriers
+  // pass tables of this and the next tile, their barriers: written, and read to the end by this CTA's producer
+  const uint32_t tab0 = bars + 16 * S + 48, tabread0 = tab0 + 16;
   uint8_t* tab_ptr = bar_ptr + 256;
   static_assert(256 + 2 * kPairTabBytes <= 1024, "barrier block");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -141,6 +142,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       mbar_init(tfull0 + 8 * a, 1);    // each CTA's own, by commit
       mbar_init(tempty0 + 8 * a, 16);  // used in the first CTA: one arrival per epilogue warp of the pair
       mbar_init(tab0 + 8 * a, 1);
+      mbar_init(tabread0 + 8 * a, 1);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -214,6 +216,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
             }
           }
         }
+        if (ok) mbar_arrive(tabread0 + 8 * (lt & 1u));
       }
     }
   } else if (warp == 1) {
@@ -274,6 +277,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
             }
           }
         }
+        __syncwarp();   // every lane has read the tile's passes
         if (ok && leader) tc_commit_pair(tfull0 + 8 * acc);
       }
     }
@@ -285,17 +289,21 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
     const uint32_t buf = out0 + (uint32_t)(wh * 4 + q) * 4096u;
     uint32_t lt = 0, n_st = 0;
     bool ok = true;
-    // Passes of tile i into table i & 1.  Written when the epilogue of tile i - 2 is over at the earliest: its
-    // accumulator was complete, so nobody reads that tile's table any more.
-    auto scout = [&](const PairTile& n, uint32_t i) {
+    // Passes of tile i into table i & 1.  The readers of tile i - 2's passes there are through: the MMA warp, whose
+    // reads come before the commit of the accumulator that this warp has waited for, and the producer, whose last entries
+    // may be passes without an adapter, which no copy and so no accumulator depends on: it says when it has read them.
+    auto scout = [&](const PairTile& n, uint32_t i) -> bool {
+      if (!mbar_wait_warp(tabread0 + 8 * (i & 1u), ((i >> 1) & 1u) ^ 1u, abort_flag, p.status, 67)) return false;
       pair_passes(p, n, EPI == PAIR_SWIGLU, lane, tab_ptr + (i & 1u) * kPairTabBytes);
       __syncwarp();
       if (lane == 0) mbar_arrive(tab0 + 8 * (i & 1u));
+      return true;
     };
-    if (kTail && warp == 2 && p.tail_r > 0 && pair < total) scout(pair_tile(p, pair, tiles_m), 0);
+    if (kTail && warp == 2 && p.tail_r > 0 && pair < total) ok = scout(pair_tile(p, pair, tiles_m), 0);
     for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
       const PairTile t = pair_tile(p, tile, tiles_m);
-      if (kTail && warp == 2 && p.tail_r > 0 && tile + n_pairs < total) scout(pair_tile(p, tile + n_pairs, tiles_m), lt + 1);
+      if (kTail && warp == 2 && p.tail_r > 0 && tile + n_pairs < total &&
+          !(ok = scout(pair_tile(p, tile + n_pairs, tiles_m), lt + 1))) break;
       const int row0 = rank == 0 ? t.row0[0] : t.row0[1], rows = rank == 0 ? t.rows[0] : t.rows[1];
       int n = p.N[0];
       __nv_bfloat16* y = p.y[0];
