@@ -321,6 +321,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
           const float inv = (4 * lane < p.bn / 2 && k0 + i < n) ? __ldg(p.inv_norm + k0 + i) : 0.f;
           e[i] = inv > 0.f ? inv : __int_as_float(0x7FC00000);
         }
+        __syncwarp();   // the other lanes have read the last tile's values
         *reinterpret_cast<float4*>(smem_raw + (buf - raw) + 16 * lane) = v;
         __syncwarp();
       }
