@@ -332,7 +332,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     uint32_t nq = 0;   // Q tiles staged
     auto q_stage = [&](const AttItem& n) {
       uint8_t* qrow = base_ptr + (sQ - base) + (nq & 1u) * kAtTile;
-      ok = mbar_wait(qraw, nq & 1u, abort_flag, p.status, 46) && ok;
+      ok = mbar_wait_warp(qraw, nq & 1u, abort_flag, p.status, 46) && ok;
       ++nq;
       const int npos = n.q0 + row_pos;
       const bool nlive = npos < n.L;
@@ -342,7 +342,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       c[2] = *reinterpret_cast<const uint4*>(qrow + at_swz(row, i0c + 4));
       c[3] = *reinterpret_cast<const uint4*>(qrow + at_swz(row, i0c + 5));
       // the (cos, sin) rows of the item's positions: staged by the producer when they fit, else from the table
-      if (p.rope_smem) ok = mbar_wait(rfull, rq & 1u, abort_flag, p.status, 45) && ok;
+      if (p.rope_smem) ok = mbar_wait_warp(rfull, rq & 1u, abort_flag, p.status, 45) && ok;
       if (nlive) {
         const float4* rt = p.rope_smem ? reinterpret_cast<const float4*>(base_ptr + (sRope - base) + row_pos * 256)
                                        : reinterpret_cast<const float4*>(p.rope + (size_t)npos * 32);

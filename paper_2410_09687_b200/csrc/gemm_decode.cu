@@ -172,7 +172,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
         if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
       }
     }
-    ok = ok && mbar_wait(done, 0, abort_flag, p.status, 53);
+    ok = ok && mbar_wait_warp(done, 0, abort_flag, p.status, 53);
     tc_fence_after();
   }
   // ---------------------------------------------------------------- epilogue

@@ -119,7 +119,9 @@ __device__ __forceinline__ bool mbar_wait_cluster_warp(uint32_t bar, uint32_t pa
   return __all_sync(0xffffffffu, mbar_wait_cluster(bar, parity, abort_flag, st, site));
 }
 
-// mbar_wait by a whole warp: the answer is the same for every lane, and the warp is converged afterwards.
+// mbar_wait by a whole warp: the answer is the same for every lane, and the warp is converged afterwards.  Needed
+// wherever warp-wide instructions follow: were the barrier to complete just as the limit expires, some lanes would go on
+// and wait in one of those for lanes that have given up.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, DeviceStatus* st,
                                                int site) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, st, site));

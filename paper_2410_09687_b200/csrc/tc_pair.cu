@@ -325,7 +325,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
         *reinterpret_cast<float4*>(smem_raw + (buf - raw) + 16 * lane) = v;
         __syncwarp();
       }
-      if (!(ok = mbar_wait(tfull0 + 8 * acc, aph, abort_flag, p.status, 64))) break;
+      if (!(ok = mbar_wait_warp(tfull0 + 8 * acc, aph, abort_flag, p.status, 64))) break;
       tc_fence_after();
       const bool row_ok = trow < rows;
       const size_t grow = (size_t)(row0 + trow);
