@@ -425,7 +425,6 @@ class KMeansWorkload:
         self.points = [rc.queries] + [torch.roll(rc.queries, shifts=i * 4099, dims=0).contiguous() for i in range(1, ROTATE)]
         self.assign = torch.empty(N, dtype=torch.int32, device=dev)
         self.plan = moin.Plan(N, K, dev, moin.PLAN_SEGMENTS)
-        self.router.workspace(N)
         self.unit, self.units_per_step = "points", N
         self.h_x = [self.points[0].cpu().pin_memory()]
         self.h_c = torch.empty(K, D, dtype=torch.bfloat16).pin_memory()

@@ -28,10 +28,11 @@
  *     hang: an out-of-range id means "no adapter" and is counted, a wait that runs out sets a
  *     flag, the kernel returns; both are read back with moin_device_status.
  *   - Results are deterministic: identical inputs give bit-identical outputs run to run.
- *   - Devices and threads: the library keeps its host-side state (side streams, events, the address of the
- *     status block, kernel attributes) per device ordinal and sets it up on the first call made with that
- *     device current, so one process may drive several GPUs; calls that target the SAME device must come
- *     from one host thread at a time (the per-device record and the side streams are not locked).
+ *   - Devices and threads: the library keeps its host-side state (the address of the status block, kernel
+ *     attributes) per device ordinal and sets it up on the first call made with that device current, so one
+ *     process may drive several GPUs; calls that target the SAME device must come from one host thread at a
+ *     time (the per-device record is not locked).  Calls on different streams may overlap on the GPU as long
+ *     as they share no output and no workspace.
  *   - Arithmetic: bf16 operands, fp32 accumulation, one rounding to bf16 at the output.
  */
 #ifndef MOIN_H_
@@ -140,7 +141,8 @@ moin_status moin_router_prepare(const void* centroids, int32_t K, int32_t D, flo
 size_t moin_route_workspace_bytes(int32_t Q, int32_t K, int32_t D);
 /* queries [Q, D] bf16 -> out_expert[Q] (int32: centroid_to_expert[id] if the map is given, else id),
  * out_centroid[Q] (nullable, int32 id), out_best_sim[Q] (nullable, fp32 cosine of the winner).
- * Q == 0 is a no-op.  Workspace contents are scratch. */
+ * Q == 0 is a no-op.  Workspace contents are scratch, also for a single query (the keys of a table cut into parts):
+ * calls that may overlap on the GPU - on two streams, or captured in two graphs - need a workspace each. */
 moin_status moin_route(const moin_router* router, const void* queries, int32_t Q, int32_t* out_expert,
                        int32_t* out_centroid, float* out_best_sim, void* workspace, size_t workspace_bytes,
                        moin_stream stream);

@@ -221,13 +221,20 @@ class Router:
         _check(lib().moin_router_prepare(_ptr(centroids), self.K, self.D, _ptr(self.inv_norm), _stream(stream)),
                "moin_router_prepare")
         self.c = _Router(_ptr(centroids), _ptr(self.inv_norm), _ptr(centroid_to_expert), self.K, self.D)
-        self._ws: Optional[torch.Tensor] = None
 
-    def workspace(self, Q: int) -> torch.Tensor:
-        n = lib().moin_route_workspace_bytes(Q, self.K, self.D)
-        if self._ws is None or self._ws.numel() < n:
-            self._ws = torch.empty(n, dtype=torch.uint8, device=self.centroids.device)
-        return self._ws
+    def workspace(self, Q: int, stream=None) -> torch.Tensor:
+        """Scratch of one call on ``stream``.  Every call has its own: calls over one table may overlap (several workers,
+        streams or captured graphs), and each keeps its keys there."""
+        return _scratch(lib().moin_route_workspace_bytes(Q, self.K, self.D), self.centroids.device, stream)
+
+
+def _scratch(nbytes: int, device, stream: Optional[torch.cuda.Stream]) -> torch.Tensor:
+    """A block of the caching allocator that belongs to the stream the call goes to: dropped when the call returns, it is
+    handed out again only to work behind the call."""
+    if stream is None:
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    with torch.cuda.stream(stream):
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
 
 
 def route(router: Router, queries: torch.Tensor, out_expert: Optional[torch.Tensor] = None,
@@ -237,7 +244,7 @@ def route(router: Router, queries: torch.Tensor, out_expert: Optional[torch.Tens
     Q = queries.shape[0]
     if out_expert is None:
         out_expert = torch.empty(Q, dtype=torch.int32, device=queries.device)
-    ws = router.workspace(Q)
+    ws = router.workspace(Q, stream)
     _check(lib().moin_route(ctypes.byref(router.c), _ptr(queries), Q, _ptr(out_expert), _ptr(out_centroid),
                             _ptr(out_best_sim), _ptr(ws), ws.numel(), _stream(stream)), "moin_route")
     return out_expert
@@ -250,8 +257,7 @@ def route_top2(router: Router, queries: torch.Tensor, stream=None) -> dict:
     out = {"expert": torch.empty(Q, dtype=torch.int32, device=dev), "centroid": torch.empty(Q, dtype=torch.int32, device=dev),
            "second": torch.empty(Q, dtype=torch.int32, device=dev), "best": torch.empty(Q, dtype=torch.float32, device=dev),
            "margin": torch.empty(Q, dtype=torch.float32, device=dev)}
-    n = lib().moin_route_top2_workspace_bytes(Q, router.K, router.D)
-    ws = torch.empty(max(n, 256), dtype=torch.uint8, device=dev)
+    ws = _scratch(lib().moin_route_top2_workspace_bytes(Q, router.K, router.D), dev, stream)
     _check(lib().moin_route_top2(ctypes.byref(router.c), _ptr(queries), Q, _ptr(out["expert"]), _ptr(out["centroid"]),
                                  _ptr(out["second"]), _ptr(out["best"]), _ptr(out["margin"]), _ptr(ws), ws.numel(),
                                  _stream(stream)), "moin_route_top2")
