@@ -272,9 +272,10 @@ def route_static(router: Router, queries: torch.Tensor, out_expert: torch.Tensor
                  stream=None) -> torch.Tensor:
     """moin_route_static: the router for callers that may not allocate device memory.
 
-    Same result as ``route``; the scratch lives inside the library (at most ROUTE_STATIC_MAX_Q queries per
-    call).  This wrapper allocates nothing either: the caller passes every output tensor.  Calls share
-    the built-in scratch, so calls that overlap on the GPU race - keep them ordered on one stream."""
+    Same result as ``route``; small problems need no scratch, that of larger ones lives inside the library (at most
+    ROUTE_STATIC_MAX_Q queries per call).  This wrapper allocates nothing either: the caller passes every output tensor.
+    Calls that use the built-in scratch share it (include/moin.h says which), so such calls race when they overlap on the
+    GPU - keep them ordered on one stream."""
     assert queries.dtype == torch.bfloat16 and queries.dim() == 2 and queries.shape[1] == router.D
     _check(lib().moin_route_static(ctypes.byref(router.c), _ptr(queries), queries.shape[0], _ptr(out_expert),
                                    _ptr(out_centroid), _ptr(out_best_sim), _stream(stream)), "moin_route_static")

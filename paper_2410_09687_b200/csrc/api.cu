@@ -211,6 +211,12 @@ size_t moin_route_workspace_bytes(int32_t Q, int32_t K, int32_t D) {
 // Kernel choice shared by moin_route and moin_route_static, so that both compute the same values for the same
 // shapes and options: 0 = cluster kernel (few queries; one 64-bit key of scratch per query and part when it cuts the
 // table), 1 = tensor-core GEMM with one 64-bit key of scratch per query, 2 = CUDA-core kernel (no scratch).
+// 0 and 1 have a form without scratch that gives the same bits and is slower; small problems are served by it where
+// there is none: up to 1024 queries against 1024 centroids, and up to 65 535 products.
+static bool route_without_scratch(const HostState* hs, int choice, int Q, int K, int D) {
+  if (choice != 1) return true;
+  return hs->gemm_impl == 0 && ((Q <= 1024 && K <= 1024 && D <= 3168) || (long long)Q * K < (1ll << 16));
+}
 static moin_status route_choice(const HostState* hs, int Q, int K, int D, int* choice) {
   const bool tc_ok = tc_router_supported(Q, K, D);
   bool use_tc = tc_ok && (long long)Q * K >= (1ll << 12);
@@ -229,10 +235,18 @@ static moin_status route_launch(HostState* hs, int choice, const moin_router* ro
                                 unsigned long long* keys, cudaStream_t s) {
   const int K = router->K, D = router->D;
   if (choice == 0) {
-    ProfScope prof(MOIN_K_ROUTE_CLUSTER, route_parts(Q, K, D) > 1 ? 2 : 1, s);
+    ProfScope prof(MOIN_K_ROUTE_CLUSTER, keys && route_parts(Q, K, D) > 1 ? 2 : 1, s);
     return record_cuda(launch_route_cluster((const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
                                             router->inv_norm, router->centroid_to_expert, Q, K, D, out_expert,
                                             out_centroid, out_best_sim, keys, s));
+  }
+  if (choice == 1 && !keys) {
+    ProfScope prof(MOIN_K_ROUTE_TC, out_best_sim ? 2 : 1, s);
+    moin_status st = launch_pair_router_rows(hs, (const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
+                                             router->inv_norm, router->centroid_to_expert, Q, K, D, out_expert, out_centroid,
+                                             out_best_sim, s);
+    if (st || !out_best_sim) return st;
+    return record_cuda(launch_route_cosine((const __nv_bfloat16*)queries, Q, D, out_best_sim, s));
   }
   if (choice == 1) {
     // the merge across column tiles is a max, so the keys must start from zero
@@ -276,13 +290,8 @@ moin_status moin_route(const moin_router* router, const void* queries, int32_t Q
   if ((st = route_choice(hs, Q, router->K, router->D, &choice))) return st;
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(workspace);
   if (!workspace || workspace_bytes < moin_route_workspace_bytes(Q, router->K, router->D) || !aligned16(workspace)) {
-    // small problems run without scratch: the cluster kernel with the table in one part, or the CUDA-core kernel
     keys = nullptr;
-    if (choice == 1 && hs->gemm_impl != 2) {
-      if (Q <= 1024 && router->K <= 1024 && router->D <= 3072) choice = 0;
-      else if ((long long)Q * router->K < (1ll << 16)) choice = 2;
-    }
-    if (choice == 1) return MOIN_ERR_WORKSPACE;
+    if (!route_without_scratch(hs, choice, Q, router->K, router->D)) return MOIN_ERR_WORKSPACE;
   }
   return route_launch(hs, choice, router, queries, Q, out_expert, out_centroid, out_best_sim, keys, (cudaStream_t)stream);
 }
@@ -362,7 +371,7 @@ moin_status moin_route_static(const moin_router* router, const void* queries, in
   int choice;
   if ((st = route_choice(hs, Q, router->K, router->D, &choice))) return st;
   unsigned long long* keys = nullptr;
-  if (choice == 1 || (choice == 0 && route_parts(Q, router->K, router->D) > 1)) {
+  if (!route_without_scratch(hs, choice, Q, router->K, router->D)) {
     if (g_route_static_ptr[hs->device] == nullptr) {   // set-up: once per device, that device is current here
       void* p = nullptr;
       cudaError_t e = cudaGetSymbolAddress(&p, g_route_static_keys);

@@ -228,8 +228,8 @@ bool route_cluster_supported(int Q, int K, int D);
 cudaError_t launch_route_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                  const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
                                  float* out_best, unsigned long long* part_keys, cudaStream_t stream);
-// Parts the cluster kernel cuts the table into, given route_parts(Q, K, D) * Q keys of scratch (top-2: twice as many);
-// with part_keys == nullptr it takes the table in one part.
+// Parts the cluster kernel cuts the table into: a cluster each, given route_parts(Q, K, D) * Q keys of scratch (top-2:
+// twice as many); with part_keys == nullptr one cluster walks them all, with the same results to the bit.
 constexpr int kRouteMaxParts = 12;
 int route_parts(int Q, int K, int D);
 cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
@@ -240,6 +240,8 @@ cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat1
 // the next one set up under it (K-means iteration 83 -> 80.6 us, 200
 // queries x 5000 x 768 12.3 -> 11.8 us).
 cudaError_t launch_clear_keys(unsigned long long* keys, size_t n, cudaStream_t stream);
+// out_best[i] /= |q_i| (-inf stays)
+cudaError_t launch_route_cosine(const __nv_bfloat16* q, int Q, int D, float* out_best, cudaStream_t stream);
 cudaError_t launch_route_finish(const unsigned long long* keys, const __nv_bfloat16* q, const int* cmap, int Q, int D,
                                 int* out_expert, int* out_centroid, float* out_best, cudaStream_t stream);
 
@@ -247,7 +249,7 @@ cudaError_t launch_route_finish(const unsigned long long* keys, const __nv_bfloa
 // that device current.  The status block's address and the kernels' shared-memory opt-ins belong to one device, so
 // nothing here is shared between devices.
 constexpr int kMaxDevices = 64;
-constexpr int kOptinSlots = 48;
+constexpr int kOptinSlots = 18;
 struct HostState {
   DeviceStatus* status = nullptr;  // device address of the status block
   int device = -1;
@@ -261,8 +263,8 @@ moin_status record_cuda(cudaError_t e);       // MOIN_OK or MOIN_ERR_CUDA (remem
 // Kernels that need more than 48 KB of dynamic shared memory opt in with cudaFuncSetAttribute; the driver keeps
 // that attribute per device, so the "already done" note is kept per device too (slot = one id per kernel).
 enum {
-  OPTIN_ROUTE_CLUSTER = 24, /* .. 27 */ OPTIN_ROUTE_SIMPLE = 28, OPTIN_ATTENTION = 29,
-  OPTIN_DECODE_GEMM = 30, OPTIN_TC_PAIR = 31 /* .. 34 */, OPTIN_TC_SHRINK = 35, OPTIN_DECODE_GEMM_FP8 = 36
+  OPTIN_ROUTE_CLUSTER = 0, /* .. 7 */ OPTIN_ROUTE_SIMPLE = 8, OPTIN_ATTENTION = 9, OPTIN_DECODE_GEMM = 10,
+  OPTIN_DECODE_GEMM_FP8 = 11, OPTIN_TC_SHRINK = 12, OPTIN_TC_PAIR = 13 /* .. 17 */
 };
 template <class Fn>
 inline cudaError_t ensure_smem_optin(int slot, Fn* fn, size_t bytes) {

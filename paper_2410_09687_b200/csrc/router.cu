@@ -165,7 +165,9 @@ route_finish_kernel(const unsigned long long* __restrict__ keys, const __nv_bflo
 // in shared memory with a 64-bit max on the (similarity, index) key, and after a cluster barrier CTA 0 reads the other
 // CTAs' keys through distributed shared memory.  A table in one part (up to 512 centroids) is finished right there:
 // one launch, no scratch.  Larger tables are cut into parts, one cluster each, whose keys go to
-// scratch and meet in a small second launch.
+// scratch and meet in a small second launch.  Without scratch (WALK) one cluster takes the whole table, a tile per warp; it
+// adds up the two halves of a row that two warps of a part would have had apart, so that the bits are the same (1 x 5000 x
+// 768: 7.7 us in ten parts, 21.7 without scratch).
 //
 // What bounds it: a few dependent memory round trips, and what the SMs of one cluster can pull - one cluster of 16
 // needs 15.3 us for 1 x 5000 x 768 (480 KB per SM), ten clusters and the second launch 7.4 us (the CUDA-core kernel
@@ -221,8 +223,8 @@ __device__ __forceinline__ void route_write(const RouteOut& out, const int* cmap
   }
 }
 
-// part_keys (nullptr when parts == 1): [parts][Q] keys, and with TOP2 [parts][Q] runner-up keys behind them
-template <int NQ, bool TOP2>
+// part_keys (nullptr when parts == 1 or WALK): [parts][Q] keys, and with TOP2 [parts][Q] runner-up keys behind them
+template <int NQ, bool TOP2, bool WALK>
 __global__ void __launch_bounds__(kRcWarps * 32)
 route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ c,
                      const float* __restrict__ inv_norm, const int* __restrict__ cmap, int Q, int K, int D, int parts,
@@ -235,16 +237,19 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const int rank = (int)cluster.block_rank(), csize = (int)cluster.num_blocks();
-  const int cl = blockIdx.x / csize, part = cl % parts, q0 = (cl / parts) * NQ;
+  const int cl = blockIdx.x / csize, part = WALK ? 0 : cl % parts, q0 = (WALK ? cl : cl / parts) * NQ;
   const int pitch = route_pitch(D);
   const int nch = D / 8, steps = (nch + 3) / 4, all_tiles = (K + 15) / 16;
-  const int tile_lo = (int)((long long)all_tiles * part / parts), tile_hi = (int)((long long)all_tiles * (part + 1) / parts);
-  // few tiles: two warps share one, half of the k range each (the parts are added in shared memory in a fixed order)
-  const int ksplit = (tile_hi - tile_lo <= csize * (kRcWarps / 2)) ? 2 : 1, tile_warps = kRcWarps / ksplit;
+  const int tile_lo = WALK ? 0 : (int)((long long)all_tiles * part / parts);
+  const int tile_hi = WALK ? all_tiles : (int)((long long)all_tiles * (part + 1) / parts);
+  // few tiles: two warps share one, half of the k range each (the halves are added in shared memory in a fixed order)
+  const bool halves = (all_tiles + parts - 1) / parts <= csize * (kRcWarps / 2);   // (the same in every part)
+  const int ksplit = halves && !WALK ? 2 : 1, tile_warps = kRcWarps / ksplit;
   const int tw = warp % tile_warps, kpart = warp / tile_warps;
   const int steps_part = (steps + ksplit - 1) / ksplit;
   const int s_lo = kpart * steps_part, s_hi = min(steps, s_lo + steps_part);
   const int nb = (steps_part + kRcBatch - 1) / kRcBatch;   // batches per tile
+  const int second = WALK && halves ? (steps + 1) / 2 : INT_MAX;   // first step of the second half
 
   uint4 a[2][kRcBatch][2];
   auto load = [&](uint4 (&r)[kRcBatch][2], int tl, int b) {
@@ -287,25 +292,35 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
   __syncthreads();
 
   // candidates of this lane: queries j*8 + 2t + e; rows in increasing order, strict '>' keeps the lowest index
-  float best[NJ][2], second[NJ][2];
-  int best_k[NJ][2], second_k[NJ][2];
+  float best[NJ][2], runner[NJ][2];
+  int best_k[NJ][2], runner_k[NJ][2];
 #pragma unroll
   for (int j = 0; j < NJ; ++j)
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      best[j][e] = second[j][e] = -INFINITY;
-      best_k[j][e] = second_k[j][e] = 0;
+      best[j][e] = runner[j][e] = -INFINITY;
+      best_k[j][e] = runner_k[j][e] = 0;
     }
   float acc[NJ][4];
 #pragma unroll
   for (int j = 0; j < NJ; ++j)
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+  float acc0[NJ][4];   // WALK: of the first half
   auto multiply = [&](uint4 (&r)[kRcBatch][2], int b) {
 #pragma unroll
     for (int u = 0; u < kRcBatch; ++u) {
       const int st = s_lo + b * kRcBatch + u;
       if (st >= s_hi) break;
+      if (WALK && st == second) {
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            acc0[j][e] = acc[j][e];
+            acc[j][e] = 0.f;
+          }
+      }
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
         const uint4 bv = *reinterpret_cast<const uint4*>(smem_raw + (size_t)(j * 8 + g) * pitch + st * 64 + t * 16);
@@ -316,12 +331,12 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
   };
   auto take = [&](float sim, int k, int j, int e) {
     if (sim > best[j][e]) {
-      if (TOP2) { second[j][e] = best[j][e]; second_k[j][e] = best_k[j][e]; }
+      if (TOP2) { runner[j][e] = best[j][e]; runner_k[j][e] = best_k[j][e]; }
       best[j][e] = sim;
       best_k[j][e] = k;
-    } else if (TOP2 && sim > second[j][e]) {
-      second[j][e] = sim;
-      second_k[j][e] = k;
+    } else if (TOP2 && sim > runner[j][e]) {
+      runner[j][e] = sim;
+      runner_k[j][e] = k;
     }
   };
   auto finish_tile = [&]() {   // (CTA-uniform trip count when two warps share a tile)
@@ -339,6 +354,12 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[j][e] += s_part[tw][j][e][lane];
       }
+    }
+    if (WALK && second < steps) {
+#pragma unroll
+      for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[j][e] += acc0[j][e];
     }
     if (kpart == 0 && tile < tile_hi) {
       // acc[j][0..1]: centroid r0, queries j*8 + 2t, 2t+1;  acc[j][2..3]: centroid r1
@@ -393,7 +414,7 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
       for (int e = 0; e < 2; ++e) {
         // key 0 = no candidate (zero-norm or padding row, NaN or -inf similarity)
         unsigned long long k1 = best[j][e] > -INFINITY ? route_key(best[j][e], best_k[j][e]) : 0ull;
-        unsigned long long k2 = (TOP2 && second[j][e] > -INFINITY) ? route_key(second[j][e], second_k[j][e]) : 0ull;
+        unsigned long long k2 = (TOP2 && runner[j][e] > -INFINITY) ? route_key(runner[j][e], runner_k[j][e]) : 0ull;
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) {
           const unsigned long long o1 = shfl_xor_u64(k1, o);
@@ -425,7 +446,7 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
       }
     }
     float ss = 0.f;
-    if (on && parts == 1 && (out.best || out.margin))
+    if (on && (parts == 1 || WALK) && (out.best || out.margin))
       for (int ch = sub; ch < nch; ch += 8) add_sq8(*reinterpret_cast<const uint4*>(smem_raw + (size_t)qi * pitch + ch * 16), ss);
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {
@@ -435,7 +456,7 @@ route_cluster_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
       ss += __shfl_xor_sync(0xffffffffu, ss, o);
     }
     if (on && sub == 0) {
-      if (parts > 1) {
+      if (parts > 1 && !WALK) {
         part_keys[(size_t)part * Q + q0 + qi] = k1;
         if (TOP2) part_keys[(size_t)(parts + part) * Q + q0 + qi] = k2;
       } else {
@@ -511,19 +532,13 @@ int route_parts(int Q, int K, int D) {
   const RouteCut r = route_cut(Q, K, D);
   return r.fast ? r.parts : 1;
 }
-// without scratch the table stays in one part
-static RouteCut route_cut_scratch(int Q, int K, int D, const unsigned long long* part_keys) {
-  RouteCut r = route_cut(Q, K, D);
-  if (part_keys == nullptr) r.parts = 1;
-  return r;
-}
-
-template <int NQ, bool TOP2>
+template <int NQ, bool TOP2, bool WALK>
 static cudaError_t launch_rc(int optin, const RouteCut& cut, const __nv_bfloat16* q, const __nv_bfloat16* c,
                              const float* inv_norm, const int* cmap, int Q, int K, int D, const RouteOut& out,
                              unsigned long long* part_keys, cudaStream_t stream) {
   const size_t smem = (size_t)NQ * route_pitch(D);
-  cudaError_t ce = ensure_smem_optin(optin, route_cluster_kernel<NQ, TOP2>, smem > 64 * 1024 ? smem : 64 * 1024);
+  const int clusters = WALK ? 1 : cut.parts;   // per group of queries
+  cudaError_t ce = ensure_smem_optin(optin, route_cluster_kernel<NQ, TOP2, WALK>, smem > 64 * 1024 ? smem : 64 * 1024);
   if (ce != cudaSuccess) return ce;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -532,33 +547,41 @@ static cudaError_t launch_rc(int optin, const RouteCut& cut, const __nv_bfloat16
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(cut.groups * cut.parts * cut.csize));
+  cfg.gridDim = dim3((unsigned)(cut.groups * clusters * cut.csize));
   cfg.blockDim = dim3(kRcWarps * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  ce = cudaLaunchKernelEx(&cfg, route_cluster_kernel<NQ, TOP2>, q, c, inv_norm, cmap, Q, K, D, cut.parts, part_keys, out);
-  if (ce != cudaSuccess || cut.parts == 1) return ce;
+  ce = cudaLaunchKernelEx(&cfg, route_cluster_kernel<NQ, TOP2, WALK>, q, c, inv_norm, cmap, Q, K, D, cut.parts, part_keys, out);
+  if (ce != cudaSuccess || clusters == 1) return ce;
   return launch_pdl(route_parts_kernel<TOP2>, (Q + 15) / 16, 128, 0, stream, part_keys, cut.parts, q, cmap, Q, D, out);
+}
+template <bool TOP2>
+static cudaError_t launch_rc(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm, const int* cmap, int Q,
+                             int K, int D, const RouteOut& out, unsigned long long* part_keys, cudaStream_t stream) {
+  const RouteCut cut = route_cut(Q, K, D);
+  const bool walk = cut.parts > 1 && part_keys == nullptr;
+  const int slot = OPTIN_ROUTE_CLUSTER + 4 * TOP2 + 2 * walk + (cut.nq == 8);
+  if (cut.nq == 32)
+    return walk ? launch_rc<32, TOP2, true>(slot, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream)
+                : launch_rc<32, TOP2, false>(slot, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
+  return walk ? launch_rc<8, TOP2, true>(slot, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream)
+              : launch_rc<8, TOP2, false>(slot, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
 }
 
 cudaError_t launch_route_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                  const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
                                  float* out_best, unsigned long long* part_keys, cudaStream_t stream) {
   const RouteOut out = {out_expert, out_centroid, nullptr, out_best, nullptr};
-  const RouteCut cut = route_cut_scratch(Q, K, D, part_keys);
-  if (cut.nq == 32) return launch_rc<32, false>(OPTIN_ROUTE_CLUSTER, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
-  return launch_rc<8, false>(OPTIN_ROUTE_CLUSTER + 1, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
+  return launch_rc<false>(q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
 }
 cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                       const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
                                       int* out_second, float* out_best, float* out_margin,
                                       unsigned long long* part_keys, cudaStream_t stream) {
   const RouteOut out = {out_expert, out_centroid, out_second, out_best, out_margin};
-  const RouteCut cut = route_cut_scratch(Q, K, D, part_keys);
-  if (cut.nq == 32) return launch_rc<32, true>(OPTIN_ROUTE_CLUSTER + 2, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
-  return launch_rc<8, true>(OPTIN_ROUTE_CLUSTER + 3, cut, q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
+  return launch_rc<true>(q, c, inv_norm, cmap, Q, K, D, out, part_keys, stream);
 }
 
 // ----------------------------------------------------------------------------------------
@@ -814,6 +837,21 @@ route_finish_ids_kernel(const unsigned long long* __restrict__ keys, const int* 
   const int id = (key == 0ull) ? 0 : (int)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
   if (out_centroid) out_centroid[i] = id;
   out_expert[i] = cmap ? cmap[id] : id;
+}
+
+// best[i] / |q_i| for the router without scratch, added up as in route_finish_kernel.
+__global__ void __launch_bounds__(256)
+route_cosine_kernel(const __nv_bfloat16* __restrict__ q, int Q, int D, float* __restrict__ best) {
+  pdl_begin();
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= Q) return;
+  float ss = 0.f;
+  for (int ch = lane; ch < D / 8; ch += 32) add_sq8(ldg_cached(q + (size_t)i * D + ch * 8), ss);
+  ss = warp_sum(ss);
+  if (lane == 0 && best[i] > -INFINITY) best[i] *= rsqrtf(ss);
+}
+cudaError_t launch_route_cosine(const __nv_bfloat16* q, int Q, int D, float* out_best, cudaStream_t stream) {
+  return launch_pdl(route_cosine_kernel, (unsigned)((Q + 7) / 8), 256, 0, stream, q, Q, D, out_best);
 }
 
 cudaError_t launch_route_finish(const unsigned long long* keys, const __nv_bfloat16* q, const int* cmap, int Q, int D,

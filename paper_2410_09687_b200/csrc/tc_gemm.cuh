@@ -49,6 +49,10 @@ moin_status lora_swiglu(HostState* hs, const moin_plan* plan, const moin_lora_jo
 moin_status launch_pair_router(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm, int Q,
                                int K, int D, unsigned long long* keys, cudaStream_t stream,
                                unsigned long long* keys2 = nullptr);   // keys2 != nullptr: also the runner-up
+// Without scratch: the outputs, out_best (nullable, as out_centroid) not yet divided by |q| (launch_route_cosine does).
+moin_status launch_pair_router_rows(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
+                                    const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid, float* out_best,
+                                    cudaStream_t stream);
 // Tile mode: hb = hi/lo bf16 parts of s * x A_e^T per row and run of its GEMM tile ([kTileRuns][2][T][r]); launch_pair_gemm adds hb B_e^T.
 moin_status launch_tc_shrink_group(HostState* hs, const PlanView& pv, const moin_pool* const* pools,
                                    const __nv_bfloat16* const* xs, __nv_bfloat16* const* hbs, int n_jobs, float scale,

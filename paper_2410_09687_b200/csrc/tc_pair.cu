@@ -29,7 +29,8 @@
 namespace moin {
 
 constexpr int kPairThreads = 320, kPairM = 128, kPairK = 64;
-enum { PAIR_STORE = 0, PAIR_ROUTER = 1, PAIR_ROUTER2 = 2, PAIR_SWIGLU = 3 };
+// PAIR_ROUTER_ROWS: a pair takes all column tiles of its rows and so needs no keys to meet in (see launch_pair_router_rows)
+enum { PAIR_STORE = 0, PAIR_ROUTER = 1, PAIR_ROUTER2 = 2, PAIR_SWIGLU = 3, PAIR_ROUTER_ROWS = 4 };
 
 struct PairMaps { CUtensorMap x[kPairJobs], w[kPairJobs], b[kPairJobs], h[kPairJobs], y[kPairJobs]; };
 struct PairParams {
@@ -44,6 +45,9 @@ struct PairParams {
   float* y0[kPairJobs];                  // fp32 copy, nullable (then the rows are written straight from registers)
   const float* inv_norm;                 // PAIR_ROUTER*
   unsigned long long *keys, *keys2;
+  const int* cmap;                       // PAIR_ROUTER_ROWS: outputs, the cosine still to be divided by |q|
+  int *out_expert, *out_centroid;
+  float* out_best;
   DeviceStatus* status;
 };
 
@@ -164,6 +168,12 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
   const int nkb_main = (p.K + kPairK - 1) / kPairK;
   const int nrb = (p.tail_r + kPairK - 1) / kPairK;   // 64-wide blocks of the rank
   const int pair = (int)blockIdx.x >> 1, n_pairs = (int)gridDim.x >> 1;
+  const int tn_all = p.tn_end[p.n_jobs - 1];
+  const int tile_first = EPI == PAIR_ROUTER_ROWS ? pair * tn_all : pair;
+  auto next_tile = [&](int tile) {
+    if (EPI != PAIR_ROUTER_ROWS) return tile + n_pairs;
+    return (tile + 1) % tn_all ? tile + 1 : tile + 1 + (n_pairs - 1) * tn_all;
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -173,7 +183,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       const uint32_t tx_tail = EPI == PAIR_SWIGLU ? (uint32_t)(2 * kPairM + p.bn / 2) * kPairK * 2 : tx;
       uint32_t it = 0, lt = 0;
       bool ok = true;
-      for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
+      for (int tile = tile_first; tile < total && ok; tile = next_tile(tile), ++lt) {
         const PairTile t = pair_tile(p, tile, tiles_m);
         const int row0 = rank == 0 ? t.row0[0] : t.row0[1];
         const CUtensorMap* mx = &maps.x[t.job];
@@ -227,7 +237,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       const bool leader = elect_one();
       uint32_t it = 0, lt = 0;
       bool ok = true;
-      for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
+      for (int tile = tile_first; tile < total && ok; tile = next_tile(tile), ++lt) {
         const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
         if (!(ok = mbar_wait_cluster_warp(tempty0 + 8 * acc, aph ^ 1u, abort_flag, p.status, 62))) break;
         tc_fence_after();
@@ -288,6 +298,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
     const int wh = (warp - 2) >> 2;     // two warps per quarter, every other 64 columns each
     const uint32_t buf = out0 + (uint32_t)(wh * 4 + q) * 4096u;
     uint32_t lt = 0, n_st = 0;
+    unsigned long long row_key = 0ull;   // PAIR_ROUTER_ROWS: of this thread's row, over the column tiles so far
     bool ok = true;
     // Passes of tile i into table i & 1.  The readers of tile i - 2's passes there are through: the MMA warp, whose
     // reads come before the commit of the accumulator that this warp has waited for, and the producer, whose last entries
@@ -300,7 +311,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       return true;
     };
     if (kTail && warp == 2 && p.tail_r > 0 && pair < total) ok = scout(pair_tile(p, pair, tiles_m), 0);
-    for (int tile = pair; tile < total && ok; tile += n_pairs, ++lt) {
+    for (int tile = tile_first; tile < total && ok; tile = next_tile(tile), ++lt) {
       const PairTile t = pair_tile(p, tile, tiles_m);
       if (kTail && warp == 2 && p.tail_r > 0 && tile + n_pairs < total &&
           !(ok = scout(pair_tile(p, tile + n_pairs, tiles_m), lt + 1))) break;
@@ -312,8 +323,9 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       for (int j = 1; j < kPairJobs; ++j)
         if (t.job == j) { n = p.N[j]; y = p.y[j]; y0 = p.y0[j]; }
       const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
-      if (EPI == PAIR_ROUTER || EPI == PAIR_ROUTER2) {   // 1/|c_k| of this warp's columns; NaN where there is no candidate: it loses every maximum
-        const int k0 = t.n0 + wh * (p.bn / 2) + 4 * lane;
+      // 1/|c_k| of the columns of half h; NaN where there is no candidate: it loses every maximum
+      auto stage_norms = [&](int h) {
+        const int k0 = t.n0 + h * (p.bn / 2) + 4 * lane;
         float4 v;
         float* e = reinterpret_cast<float*>(&v);
 #pragma unroll
@@ -321,10 +333,11 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
           const float inv = (4 * lane < p.bn / 2 && k0 + i < n) ? __ldg(p.inv_norm + k0 + i) : 0.f;
           e[i] = inv > 0.f ? inv : __int_as_float(0x7FC00000);
         }
-        __syncwarp();   // the other lanes have read the last tile's values
+        __syncwarp();   // the other lanes have read the last values
         *reinterpret_cast<float4*>(smem_raw + (buf - raw) + 16 * lane) = v;
         __syncwarp();
-      }
+      };
+      if (EPI == PAIR_ROUTER || EPI == PAIR_ROUTER2) stage_norms(wh);
       if (!(ok = mbar_wait_warp(tfull0 + 8 * acc, aph, abort_flag, p.status, 64))) break;
       tc_fence_after();
       const bool row_ok = trow < rows;
@@ -332,6 +345,66 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * kPairMaxN;
       float best = -INFINITY, second = -INFINITY;
       int best_k = 0, second_k = 0;
+      auto release = [&]() {   // the accumulator has been read
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(map_rank(tempty0 + 8 * acc, 0));
+      };
+      auto row_best = [&](int h, bool last) {   // best (and second) score of this thread's row among the columns of half h
+        // The row's (up to) 128 scores go to registers at once, which frees the accumulator; then the maximum (two
+        // columns per instruction) and the first column that holds it.  A running (maximum, index) pair column by
+        // column takes eight instructions a column and bounded the launch: 65536 x 5000 x 768 400 us with 128 x 256 tiles
+        // of single CTAs, 455 us with pairs, now 373 us = 1.35 PFLOP/s, the power limit.
+        uint32_t f[4][32];
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+          if (32 * g < p.bn / 2) tmem_ld32(taddr + h * (p.bn / 2) + 32 * g, f[g]);
+        tmem_ld_wait();
+        if (last) release();
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          if (32 * g < p.bn / 2) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+              const float4 inv = lds_f4(buf + 4u * (32 * g + j));
+              const float f0 = __uint_as_float(f[g][j]) * inv.x, f1 = __uint_as_float(f[g][j + 1]) * inv.y;
+              const float f2 = __uint_as_float(f[g][j + 2]) * inv.z, f3 = __uint_as_float(f[g][j + 3]) * inv.w;
+              best = fmax3(best, fmax3(f0, f1, f2), f3);
+              f[g][j] = __float_as_uint(f0); f[g][j + 1] = __float_as_uint(f1);
+              f[g][j + 2] = __float_as_uint(f2); f[g][j + 3] = __float_as_uint(f3);
+            }
+          }
+        }
+#pragma unroll
+        for (int g = 3; g >= 0; --g) {
+          if (32 * g < p.bn / 2) {
+#pragma unroll
+            for (int j = 31; j >= 0; --j) best_k = (__uint_as_float(f[g][j]) == best) ? 32 * g + j : best_k;   // lowest index wins
+          }
+        }
+        if (EPI == PAIR_ROUTER2) {   // the same once more without the winner
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            if (32 * g < p.bn / 2) {
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) {
+                if (32 * g + j == best_k) f[g][j] = 0x7FC00000u;
+                if (32 * g + j + 1 == best_k) f[g][j + 1] = 0x7FC00000u;
+                second = fmax3(second, __uint_as_float(f[g][j]), __uint_as_float(f[g][j + 1]));
+              }
+            }
+          }
+#pragma unroll
+          for (int g = 3; g >= 0; --g) {
+            if (32 * g < p.bn / 2) {
+#pragma unroll
+              for (int j = 31; j >= 0; --j) second_k = (__uint_as_float(f[g][j]) == second) ? 32 * g + j : second_k;
+            }
+          }
+          second_k += t.n0 + h * (p.bn / 2);
+        }
+        best_k += t.n0 + h * (p.bn / 2);
+      };
       if (EPI == PAIR_STORE || EPI == PAIR_SWIGLU) {
         // Full 32-row groups leave through shared memory (128-byte swizzled rows) as tiled stores of whole lines: a
         // warp's 16-byte pieces straight from registers are 32 partial-line requests per instruction, beside the
@@ -396,67 +469,37 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
             ++n_st;
           }
         }
-      } else {
-        // The row's (up to) 128 scores go to registers at once, which frees the accumulator; then the maximum (two
-        // columns per instruction) and the first column that holds it.  A running (maximum, index) pair column by
-        // column takes eight instructions a column and bounded the launch: 65536 x 5000 x 768 400 us with 128 x 256 tiles
-        // of single CTAs, 455 us with pairs, now 373 us = 1.35 PFLOP/s, the power limit.
-        uint32_t f[4][32];
-#pragma unroll
-        for (int g = 0; g < 4; ++g)
-          if (32 * g < p.bn / 2) tmem_ld32(taddr + wh * (p.bn / 2) + 32 * g, f[g]);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_rank(tempty0 + 8 * acc, 0));
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          if (32 * g < p.bn / 2) {
-#pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-              const float4 inv = lds_f4(buf + 4u * (32 * g + j));
-              const float f0 = __uint_as_float(f[g][j]) * inv.x, f1 = __uint_as_float(f[g][j + 1]) * inv.y;
-              const float f2 = __uint_as_float(f[g][j + 2]) * inv.z, f3 = __uint_as_float(f[g][j + 3]) * inv.w;
-              best = fmax3(best, fmax3(f0, f1, f2), f3);
-              f[g][j] = __float_as_uint(f0); f[g][j + 1] = __float_as_uint(f1);
-              f[g][j + 2] = __float_as_uint(f2); f[g][j + 3] = __float_as_uint(f3);
-            }
-          }
-        }
-#pragma unroll
-        for (int g = 3; g >= 0; --g) {
-          if (32 * g < p.bn / 2) {
-#pragma unroll
-            for (int j = 31; j >= 0; --j) best_k = (__uint_as_float(f[g][j]) == best) ? 32 * g + j : best_k;   // lowest index wins
-          }
-        }
-        if (EPI == PAIR_ROUTER2) {   // the same once more without the winner
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            if (32 * g < p.bn / 2) {
-#pragma unroll
-              for (int j = 0; j < 32; j += 2) {
-                if (32 * g + j == best_k) f[g][j] = 0x7FC00000u;
-                if (32 * g + j + 1 == best_k) f[g][j + 1] = 0x7FC00000u;
-                second = fmax3(second, __uint_as_float(f[g][j]), __uint_as_float(f[g][j + 1]));
-              }
-            }
-          }
-#pragma unroll
-          for (int g = 3; g >= 0; --g) {
-            if (32 * g < p.bn / 2) {
-#pragma unroll
-              for (int j = 31; j >= 0; --j) second_k = (__uint_as_float(f[g][j]) == second) ? 32 * g + j : second_k;
-            }
-          }
-          second_k += t.n0 + wh * (p.bn / 2);
-        }
-        best_k += t.n0 + wh * (p.bn / 2);
       }
-      if (EPI == PAIR_STORE || EPI == PAIR_SWIGLU) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_rank(tempty0 + 8 * acc, 0));
+      if (EPI == PAIR_STORE || EPI == PAIR_SWIGLU) release();
+      if (EPI == PAIR_ROUTER || EPI == PAIR_ROUTER2) row_best(wh, true);
+      if (EPI == PAIR_ROUTER_ROWS) {   // both halves by one warp, whose keys stay in registers
+        if (wh != 0) {
+          release();
+          continue;
+        }
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          stage_norms(h);
+          best = -INFINITY;
+          best_k = 0;
+          row_best(h, h == 1);
+          if (best > -INFINITY) {
+            const unsigned long long key =
+                ((unsigned long long)pair_orderable(best) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k);
+            row_key = key > row_key ? key : row_key;
+          }
+        }
+        if ((tile + 1) % tn_all == 0) {
+          if (row_ok) {
+            const int id = row_key == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)(row_key & 0xFFFFFFFFull));
+            const uint32_t u = (uint32_t)(row_key >> 32);
+            if (p.out_centroid) p.out_centroid[grow] = id;
+            p.out_expert[grow] = p.cmap ? p.cmap[id] : id;
+            if (p.out_best)
+              p.out_best[grow] = row_key == 0ull ? -INFINITY : __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u);
+          }
+          row_key = 0ull;
+        }
       }
       if (EPI == PAIR_ROUTER && row_ok && best > -INFINITY)
         atomicMax(p.keys + grow, ((unsigned long long)pair_orderable(best) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k));
@@ -613,6 +656,25 @@ moin_status launch_pair_router(HostState* hs, const __nv_bfloat16* q, const __nv
   const long tiles = (tiles_m + 1) / 2 * p.tn_end[0];
   if (keys2 != nullptr) return launch_pair<PAIR_ROUTER2>(hs, maps, p, tiles, stream);
   return launch_pair<PAIR_ROUTER>(hs, maps, p, tiles, stream);
+}
+
+// The same without scratch: outputs written by the pair, except that out_best still lacks the division by |q|.  For few
+// queries only, as a pair then walks the table alone (the keys' way has a clearing and a finishing launch and more SMs:
+// 400 x 500 x 768 8.8 us with keys, 13.3 without, 1024 x 1000 x 768 9.9 and 20.6; the cluster kernel in waves 10 and 37).
+// The scores and their order of merging are those of launch_pair_router, and so are the results, to the bit.
+moin_status launch_pair_router_rows(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
+                                    const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid, float* out_best,
+                                    cudaStream_t stream) {
+  PairMaps maps;
+  PairParams p = {};
+  p.M = Q; p.K = D; p.n_jobs = 1; p.status = hs->status; p.inv_norm = inv_norm;
+  p.bn = p.cols = K > 192 ? 256 : (K + 63) / 64 * 64;
+  p.N[0] = K; p.tn_end[0] = (K + p.bn - 1) / p.bn;
+  p.cmap = cmap; p.out_expert = out_expert; p.out_centroid = out_centroid; p.out_best = out_best;
+  moin_status st = make_map(&maps.x[0], q, Q, D, kPairM);
+  if (!st) st = make_map(&maps.w[0], c, K, D, p.bn / 2);
+  if (st) return st;
+  return launch_pair<PAIR_ROUTER_ROWS>(hs, maps, p, (Q + 2 * kPairM - 1) / (2 * kPairM), stream);
 }
 
 }  // namespace moin
