@@ -138,6 +138,7 @@ typedef struct {
 /* Fills inv_norm[K] (fp32, device) from centroids[K, D].  Once per centroid table. */
 moin_status moin_router_prepare(const void* centroids, int32_t K, int32_t D, float* inv_norm, moin_stream stream);
 
+/* Enough for Q queries and for any smaller batch. */
 size_t moin_route_workspace_bytes(int32_t Q, int32_t K, int32_t D);
 /* queries [Q, D] bf16 -> out_expert[Q] (int32: centroid_to_expert[id] if the map is given, else id),
  * out_centroid[Q] (nullable, int32 id), out_best_sim[Q] (nullable, fp32 cosine of the winner).
@@ -154,7 +155,8 @@ moin_status moin_route(const moin_router* router, const void* queries, int32_t Q
  * moin_route, plus
  *   out_second  [Q] int32, nullable: centroid index of the second-best similarity, -1 if there is none
  *   out_margin  [Q] fp32,  nullable: cos(best) - cos(second), +inf if there is no second candidate
- * out_expert and out_centroid may be NULL here.  Workspace: moin_route_top2_workspace_bytes. */
+ * out_expert and out_centroid may be NULL here.  Workspace: moin_route_top2_workspace_bytes (as above, also for any
+ * smaller batch). */
 size_t moin_route_top2_workspace_bytes(int32_t Q, int32_t K, int32_t D);
 moin_status moin_route_top2(const moin_router* router, const void* queries, int32_t Q, int32_t* out_expert,
                             int32_t* out_centroid, int32_t* out_second, float* out_best_sim, float* out_margin,

@@ -203,9 +203,18 @@ moin_status moin_router_prepare(const void* centroids, int32_t K, int32_t D, flo
   return record_cuda(launch_inv_norm((const __nv_bfloat16*)centroids, K, D, inv_norm, (cudaStream_t)stream));
 }
 
+// What one call needs, and what covers every smaller batch too (a few queries over a table cut into parts need more keys
+// than many over an uncut one).
+static size_t route_need(int Q, int K, int D) {
+  return align_up((size_t)Q * (size_t)route_parts(Q, K, D) * sizeof(unsigned long long), 256);
+}
+static size_t route_cover(int Q) {
+  return align_up((size_t)(Q > kRouteMaxPartKeys ? Q : kRouteMaxPartKeys) * sizeof(unsigned long long), 256);
+}
+
 size_t moin_route_workspace_bytes(int32_t Q, int32_t K, int32_t D) {
-  if (Q <= 0) return 256;
-  return align_up((size_t)Q * (size_t)route_parts(Q, K, D) * sizeof(unsigned long long), 256) + 256;
+  (void)K; (void)D;
+  return Q <= 0 ? 256 : route_cover(Q) + 256;
 }
 
 // Kernel choice shared by moin_route and moin_route_static, so that both compute the same values for the same
@@ -289,7 +298,7 @@ moin_status moin_route(const moin_router* router, const void* queries, int32_t Q
   int choice;
   if ((st = route_choice(hs, Q, router->K, router->D, &choice))) return st;
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(workspace);
-  if (!workspace || workspace_bytes < moin_route_workspace_bytes(Q, router->K, router->D) || !aligned16(workspace)) {
+  if (!workspace || workspace_bytes < route_need(Q, router->K, router->D) + 256 || !aligned16(workspace)) {
     keys = nullptr;
     if (!route_without_scratch(hs, choice, Q, router->K, router->D)) return MOIN_ERR_WORKSPACE;
   }
@@ -297,8 +306,8 @@ moin_status moin_route(const moin_router* router, const void* queries, int32_t Q
 }
 
 size_t moin_route_top2_workspace_bytes(int32_t Q, int32_t K, int32_t D) {
-  if (Q <= 0) return 256;
-  return 2 * align_up((size_t)Q * (size_t)route_parts(Q, K, D) * sizeof(unsigned long long), 256) + 256;
+  (void)K; (void)D;
+  return Q <= 0 ? 256 : 2 * route_cover(Q) + 256;
 }
 
 moin_status moin_route_top2(const moin_router* router, const void* queries, int32_t Q, int32_t* out_expert,
@@ -321,7 +330,7 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
     if (!tc_ok) return MOIN_ERR_BAD_SHAPE;
     use_tc = true;
   }
-  const bool fits = workspace && workspace_bytes >= moin_route_top2_workspace_bytes(Q, K, D) && aligned16(workspace);
+  const bool fits = workspace && workspace_bytes >= 2 * route_need(Q, K, D) + 256 && aligned16(workspace);
   if (use_tc && !fits && !(hs->gemm_impl == 0 && route_cluster_supported(Q, K, D))) {
     if (hs->gemm_impl == 2 || (long long)Q * K >= (1ll << 16)) return MOIN_ERR_WORKSPACE;
     use_tc = false;

@@ -231,6 +231,7 @@ cudaError_t launch_route_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c,
 // Parts the cluster kernel cuts the table into: a cluster each, given route_parts(Q, K, D) * Q keys of scratch (top-2:
 // twice as many); with part_keys == nullptr one cluster walks them all, with the same results to the bit.
 constexpr int kRouteMaxParts = 12;
+constexpr int kRouteMaxPartKeys = 12 * 32;   // queries x parts where there is more than one: at most 12 clusters of up to 32 queries
 int route_parts(int Q, int K, int D);
 cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                       const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,

@@ -517,7 +517,7 @@ static RouteCut route_cut(int Q, int K, int D) {
   // One tile per warp pair of a cluster of 8 = 512 centroids per part, while all clusters are resident at once: a
   // cluster of 8 one-per-SM CTAs needs 8 free SMs of one GPC, and 16 of them take two waves (500 centroids x 768,
   // 256 queries = 8 clusters 9.8 us, 512 queries = 16 clusters 18.4 us).
-  constexpr int kResident = 12;
+  constexpr int kResident = kRouteMaxPartKeys / 32;
   while (r.parts < kRouteMaxParts && K > 512 * r.parts && r.groups * (r.parts + 1) <= kResident) ++r.parts;
   const int tiles = (K + 512 * r.parts - 1) / (512 * r.parts);   // tiles per warp pair
   // Against the tensor-core GEMM with its clearing and finishing launches (11.8 us up to 128 queries, 14.4 at 256 x
