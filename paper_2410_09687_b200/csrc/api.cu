@@ -500,8 +500,8 @@ size_t moin_lora_linear_workspace_bytes(int32_t T, int32_t d_in, int32_t d_out, 
   (void)d_in;
   size_t seg = align_up((size_t)T * (size_t)(r > 0 ? r : 8) * sizeof(float), 256) +
                align_up((size_t)T * (size_t)d_out * sizeof(float), 256);
-  // hi and lo parts of s * (x A^T), under each of the runs of a row tile
-  size_t tiles = align_up(2 * kTileRuns * Tp * (size_t)(r > 64 ? r : 64) * sizeof(__nv_bfloat16), 256);
+  // hi and lo parts of s * (x A^T)
+  size_t tiles = align_up(2 * Tp * (size_t)(r > 64 ? r : 64) * sizeof(__nv_bfloat16), 256);
   return (seg > tiles ? seg : tiles) + 256;
 }
 

@@ -45,7 +45,6 @@ struct PlanView {   // pointers into the plan buffer
   int* run_row0;     // [T + 1] their first rows
   int* grid_run;     // [grid tiles] run of the grid tile's first row
   int* grid_nrun;    // [grid tiles] runs in it
-  int* tile_run;     // [T]   run of row tile i
   int* rank;         // [T]   scratch
   int* key;          // [T]   scratch
   int* keybase;      // [E+1] scratch
@@ -79,7 +78,6 @@ inline PlanView plan_view(void* buffer, int T, int E, size_t* total_words = null
   v.run_row0 = take(T + 2);
   v.grid_run = take(T / kTileRows + 2);
   v.grid_nrun = take(T / kTileRows + 2);
-  v.tile_run = take(T + 1);
   v.rank = take(T);
   v.key = take(T);
   v.keybase = take(E + 2);

@@ -250,7 +250,6 @@ __device__ __forceinline__ void plan_tiles(const PlanView& v, const int* key, in
         prev = k[i];
         if ((t + i) % kTileRows == 0) v.grid_run[(t + i) / kTileRows] = ord - 1;
         if (((t + i - rs) % kTileRows) == 0) {
-          v.tile_run[idx] = ord - 1;
           v.tile_row0[idx] = t + i;
           if (row0 != v.tile_row0) row0[idx] = t + i;
           v.tile_expert[idx] = (k[i] == E) ? -1 : k[i];

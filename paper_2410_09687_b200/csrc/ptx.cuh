@@ -226,6 +226,14 @@ __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t tmem_d, uint64_t adesc
   asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
                ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
 }
+// accumulates; accumulator rows whose bit is set in `out` (256 rows, the first CTA's first) stay as they are
+__device__ __forceinline__ void tc_mma_bf16_pair_rows(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                      const uint32_t (&out)[8]) {
+  asm volatile("{\n .reg .pred p;\n setp.eq.b32 p, 0, 0;\n"
+               " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, {%4, %5, %6, %7, %8, %9, %10, %11}, p;\n}\n"
+               ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(out[0]), "r"(out[1]), "r"(out[2]), "r"(out[3]),
+                 "r"(out[4]), "r"(out[5]), "r"(out[6]), "r"(out[7]) : "memory");
+}
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "

@@ -33,7 +33,7 @@ inline bool decode_fp8_supported(const HostState* hs, int T) { return hs->gemm_i
 moin_status lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, const float* const* w_scale, int n_jobs,
                               float scale, void* workspace, size_t workspace_bytes, moin_stream stream);
 // Long-run GEMMs on CTA pairs (tc_pair.cu): y_j = x_j W_j^T for up to kPairJobs projections of one K; with a plan the
-// low-rank term s x A_e^T B_e^T is added from hb (hi / lo parts of s x A_e^T, [kTileRuns][2][M][r], all jobs of the same r).
+// low-rank term s x A_e^T B_e^T is added from hb (hi / lo parts of s x A_e^T, [2][M][r], all jobs of the same r).
 constexpr int kPairJobs = 3;
 struct PairJob { const __nv_bfloat16 *x, *W, *hb; __nv_bfloat16* y; float* y0; const moin_pool* pool; int N; };   // y0: fp32 copy or nullptr
 moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* jobs, int n_jobs, int M, int K,
@@ -53,7 +53,7 @@ moin_status launch_pair_router(HostState* hs, const __nv_bfloat16* q, const __nv
 moin_status launch_pair_router_rows(HostState* hs, const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                     const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid, float* out_best,
                                     cudaStream_t stream);
-// Tile mode: hb = hi/lo bf16 parts of s * x A_e^T per row and run of its GEMM tile ([kTileRuns][2][T][r]); launch_pair_gemm adds hb B_e^T.
+// Tile mode: hb = hi/lo bf16 parts of s * x A_e^T ([2][T][r]); launch_pair_gemm adds hb B_e^T.
 moin_status launch_tc_shrink_group(HostState* hs, const PlanView& pv, const moin_pool* const* pools,
                                    const __nv_bfloat16* const* xs, __nv_bfloat16* const* hbs, int n_jobs, float scale,
                                    cudaStream_t stream);

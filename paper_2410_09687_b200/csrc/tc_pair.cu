@@ -12,9 +12,9 @@
 //
 // Row tiles are the regular grid of 128 rows, also with a batch plan: a tile may hold up to kTileRuns runs of one expert
 // (the plan cuts a grid tile of more).  With adapters every tile ends with extra K blocks [hi(s h) | lo(s h)] x
-// [B_e ; B_e], one pass per run, that add the low-rank term inside the accumulator; the rows of the other runs are zero in
-// a pass (the shrink writes h under the number of a row's run in its tile and zeros under the others), and so are those of
-// a CTA that has no row of the run (a copy that starts past the last row fills zeros).  Tiles that began anew with each
+// [B_e ; B_e], one pass per run, that add the low-rank term inside the accumulator; a pass's MMAs leave out the
+// accumulator rows of the other runs (disable-output-lane), whatever lies in their h and whatever B_e holds: an adapter
+// with an infinity or a NaN in it spoils the rows of its own run only.  Tiles that began anew with each
 // run instead multiplied up to a fifth of padding: 11 prompts of 65 to 600 tokens, forward 10.34 -> 8.98 ms; nine, a
 // block's projections 464 -> 400 us.
 //
@@ -36,7 +36,7 @@ struct PairMaps { CUtensorMap x[kPairJobs], w[kPairJobs], b[kPairJobs], h[kPairJ
 struct PairParams {
   int M, K, n_jobs, bn, cols;            // bn: tile width, a multiple of 16 up to 256; cols: output columns of it
   int N[kPairJobs], tn_end[kPairJobs];   // columns, column tiles of jobs 0 .. j
-  const int *header, *run_expert;        // plan (header == nullptr: regular grid over M, no runs)
+  const int *header, *run_expert, *run_row0;   // plan (header == nullptr: regular grid over M, no runs)
   const int4* gemm_tab;
   int tail_r;                            // stored rank of the appended low-rank blocks (0 = none)
   const int* slot_of_expert[kPairJobs];
@@ -94,26 +94,37 @@ __device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int
 // pass i (SWIGLU: lanes 8 .. 15 for the up projection), and leaves the result in shared memory.  (In the producer and the
 // MMA warp themselves, at the start of a tile or in steps between the quarters of its main loop, it cost 2 to 5 percent.)
 constexpr int kPairPasses = 2 * kTileRuns;
-struct PairPass { int slot, rank, run[2]; };   // adapter or -1; per CTA the number under which hb has the run's rows or -1
+struct PairPass { int slot, rank, rows[2]; };   // adapter or -1; per CTA the run's rows of the tile: first | end << 16
 constexpr uint32_t kPairTabBytes = 2 * kPairPasses * sizeof(PairPass) + 16;   // passes, then their number
 __device__ __forceinline__ void pair_passes(const PairParams& p, const PairTile& t, bool two_jobs, int lane, uint8_t* tab) {
   const int shared = t.n_run[0] > 0 && t.n_run[1] > 0 && t.run0[0] + t.n_run[0] - 1 == t.run0[1];
   const int n = t.n_run[0] + t.n_run[1] - shared;
   const int i = lane % kPairPasses, job = two_jobs ? lane / kPairPasses : t.job;
   if (lane < (two_jobs ? 2 : 1) * kPairPasses && i < n) {
-    const int k1 = i - t.n_run[0] + shared;   // run of the second CTA's rows
-    PairPass q = {-1, p.tail_r, {i < t.n_run[0] ? i : -1, k1 >= 0 ? k1 : -1}};
+    const int run = i < t.n_run[0] ? t.run0[0] + i : t.run0[1] + i - t.n_run[0] + shared;
+    const int r0 = __ldg(p.run_row0 + run), r1 = __ldg(p.run_row0 + run + 1);
+    PairPass q = {-1, p.tail_r, {0, 0}};
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      q.rows[c] = min(max(r0 - t.row0[c], 0), t.rows[c]) | min(max(r1 - t.row0[c], 0), t.rows[c]) << 16;
     const int* slots = p.slot_of_expert[0];
     const int* ranks = p.slot_rank[0];
 #pragma unroll
     for (int j = 1; j < kPairJobs; ++j)
       if (job == j) { slots = p.slot_of_expert[j]; ranks = p.slot_rank[j]; }
-    const int e = __ldg(p.run_expert + (i < t.n_run[0] ? t.run0[0] + i : t.run0[1] + k1));
+    const int e = __ldg(p.run_expert + run);
     if (e >= 0) q.slot = __ldg(slots + e);
     if (q.slot >= 0 && ranks) q.rank = min(__ldg(ranks + q.slot), p.tail_r);
     reinterpret_cast<PairPass*>(tab)[lane] = q;
   }
   if (lane == 0) *reinterpret_cast<int*>(tab + 2 * kPairPasses * sizeof(PairPass)) = n;
+}
+
+// disable-output-lane word of 32 accumulator rows of which first .. end - 1 (counted from the word's first row) take part
+__device__ __forceinline__ uint32_t lanes_out(int first, int end) {
+  const uint32_t below_end = end <= 0 ? 0u : end >= 32 ? ~0u : (1u << end) - 1u;
+  const uint32_t below_first = first <= 0 ? 0u : first >= 32 ? ~0u : (1u << first) - 1u;
+  return ~(below_end & ~below_first);
 }
 
 template <int EPI>
@@ -209,7 +220,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
           for (int jj = 1; jj < kPairJobs; ++jj)
             if (job == jj) n = p.N[jj];
           for (int i = 0; i < n_pass && ok; ++i) {
-            const int slot = pass[i].slot, run = pass[i].run[rank];
+            const int slot = pass[i].slot;
             if (slot < 0) continue;
             const int b0 = slot * n + t.n0 + (int)rank * (p.cols / 2);
             for (int j = 0; j < 2 * nrb; ++j, ++it) {
@@ -219,9 +230,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
               const uint32_t bar = map_rank(full0 + 8 * s, 0);
               if (rank == 0) mbar_expect_tx(full0 + 8 * s, tx_tail);
               const int lo = j >= nrb ? 1 : 0, rb = j - lo * nrb;   // hi blocks first, then lo blocks
-              // rows of the run under its number; a CTA without rows of it starts past the last row: zeros
-              const int h0 = run >= 0 ? (2 * run + lo) * p.M + row0 : 2 * kTileRuns * p.M;
-              tma_load_2d_pair(sa, &maps.h[job], bar, rb * kPairK, h0);
+              tma_load_2d_pair(sa, &maps.h[job], bar, rb * kPairK, lo * p.M + row0);   // (all rows: the MMAs choose)
               tma_load_2d_pair(sb, &maps.b[job], bar, rb * kPairK, b0);
             }
           }
@@ -270,6 +279,12 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
             for (int i = 0; i < n_pass && ok; ++i) {
               const int slot = pass[i].slot, rk = pass[i].rank;
               if (slot < 0) continue;
+              uint32_t out[8];   // rows of the other runs, first CTA's then second's
+#pragma unroll
+              for (int w = 0; w < 8; ++w) {
+                const int rows = pass[i].rows[w >> 2];
+                out[w] = lanes_out((rows & 0xFFFF) - 32 * (w & 3), (rows >> 16) - 32 * (w & 3));
+              }
               for (int j = 0; j < 2 * nrb; ++j, ++it) {
                 const uint32_t s = it % S, ph = (it / S) & 1u;
                 if (!(ok = mbar_wait_cluster_warp(full0 + 8 * s, ph, abort_flag, p.status, 63))) break;
@@ -280,7 +295,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
                 const int nk16 = (min(kPairK, rk - rb * kPairK) + 15) / 16;   // beyond the rank: no MMA
                 if (leader) {
                   for (int k = 0; k < nk16; ++k)
-                    tc_mma_bf16_pair(tmem_g, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc_tail, 1u);
+                    tc_mma_bf16_pair_rows(tmem_g, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc_tail, out);
                   tc_commit_pair(empty0 + 8 * s);
                 }
               }
@@ -581,7 +596,7 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
   PairParams p = {};
   p.M = M; p.K = K; p.n_jobs = n_jobs; p.bn = p.cols = bn; p.status = hs->status;
   if (pv) {
-    p.header = pv->header; p.gemm_tab = pv->gemm_tab; p.run_expert = pv->run_expert;
+    p.header = pv->header; p.gemm_tab = pv->gemm_tab; p.run_expert = pv->run_expert; p.run_row0 = pv->run_row0;
     p.tail_r = jobs[0].pool->r;
   }
   int tn = 0;
@@ -592,7 +607,7 @@ moin_status launch_pair_gemm(HostState* hs, const PlanView* pv, const PairJob* j
     if (!st) st = make_map(&maps.y[j], g.y, M, g.N, 32);
     if (!st && pv) {
       const int r = g.pool->r;
-      st = make_map(&maps.h[j], g.hb, 2ull * kTileRuns * M, r, kPairM);
+      st = make_map(&maps.h[j], g.hb, 2ull * M, r, kPairM);
       if (!st) st = make_map(&maps.b[j], g.pool->B, (uint64_t)g.pool->n_slots * g.N, r, bn / 2);
       p.slot_of_expert[j] = g.pool->slot_of_expert;
       p.slot_rank[j] = g.pool->slot_rank;
@@ -624,7 +639,7 @@ moin_status launch_pair_swiglu(HostState* hs, const PlanView* pv, const PairJob*
   moin_status st = make_map(&maps.x[0], jobs[0].x, M, K, kPairM);
   if (!st) st = make_map(&maps.y[0], jobs[0].y, M, F, 32);
   if (pv) {
-    p.header = pv->header; p.gemm_tab = pv->gemm_tab; p.run_expert = pv->run_expert;
+    p.header = pv->header; p.gemm_tab = pv->gemm_tab; p.run_expert = pv->run_expert; p.run_row0 = pv->run_row0;
     p.tail_r = jobs[0].pool->r;
   }
   for (int j = 0; j < 2 && !st; ++j) {
@@ -632,7 +647,7 @@ moin_status launch_pair_swiglu(HostState* hs, const PlanView* pv, const PairJob*
     st = make_map(&maps.w[j], g.W, F, K, p.cols);
     if (!st && pv) {
       const int r = g.pool->r;
-      st = make_map(&maps.h[j], g.hb, 2ull * kTileRuns * M, r, kPairM);
+      st = make_map(&maps.h[j], g.hb, 2ull * M, r, kPairM);
       if (!st) st = make_map(&maps.b[j], g.pool->B, (uint64_t)g.pool->n_slots * F, r, p.cols / 2);
       p.slot_of_expert[j] = g.pool->slot_of_expert;
       p.slot_rank[j] = g.pool->slot_rank;

@@ -25,10 +25,10 @@ struct TsMaps { CUtensorMap x, a[kTcMaxShrinkJobs]; };
 struct TsParams {
   int T, K, r, n_jobs, N;                   // N: the jobs' ranks together, a multiple of 16
   int stages, stage_bytes, tmem_cols, ks;
-  const int *header, *tile_row0, *tile_rows, *tile_expert, *tile_run, *grid_run, *grid_nrun;
+  const int *header, *tile_row0, *tile_rows, *tile_expert;
   const int* slot_of_expert[kTcMaxShrinkJobs];
   const int* slot_rank[kTcMaxShrinkJobs];   // nullable: the stored rank
-  __nv_bfloat16* hb[kTcMaxShrinkJobs];      // [kTileRuns][2][T][r]: hi, lo of a row, under the number of its run in its GEMM tile
+  __nv_bfloat16* hb[kTcMaxShrinkJobs];      // [2][T][r]: hi, lo (rows without an adapter are not written)
   int act;
   float scale;
   DeviceStatus* status;
@@ -82,9 +82,6 @@ tc_shrink_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__ Ts
   bool ok = true;
   for (int tm = cluster; tm < total; tm += n_clusters) {
     const int row0 = __ldg(p.tile_row0 + tm), rows = __ldg(p.tile_rows + tm), e = __ldg(p.tile_expert + tm);
-    // its rows lie in one or two GEMM grid tiles: how many runs the GEMM tile there has, and which of them this one is
-    const int tile_run = __ldg(p.tile_run + tm), g0 = row0 / kTileRows, g1 = (row0 + rows - 1) / kTileRows;
-    const int first[2] = {__ldg(p.grid_run + g0), __ldg(p.grid_run + g1)}, runs[2] = {__ldg(p.grid_nrun + g0), __ldg(p.grid_nrun + g1)};
     int slot[kTcMaxShrinkJobs];
     bool any = false;
 #pragma unroll
@@ -159,20 +156,7 @@ tc_shrink_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__ Ts
 #pragma unroll
       for (int jj = 1; jj < kTcMaxShrinkJobs; ++jj)
         if (j == jj) { sl = slot[jj]; ranks = p.slot_rank[jj]; hb = p.hb[jj]; }
-      if (row >= rows || *abort_flag) continue;
-      // The GEMM's tile multiplies its runs one after the other, each under its own number: this row's values under the
-      // number of its run, zeros under the others of the tile.
-      const bool g = row0 + row >= g1 * kTileRows;
-      const int in_grid = tile_run - (g ? first[1] : first[0]), my_run = in_grid % kTileRuns;
-      const int n_run = min(kTileRuns, (g ? runs[1] : runs[0]) - (in_grid - my_run));
-      __nv_bfloat16* dst = hb + (size_t)(row0 + row) * (size_t)p.r + cj;
-      const size_t part = (size_t)p.T * (size_t)p.r;
-      for (int k = 0; k < n_run; ++k)
-        if (k != my_run) {
-          *reinterpret_cast<uint4*>(dst + 2 * k * part) = make_uint4(0u, 0u, 0u, 0u);
-          *reinterpret_cast<uint4*>(dst + (2 * k + 1) * part) = make_uint4(0u, 0u, 0u, 0u);
-        }
-      if (sl < 0) continue;
+      if (row >= rows || sl < 0 || *abort_flag) continue;
       const int r_use = ranks ? min(__ldg(ranks + sl), p.r) : p.r;
       const uint32_t off = (uint32_t)(row * pitch + c8 * 8) * 4u;
       float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -200,8 +184,9 @@ tc_shrink_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__ Ts
       l.y = pack_bf16(f[2] - bf16_lo(h.y), f[3] - bf16_hi(h.y));
       l.z = pack_bf16(f[4] - bf16_lo(h.z), f[5] - bf16_hi(h.z));
       l.w = pack_bf16(f[6] - bf16_lo(h.w), f[7] - bf16_hi(h.w));
-      *reinterpret_cast<uint4*>(dst + 2 * my_run * part) = h;
-      *reinterpret_cast<uint4*>(dst + (2 * my_run + 1) * part) = l;
+      __nv_bfloat16* dst = hb + (size_t)(row0 + row) * (size_t)p.r + cj;
+      *reinterpret_cast<uint4*>(dst) = h;
+      *reinterpret_cast<uint4*>(dst + (size_t)p.T * (size_t)p.r) = l;
     }
     if (any) {   // the parts have been read everywhere: the next item's copies may overwrite them
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -229,7 +214,6 @@ static moin_status launch_set(HostState* hs, const PlanView& pv, const moin_pool
   p.T = T; p.K = K; p.r = r; p.n_jobs = n_jobs; p.N = (n_jobs * r + 15) / 16 * 16;
   p.scale = scale; p.act = pools[0]->activation; p.status = hs->status;
   p.header = pv.header; p.tile_row0 = pv.tile_row0; p.tile_rows = pv.tile_rows; p.tile_expert = pv.tile_expert;
-  p.tile_run = pv.tile_run; p.grid_run = pv.grid_run; p.grid_nrun = pv.grid_nrun;
   moin_status st = make_map(&maps.x, x, T, K, kTsM);
   for (int j = 0; j < n_jobs && !st; ++j) {
     st = make_map(&maps.a[j], pools[j]->A, (uint64_t)pools[j]->n_slots * r, K, r);   // one slot's rows
