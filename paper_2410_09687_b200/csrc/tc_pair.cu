@@ -447,8 +447,8 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
                 const uint32_t gw = pack_bf16(__uint_as_float(v[j]), __uint_as_float(v[j + 1]));
                 const uint32_t uw = pack_bf16(__uint_as_float(u[j]), __uint_as_float(u[j + 1]));
                 const float g0 = bf16_lo(gw), g1 = bf16_hi(gw);
-                v[j] = __float_as_uint(__fdividef(g0, 1.f + __expf(-g0)) * bf16_lo(uw));
-                v[j + 1] = __float_as_uint(__fdividef(g1, 1.f + __expf(-g1)) * bf16_hi(uw));
+                v[j] = __float_as_uint(g0 / (1.f + __expf(-g0)) * bf16_lo(uw));
+                v[j + 1] = __float_as_uint(g1 / (1.f + __expf(-g1)) * bf16_hi(uw));
               }
             } else {
               tmem_ld_wait();
