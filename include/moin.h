@@ -144,7 +144,8 @@ size_t moin_route_workspace_bytes(int32_t Q, int32_t K, int32_t D);
  * out_centroid[Q] (nullable, int32 id), out_best_sim[Q] (nullable, fp32 cosine of the winner).
  * Q == 0 is a no-op.  Workspace contents are scratch, also for a single query (the keys of a table cut into parts):
  * calls that may overlap on the GPU - on two streams, or captured in two graphs - need a workspace each.  Without one
- * (NULL, or too small) small problems are served all the same, some of them slower (see moin_route_static for which). */
+ * (NULL, or too small) small problems are served all the same, some of them slower: those that moin_route_static names,
+ * and a few hundred queries against any table. */
 moin_status moin_route(const moin_router* router, const void* queries, int32_t Q, int32_t* out_expert,
                        int32_t* out_centroid, float* out_best_sim, void* workspace, size_t workspace_bytes,
                        moin_stream stream);
@@ -167,19 +168,19 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
  * serving worker whose memory pool was sized and frozen at start-up, or a plug-in that runs inside
  * someone else's CUDA context and is forbidden to call cudaMalloc.)
  *
- * It computes what moin_route computes - same arguments minus the workspace, same ids and the same cosines.  What
- * moin_route serves without scratch (a workspace of NULL) is served without it here too: a few hundred queries, up to
- * 1024 queries against up to 1024 topics of up to 3168 dimensions, and problems of fewer than 65 536 query-topic
- * products.  For larger ones the per-query scratch of the tensor-core router lives in a fixed array inside the library
- * image (MOIN_ROUTE_STATIC_MAX_Q * 8 bytes = 512 KiB, held by every GPU that loads the library until the process exits),
- * which the others do not touch.  The call performs no cudaMalloc/cudaFree and calls no allocating routine.
+ * It computes what moin_route computes - same arguments minus the workspace, same ids and the same cosines.  Small
+ * problems - up to 1024 queries against up to 1024 topics of up to 3168 dimensions, and those of fewer than 65 536
+ * query-topic products - are served without scratch, as by moin_route with a workspace of NULL.  For larger ones the
+ * router's scratch lives in a fixed array inside the library image (MOIN_ROUTE_STATIC_MAX_Q * 8 bytes = 512 KiB, held
+ * by every GPU that loads the library until the process exits), which the small ones do not touch.  The call performs
+ * no cudaMalloc/cudaFree and calls no allocating routine.
  *   - Q > MOIN_ROUTE_STATIC_MAX_Q returns MOIN_ERR_WORKSPACE and launches nothing.
  *   - The first call on each device that needs the array looks up its device address (with that device
  *     current); make that first call outside any stream capture, and from one host thread at a time (the
  *     look-up is not guarded against two threads making their first call together).
  *   - The calls that need the array share it; it keeps the previous call's contents, and the part a call uses is
- *     cleared on `stream` before use.  Two such calls whose GPU work overlaps (different streams, no ordering
- *     between them) race on it: order them, or use moin_route with separate workspaces. */
+ *     cleared or overwritten on `stream` before use.  Two such calls whose GPU work overlaps (different streams,
+ *     no ordering between them) race on it: order them, or use moin_route with separate workspaces. */
 enum { MOIN_ROUTE_STATIC_MAX_Q = 65536 };
 moin_status moin_route_static(const moin_router* router, const void* queries, int32_t Q, int32_t* out_expert,
                               int32_t* out_centroid, float* out_best_sim, moin_stream stream);

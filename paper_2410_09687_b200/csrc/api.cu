@@ -220,10 +220,9 @@ size_t moin_route_workspace_bytes(int32_t Q, int32_t K, int32_t D) {
 // Kernel choice shared by moin_route and moin_route_static, so that both compute the same values for the same
 // shapes and options: 0 = cluster kernel (few queries; one 64-bit key of scratch per query and part when it cuts the
 // table), 1 = tensor-core GEMM with one 64-bit key of scratch per query, 2 = CUDA-core kernel (no scratch).
-// 0 and 1 have a form without scratch that gives the same bits and is slower; small problems are served by it where
-// there is none: up to 1024 queries against 1024 centroids, and up to 65 535 products.
-static bool route_without_scratch(const HostState* hs, int choice, int Q, int K, int D) {
-  if (choice != 1) return true;
+// 0 and 1 have a form without scratch that gives the same bits and is slower.  Small problems have always been served
+// without: up to 1024 queries against 1024 centroids, and up to 65 535 products; with few queries any table can be.
+static bool route_small(const HostState* hs, int Q, int K, int D) {
   return hs->gemm_impl == 0 && ((Q <= 1024 && K <= 1024 && D <= 3168) || (long long)Q * K < (1ll << 16));
 }
 static moin_status route_choice(const HostState* hs, int Q, int K, int D, int* choice) {
@@ -300,7 +299,7 @@ moin_status moin_route(const moin_router* router, const void* queries, int32_t Q
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(workspace);
   if (!workspace || workspace_bytes < route_need(Q, router->K, router->D) + 256 || !aligned16(workspace)) {
     keys = nullptr;
-    if (!route_without_scratch(hs, choice, Q, router->K, router->D)) return MOIN_ERR_WORKSPACE;
+    if (choice == 1 && !route_small(hs, Q, router->K, router->D)) return MOIN_ERR_WORKSPACE;
   }
   return route_launch(hs, choice, router, queries, Q, out_expert, out_centroid, out_best_sim, keys, (cudaStream_t)stream);
 }
@@ -380,7 +379,8 @@ moin_status moin_route_static(const moin_router* router, const void* queries, in
   int choice;
   if ((st = route_choice(hs, Q, router->K, router->D, &choice))) return st;
   unsigned long long* keys = nullptr;
-  if (!route_without_scratch(hs, choice, Q, router->K, router->D)) {
+  const bool scratch = choice == 1 || (choice == 0 && route_parts(Q, router->K, router->D) > 1);
+  if (scratch && !route_small(hs, Q, router->K, router->D)) {
     if (g_route_static_ptr[hs->device] == nullptr) {   // set-up: once per device, that device is current here
       void* p = nullptr;
       cudaError_t e = cudaGetSymbolAddress(&p, g_route_static_keys);
