@@ -587,8 +587,10 @@ cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat1
 // ----------------------------------------------------------------------------------------
 // K-means update: centroid of every non-empty cluster = mean of its member rows, its inverse norm with it; a cluster
 // without members keeps its centroid.  One CTA per segment of the plan built from the assignments (segment = cluster
-// id, start, length in `perm`, members in increasing point order); it also copies the empty clusters between its own
-// id and the one before, so one launch covers the table.
+// id, start, length in `perm`, members in increasing point order); the CTAs behind those copy the clusters without a
+// segment, a warp for each kMeanEmpties clusters, so one launch covers the table however the points are spread.  (The
+// empty clusters next to a segment copied by the segment's CTA: 40000 points in the first 500 of 1000 clusters 77 us,
+// no point in any 134 us, now 16 and 8.)
 //
 // HBM-bound (every point is read once) as long as enough rows are in flight: warp (g, p) of a CTA adds part p of the
 // members in column group g (256 columns, 8 a lane; up to 128 columns several members at once), eight rows in flight,
@@ -596,11 +598,11 @@ cudaError_t launch_route_top2_cluster(const __nv_bfloat16* q, const __nv_bfloat1
 // all the members four at a time took 26.5 us for 40000 x 768 in 1000 clusters and 66.7 us for 6141 in 28, now 19.3
 // and 9.0 us, with the copy of the table and the norms (4.4 us, two launches) in the same launch.
 // ----------------------------------------------------------------------------------------
-constexpr int kMeanRows = 8, kMeanMaxWarps = 16;
+constexpr int kMeanRows = 8, kMeanMaxWarps = 16, kMeanEmpties = 8;
 __global__ void __launch_bounds__(kMeanMaxWarps * 32, 2)
 kmeans_update_kernel(const int* __restrict__ header, const int* __restrict__ perm, const int4* __restrict__ seg_tab,
                      const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* c_old, __nv_bfloat16* c_new,
-                     float* __restrict__ inv_new, int K, int D, int G, int P) {
+                     float* __restrict__ inv_new, int K, int D, int G, int P, int seg_ctas) {
   __shared__ float4 s_acc[kMeanMaxWarps][2][32];
   __shared__ float s_ss[kMeanMaxWarps];
   pdl_begin();
@@ -609,12 +611,37 @@ kmeans_update_kernel(const int* __restrict__ header, const int* __restrict__ per
   const int g = warp % G, part = warp / G, nch = D / 8;
   const int lpr = nch <= 8 ? 8 : nch <= 16 ? 16 : 32, rows = 32 / lpr;   // lanes per row, members taken at once
   const int sub = lane / lpr, lc = lane % lpr;
-  for (int seg = blockIdx.x; seg < max(nseg, 1); seg += gridDim.x) {
-    const int4 e = nseg > 0 ? __ldg(seg_tab + seg) : make_int4(K, 0, 0, 0);   // (cluster, start, length, -)
+  if ((int)blockIdx.x >= seg_ctas) {   // clusters m0 .. m0 + kMeanEmpties - 1 as far as they are empty
+    const int m0 = (((int)blockIdx.x - seg_ctas) * n_warps + warp) * kMeanEmpties;
+    if (m0 >= K || blockIdx.y > 0) return;
+    int lo = 0, hi = nseg;   // first segment of a cluster >= m0: the lanes probe 32 places at a time
+    while (lo < hi) {
+      const int step = (hi - lo + 32) / 33, at = lo + (lane + 1) * step - 1;
+      const int below = __popc(__ballot_sync(0xffffffffu, at < hi && __ldg(seg_tab + min(at, hi - 1)).x < m0));
+      lo = min(hi, lo + below * step);
+      if (below < 32) hi = min(hi, lo + step - 1);
+    }
+    const int k = lo + lane < nseg && lane < kMeanEmpties ? __ldg(seg_tab + lo + lane).x : K;
+    const uint32_t full = __reduce_or_sync(0xffffffffu, k < m0 + kMeanEmpties ? 1u << (k - m0) : 0u);
+    for (int m = m0; m < min(K, m0 + kMeanEmpties); ++m) {
+      if ((full >> (m - m0)) & 1u) continue;
+      float s2 = 0.f;
+      for (int ch = lane; ch < nch; ch += 32) {
+        const uint4 v = *reinterpret_cast<const uint4*>(c_old + (size_t)m * D + ch * 8);
+        if (c_new != c_old) *reinterpret_cast<uint4*>(c_new + (size_t)m * D + ch * 8) = v;
+        add_sq8(v, s2);
+      }
+      s2 = warp_sum(s2);
+      if (inv_new != nullptr && lane == 0) inv_new[m] = s2 > 0.f ? rsqrtf(s2) : 0.f;
+    }
+    return;
+  }
+  for (int seg = blockIdx.x; seg < nseg; seg += seg_ctas) {
+    const int4 e = __ldg(seg_tab + seg);   // (cluster, start, length, -)
     const int k = e.x, lo = e.y + (int)((long long)e.z * part / P), hi = e.y + (int)((long long)e.z * (part + 1) / P);
     float ss = 0.f;
     const int c_step = 32 * G * gridDim.y;   // (gridDim.y > 1: the column groups are spread over CTAs, norms come later)
-    for (int c0 = 32 * G * blockIdx.y; c0 < nch && nseg > 0; c0 += c_step) {
+    for (int c0 = 32 * G * blockIdx.y; c0 < nch; c0 += c_step) {
       const int ch = c0 + g * 32 + lc;
       const bool on = ch < nch;
       float acc[8];
@@ -664,7 +691,7 @@ kmeans_update_kernel(const int* __restrict__ header, const int* __restrict__ per
       }
       __syncthreads();
     }
-    if (inv_new != nullptr && nseg > 0) {
+    if (inv_new != nullptr) {
       ss = warp_sum(ss);
       if (lane == 0) s_ss[warp] = ss;
       __syncthreads();
@@ -674,20 +701,6 @@ kmeans_update_kernel(const int* __restrict__ header, const int* __restrict__ per
         inv_new[k] = t > 0.f ? rsqrtf(t) : 0.f;
       }
       __syncthreads();
-    }
-    // empty clusters next to this one: a warp each
-    const int e_lo = seg > 0 ? __ldg(seg_tab + seg - 1).x + 1 : 0;
-    const int e_hi = seg + 1 >= nseg ? K : k;          // (the last segment takes those behind it as well)
-    for (int m = e_lo + warp; m < e_hi && blockIdx.y == 0; m += n_warps) {
-      if (m == k) continue;
-      float s2 = 0.f;
-      for (int ch = lane; ch < nch; ch += 32) {
-        const uint4 v = *reinterpret_cast<const uint4*>(c_old + (size_t)m * D + ch * 8);
-        if (c_new != c_old) *reinterpret_cast<uint4*>(c_new + (size_t)m * D + ch * 8) = v;
-        add_sq8(v, s2);
-      }
-      s2 = warp_sum(s2);
-      if (inv_new != nullptr && lane == 0) inv_new[m] = s2 > 0.f ? rsqrtf(s2) : 0.f;
     }
   }
 }
@@ -701,10 +714,10 @@ cudaError_t launch_kmeans_update(const PlanView& pv, const __nv_bfloat16* x, con
   const int G = split ? 1 : groups < 4 ? groups : 4;
   int P = pv.T / pv.E / 16;   // sixteen members per warp
   P = P < 1 ? 1 : P > kMeanMaxWarps / G ? kMeanMaxWarps / G : P;
-  long grid = pv.Smax < (long)n_sms * 16 ? pv.Smax : (long)n_sms * 16;
-  if (grid < 1) grid = 1;
-  launch_pdl(kmeans_update_kernel, dim3((unsigned)grid, split ? (unsigned)groups : 1u), 32 * G * P, 0, stream,
-             pv.header, pv.perm, pv.seg_tab, x, c_old, c_new, split ? nullptr : inv_new, pv.E, D, G, P);
+  const int seg_ctas = pv.Smax < n_sms * 16 ? pv.Smax : n_sms * 16;
+  const int empty_warps = (pv.E + kMeanEmpties - 1) / kMeanEmpties, empty_ctas = (empty_warps + G * P - 1) / (G * P);
+  launch_pdl(kmeans_update_kernel, dim3((unsigned)(seg_ctas + empty_ctas), split ? (unsigned)groups : 1u), 32 * G * P, 0, stream,
+             pv.header, pv.perm, pv.seg_tab, x, c_old, c_new, split ? nullptr : inv_new, pv.E, D, G, P, seg_ctas);
   if (split && inv_new != nullptr) return launch_inv_norm(c_new, pv.E, D, inv_new, stream);
   return cudaGetLastError();
 }
