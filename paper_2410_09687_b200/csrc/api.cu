@@ -541,12 +541,20 @@ static moin_status pick_gemm(const HostState* hs, int T, int d_in, int d_out, bo
   return MOIN_OK;
 }
 
-// y (and y0) = x W^T for one projection: few tokens, the token-wide kernel (W is read once); many, CTA pairs.
+// y (and y0) = x W^T for one projection: few tokens, the token-wide kernel (W is read once); many, CTA pairs.  Without
+// adapters beside it the token-wide kernel's x traffic and its epilogue weigh from some tokens x features on, more of them
+// the longer the reduction: us of the two kernels at 128 tokens 2048 -> 2048 7.1 / 10.2, 2048 -> 5632 13.5 / 11.2, 2048 ->
+// 32000 38.6 / 29.0; at 256 tokens 64 -> 4096 7.1 / 4.4, 2048 -> 2048 9.9 / 10.3, 2048 -> 4096 15.0 / 10.9, 5632 -> 2048
+// 14.4 / 21.6; at 512 tokens 768 -> 768 7.6 / 6.2, 2048 -> 256 6.2 / 10.1, 2048 -> 2048 15.2 / 10.9.  Up to 64 tokens it
+// has two CTAs an SM and is the better one throughout (64 tokens 2048 -> 5632 7.5 / 10.7).
+static bool decode_gemm_wins(int T, int d_in, int d_out) {
+  return T <= 64 || (T <= kDecodeGemmMaxT && (long long)T * d_out < 262144 + 160ll * d_in);
+}
 static moin_status launch_base_gemm(HostState* hs, bool use_tc, const __nv_bfloat16* x, const __nv_bfloat16* W,
                                     __nv_bfloat16* y, float* y0, int T, int d_in, int d_out, cudaStream_t s) {
   ProfScope prof(use_tc ? MOIN_K_GEMM_TC : MOIN_K_GEMM_WARP, 1, s);
   if (!use_tc) return record_cuda(launch_gemm_warp(x, W, y, y0, T, d_in, d_out, s));
-  if (T <= kDecodeGemmMaxT) {
+  if (decode_gemm_wins(T, d_in, d_out)) {
     const DecodeGemmJob job = {x, W, y, y0, d_in, d_out, nullptr};
     return launch_decode_gemm(hs, &job, 1, T, s);
   }
