@@ -227,7 +227,7 @@ static bool route_small(const HostState* hs, int Q, int K, int D) {
 }
 static moin_status route_choice(const HostState* hs, int Q, int K, int D, int* choice) {
   const bool tc_ok = tc_router_supported(Q, K, D);
-  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 12);
+  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 12) && !route_few_topics(Q, K, D);
   if (hs->gemm_impl == 1) use_tc = false;
   if (hs->gemm_impl == 2) {
     if (!tc_ok) return MOIN_ERR_BAD_SHAPE;
@@ -323,7 +323,7 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
   if (st) return st;
   cudaStream_t s = (cudaStream_t)stream;
   const bool tc_ok = tc_router_supported(Q, K, D);
-  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 12);
+  bool use_tc = tc_ok && (long long)Q * K >= (1ll << 12) && !route_few_topics(Q, K, D);
   if (hs->gemm_impl == 1) use_tc = false;
   if (hs->gemm_impl == 2) {
     if (!tc_ok) return MOIN_ERR_BAD_SHAPE;

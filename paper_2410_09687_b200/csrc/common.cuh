@@ -223,6 +223,7 @@ cudaError_t launch_route_simple(const __nv_bfloat16* q, const __nv_bfloat16* c, 
                                 const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
                                 float* out_best, cudaStream_t stream);
 bool route_cluster_supported(int Q, int K, int D);
+bool route_few_topics(int Q, int K, int D);   // left to the CUDA-core kernel
 cudaError_t launch_route_cluster(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                  const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
                                  float* out_best, unsigned long long* part_keys, cudaStream_t stream);

@@ -43,6 +43,7 @@ route_simple_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
   __shared__ float s_best[4][kRouteQB];
   __shared__ int s_id[4][kRouteQB];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_begin();
   const int q0 = blockIdx.x * kRouteQB;
   const int nch = D / 8;
   for (int i = tid; i < kRouteQB * nch; i += 128) {
@@ -509,6 +510,9 @@ cudaError_t launch_clear_keys(unsigned long long* keys, size_t n, cudaStream_t s
 
 // How a problem is cut: queries per cluster, CTAs per cluster, parts of the table; fast = the rule picks this kernel.
 struct RouteCut { int nq, csize, parts, groups; bool fast; };
+// A handful of topics: the CUDA-core kernel has them done before a cluster is set up (D = 768, 1 to 384 queries x 1 topic
+// 5.4-8.7 us by the cluster kernel, 3.1-3.8 so; x 8 5.6-8.6 / 4.4-5.0; 512 x 16 8.1 by the GEMM, 7.2 so).
+bool route_few_topics(int Q, int K, int D) { return K <= 16 && K * D <= 16 * 768 && (long long)Q * K < (1ll << 16); }
 static RouteCut route_cut(int Q, int K, int D) {
   RouteCut r = {0, 8, 1, 0, false};
   if (Q < 1 || K < 1 || (D % 8) != 0 || 8 * route_pitch(D) > 200 * 1024) return r;
@@ -524,7 +528,10 @@ static RouteCut route_cut(int Q, int K, int D) {
   // 5000 x 768): 7.3 us for up to 8 queries and 9.8-10.6 us for up to 32 per cluster with one tile per warp pair,
   // 13.3 and 18.7 with two.
   r.fast = r.groups * r.parts <= kResident && tiles <= (nq == 8 ? 2 : 1);
-  if (!tc_router_supported(Q, K, D)) r.fast = r.fast || r.groups <= 64;   // else only the CUDA-core kernel is left
+  // Too narrow for the GEMM: against the CUDA-core kernel (2.2 us + 0.18 us a centroid) a wave of clusters takes 6.3 us
+  // (D = 40: 512 queries x 30 12.6 / 6.9 us, 1500 x 100 25.9 / 20.2, 1500 x 300 27 / 60).
+  if (!tc_router_supported(Q, K, D)) r.fast = r.fast || (r.groups <= 64 && K > 35 * ((r.groups + kResident - 1) / kResident));
+  if (route_few_topics(Q, K, D)) r.fast = false;
   return r;
 }
 bool route_cluster_supported(int Q, int K, int D) { return route_cut(Q, K, D).fast; }
@@ -732,6 +739,7 @@ route_top2_simple_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat1
                          const float* __restrict__ inv_norm, const int* __restrict__ cmap, int Q, int K, int D,
                          int* __restrict__ out_expert, int* __restrict__ out_centroid, int* __restrict__ out_second,
                          float* __restrict__ out_best, float* __restrict__ out_margin) {
+  pdl_begin();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= Q) return;
   const int nch = D / 8;
@@ -810,9 +818,8 @@ route_finish_top2_kernel(const unsigned long long* __restrict__ keys, const unsi
 cudaError_t launch_route_top2_simple(const __nv_bfloat16* q, const __nv_bfloat16* c, const float* inv_norm,
                                      const int* cmap, int Q, int K, int D, int* out_expert, int* out_centroid,
                                      int* out_second, float* out_best, float* out_margin, cudaStream_t stream) {
-  route_top2_simple_kernel<<<(Q + 7) / 8, 256, 0, stream>>>(q, c, inv_norm, cmap, Q, K, D, out_expert, out_centroid,
-                                                           out_second, out_best, out_margin);
-  return cudaGetLastError();
+  return launch_pdl(route_top2_simple_kernel, (Q + 7) / 8, 256, 0, stream, q, c, inv_norm, cmap, Q, K, D, out_expert,
+                    out_centroid, out_second, out_best, out_margin);
 }
 cudaError_t launch_route_finish_top2(const unsigned long long* keys, const unsigned long long* keys2,
                                      const __nv_bfloat16* q, const int* cmap, int Q, int D, int* out_expert,
@@ -834,9 +841,8 @@ cudaError_t launch_route_simple(const __nv_bfloat16* q, const __nv_bfloat16* c, 
   const size_t smem = (size_t)kRouteQB * D * 2;
   cudaError_t ce = ensure_smem_optin(OPTIN_ROUTE_SIMPLE, route_simple_kernel, 8 * 8192 * 2);
   if (ce != cudaSuccess) return ce;
-  route_simple_kernel<<<(Q + kRouteQB - 1) / kRouteQB, 128, smem, stream>>>(q, c, inv_norm, cmap, Q, K, D, out_expert,
-                                                                            out_centroid, out_best);
-  return cudaGetLastError();
+  return launch_pdl(route_simple_kernel, (Q + kRouteQB - 1) / kRouteQB, 128, smem, stream, q, c, inv_norm, cmap, Q, K, D,
+                    out_expert, out_centroid, out_best);
 }
 
 // The same without the cosine output: nothing to reduce, so one thread per query (coalesced keys and ids).
