@@ -222,19 +222,27 @@ class Router:
                "moin_router_prepare")
         self.c = _Router(_ptr(centroids), _ptr(self.inv_norm), _ptr(centroid_to_expert), self.K, self.D)
 
-    def workspace(self, Q: int, stream=None) -> torch.Tensor:
-        """Scratch of one call on ``stream``.  Every call has its own: calls over one table may overlap (several workers,
-        streams or captured graphs), and each keeps its keys there."""
-        return _scratch(lib().moin_route_workspace_bytes(Q, self.K, self.D), self.centroids.device, stream)
+        self._ws_bytes: dict = {}   # batch size -> bytes (asking the library costs half a microsecond)
+
+    def workspace_bytes(self, Q: int) -> int:
+        n = self._ws_bytes.get(Q)
+        if n is None:
+            if len(self._ws_bytes) >= 1024:
+                self._ws_bytes.clear()
+            n = self._ws_bytes[Q] = lib().moin_route_workspace_bytes(Q, self.K, self.D)
+        return n
+
+    def workspace(self, Q: int) -> torch.Tensor:
+        """Scratch for calls of the C ABI with up to Q queries that do not overlap (``route`` takes its own)."""
+        return torch.empty(self.workspace_bytes(Q), dtype=torch.uint8, device=self.centroids.device)
 
 
-def _scratch(nbytes: int, device, stream: Optional[torch.cuda.Stream]) -> torch.Tensor:
-    """A block of the caching allocator that belongs to the stream the call goes to: dropped when the call returns, it is
-    handed out again only to work behind the call."""
-    if stream is None:
-        return torch.empty(nbytes, dtype=torch.uint8, device=device)
-    with torch.cuda.stream(stream):
-        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+# Scratch of one call: a block of torch's caching allocator that belongs to the stream the call goes to, so that, given
+# back when the call has returned, it is handed out again only to work behind it.  Every call has its own: calls over one table may
+# overlap (several workers, streams or captured graphs), and each keeps its keys there.  (The raw calls, on the current
+# device as the library's own: half a microsecond, where a tensor takes 1.6.)
+_scratch_alloc = torch._C._cuda_cudaCachingAllocator_raw_alloc
+_scratch_free = torch._C._cuda_cudaCachingAllocator_raw_delete
 
 
 def route(router: Router, queries: torch.Tensor, out_expert: Optional[torch.Tensor] = None,
@@ -244,9 +252,13 @@ def route(router: Router, queries: torch.Tensor, out_expert: Optional[torch.Tens
     Q = queries.shape[0]
     if out_expert is None:
         out_expert = torch.empty(Q, dtype=torch.int32, device=queries.device)
-    ws = router.workspace(Q, stream)
-    _check(lib().moin_route(ctypes.byref(router.c), _ptr(queries), Q, _ptr(out_expert), _ptr(out_centroid),
-                            _ptr(out_best_sim), _ptr(ws), ws.numel(), _stream(stream)), "moin_route")
+    n, s = router.workspace_bytes(Q), _stream(stream)
+    ws = _scratch_alloc(n, s)
+    try:
+        _check(lib().moin_route(ctypes.byref(router.c), _ptr(queries), Q, _ptr(out_expert), _ptr(out_centroid),
+                                _ptr(out_best_sim), ws, n, s), "moin_route")
+    finally:
+        _scratch_free(ws)
     return out_expert
 
 
@@ -257,10 +269,14 @@ def route_top2(router: Router, queries: torch.Tensor, stream=None) -> dict:
     out = {"expert": torch.empty(Q, dtype=torch.int32, device=dev), "centroid": torch.empty(Q, dtype=torch.int32, device=dev),
            "second": torch.empty(Q, dtype=torch.int32, device=dev), "best": torch.empty(Q, dtype=torch.float32, device=dev),
            "margin": torch.empty(Q, dtype=torch.float32, device=dev)}
-    ws = _scratch(lib().moin_route_top2_workspace_bytes(Q, router.K, router.D), dev, stream)
-    _check(lib().moin_route_top2(ctypes.byref(router.c), _ptr(queries), Q, _ptr(out["expert"]), _ptr(out["centroid"]),
-                                 _ptr(out["second"]), _ptr(out["best"]), _ptr(out["margin"]), _ptr(ws), ws.numel(),
-                                 _stream(stream)), "moin_route_top2")
+    n, s = lib().moin_route_top2_workspace_bytes(Q, router.K, router.D), _stream(stream)
+    ws = _scratch_alloc(n, s)
+    try:
+        _check(lib().moin_route_top2(ctypes.byref(router.c), _ptr(queries), Q, _ptr(out["expert"]), _ptr(out["centroid"]),
+                                     _ptr(out["second"]), _ptr(out["best"]), _ptr(out["margin"]), ws, n, s),
+               "moin_route_top2")
+    finally:
+        _scratch_free(ws)
     return out
 
 
