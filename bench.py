@@ -910,8 +910,8 @@ def main():
 
     # per-kernel timing -> roofline of the dominant kernel
     agg, launches_per_step = profile_pass(moin, wl.step, min(args.steps, 20))
-    # dominant kernel = most device time among the kernels on the call's own stream; in the short-segment
-    # (decode) path the base GEMMs run on side streams beside the shrink, so their brackets overlap it
+    # dominant kernel = most device time among the kernels that carry the step; in the short-segment (decode)
+    # path the base GEMM is the one that the adapter streams run beside
     on_path = {k: v for k, v in agg.items() if not (kind == "decode" and k in ("gemm_tc", "gemm_warp"))}
     top = max(on_path.items(), key=lambda kv: kv[1]["ms"])[0]
     kernels = {k: {"launches": a["launches"], "ms_per_launch": a["ms"] / max(a["launches"], 1)} for k, a in agg.items()}

@@ -258,9 +258,11 @@ static moin_status route_launch(HostState* hs, int choice, const moin_router* ro
   }
   if (choice == 1) {
     // the merge across column tiles is a max, so the keys must start from zero
-    cudaError_t e = launch_clear_keys(keys, (size_t)Q, s);
-    if (e != cudaSuccess) return record_cuda(e);
     moin_status st;
+    {
+      ProfScope prof(MOIN_K_ROUTE_FINISH, 1, s);   // (with the finishing pass: the keys' own kernels)
+      if ((st = record_cuda(launch_clear_keys(keys, (size_t)Q, s)))) return st;
+    }
     {
       ProfScope prof(MOIN_K_ROUTE_TC, 1, s);
       st = launch_pair_router(hs, (const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
@@ -335,7 +337,7 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
     use_tc = false;
   }
   if (hs->gemm_impl == 0 && route_cluster_supported(Q, K, D)) {
-    ProfScope prof(MOIN_K_ROUTE_CLUSTER, route_parts(Q, K, D) > 1 ? 2 : 1, s);
+    ProfScope prof(MOIN_K_ROUTE_CLUSTER, fits && route_parts(Q, K, D) > 1 ? 2 : 1, s);
     return record_cuda(launch_route_top2_cluster((const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids,
                                                  router->inv_norm, router->centroid_to_expert, Q, K, D, out_expert,
                                                  out_centroid, out_second, out_best_sim, out_margin,
@@ -350,8 +352,10 @@ moin_status moin_route_top2(const moin_router* router, const void* queries, int3
   const size_t half = align_up((size_t)Q * sizeof(unsigned long long), 256);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(workspace);
   unsigned long long* keys2 = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(workspace) + half);
-  cudaError_t e = launch_clear_keys(keys, 2 * half / sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return record_cuda(e);
+  {
+    ProfScope prof(MOIN_K_ROUTE_FINISH, 1, s);
+    if ((st = record_cuda(launch_clear_keys(keys, 2 * half / sizeof(unsigned long long), s)))) return st;
+  }
   {
     ProfScope prof(MOIN_K_ROUTE_TC, 1, s);
     st = launch_pair_router(hs, (const __nv_bfloat16*)queries, (const __nv_bfloat16*)router->centroids, router->inv_norm,
@@ -408,7 +412,7 @@ moin_status moin_kmeans_update(const moin_plan* plan, const void* x, const void*
   const int K = plan->E;
   if (plan->T > 0) {
     PlanView pv = plan_view(plan->buffer, plan->T, plan->E);
-    ProfScope prof(MOIN_K_KMEANS_UPDATE, 1, s);
+    ProfScope prof(MOIN_K_KMEANS_UPDATE, inv_norm_new && kmeans_update_split(K, D, hs->n_sms) ? 2 : 1, s);
     return record_cuda(launch_kmeans_update(pv, (const __nv_bfloat16*)x, (const __nv_bfloat16*)centroids_old,
                                             (__nv_bfloat16*)centroids_new, inv_norm_new, D, hs->n_sms, s));
   }

@@ -8,7 +8,8 @@
 // The time of an item is a chain of hand-overs (scores, softmax, product), not any unit's throughput, so a CTA keeps two
 // chains going: the even key tiles are one STREAM, the odd ones another, each with its own four softmax warps, scores,
 // running maximum, row sum and accumulator; the two meet once at the end of the item.  A stream takes a thread per row and
-// one pass over its keys: p = 2^(s - m) against a maximum m that may lag behind by a factor of up to 2^8 (p is bf16 and
+// one pass over its key tiles (the scores of a tile are read from tensor memory twice, once for their maximum): p = 2^(s - m)
+// against a maximum m that may lag behind by a factor of up to 2^8 (p is bf16 and
 // its sum fp32: the relative accuracy is the same), so the accumulator is rescaled only when a row outgrows that.  P goes
 // back into tensor memory over the scores it came from, as the A operand of the second product: nothing of it passes
 // through shared memory.  Warp roles:
@@ -58,31 +59,20 @@ struct AttParams {
   DeviceStatus* status;
 };
 
-// K-major operand with 128-byte swizzle: rows of 128 bytes, 8-row groups 1024 bytes apart (same as the GEMMs).
-__device__ __forceinline__ uint64_t at_sdesc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-// D fp32, A / B bf16 K-major, M = 128, N = 64
-constexpr uint32_t kAtIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+constexpr uint32_t kAtIdesc = idesc_bf16(128, 64);
 // the same with B MN-major (V tile: one 128-byte row per key, the 64 output dims contiguous); a 16-key step of
 // such a tile is two 8-key groups = 2048 bytes further on
 constexpr uint32_t kAtIdescPV = kAtIdesc | (1u << 16);
 constexpr uint64_t kAtVStep = 2048 >> 4;
 
-__device__ __forceinline__ float fast_exp2(float x) {   // arguments are <= 0 here: 2^x in (0, 1]
+__device__ __forceinline__ float fast_exp2(float x) {   // x <= kAtLag here: 2^x up to 256, below 2^-126 zero
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
-// Two-lane fp32 arithmetic (one instruction for a pair of scores) and the three-input maximum: the softmax threads
-// are bound by the number of instructions they issue, not by any one pipe.
+// Two-lane fp32 arithmetic (one instruction for a pair of scores): the softmax threads are bound by the number of
+// instructions they issue, not by any one pipe.
 __device__ __forceinline__ uint64_t pair_f32(float lo, float hi) {
   uint64_t d;
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
@@ -101,18 +91,12 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-
 // byte offset of 16-byte chunk c of row r in a swizzled [rows x 128 bytes] tile
 __device__ __forceinline__ uint32_t at_swz(int r, int c) {
   return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4));
 }
 
-struct AttItem { int req, kvh, q0, t0, L, a0, n_tiles; bool on; };
+struct AttItem { int req, kvh, q0, t0, L, n_tiles; bool on; };
 __device__ __forceinline__ AttItem at_item(const AttParams& p, const int* cu, int idx) {
   AttItem it;
   const int per_qb = p.R * p.n_kv;
@@ -124,9 +108,8 @@ __device__ __forceinline__ AttItem at_item(const AttParams& p, const int* cu, in
   it.t0 = cu[it.req];
   it.L = cu[it.req + 1] - it.t0;
   it.on = it.q0 < it.L;
-  it.a0 = it.t0;
   const int kv_end = min(it.L, it.q0 + p.ppt);   // keys of the request this block can see
-  it.n_tiles = it.on ? (it.t0 + kv_end - it.a0 + kAtKeys - 1) / kAtKeys : 0;
+  it.n_tiles = it.on ? (kv_end + kAtKeys - 1) / kAtKeys : 0;
   return it;
 }
 
@@ -216,10 +199,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           const uint32_t s = tq % kAtRing, ph = (tq / kAtRing) & 1u;
           if (!(ok = mbar_wait(kempty + 8 * s, ph ^ 1u, abort_flag, p.status, 31))) break;
           mbar_expect_tx(kfull + 8 * s, kAtKV);
-          tma_load_2d(sK + s * kAtKV, &tmK, kfull + 8 * s, it.kvh * 64, it.a0 + j * kAtKeys);
+          tma_load_2d(sK + s * kAtKV, &tmK, kfull + 8 * s, it.kvh * 64, it.t0 + j * kAtKeys);
           if (!(ok = mbar_wait(vempty + 8 * s, ph ^ 1u, abort_flag, p.status, 32))) break;
           mbar_expect_tx(vfull + 8 * s, kAtKV);
-          tma_load_2d(sV + s * kAtKV, &tmV, vfull + 8 * s, it.kvh * 64, it.a0 + j * kAtKeys);
+          tma_load_2d(sV + s * kAtKV, &tmV, vfull + 8 * s, it.kvh * 64, it.t0 + j * kAtKeys);
         }
         it = nx;
         idx = nidx;
@@ -238,7 +221,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if (!it.on) continue;
         if (!(ok = mbar_wait_warp(qready, nit & 1u, abort_flag, p.status, 35))) break;
         tc_fence_after();
-        const uint64_t dq = at_sdesc(sQ + (nit & 1u) * kAtTile);
+        const uint64_t dq = sdesc_k128(sQ + (nit & 1u) * kAtTile);
         int tile[2] = {0, 1}, left = it.n_tiles;   // next tile of each stream; products to go
         bool scores[2] = {false, false};           // its scores have been issued
         bool o_free = false;
@@ -255,7 +238,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
               if (!__all_sync(0xffffffffu, (n_p[h] == 0 || mbar_test_wait(pvdone + 8 * h, (n_p[h] - 1) & 1u)) &&
                                                mbar_test_wait(kfull + 8 * s, ph))) continue;
               tc_fence_after();
-              const uint64_t dk = at_sdesc(sK + s * kAtKV);
+              const uint64_t dk = sdesc_k128(sK + s * kAtKV);
               if (leader) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) tc_mma_bf16(tmem + h * 64, dq + (uint64_t)(2 * k), dk + (uint64_t)(2 * k), kAtIdesc, k > 0 ? 1u : 0u);
@@ -269,7 +252,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
               if (!o_free && !(o_free = __all_sync(0xffffffffu, mbar_test_wait(ofree, (nit & 1u) ^ 1u)))) continue;
               if (!__all_sync(0xffffffffu, mbar_test_wait(pready + 8 * h, n_p[h] & 1u) && mbar_test_wait(vfull + 8 * s, ph))) continue;
               tc_fence_after();
-              const uint64_t dv = at_sdesc(sV + s * kAtKV);
+              const uint64_t dv = sdesc_k128(sV + s * kAtKV);
               const uint32_t first = tile[h] == h ? 0u : 1u;
               if (leader) {
 #pragma unroll
@@ -401,8 +384,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           if (kr + 15 <= it.q0) {
 #pragma unroll
             for (int c = 0; c < 16; c += 4) {
-              ma = max3(ma, __uint_as_float(v[c]), __uint_as_float(v[c + 1]));
-              mc = max3(mc, __uint_as_float(v[c + 2]), __uint_as_float(v[c + 3]));
+              ma = fmax3(ma, __uint_as_float(v[c]), __uint_as_float(v[c + 1]));
+              mc = fmax3(mc, __uint_as_float(v[c + 2]), __uint_as_float(v[c + 3]));
             }
           } else if (kr <= q_last) {
 #pragma unroll

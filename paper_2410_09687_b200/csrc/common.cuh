@@ -149,12 +149,25 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Router: (similarity, index) as a 64-bit key whose maximum is the best similarity, among equals the lowest index.
+__device__ __forceinline__ unsigned long long route_key(float sim, int k) {
+  uint32_t u = __float_as_uint(sim);
+  u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)k);
+}
+__device__ __forceinline__ float key_to_float(uint32_t u) {   // upper half of a key
+  u = (u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u;
+  return __uint_as_float(u);
+}
+
 // Programmatic dependent launch: the next kernel of the stream may start once every CTA has got here / this CTA goes
 // on once the kernels before it are complete and their writes visible (no-ops in an ordinary launch).  The kernels of a
 // call are launched this way, so that a kernel's launch latency and set-up lie under the tail of the one before it
 // (about 2 us each).  Rule: a kernel waits before it touches global memory and lets the next one start only after that
-// - then everything before a running kernel is complete but the kernel right before it.  The adapter shrink beside the
-// decode GEMM is the one exception; lora_stream.cu says how it keeps the order.
+// - then everything before a running kernel is complete but the kernel right before it.  Three kernels differ, and say
+// beside their code how the order is kept: the adapter shrink beside the decode GEMM, which does not wait at its start
+// (its last CTA waits at its end); the expand behind it, which reads the plan and starts on the adapters before it waits,
+// and lets the next kernel start at once; and route_parts_kernel, which reads the queries before it waits.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -201,7 +214,7 @@ struct ExpandJobs {
   const int* slot_of_expert[kMaxStreamJobs];
   const int* slot_rank[kMaxStreamJobs];   // per-slot rank (nullptr: the pool's r)
   int act[kMaxStreamJobs];                // MOIN_ACT_* applied to h
-  int r[kMaxStreamJobs], d_out[kMaxStreamJobs], rows_per_item[kMaxStreamJobs], per_seg[kMaxStreamJobs];
+  int r[kMaxStreamJobs], d_out[kMaxStreamJobs], per_seg[kMaxStreamJobs];
   int n;
 };
 cudaError_t launch_lora_shrink_stream(const PlanView& pv, ShrinkJobs jobs, int n_sms, cudaStream_t stream);
@@ -216,6 +229,7 @@ cudaError_t launch_route_finish_top2(const unsigned long long* keys, const unsig
                                      const __nv_bfloat16* q, const int* cmap, int Q, int D, int* out_expert,
                                      int* out_centroid, int* out_second, float* out_best, float* out_margin,
                                      cudaStream_t stream);
+bool kmeans_update_split(int K, int D, int n_sms);   // column groups apart, norms in a second launch
 cudaError_t launch_kmeans_update(const PlanView& pv, const __nv_bfloat16* x, const __nv_bfloat16* c_old,
                                  __nv_bfloat16* c_new, float* inv_new, int D, int n_sms, cudaStream_t stream);
 cudaError_t launch_inv_norm(const __nv_bfloat16* c, int K, int D, float* inv_norm, cudaStream_t stream);

@@ -367,7 +367,6 @@ cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float
                                       cudaStream_t stream) {
   int tps = 0, rmax = 0;
   for (int j = 0; j < jobs.n; ++j) {
-    jobs.rows_per_item[j] = 16;
     jobs.per_seg[j] = (jobs.d_out[j] + 15) / 16;   // 16-row tiles per chunk
     tps += jobs.per_seg[j];
     rmax = jobs.r[j] > rmax ? jobs.r[j] : rmax;

@@ -122,10 +122,6 @@ route_simple_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
 // Finishing pass of the tensor-core router: unpack the per-query (similarity, index) key that
 // the GEMM epilogues merged with 64-bit atomicMax, apply the centroid->expert map, and turn
 // the winning value into a cosine by dividing by |q|.  One warp per query.
-__device__ __forceinline__ float key_to_float(uint32_t u) {
-  u = (u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u;
-  return __uint_as_float(u);
-}
 __global__ void __launch_bounds__(256)
 route_finish_kernel(const unsigned long long* __restrict__ keys, const __nv_bfloat16* __restrict__ q,
                     const int* __restrict__ cmap, int Q, int D, int* __restrict__ out_expert,
@@ -179,11 +175,6 @@ route_finish_kernel(const unsigned long long* __restrict__ keys, const __nv_bflo
 // ----------------------------------------------------------------------------------------
 constexpr int kRcWarps = 8, kRcBatch = 6;
 
-__device__ __forceinline__ unsigned long long route_key(float sim, int k) {
-  uint32_t u = __float_as_uint(sim);
-  u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-  return ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)k);
-}
 __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v, int o) {
   return __shfl_xor_sync(0xffffffffu, v, o);
 }
@@ -712,12 +703,13 @@ kmeans_update_kernel(const int* __restrict__ header, const int* __restrict__ per
   }
 }
 
+// Enough clusters to fill the GPU: a CTA takes whole rows and the norm with them.  Fewer: its column groups go to
+// CTAs of their own (65536 x 768 in 20 clusters: 446 us whole rows, 92 us) and the norms to a second launch.
+bool kmeans_update_split(int K, int D, int n_sms) { return K < 2 * n_sms && D > 256; }
 cudaError_t launch_kmeans_update(const PlanView& pv, const __nv_bfloat16* x, const __nv_bfloat16* c_old,
                                  __nv_bfloat16* c_new, float* inv_new, int D, int n_sms, cudaStream_t stream) {
-  // Enough clusters to fill the GPU: a CTA takes whole rows and the norm with them.  Fewer: its column groups go to
-  // CTAs of their own (65536 x 768 in 20 clusters: 446 us whole rows, 92 us) and the norms to a second launch.
   const int nch = D / 8, groups = (nch + 31) / 32;
-  const bool split = pv.E < 2 * n_sms && groups > 1;
+  const bool split = kmeans_update_split(pv.E, D, n_sms);
   const int G = split ? 1 : groups < 4 ? groups : 4;
   int P = pv.T / pv.E / 16;   // sixteen members per warp
   P = P < 1 ? 1 : P > kMeanMaxWarps / G ? kMeanMaxWarps / G : P;

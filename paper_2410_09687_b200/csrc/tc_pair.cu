@@ -55,11 +55,6 @@ constexpr int kPairMaxN = 256, kPairStageBytes = (kPairM + kPairMaxN / 2) * kPai
 constexpr int kPairOutBytes = 8 * 32 * 128;   // epilogue staging: [32 rows x 64 columns] bf16 per warp
 constexpr size_t kPairSmem = (size_t)kPairStages * kPairStageBytes + 1024 /*align*/ + 1024 /*barriers*/ + kPairOutBytes;
 
-__device__ __forceinline__ uint32_t pair_orderable(float f) {
-  const uint32_t u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
 // What a tile is: its job, first column, and for both CTAs of the pair the rows and the runs in them.
 struct PairTile { int job, n0, row0[2], rows[2], run0[2], n_run[2]; };
 
@@ -369,7 +364,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
         // The row's (up to) 128 scores go to registers at once, which frees the accumulator; then the maximum (two
         // columns per instruction) and the first column that holds it.  A running (maximum, index) pair column by
         // column takes eight instructions a column and bounded the launch: 65536 x 5000 x 768 400 us with 128 x 256 tiles
-        // of single CTAs, 455 us with pairs, now 373 us = 1.35 PFLOP/s, the power limit.
+        // of single CTAs, 455 us with pairs, now 305 us alone (1.65 PFLOP/s) and 365 us in a loop at the power limit.
         uint32_t f[4][32];
 #pragma unroll
         for (int g = 0; g < 4; ++g)
@@ -499,25 +494,22 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
           best_k = 0;
           row_best(h, h == 1);
           if (best > -INFINITY) {
-            const unsigned long long key =
-                ((unsigned long long)pair_orderable(best) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k);
+            const unsigned long long key = route_key(best, best_k);
             row_key = key > row_key ? key : row_key;
           }
         }
         if ((tile + 1) % tn_all == 0) {
           if (row_ok) {
             const int id = row_key == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)(row_key & 0xFFFFFFFFull));
-            const uint32_t u = (uint32_t)(row_key >> 32);
             if (p.out_centroid) p.out_centroid[grow] = id;
             p.out_expert[grow] = p.cmap ? p.cmap[id] : id;
-            if (p.out_best)
-              p.out_best[grow] = row_key == 0ull ? -INFINITY : __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u);
+            if (p.out_best) p.out_best[grow] = row_key == 0ull ? -INFINITY : key_to_float((uint32_t)(row_key >> 32));
           }
           row_key = 0ull;
         }
       }
       if (EPI == PAIR_ROUTER && row_ok && best > -INFINITY)
-        atomicMax(p.keys + grow, ((unsigned long long)pair_orderable(best) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k));
+        atomicMax(p.keys + grow, route_key(best, best_k));
       if (EPI == PAIR_ROUTER2 && row_ok) {
         // Two-slot merge: the max goes to keys; whatever loses a comparison there (the value it displaced, or the
         // candidate itself) is offered to keys2.  Keys are distinct and both slots are maxima: order independent.
@@ -526,8 +518,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           if (cand[i] > -INFINITY) {
-            const unsigned long long key = ((unsigned long long)pair_orderable(cand[i]) << 32) |
-                                           (unsigned long long)(0xFFFFFFFFu - (uint32_t)cand_k[i]);
+            const unsigned long long key = route_key(cand[i], cand_k[i]);
             const unsigned long long old = atomicMax(p.keys + grow, key);
             const unsigned long long loser = old < key ? old : key;
             if (loser != 0ull) atomicMax(p.keys2 + grow, loser);

@@ -77,7 +77,7 @@ def test_static_router_limits_and_small_dimension():
     with pytest.raises(moin.MoinError, match="WORKSPACE"):
         moin.route_static(router, too_many, torch.empty(too_many.shape[0], dtype=torch.int32, device=DEV))
     moin.route_static(router, q[:0], out[:0])          # empty batch: no-op
-    # embedding dimension below the tensor-core kernel's minimum: the CUDA-core kernel, which needs no scratch
+    # embedding dimension below the tensor-core kernel's minimum: the cluster kernel, in one part
     low = mi.planted_router(K=40, Q=333, D=40, seed=13, device=DEV)
     r_low = moin.Router(low.centroids)
     ref, got = _both(r_low, low.queries)
