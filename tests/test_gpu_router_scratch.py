@@ -16,7 +16,8 @@ from gpu_util import DEV, assert_router_matches
 pytestmark = pytest.mark.gpu
 
 # cluster kernel (one part; parts of equal and of unequal numbers of tiles, with the reduction split or not; rows too long for
-# 32 queries), GEMM (one column tile of each width; several; more than one block of 256 rows; K above 1024; long rows)
+# 32 queries), GEMM (one column tile of each width; several; more than one block of 256 rows; K above 1024 and above what the
+# cluster kernel takes; long rows), CUDA cores
 SHAPES = [(24, 500, 768), (1, 5000, 768), (8, 5000, 216), (32, 1025, 40), (100, 1030, 384), (3, 13000, 64), (12, 600, 3200),
           (400, 60, 64), (400, 190, 72), (513, 256, 768), (777, 300, 128), (1024, 1024, 768), (1024, 1000, 3168), (385, 1, 64),
           (2000, 30, 200), (9, 7000, 64), (16000, 4, 64)]
@@ -57,6 +58,21 @@ def test_same_bits_without_scratch(Q, K, D):
     ref = oracle.route(mi.bf16_bits(queries[torch.from_numpy(rows)]), mi.bf16_bits(centroids))
     assert_router_matches(c.cpu().numpy()[rows], ref)
     assert moin.device_status()["timeout_flag"] == 0
+
+
+@pytest.mark.parametrize("Q,K,D", [(24, 500, 768), (1, 5000, 768), (8, 5000, 216), (32, 1025, 40), (100, 1030, 384), (3, 12000, 64)])
+def test_runner_up_without_scratch(Q, K, D):
+    # the cluster kernel (up to 2 x 12 parts of 512 topics for a few queries), whose two forms give the same bits
+    case = mi.planted_router(K=K, Q=Q, D=D, seed=61 + Q, unit_centroid_noise=True)
+    router, q = moin.Router(case.centroids.to(DEV)), case.queries.to(DEV)
+    want = moin.route_top2(router, q)
+    got = {k: torch.full_like(v, 7) for k, v in want.items()}
+    st = moin.lib().moin_route_top2(ctypes.byref(router.c), q.data_ptr(), Q, *[got[k].data_ptr() for k in ("expert", "centroid", "second", "best", "margin")],
+                                    None, 0, binding._stream(None))
+    assert st == 0 and all(torch.equal(got[k], want[k]) for k in want)
+    ref = oracle.route(mi.bf16_bits(case.queries), mi.bf16_bits(case.centroids))
+    assert_router_matches(got["centroid"].cpu().numpy(), ref)
+    assert (np.abs(got["margin"].cpu().numpy() - ref["margin"]) <= 2e-5).all()
 
 
 def test_static_calls_overlap():
