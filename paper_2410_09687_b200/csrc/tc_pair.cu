@@ -89,37 +89,50 @@ __device__ __forceinline__ PairTile pair_tile(const PairParams& p, int tile, int
 // pass i (SWIGLU: lanes 8 .. 15 for the up projection), and leaves the result in shared memory.  (In the producer and the
 // MMA warp themselves, at the start of a tile or in steps between the quarters of its main loop, it cost 2 to 5 percent.)
 constexpr int kPairPasses = 2 * kTileRuns;
-struct PairPass { int slot, rank, rows[2]; };   // adapter or -1; per CTA the run's rows of the tile: first | end << 16
-constexpr uint32_t kPairTabBytes = 2 * kPairPasses * sizeof(PairPass) + 16;   // passes, then their number
-__device__ __forceinline__ void pair_passes(const PairParams& p, const PairTile& t, bool two_jobs, int lane, uint8_t* tab) {
+// What the passes leave out stands there word for word as the MMAs take it.
+struct PairTable {
+  struct { int slot, rank; } pass[2 * kPairPasses];   // adapter or -1, its rank
+  uint32_t out[kPairPasses][8];                       // accumulator rows of other runs, first CTA's then second's
+  int n, has[2], pad;                                 // passes; bit i: the CTA has rows of pass i's run
+};
+// disable-output-lane word of 32 accumulator rows of which first .. end - 1 (counted from the word's first row) take part
+__device__ __forceinline__ uint32_t lanes_out(int first, int end) {
+  const uint32_t below_end = end <= 0 ? 0u : end >= 32 ? ~0u : (1u << end) - 1u;
+  const uint32_t below_first = first <= 0 ? 0u : first >= 32 ? ~0u : (1u << first) - 1u;
+  return ~(below_end & ~below_first);
+}
+__device__ __forceinline__ void pair_passes(const PairParams& p, const PairTile& t, bool two_jobs, int lane, PairTable* tab) {
   const int shared = t.n_run[0] > 0 && t.n_run[1] > 0 && t.run0[0] + t.n_run[0] - 1 == t.run0[1];
   const int n = t.n_run[0] + t.n_run[1] - shared;
   const int i = lane % kPairPasses, job = two_jobs ? lane / kPairPasses : t.job;
+  const int run = i < t.n_run[0] ? t.run0[0] + i : t.run0[1] + i - t.n_run[0] + shared;
+  bool has = false;
   if (lane < (two_jobs ? 2 : 1) * kPairPasses && i < n) {
-    const int run = i < t.n_run[0] ? t.run0[0] + i : t.run0[1] + i - t.n_run[0] + shared;
-    const int r0 = __ldg(p.run_row0 + run), r1 = __ldg(p.run_row0 + run + 1);
-    PairPass q = {-1, p.tail_r, {0, 0}};
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-      q.rows[c] = min(max(r0 - t.row0[c], 0), t.rows[c]) | min(max(r1 - t.row0[c], 0), t.rows[c]) << 16;
+    int slot = -1, rank = p.tail_r;
     const int* slots = p.slot_of_expert[0];
     const int* ranks = p.slot_rank[0];
 #pragma unroll
     for (int j = 1; j < kPairJobs; ++j)
       if (job == j) { slots = p.slot_of_expert[j]; ranks = p.slot_rank[j]; }
     const int e = __ldg(p.run_expert + run);
-    if (e >= 0) q.slot = __ldg(slots + e);
-    if (q.slot >= 0 && ranks) q.rank = min(__ldg(ranks + q.slot), p.tail_r);
-    reinterpret_cast<PairPass*>(tab)[lane] = q;
+    if (e >= 0) slot = __ldg(slots + e);
+    if (slot >= 0 && ranks) rank = min(__ldg(ranks + slot), p.tail_r);
+    tab->pass[lane].slot = slot;
+    tab->pass[lane].rank = rank;
+  } else if (lane >= 2 * kPairPasses && i < n) {   // lanes 16 .. 23: the first CTA's rows, 24 .. 31: the second's
+    const int c = lane >= 3 * kPairPasses;
+    const int row0 = c ? t.row0[1] : t.row0[0], rows = c ? t.rows[1] : t.rows[0];
+    const int first = __ldg(p.run_row0 + run) - row0, end = min(__ldg(p.run_row0 + run + 1) - row0, rows);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) tab->out[i][4 * c + w] = lanes_out(first - 32 * w, end - 32 * w);
+    has = first < rows && end > 0;
   }
-  if (lane == 0) *reinterpret_cast<int*>(tab + 2 * kPairPasses * sizeof(PairPass)) = n;
-}
-
-// disable-output-lane word of 32 accumulator rows of which first .. end - 1 (counted from the word's first row) take part
-__device__ __forceinline__ uint32_t lanes_out(int first, int end) {
-  const uint32_t below_end = end <= 0 ? 0u : end >= 32 ? ~0u : (1u << end) - 1u;
-  const uint32_t below_first = first <= 0 ? 0u : first >= 32 ? ~0u : (1u << first) - 1u;
-  return ~(below_end & ~below_first);
+  const uint32_t in = __ballot_sync(0xffffffffu, has);
+  if (lane == 0) {
+    tab->n = n;
+    tab->has[0] = (int)(in >> (2 * kPairPasses)) & ((1 << kPairPasses) - 1);
+    tab->has[1] = (int)(in >> (3 * kPairPasses));
+  }
 }
 
 template <int EPI>
@@ -138,8 +151,8 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
   constexpr bool kTail = EPI == PAIR_STORE || EPI == PAIR_SWIGLU;   // low-rank blocks at the end of a tile
   // pass tables of this and the next tile, their barriers: written, and read to the end by this CTA's producer
   const uint32_t tab0 = bars + 16 * S + 48, tabread0 = tab0 + 16;
-  uint8_t* tab_ptr = bar_ptr + 256;
-  static_assert(256 + 2 * kPairTabBytes <= 1024, "barrier block");
+  PairTable* tabs = reinterpret_cast<PairTable*>(bar_ptr + 192);
+  static_assert(16 * S + 80 <= 192 && 192 + 2 * sizeof(PairTable) <= 1024 && sizeof(PairTable) % 16 == 0, "barrier block");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
 
@@ -206,16 +219,16 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
         }
         if (!kTail || p.tail_r == 0 || !ok) continue;
         if (!(ok = mbar_wait(tab0 + 8 * (lt & 1u), (lt >> 1) & 1u, abort_flag, p.status, 65))) break;
-        const volatile PairPass* pass = reinterpret_cast<const volatile PairPass*>(tab_ptr + (lt & 1u) * kPairTabBytes);
-        const int n_pass = *reinterpret_cast<const volatile int*>(pass + 2 * kPairPasses);
-        for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g, pass += kPairPasses) {
+        const volatile PairTable* tab = tabs + (lt & 1u);
+        const int n_pass = tab->n, has = tab->has[rank];
+        for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g) {
           const int job = EPI == PAIR_SWIGLU ? g : t.job;
           int n = p.N[0];
 #pragma unroll
           for (int jj = 1; jj < kPairJobs; ++jj)
             if (job == jj) n = p.N[jj];
           for (int i = 0; i < n_pass && ok; ++i) {
-            const int slot = pass[i].slot;
+            const int slot = tab->pass[g * kPairPasses + i].slot;
             if (slot < 0) continue;
             const int b0 = slot * n + t.n0 + (int)rank * (p.cols / 2);
             for (int j = 0; j < 2 * nrb; ++j, ++it) {
@@ -225,7 +238,9 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
               const uint32_t bar = map_rank(full0 + 8 * s, 0);
               if (rank == 0) mbar_expect_tx(full0 + 8 * s, tx_tail);
               const int lo = j >= nrb ? 1 : 0, rb = j - lo * nrb;   // hi blocks first, then lo blocks
-              tma_load_2d_pair(sa, &maps.h[job], bar, rb * kPairK, lo * p.M + row0);   // (all rows: the MMAs choose)
+              // all rows of the tile: the MMAs choose; a CTA without any of the run's starts past the last: nothing is read
+              // (14 prompts of 202 to 262 tokens, rank 8, gate/up launch 121 us when it reads them, 117 so)
+              tma_load_2d_pair(sa, &maps.h[job], bar, rb * kPairK, (has >> i) & 1 ? lo * p.M + row0 : 2 * p.M);
               tma_load_2d_pair(sb, &maps.b[job], bar, rb * kPairK, b0);
             }
           }
@@ -267,19 +282,16 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
         }
         if (kTail && p.tail_r > 0 && ok) {
           if (!(ok = mbar_wait_warp(tab0 + 8 * (lt & 1u), (lt >> 1) & 1u, abort_flag, p.status, 66))) break;
-          const volatile PairPass* pass = reinterpret_cast<const volatile PairPass*>(tab_ptr + (lt & 1u) * kPairTabBytes);
-          const int n_pass = *reinterpret_cast<const volatile int*>(pass + 2 * kPairPasses);
-          for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g, pass += kPairPasses) {
+          const volatile PairTable* tab = tabs + (lt & 1u);
+          const int n_pass = tab->n;
+          for (int g = 0; g < (EPI == PAIR_SWIGLU ? 2 : 1) && ok; ++g) {
             const uint32_t tmem_g = tmem_d + g * (p.bn / 2);
             for (int i = 0; i < n_pass && ok; ++i) {
-              const int slot = pass[i].slot, rk = pass[i].rank;
+              const int slot = tab->pass[g * kPairPasses + i].slot, rk = tab->pass[g * kPairPasses + i].rank;
               if (slot < 0) continue;
-              uint32_t out[8];   // rows of the other runs, first CTA's then second's
-#pragma unroll
-              for (int w = 0; w < 8; ++w) {
-                const int rows = pass[i].rows[w >> 2];
-                out[w] = lanes_out((rows & 0xFFFF) - 32 * (w & 3), (rows >> 16) - 32 * (w & 3));
-              }
+              const uint32_t words = bars + 192 + (lt & 1u) * (uint32_t)sizeof(PairTable) + (uint32_t)offsetof(PairTable, out) + 32u * i;
+              const uint4 first = lds_u4(words), second = lds_u4(words + 16);
+              const uint32_t out[8] = {first.x, first.y, first.z, first.w, second.x, second.y, second.z, second.w};
               for (int j = 0; j < 2 * nrb; ++j, ++it) {
                 const uint32_t s = it % S, ph = (it / S) & 1u;
                 if (!(ok = mbar_wait_cluster_warp(full0 + 8 * s, ph, abort_flag, p.status, 63))) break;
@@ -315,7 +327,7 @@ tc_pair_kernel(const __grid_constant__ PairMaps maps, const PairParams p) {
     // may be passes without an adapter, which no copy and so no accumulator depends on: it says when it has read them.
     auto scout = [&](const PairTile& n, uint32_t i) -> bool {
       if (!mbar_wait_warp(tabread0 + 8 * (i & 1u), ((i >> 1) & 1u) ^ 1u, abort_flag, p.status, 67)) return false;
-      pair_passes(p, n, EPI == PAIR_SWIGLU, lane, tab_ptr + (i & 1u) * kPairTabBytes);
+      pair_passes(p, n, EPI == PAIR_SWIGLU, lane, tabs + (i & 1u));
       __syncwarp();
       if (lane == 0) mbar_arrive(tab0 + 8 * (i & 1u));
       return true;
