@@ -426,6 +426,19 @@ static DecoderWorkspace carve(const moin_model* m, int R, int T, int max_seqlen,
   return w;
 }
 
+// One expert per request: tiles or segments for T tokens of R requests?  Tiles pay a pass over a row tile for every run in it, and
+// on an 8-bit base the conversion of all weights (0.6 ms a forward); segments read an adapter again for every eight tokens.
+// Segments / tiles, ms a forward, rank 16; 64: 2 x 64 tokens 1.83 / 2.59; 1.91 / 2.75, 3 x 100 2.88 / 3.01; 3.09 / 3.17, 4 x 100
+// 3.37 / 3.10; 3.68 / 3.28, 10 x 100 5.65 / 3.65; 6.83 / 3.94; 12 x 40 3.25 / 3.67; 3.99 / 3.54, 20 x 40 4.39 / 4.59; 6.20 / 4.67;
+// 28 x 36 5.30 / 5.97; 7.23 / 6.09; 71 x 28 (segments beyond kDecodeSegMaxT) 10.2 / 9.7; 14.1 / 10.4.  8-bit base: 2 x 64 1.82 / 3.55;
+// 2.02 / 3.69, 5 x 100 3.38 / 4.20; 4.13 / 4.38, 8 x 100 4.91 / 4.75; 6.12 / 5.04, 25 x 56 6.77 / 6.39 (rank 16).
+static bool forward_tiles(int T, int R, bool coded) {
+  const int mean = T / R;
+  if (mean >= 64) return T >= (coded ? 600 : 384);
+  if (T > kDecodeSegMaxT) return mean >= 28;
+  return mean >= 40 && T >= (coded ? 1400 : 480);
+}
+
 }  // namespace moin
 
 using namespace moin;
@@ -472,7 +485,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     plan.buffer = w.plan; plan.buffer_bytes = w.plan_bytes; plan.T = T; plan.E = m->E;
     // one expert per request: the run lengths are the request lengths; one per token: they depend on the ids, so
     // the plan decides after it has grouped them (reads its header back: one synchronisation of the stream)
-    plan.mode = token_expert_in ? MOIN_PLAN_AUTO : ((T / R >= 64) ? MOIN_PLAN_TILES : MOIN_PLAN_SEGMENTS);
+    plan.mode = token_expert_in ? MOIN_PLAN_AUTO : (forward_tiles(T, R, m->W8 != nullptr) ? MOIN_PLAN_TILES : MOIN_PLAN_SEGMENTS);
     st = moin_plan_build(w.token_expert, &plan, stream);
     if (st) return st;
   }
@@ -503,10 +516,11 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     }
     return dq.n ? launch_dequant(dq, d_in, s) : MOIN_OK;
   };
+  const int max_adapters = token_expert_in ? T : R;
   // projections of a block that read the same input and do not depend on one another go out as one group
   auto proj_group = [&](int layer, int p0, int n, const void* in, int d_in, const int* d_out, void* const* outs) -> moin_status {
     // few tokens in short segments: the GEMM converts the codes itself (gemm_decode.cu has both sides' times)
-    bool coded = m->W8 && decode_fp8_supported(hs, T) && (!lora || plan.mode == MOIN_PLAN_SEGMENTS);
+    bool coded = m->W8 && decode_fp8_supported(hs, T, lora) && (!lora || plan.mode == MOIN_PLAN_SEGMENTS);
     for (int j = 0; j < n && coded; ++j) coded = m->W8[layer * 7 + p0 + j] && m->W_scale && m->W_scale[layer * 7 + p0 + j];
     if (coded) {
       moin_lora_job jobs[MOIN_MAX_GROUP];
@@ -517,9 +531,9 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
         if (lora) jobs[j] = {in, m->W8[i], &m->pools[i], outs[j]};
         else gemm[j] = {(const __nv_bfloat16*)in, m->W8[i], (__nv_bfloat16*)outs[j], nullptr, d_in, d_out[j], m->W_scale[i]};
       }
-      if (lora) return lora_linear_group(&plan, jobs, m->W_scale + layer * 7 + p0, n, m->lora_scale, w.lora, w.lora_bytes, stream);
+      if (lora) return lora_linear_group(&plan, jobs, m->W_scale + layer * 7 + p0, n, max_adapters, m->lora_scale, w.lora, w.lora_bytes, stream);
       ProfScope prof(MOIN_K_GEMM_TC, 1, s);
-      return launch_decode_gemm(hs, gemm, n, T, s);
+      return launch_decode_gemm(hs, gemm, n, T, false, s);
     }
     const void* W[MOIN_MAX_GROUP];
     moin_status e = weights(layer, p0, n, d_in, d_out, W);
@@ -533,7 +547,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
         jobs[i] = {in, W[i], &m->pools[layer * 7 + p0 + i], outs[i]};
       }
     }
-    return lora ? moin_lora_linear_group(&plan, jobs, n, m->lora_scale, w.lora, w.lora_bytes, stream) : MOIN_OK;
+    return lora ? lora_linear_group(&plan, jobs, nullptr, n, max_adapters, m->lora_scale, w.lora, w.lora_bytes, stream) : MOIN_OK;
   };
   const float scale_log2 = 1.4426950408889634f / sqrtf(64.f);
   const __nv_bfloat16* pending = nullptr;

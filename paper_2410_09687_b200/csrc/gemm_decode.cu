@@ -237,7 +237,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   }
 }
 
-moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, cudaStream_t stream) {
+moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, bool small_tiles, cudaStream_t stream) {
   DgMaps maps;
   DgParams p = {};
   p.n_jobs = n_jobs; p.T = T; p.status = hs->status;
@@ -248,10 +248,13 @@ moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_j
   // SMs, whatever the tokens (forwards of 112 / 303 / 495 tokens with half 1933 / 3263 / 4020 us, all 1871 / 2665 /
   // 3525, twice 1992 / 2795 / 3516).
   const bool fp8 = jobs[0].w_scale != nullptr;
-  const int max_n = fp8 ? kDgFp8MaxN : kDgMaxN;
+  // A few narrow adapters leave the memory to the GEMM, and its tiles of 64 tokens, two CTAs an SM, the epilogues short: forwards
+  // in segments of 24 tokens, tiles of up to 256 / of 64, ms: rank 16 288 tokens 2.81 / 2.51, 504 3.75 / 3.32, 792 5.04 / 4.39, 1392
+  // 6.97 / 6.86, 1992 8.72 / 9.82; rank 32 2.86 / 2.58, 3.87 / 3.52, 5.30 / 4.77; rank 64 504 4.41 / 4.30, 1008 7.33 / 7.42.
+  const int max_n = small_tiles ? 64 : fp8 ? kDgFp8MaxN : kDgMaxN;
   const int chunks0 = (T + max_n - 1) / max_n;
   const bool small = (T + chunks0 - 1) / chunks0 <= 64;
-  const int limit = fp8 ? hs->n_sms : small ? 2 * hs->n_sms : hs->n_sms / 2;
+  const int limit = fp8 || (small_tiles && T > 512) ? hs->n_sms : small ? 2 * hs->n_sms : hs->n_sms / 2;
   int items = 0;   // CTAs with one token tile per 256 tokens
   p.cluster = 1;
   for (int j = 0; j < n_jobs; ++j) {

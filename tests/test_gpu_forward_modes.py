@@ -1,0 +1,50 @@
+"""Decoder forwards on both sides of the rules that choose between segments and tiles, and in segments between the kernels of
+the base GEMM: tokens and mean lengths at their edges, block by block against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import moin_inputs as mi
+import oracle
+import paper_2410_09687_b200 as moin
+from gpu_util import DEV, REL_FRO
+from test_gpu_decoder import gpu_model, oracle_weights, rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("r", [16, 40])
+@pytest.mark.parametrize("lengths", [[64] * 5 + [63], [64] * 6, [40] * 11 + [39], [40] * 12, [6] * 43, [24] * 22, [9] * 170, [28] * 73,
+                                     [27] * 76, [29] * 71])
+def test_block(lengths, r):
+    cfg = mi.DecoderConfig(n_layers=1, hidden=256, n_heads=4, n_kv_heads=2, head_dim=64, ffn=576, vocab=512, E=9, r=r, scale=2.0)
+    model = mi.decoder_model(cfg, seed=23, missing=(4,))
+    orc = oracle.DecoderOracle(cfg, oracle_weights(model))
+    batch = mi.decoder_batch(cfg, lengths, seed=r, req_expert=[(5 * i) % 10 - 1 for i in range(len(lengths))])
+    args = (batch.tokens.numpy(), batch.cu_seqlens.numpy(), batch.req_expert.numpy())
+    h_in = orc.forward(*args, layer_begin=0, layer_end=0, want_hidden=True, want_logits=False)["hidden"]
+    ref = orc.forward(*args, layer_begin=0, layer_end=1, round_storage=True, hidden_in=h_in, want_hidden=True, want_logits=False)["hidden"]
+    hin = torch.from_numpy(h_in).to(torch.float32).to(DEV)
+    hid = torch.empty(batch.T, cfg.hidden, dtype=torch.float32, device=DEV)
+    moin.decoder_forward(gpu_model(model), batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths),
+                         logits_mode=moin.LOGITS_NONE, hidden_in=hin, hidden_out=hid)
+    assert moin.device_status()["timeout_flag"] == 0
+    # as test_gpu_decoder's blocks: one block against the oracle that rounds where the library stores
+    assert rel(hid.double().cpu().numpy() - hin.double().cpu().numpy(), ref - h_in) <= REL_FRO
+
+
+@pytest.mark.parametrize("lengths", [[37] * 56, [9] * 70, [2] * 513])   # codes converted by the GEMM beyond 512 tokens, and no longer
+def test_coded_base(lengths):
+    from test_gpu_quant import quantise
+    from test_gpu_quant_group import _decoder
+    cfg = mi.DecoderConfig(n_layers=1, hidden=320, n_heads=5, n_kv_heads=1, head_dim=64, ffn=1088, vocab=512, E=4, r=16, scale=2.0)
+    model = mi.decoder_model(cfg, seed=4)
+    q = {p: quantise(model.W[0][p]) for p in oracle.PROJ_ORDER}
+    same = {p: torch.from_numpy(oracle.dequant_fp8(c.numpy(), s.numpy()).view(np.int16)).view(torch.bfloat16).to(DEV) for p, (c, s) in q.items()}
+    coded = _decoder(cfg, model, [{}], [{p: c.to(DEV) for p, (c, s) in q.items()}], [{p: s.to(DEV) for p, (c, s) in q.items()}])
+    batch = mi.decoder_batch(cfg, lengths, seed=6, req_expert=[i % 4 for i in range(len(lengths))])
+    args = [batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths)]
+    got, want = (moin.decoder_forward(m, *args).double() for m in (coded, _decoder(cfg, model, [same])))
+    # the same bf16 weights, sums of 32-bit products in another order: two bf16 roundings of a chain of four projections
+    assert ((got - want).norm() / want.norm()).item() <= REL_FRO * 2 ** 0.5
+    assert moin.device_status()["timeout_flag"] == 0
