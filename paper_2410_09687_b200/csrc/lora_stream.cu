@@ -13,8 +13,11 @@
 
 namespace moin {
 
-constexpr int kShrinkThreads = 128;      // 4 warps split the reduction dimension
-constexpr int kShrinkWarps = kShrinkThreads / 32;
+// Warps that split the reduction: four, so that the CTAs of many items share an SM; up to kShrinkFewT tokens, whose items leave
+// the SMs empty and whose time is a warp's chain of loads, eight.  Decode step of 6 tokens of rank 16 60.0 -> 55.3 us, of one of
+// rank 64 53.8 -> 52.8, forward of 14 tokens on the 8-bit base 1465 -> 1383; with eight throughout 100 tokens 135.7 -> 137.2, 256
+// 230 -> 246, forward of 112 tokens 1829 -> 1872; with sixteen 12 tokens and more are slower.
+constexpr int kShrinkWarps = 4, kShrinkFewWarps = 8, kShrinkFewT = 16;
 constexpr int kShrinkUnroll = 4;         // 32-wide k steps in flight per warp
 constexpr int kExpandThreads = 128;      // 4 warps
 constexpr int kExpandFirst = 4;          // 16-row tiles prefetched while a warp waits for the shrink
@@ -81,10 +84,11 @@ __device__ __forceinline__ SegMeta load_seg(const int4* __restrict__ chunk_tab, 
 // the hardware's block scheduler hands the items out as slots free up, so a launch ends evenly whatever
 // the base GEMM beside it occupies, and a CTA's metadata hops (segment count, table entry,
 // slot) hide behind the streams of the other CTAs on its SM.
-__global__ void __launch_bounds__(kShrinkThreads, 6)
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 24 / WARPS)
 lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict__ perm,
                           const int4* __restrict__ chunk_tab, const ShrinkJobs jobs) {
-  __shared__ float red[kShrinkWarps][32][4];
+  __shared__ float red[WARPS][32][4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   pdl_launch_dependents();
@@ -112,12 +116,12 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
       const bool vx = g < cur.n;
       float c[4] = {0.f, 0.f, 0.f, 0.f};
       const __nv_bfloat16* x_row = nullptr;
-      for (int base = 0; base < steps; base += kShrinkWarps * kShrinkUnroll) {
+      for (int base = 0; base < steps; base += WARPS * kShrinkUnroll) {
         uint4 a0[kShrinkUnroll], a1[kShrinkUnroll], xv[kShrinkUnroll];
         const uint4 z = make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int u = 0; u < kShrinkUnroll; ++u) {  // adapter bytes first: they come from HBM
-          const int i = base + u * kShrinkWarps + warp;
+          const int i = base + u * WARPS + warp;
           const bool vi = i < steps;
           a0[u] = (vi && v0) ? ldg_stream(a_row0 + i * 32) : z;
           a1[u] = (vi && v1) ? ldg_stream(a_row1 + i * 32) : z;
@@ -125,7 +129,7 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
         if (x_row == nullptr) x_row = x + (size_t)(vx ? perm[cur.s0 + g] : 0) * (size_t)d_in + 8 * t;
 #pragma unroll
         for (int u = 0; u < kShrinkUnroll; ++u) {
-          const int i = base + u * kShrinkWarps + warp;
+          const int i = base + u * WARPS + warp;
           xv[u] = (i < steps && vx) ? ldg_cached(x_row + i * 32) : z;
         }
 #pragma unroll
@@ -145,7 +149,7 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
         for (int j = 0; j < 4; ++j) {
           float acc = red[0][lane][j];
 #pragma unroll
-          for (int w = 1; w < kShrinkWarps; ++w) acc += red[w][lane][j];
+          for (int w = 1; w < WARPS; ++w) acc += red[w][lane][j];
           s[j] = acc;
         }
         // c0:(rho0, col 2t) c1:(rho0, col 2t+1) c2:(rho1, col 2t) c3:(rho1, col 2t+1)
@@ -359,8 +363,11 @@ cudaError_t launch_lora_shrink_stream(const PlanView& pv, ShrinkJobs jobs, int n
     items += (long)pv.Cmax * jobs.per_seg[j];
   }
   // one CTA per item (capped; CTAs stride over the items beyond the cap)
-  return launch_pdl(lora_shrink_stream_kernel, stream_grid(items, n_sms, 1024), kShrinkThreads, 0, stream, pv.header,
-                    pv.perm, pv.chunk_tab, jobs);
+  auto go = [&](auto* fn, int warps) {
+    return launch_pdl(fn, stream_grid(items, n_sms, 1024), 32 * warps, 0, stream, pv.header, pv.perm, pv.chunk_tab, jobs);
+  };
+  return pv.T <= kShrinkFewT ? go(lora_shrink_stream_kernel<kShrinkFewWarps>, kShrinkFewWarps)
+                             : go(lora_shrink_stream_kernel<kShrinkWarps>, kShrinkWarps);
 }
 
 cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float scale, int n_sms,
