@@ -560,7 +560,7 @@ static moin_status launch_base_gemm(HostState* hs, bool use_tc, const __nv_bfloa
   if (!use_tc) return record_cuda(launch_gemm_warp(x, W, y, y0, T, d_in, d_out, s));
   if (decode_gemm_wins(T, d_in, d_out)) {
     const DecodeGemmJob job = {x, W, y, y0, d_in, d_out, nullptr};
-    return launch_decode_gemm(hs, &job, 1, T, false, s);
+    return launch_decode_gemm(hs, &job, 1, T, false, false, s);
   }
   const PairJob job = {x, W, nullptr, y, y0, nullptr, d_out};
   return launch_pair_gemm(hs, nullptr, &job, 1, T, d_in, s);
@@ -576,13 +576,13 @@ size_t moin_lora_linear_group_workspace_bytes(int32_t T, const moin_lora_job* jo
 
 moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, int32_t n_jobs, float scale,
                                    void* workspace, size_t workspace_bytes, moin_stream stream) {
-  return lora_linear_group(plan, jobs, nullptr, n_jobs, plan ? plan->T : 0, scale, workspace, workspace_bytes, stream);
+  return lora_linear_group(plan, jobs, nullptr, n_jobs, plan ? plan->T : 0, false, scale, workspace, workspace_bytes, stream);
 }
 
 }  // extern "C"
 
 moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, const float* const* w_scale,
-                                    int n_jobs, int max_adapters, float scale, void* workspace, size_t workspace_bytes,
+                                    int n_jobs, int max_adapters, bool w_early, float scale, void* workspace, size_t workspace_bytes,
                                     moin_stream stream) {
   if (!plan || !jobs || n_jobs < 1 || n_jobs > MOIN_MAX_GROUP) return MOIN_ERR_INVALID_ARG;
   int T = 0, d_in[kMaxStreamJobs], d_out[kMaxStreamJobs], r[kMaxStreamJobs];
@@ -670,7 +670,7 @@ moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* 
     // few narrow adapters in a batch of some size (gemm_decode.cu has the figures)
     bool small_tiles = !w_scale && T > 256 && T <= 1536 && 6ll * max_adapters <= T;
     for (int j = 0; j < n_jobs; ++j) small_tiles = small_tiles && r[j] <= 32;
-    st = launch_decode_gemm(hs, gj, n_jobs, T, small_tiles, s);
+    st = launch_decode_gemm(hs, gj, n_jobs, T, small_tiles, w_early, s);
   } else {
     for (int j = 0; j < n_jobs && !st; ++j)
       st = launch_base_gemm(hs, use_tc[j], (const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W,

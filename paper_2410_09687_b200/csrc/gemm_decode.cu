@@ -31,7 +31,7 @@ constexpr int kDgFp8MaxN = 128, kDgFp8Cols = 256, kDgFp8Smem = 104 * 1024;
 
 struct DgMaps { CUtensorMap w[kMaxStreamJobs], x[kMaxStreamJobs]; };
 struct DgParams {
-  int n_jobs, T, nt, n_chunks, stages, tmem_cols, cluster;   // nt tokens per tile, n_chunks tiles over the tokens
+  int n_jobs, T, nt, n_chunks, stages, tmem_cols, cluster, w_early;   // nt tokens per tile, n_chunks tiles over the tokens
   int cta_end[kMaxStreamJobs];   // CTAs of jobs 0 .. j (each job's padded to whole clusters)
   int ks[kMaxStreamJobs], tiles[kMaxStreamJobs], K[kMaxStreamJobs], d_out[kMaxStreamJobs];
   __nv_bfloat16* y[kMaxStreamJobs];
@@ -79,6 +79,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   const bool on = tile < n_tiles;                                      // (the last cluster of a job may be padded)
   const int tok0 = (item - tile * p.n_chunks) * p.nt, f0 = tile * kDgM;
   const int nkb = on ? K / kDgK : 0, kb0 = nkb * rank / ks, kb1 = nkb * (rank + 1) / ks;
+  const int n_early = p.w_early ? min(S, kb1 - kb0) : 0;   // k-blocks whose weights do not wait for the kernel before
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -89,6 +90,12 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
     mbar_init(done, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // Weights older than the kernel before this one (the caller knows): the first stages' are on their way while that one ends.
+    // Forward of 112 tokens on the 8-bit base 1829 -> 1777 us, on the bf16 base 1751 -> 1744, of 14 tokens 1465 -> 1451.
+    for (int s = 0; s < n_early; ++s) {
+      mbar_expect_tx(full0 + 8 * s, stage_bytes);
+      tma_load_2d(ring + s * stage_bytes, &maps.w[job], full0 + 8 * s, (kb0 + s) * kDgK, f0);
+    }
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(tmem_slot), p.tmem_cols);
@@ -112,8 +119,10 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
         if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 51)) break;
         const uint32_t sa = ring + s * stage_bytes, full = full0 + 8 * s;
         if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
-        mbar_expect_tx(full, stage_bytes);
-        tma_load_2d(sa, mw, full, kb * kDgK, f0);
+        if (kb - kb0 >= n_early) {
+          mbar_expect_tx(full, stage_bytes);
+          tma_load_2d(sa, mw, full, kb * kDgK, f0);
+        }
         tma_load_2d(sa + kWBytes, mx, full, kb * kDgK, tok0);
       }
     }
@@ -237,10 +246,10 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   }
 }
 
-moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, bool small_tiles, cudaStream_t stream) {
+moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, bool small_tiles, bool w_early, cudaStream_t stream) {
   DgMaps maps;
   DgParams p = {};
-  p.n_jobs = n_jobs; p.T = T; p.status = hs->status;
+  p.n_jobs = n_jobs; p.T = T; p.status = hs->status; p.w_early = w_early;
   // Split a projection's reduction until its own CTAs fill their share of the SM slots or a CTA is down to four 64-wide
   // blocks (from the shape alone: the same bits in any group).  Beside many tokens' adapters the share is half of the
   // SMs (decode step of 256 tokens with half / all / a quarter: 237 / 264 / 248 us); up to 64 tokens two CTAs fit an SM
