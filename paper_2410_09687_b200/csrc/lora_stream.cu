@@ -13,12 +13,13 @@
 
 namespace moin {
 
-// Warps that split the reduction: four, so that the CTAs of many items share an SM; up to kShrinkFewT tokens, whose items leave
-// the SMs empty and whose time is a warp's chain of loads, eight.  Decode step of 6 tokens of rank 16 60.0 -> 55.3 us, of one of
-// rank 64 53.8 -> 52.8, forward of 14 tokens on the 8-bit base 1465 -> 1383; with eight throughout 100 tokens 135.7 -> 137.2, 256
-// 230 -> 246, forward of 112 tokens 1829 -> 1872; with sixteen 12 tokens and more are slower.
-constexpr int kShrinkWarps = 4, kShrinkFewWarps = 8, kShrinkFewT = 16;
-constexpr int kShrinkUnroll = 4;         // 32-wide k steps in flight per warp
+// Four warps split the reduction, 32-wide k steps dealt to them in turn.  Many items: 16 adapter rows an item and four steps a warp
+// in flight, so that six CTAs share an SM.  Up to kShrinkFewT tokens the items leave the SMs empty and the time is a warp's chain
+// of loads: half the rows an item (the other half of the MMA's rows idle) and twice the steps in flight, the sums of a row in the
+// same order.  Decode steps, us, many / few: 6 tokens of rank 16 54.8 / 53.1, of rank 64 61.4 / 57.9, 16 of rank 64 80.6 / 74.2, 1 of
+// rank 128 60.1 / 55.3; forward of 14 tokens on the 8-bit base 1440 / 1360, of 6 1379 / 1239.  (Eight warps: as fast, but another
+// order of the sums; with more tokens they are slower: 256 tokens 230 -> 246.)
+constexpr int kShrinkWarps = 4, kShrinkFewT = 16;
 constexpr int kExpandThreads = 128;      // 4 warps
 constexpr int kExpandFirst = 4;          // 16-row tiles prefetched while a warp waits for the shrink
 
@@ -79,16 +80,16 @@ __device__ __forceinline__ SegMeta load_seg(const int4* __restrict__ chunk_tab, 
 }
 
 // h[pos][rho] = sum_i A[slot][rho][i] * x[perm[pos]][i]      (fp32, pos = position in sorted order)
-// Work item = (job, chunk, group of 16 adapter rows); the CTA's warps interleave over k.
+// Work item = (job, chunk, group of ROWS adapter rows: 16, or 8); the CTA's warps interleave over k.
 // Small CTAs (4 warps, 80 registers: six per SM, and room beside a base-GEMM CTA) and one CTA per item:
 // the hardware's block scheduler hands the items out as slots free up, so a launch ends evenly whatever
 // the base GEMM beside it occupies, and a CTA's metadata hops (segment count, table entry,
 // slot) hide behind the streams of the other CTAs on its SM.
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, 24 / WARPS)
+template <int ROWS, int UNROLL>
+__global__ void __launch_bounds__(kShrinkWarps * 32, UNROLL == 4 ? 6 : 3)
 lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict__ perm,
                           const int4* __restrict__ chunk_tab, const ShrinkJobs jobs) {
-  __shared__ float red[WARPS][32][4];
+  __shared__ float red[kShrinkWarps][32][4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   pdl_launch_dependents();
@@ -102,38 +103,38 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
   for (; item < items; item += gridDim.x) {
     const SegMeta cur = nxt;
     nxt = load_seg(chunk_tab, jobs, item + gridDim.x, items, nchunk);  // lookahead
-    if (cur.slot < 0 || cur.sub * 16 >= cur.r_use) continue;  // uniform per CTA: no adapter, or rows beyond its rank
+    if (cur.slot < 0 || cur.sub * ROWS >= cur.r_use) continue;  // uniform per CTA: no adapter, or rows beyond its rank
     const int r = pick(jobs.r, cur.job), d_in = pick(jobs.d_in, cur.job);
     const __nv_bfloat16* __restrict__ x = pick(jobs.x, cur.job);
     const __nv_bfloat16* __restrict__ A = pick(jobs.A, cur.job);
     float* __restrict__ h = pick(jobs.h, cur.job);
     const int steps = d_in >> 5;  // 32 k per step
-    const int rho0 = cur.sub * 16 + g, rho1 = rho0 + 8;
-    const bool v0 = rho0 < cur.r_use, v1 = rho1 < cur.r_use;   // rows beyond the slot's rank are not read
+    const int rho0 = cur.sub * ROWS + g, rho1 = rho0 + 8;
+    const bool v0 = rho0 < cur.r_use, v1 = ROWS == 16 && rho1 < cur.r_use;   // rows beyond the slot's rank are not read
     const __nv_bfloat16* a_row0 = A + ((size_t)cur.slot * r + (v0 ? rho0 : 0)) * (size_t)d_in + 8 * t;
     const __nv_bfloat16* a_row1 = A + ((size_t)cur.slot * r + (v1 ? rho1 : 0)) * (size_t)d_in + 8 * t;
     {
       const bool vx = g < cur.n;
       float c[4] = {0.f, 0.f, 0.f, 0.f};
       const __nv_bfloat16* x_row = nullptr;
-      for (int base = 0; base < steps; base += WARPS * kShrinkUnroll) {
-        uint4 a0[kShrinkUnroll], a1[kShrinkUnroll], xv[kShrinkUnroll];
+      for (int base = 0; base < steps; base += kShrinkWarps * UNROLL) {
+        uint4 a0[UNROLL], a1[UNROLL], xv[UNROLL];
         const uint4 z = make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int u = 0; u < kShrinkUnroll; ++u) {  // adapter bytes first: they come from HBM
-          const int i = base + u * WARPS + warp;
+        for (int u = 0; u < UNROLL; ++u) {  // adapter bytes first: they come from HBM
+          const int i = base + u * kShrinkWarps + warp;
           const bool vi = i < steps;
           a0[u] = (vi && v0) ? ldg_stream(a_row0 + i * 32) : z;
           a1[u] = (vi && v1) ? ldg_stream(a_row1 + i * 32) : z;
         }
         if (x_row == nullptr) x_row = x + (size_t)(vx ? perm[cur.s0 + g] : 0) * (size_t)d_in + 8 * t;
 #pragma unroll
-        for (int u = 0; u < kShrinkUnroll; ++u) {
-          const int i = base + u * WARPS + warp;
+        for (int u = 0; u < UNROLL; ++u) {
+          const int i = base + u * kShrinkWarps + warp;
           xv[u] = (i < steps && vx) ? ldg_cached(x_row + i * 32) : z;
         }
 #pragma unroll
-        for (int u = 0; u < kShrinkUnroll; ++u) {
+        for (int u = 0; u < UNROLL; ++u) {
           mma_bf16_16816(c, a0[u].x, a1[u].x, a0[u].y, a1[u].y, xv[u].x, xv[u].y);
           mma_bf16_16816(c, a0[u].z, a1[u].z, a0[u].w, a1[u].w, xv[u].z, xv[u].w);
         }
@@ -149,7 +150,7 @@ lora_shrink_stream_kernel(const int* __restrict__ header, const int* __restrict_
         for (int j = 0; j < 4; ++j) {
           float acc = red[0][lane][j];
 #pragma unroll
-          for (int w = 1; w < WARPS; ++w) acc += red[w][lane][j];
+          for (int w = 1; w < kShrinkWarps; ++w) acc += red[w][lane][j];
           s[j] = acc;
         }
         // c0:(rho0, col 2t) c1:(rho0, col 2t+1) c2:(rho1, col 2t) c3:(rho1, col 2t+1)
@@ -357,17 +358,18 @@ static int stream_grid(long max_items, int n_sms, int ctas_per_sm) {
 }
 
 cudaError_t launch_lora_shrink_stream(const PlanView& pv, ShrinkJobs jobs, int n_sms, cudaStream_t stream) {
+  const bool few = pv.T <= kShrinkFewT;
+  const int rows = few ? 8 : 16;
   long items = 0;
   for (int j = 0; j < jobs.n; ++j) {
-    jobs.per_seg[j] = (jobs.r[j] + 15) / 16;
+    jobs.per_seg[j] = (jobs.r[j] + rows - 1) / rows;
     items += (long)pv.Cmax * jobs.per_seg[j];
   }
   // one CTA per item (capped; CTAs stride over the items beyond the cap)
-  auto go = [&](auto* fn, int warps) {
-    return launch_pdl(fn, stream_grid(items, n_sms, 1024), 32 * warps, 0, stream, pv.header, pv.perm, pv.chunk_tab, jobs);
+  auto go = [&](auto* fn) {
+    return launch_pdl(fn, stream_grid(items, n_sms, 1024), 32 * kShrinkWarps, 0, stream, pv.header, pv.perm, pv.chunk_tab, jobs);
   };
-  return pv.T <= kShrinkFewT ? go(lora_shrink_stream_kernel<kShrinkFewWarps>, kShrinkFewWarps)
-                             : go(lora_shrink_stream_kernel<kShrinkWarps>, kShrinkWarps);
+  return few ? go(lora_shrink_stream_kernel<8, 8>) : go(lora_shrink_stream_kernel<16, 4>);
 }
 
 cudaError_t launch_lora_expand_stream(const PlanView& pv, ExpandJobs jobs, float scale, int n_sms,
