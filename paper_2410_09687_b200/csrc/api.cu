@@ -576,14 +576,14 @@ size_t moin_lora_linear_group_workspace_bytes(int32_t T, const moin_lora_job* jo
 
 moin_status moin_lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, int32_t n_jobs, float scale,
                                    void* workspace, size_t workspace_bytes, moin_stream stream) {
-  return lora_linear_group(plan, jobs, nullptr, n_jobs, plan ? plan->T : 0, false, scale, workspace, workspace_bytes, stream);
+  return lora_linear_group(plan, jobs, n_jobs, nullptr, scale, workspace, workspace_bytes, stream);
 }
 
 }  // extern "C"
 
-moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, const float* const* w_scale,
-                                    int n_jobs, int max_adapters, bool w_early, float scale, void* workspace, size_t workspace_bytes,
-                                    moin_stream stream) {
+moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, int n_jobs, const ForwardGroup* forward,
+                                    float scale, void* workspace, size_t workspace_bytes, moin_stream stream) {
+  const float* const* w_scale = forward ? forward->w_scale : nullptr;
   if (!plan || !jobs || n_jobs < 1 || n_jobs > MOIN_MAX_GROUP) return MOIN_ERR_INVALID_ARG;
   int T = 0, d_in[kMaxStreamJobs], d_out[kMaxStreamJobs], r[kMaxStreamJobs];
   for (int j = 0; j < n_jobs; ++j) {
@@ -658,7 +658,7 @@ moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* 
     h[j] = reinterpret_cast<float*>(ws_job[j]);   // [T][r] shrink results
     y0[j] = reinterpret_cast<float*>(ws_job[j] + align_up((size_t)T * (size_t)r[j] * sizeof(float), 256));
   }
-  bool grouped = T <= kDecodeSegMaxT;
+  bool grouped = T <= (forward ? kDecodeSegMaxT : kDecodeGemmMaxT);
   for (int j = 0; j < n_jobs; ++j) grouped = grouped && use_tc[j];
   if (w_scale && !grouped) return MOIN_ERR_BAD_SHAPE;   // (decode_fp8_supported says so before)
   if (grouped) {
@@ -668,9 +668,9 @@ moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* 
       gj[j] = {(const __nv_bfloat16*)jobs[j].x, jobs[j].W, (__nv_bfloat16*)jobs[j].y, y0[j], d_in[j], d_out[j],
                w_scale ? w_scale[j] : nullptr};
     // few narrow adapters in a batch of some size (gemm_decode.cu has the figures)
-    bool small_tiles = !w_scale && T > 256 && T <= 1536 && 6ll * max_adapters <= T;
+    bool small_tiles = forward && !w_scale && T > 256 && T <= 1536 && 6ll * forward->max_adapters <= T;
     for (int j = 0; j < n_jobs; ++j) small_tiles = small_tiles && r[j] <= 32;
-    st = launch_decode_gemm(hs, gj, n_jobs, T, small_tiles, w_early, s);
+    st = launch_decode_gemm(hs, gj, n_jobs, T, small_tiles, forward && forward->w_early, s);
   } else {
     for (int j = 0; j < n_jobs && !st; ++j)
       st = launch_base_gemm(hs, use_tc[j], (const __nv_bfloat16*)jobs[j].x, (const __nv_bfloat16*)jobs[j].W,

@@ -531,7 +531,8 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
         if (lora) jobs[j] = {in, m->W8[i], &m->pools[i], outs[j]};
         else gemm[j] = {(const __nv_bfloat16*)in, m->W8[i], (__nv_bfloat16*)outs[j], nullptr, d_in, d_out[j], m->W_scale[i]};
       }
-      if (lora) return lora_linear_group(&plan, jobs, m->W_scale + layer * 7 + p0, n, max_adapters, true, m->lora_scale, w.lora, w.lora_bytes, stream);
+      const ForwardGroup fwd = {m->W_scale + layer * 7 + p0, max_adapters, true};
+      if (lora) return lora_linear_group(&plan, jobs, n, &fwd, m->lora_scale, w.lora, w.lora_bytes, stream);
       ProfScope prof(MOIN_K_GEMM_TC, 1, s);
       return launch_decode_gemm(hs, gemm, n, T, false, true, s);
     }
@@ -549,7 +550,8 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
         jobs[i] = {in, W[i], &m->pools[layer * 7 + p0 + i], outs[i]};
       }
     }
-    return lora ? lora_linear_group(&plan, jobs, nullptr, n, max_adapters, !converted, m->lora_scale, w.lora, w.lora_bytes, stream) : MOIN_OK;
+    const ForwardGroup fwd = {nullptr, max_adapters, !converted};
+    return lora ? lora_linear_group(&plan, jobs, n, &fwd, m->lora_scale, w.lora, w.lora_bytes, stream) : MOIN_OK;
   };
   const float scale_log2 = 1.4426950408889634f / sqrtf(64.f);
   const __nv_bfloat16* pending = nullptr;

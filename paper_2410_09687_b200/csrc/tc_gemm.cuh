@@ -30,17 +30,22 @@ constexpr int kDecodeGemmMaxT = 512, kDecodeFp8MaxT = 512;
 // a launch a projection, store the fp32 copy from registers and leave the shrink no SM.  Forwards in segments of 12 tokens by
 // pairs / by this kernel, ms: rank 64 636 tokens 7.35 / 5.54, 1020 9.54 / 7.82, 1992 14.5 / 12.9; rank 16 4.84 / 4.53, 5.86 / 5.91,
 // 10.4 / 8.7; 8-bit base, rank 16 5.72 / 4.31, 6.77 / 5.72, 11.3 / 9.2.
+// A forward's groups only, which together gain: a layer call may be one projection by itself, or of a batch of which few tokens
+// have an adapter, and loses (1024 tokens in runs of 12, pairs / this kernel, us: 2048 -> 2048 of rank 16 25.9 / 31.2, of rank 64
+// with an adapter for a tenth of the tokens 20.7 / 26.8; 704 -> 760 14.5 / 18.6).
 constexpr int kDecodeSegMaxT = 2048;
 // small_tiles: the rule for a few narrow adapters (see there).  w_early: the kernel right before in the stream is one of this
 // library's that writes no weights, so W is complete when this one starts; never for a call whose neighbours are not known.
 moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, bool small_tiles, bool w_early, cudaStream_t stream);
-// moin_lora_linear_group on a base of 8-bit codes: jobs[j].W points to them and w_scale[j] to their row scales (nullptr:
-// bf16 weights).  Short segments and few tokens only.  max_adapters: at most so many different ones in the batch.
+// moin_lora_linear_group, and what a decoder forward says beside it (nullptr: a layer call).  w_scale != nullptr: a base of 8-bit
+// codes, jobs[j].W points to them and w_scale[j] to their row scales; short segments and few tokens only.  max_adapters: at most
+// so many different ones in the batch.
+struct ForwardGroup { const float* const* w_scale; int max_adapters; bool w_early; };
 inline bool decode_fp8_supported(const HostState* hs, int T, bool segments) {
   return hs->gemm_impl != 1 && T <= (segments ? kDecodeSegMaxT : kDecodeFp8MaxT);
 }
-moin_status lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, const float* const* w_scale, int n_jobs,
-                              int max_adapters, bool w_early, float scale, void* workspace, size_t workspace_bytes, moin_stream stream);
+moin_status lora_linear_group(const moin_plan* plan, const moin_lora_job* jobs, int n_jobs, const ForwardGroup* forward, float scale,
+                              void* workspace, size_t workspace_bytes, moin_stream stream);
 // Long-run GEMMs on CTA pairs (tc_pair.cu): y_j = x_j W_j^T for up to kPairJobs projections of one K; with a plan the
 // low-rank term s x A_e^T B_e^T is added from hb (hi / lo parts of s x A_e^T, [2][M][r], all jobs of the same r).
 constexpr int kPairJobs = 3;
