@@ -667,8 +667,7 @@ moin_status moin::lora_linear_group(const moin_plan* plan, const moin_lora_job* 
     for (int j = 0; j < n_jobs; ++j)
       gj[j] = {(const __nv_bfloat16*)jobs[j].x, jobs[j].W, (__nv_bfloat16*)jobs[j].y, y0[j], d_in[j], d_out[j],
                w_scale ? w_scale[j] : nullptr};
-    // few narrow adapters in a batch of some size (gemm_decode.cu has the figures)
-    bool small_tiles = forward && !w_scale && T > 256 && T <= 1536 && 6ll * forward->max_adapters <= T;
+    bool small_tiles = forward && !w_scale && T > 256 && T <= 1280;   // (gemm_decode.cu has the figures)
     for (int j = 0; j < n_jobs; ++j) small_tiles = small_tiles && r[j] <= 32;
     st = launch_decode_gemm(hs, gj, n_jobs, T, small_tiles, forward && forward->w_early, s);
   } else {

@@ -516,7 +516,6 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     }
     return dq.n ? launch_dequant(dq, d_in, s) : MOIN_OK;
   };
-  const int max_adapters = token_expert_in ? T : R;
   // projections of a block that read the same input and do not depend on one another go out as one group
   auto proj_group = [&](int layer, int p0, int n, const void* in, int d_in, const int* d_out, void* const* outs) -> moin_status {
     // few tokens in short segments: the GEMM converts the codes itself (gemm_decode.cu has both sides' times)
@@ -531,7 +530,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
         if (lora) jobs[j] = {in, m->W8[i], &m->pools[i], outs[j]};
         else gemm[j] = {(const __nv_bfloat16*)in, m->W8[i], (__nv_bfloat16*)outs[j], nullptr, d_in, d_out[j], m->W_scale[i]};
       }
-      const ForwardGroup fwd = {m->W_scale + layer * 7 + p0, max_adapters, true};
+      const ForwardGroup fwd = {m->W_scale + layer * 7 + p0, true};
       if (lora) return lora_linear_group(&plan, jobs, n, &fwd, m->lora_scale, w.lora, w.lora_bytes, stream);
       ProfScope prof(MOIN_K_GEMM_TC, 1, s);
       return launch_decode_gemm(hs, gemm, n, T, false, true, s);
@@ -550,7 +549,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
         jobs[i] = {in, W[i], &m->pools[layer * 7 + p0 + i], outs[i]};
       }
     }
-    const ForwardGroup fwd = {nullptr, max_adapters, !converted};
+    const ForwardGroup fwd = {nullptr, !converted};
     return lora ? lora_linear_group(&plan, jobs, n, &fwd, m->lora_scale, w.lora, w.lora_bytes, stream) : MOIN_OK;
   };
   const float scale_log2 = 1.4426950408889634f / sqrtf(64.f);

@@ -5,8 +5,8 @@
 // every byte of W is read once per call whatever the number of tokens, and 24 tokens cost a tile of 32 and not of
 // 128.  The reduction of a narrow projection (2048 -> 256 is two tiles) is cut over `ks` CTAs of a cluster.  The
 // partial sums meet through distributed shared memory - every CTA owns 1/ks of the tokens and adds the parts in rank
-// order, so the result does not depend on timing; a job's ks depends on its own shape only, so a projection gives the
-// same bits alone and in a group.
+// order, so the result does not depend on timing; a job's ks depends on its own shape, the tokens and the token tile of the
+// launch, so with the same tile a projection gives the same bits alone and in a group.
 //   warp 0     TMA producer (one thread): [128 x 64] box of W and [nt x 64] box of x per stage
 //   warp 1     allocates TMEM, issues the MMAs (one elected lane)
 //   warps 2-5  read the accumulator (TMEM lane = feature, column = token); all warps store
@@ -251,15 +251,16 @@ moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_j
   DgParams p = {};
   p.n_jobs = n_jobs; p.T = T; p.status = hs->status; p.w_early = w_early;
   // Split a projection's reduction until its own CTAs fill their share of the SM slots or a CTA is down to four 64-wide
-  // blocks (from the shape alone: the same bits in any group).  Beside many tokens' adapters the share is half of the
+  // blocks (its own, whatever else is in the group).  Beside many tokens' adapters the share is half of the
   // SMs (decode step of 256 tokens with half / all / a quarter: 237 / 264 / 248 us); up to 64 tokens two CTAs fit an SM
   // and there is little to stream beside them (step of 24 tokens with half / all: 88 / 87 us).  8-bit codes: once all
   // SMs, whatever the tokens (forwards of 112 / 303 / 495 tokens with half 1933 / 3263 / 4020 us, all 1871 / 2665 /
   // 3525, twice 1992 / 2795 / 3516).
   const bool fp8 = jobs[0].w_scale != nullptr;
-  // A few narrow adapters leave the memory to the GEMM, and its tiles of 64 tokens, two CTAs an SM, the epilogues short: forwards
-  // in segments of 24 tokens, tiles of up to 256 / of 64, ms: rank 16 288 tokens 2.81 / 2.51, 504 3.75 / 3.32, 792 5.04 / 4.39, 1392
-  // 6.97 / 6.86, 1992 8.72 / 9.82; rank 32 2.86 / 2.58, 3.87 / 3.52, 5.30 / 4.77; rank 64 504 4.41 / 4.30, 1008 7.33 / 7.42.
+  // Narrow adapters leave the memory to the GEMM, and its tiles of 64 tokens, two CTAs an SM, the epilogues short: forwards of 300
+  // to 512 tokens in segments of 1 to 24, tiles of 64 over tiles of up to 256: rank 8 0.85 to 0.93, 16 0.87 to 0.97, 32 0.89 to
+  // 1.01, 40 0.92 to 1.10, 64 0.97 to 1.23.  Segments of 12, up to 256 / of 64, ms: rank 16 1020 tokens 5.96 / 5.50, 1404 7.05 / 6.89,
+  // 2004 8.84 / 9.90; rank 32 6.29 / 6.18, 7.70 / 7.94, 9.92 / 11.4; rank 64 7.83 / 8.08, 9.98 / 11.3, 13.2 / 14.8.
   const int max_n = small_tiles ? 64 : fp8 ? kDgFp8MaxN : kDgMaxN;
   const int chunks0 = (T + max_n - 1) / max_n;
   const bool small = (T + chunks0 - 1) / chunks0 <= 64;

@@ -28,19 +28,20 @@ struct DecodeGemmJob { const __nv_bfloat16* x; const void* W; __nv_bfloat16* y; 
 constexpr int kDecodeGemmMaxT = 512, kDecodeFp8MaxT = 512;
 // Beside the adapters of short segments it takes more tokens: one launch for a group and the shrink under it, where CTA pairs take
 // a launch a projection, store the fp32 copy from registers and leave the shrink no SM.  Forwards in segments of 12 tokens by
-// pairs / by this kernel, ms: rank 64 636 tokens 7.35 / 5.54, 1020 9.54 / 7.82, 1992 14.5 / 12.9; rank 16 4.84 / 4.53, 5.86 / 5.91,
-// 10.4 / 8.7; 8-bit base, rank 16 5.72 / 4.31, 6.77 / 5.72, 11.3 / 9.2.
+// pairs / by this kernel, ms: rank 64 636 tokens 7.41 / 5.64, 1020 9.43 / 7.83, 2004 14.7 / 13.2; rank 16 4.85 / 4.01, 5.82 / 5.50,
+// 10.4 / 8.8; 8-bit base, rank 64 8.28 / 5.78, 10.2 / 8.40, 15.6 / 13.9.  Beyond 2048 tokens it gives nothing at rank 8 (2400 to 4000
+// tokens x 0.96 to 1.01) and 128 (0.96 to 1.06), 2 to 8 % between.  With an adapter for three requests in ten the gain is smaller
+// (rank 64 5.46 / 5.57 at 800 tokens, 6.04 / 6.37 at 1024, 8.98 / 7.60 at 1400).
 // A forward's groups only, which together gain: a layer call may be one projection by itself, or of a batch of which few tokens
 // have an adapter, and loses (1024 tokens in runs of 12, pairs / this kernel, us: 2048 -> 2048 of rank 16 25.9 / 31.2, of rank 64
 // with an adapter for a tenth of the tokens 20.7 / 26.8; 704 -> 760 14.5 / 18.6).
 constexpr int kDecodeSegMaxT = 2048;
-// small_tiles: the rule for a few narrow adapters (see there).  w_early: the kernel right before in the stream is one of this
+// small_tiles: the rule for narrow adapters (see there).  w_early: the kernel right before in the stream is one of this
 // library's that writes no weights, so W is complete when this one starts; never for a call whose neighbours are not known.
 moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, bool small_tiles, bool w_early, cudaStream_t stream);
 // moin_lora_linear_group, and what a decoder forward says beside it (nullptr: a layer call).  w_scale != nullptr: a base of 8-bit
-// codes, jobs[j].W points to them and w_scale[j] to their row scales; short segments and few tokens only.  max_adapters: at most
-// so many different ones in the batch.
-struct ForwardGroup { const float* const* w_scale; int max_adapters; bool w_early; };
+// codes, jobs[j].W points to them and w_scale[j] to their row scales; short segments and few tokens only.
+struct ForwardGroup { const float* const* w_scale; bool w_early; };
 inline bool decode_fp8_supported(const HostState* hs, int T, bool segments) {
   return hs->gemm_impl != 1 && T <= (segments ? kDecodeSegMaxT : kDecodeFp8MaxT);
 }

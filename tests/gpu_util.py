@@ -63,3 +63,17 @@ def assert_router_matches(ids_gpu: np.ndarray, ref: dict, key="centroid"):
     bad = diff & ~near
     assert not bad.any(), f"{int(bad.sum())} router mismatches outside near-ties, e.g. query {np.nonzero(bad)[0][:5]}"
     return int(near.sum()), int((diff & near).sum())
+
+
+def kernel_launches(call) -> dict:
+    """Launches by kernel group (the library's profiling names) of what `call` does."""
+    moin.profile_enable(4096)
+    try:
+        moin.profile_read()
+        call()
+        out = {}
+        for rec in moin.profile_read():
+            out[rec["kernel"]] = out.get(rec["kernel"], 0) + rec["launches"]
+        return out
+    finally:
+        moin.profile_enable(0)

@@ -7,16 +7,13 @@ import torch
 import moin_inputs as mi
 import oracle
 import paper_2410_09687_b200 as moin
-from gpu_util import DEV, REL_FRO
+from gpu_util import DEV, REL_FRO, kernel_launches
 from test_gpu_decoder import gpu_model, oracle_weights, rel
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("r", [16, 40])
-@pytest.mark.parametrize("lengths", [[64] * 5 + [63], [64] * 6, [40] * 11 + [39], [40] * 12, [6] * 43, [24] * 22, [9] * 170, [28] * 73,
-                                     [27] * 76, [29] * 71])
-def test_block(lengths, r):
+def _block(lengths, r):
     cfg = mi.DecoderConfig(n_layers=1, hidden=256, n_heads=4, n_kv_heads=2, head_dim=64, ffn=576, vocab=512, E=9, r=r, scale=2.0)
     model = mi.decoder_model(cfg, seed=23, missing=(4,))
     orc = oracle.DecoderOracle(cfg, oracle_weights(model))
@@ -26,11 +23,28 @@ def test_block(lengths, r):
     ref = orc.forward(*args, layer_begin=0, layer_end=1, round_storage=True, hidden_in=h_in, want_hidden=True, want_logits=False)["hidden"]
     hin = torch.from_numpy(h_in).to(torch.float32).to(DEV)
     hid = torch.empty(batch.T, cfg.hidden, dtype=torch.float32, device=DEV)
-    moin.decoder_forward(gpu_model(model), batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths),
-                         logits_mode=moin.LOGITS_NONE, hidden_in=hin, hidden_out=hid)
+    args = (gpu_model(model), batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths))
+    run = lambda: moin.decoder_forward(*args, logits_mode=moin.LOGITS_NONE, hidden_in=hin, hidden_out=hid)
+    run()
     assert moin.device_status()["timeout_flag"] == 0
     # as test_gpu_decoder's blocks: one block against the oracle that rounds where the library stores
     assert rel(hid.double().cpu().numpy() - hin.double().cpu().numpy(), ref - h_in) <= REL_FRO
+    return kernel_launches(run)
+
+
+@pytest.mark.parametrize("r", [16, 40])
+@pytest.mark.parametrize("lengths", [[64] * 5 + [63], [64] * 6, [40] * 11 + [39], [40] * 12, [6] * 43, [24] * 22, [9] * 170, [28] * 73,
+                                     [27] * 76, [29] * 71])
+def test_block(lengths, r):
+    _block(lengths, r)
+
+
+@pytest.mark.parametrize("r", [32, 48])   # tiles of 64 tokens up to rank 32
+@pytest.mark.parametrize("T", [256, 257, 513, 1280, 1281, 2047, 2048, 2049])
+def test_segments(T, r):
+    n = _block([min(9, T - i) for i in range(0, T, 9)], r)
+    assert n["lora_expand_stream"] == 4 and "lora_fused_tc" not in n
+    assert n["gemm_tc"] == (4 if T <= 2048 else 7)   # a launch a group, or one a projection
 
 
 @pytest.mark.parametrize("lengths", [[37] * 56, [9] * 70, [2] * 513])   # codes converted by the GEMM beyond 512 tokens, and no longer
