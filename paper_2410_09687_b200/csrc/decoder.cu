@@ -426,17 +426,21 @@ static DecoderWorkspace carve(const moin_model* m, int R, int T, int max_seqlen,
   return w;
 }
 
-// One expert per request: tiles or segments for T tokens of R requests?  Tiles pay a pass over a row tile for every run in it, and
-// on an 8-bit base the conversion of all weights (0.6 ms a forward); segments read an adapter again for every eight tokens.
-// Segments / tiles, ms a forward, rank 16; 64: 2 x 64 tokens 1.83 / 2.59; 1.91 / 2.75, 3 x 100 2.88 / 3.01; 3.09 / 3.17, 4 x 100
-// 3.37 / 3.10; 3.68 / 3.28, 10 x 100 5.65 / 3.65; 6.83 / 3.94; 12 x 40 3.25 / 3.67; 3.99 / 3.54, 20 x 40 4.39 / 4.59; 6.20 / 4.67;
-// 28 x 36 5.30 / 5.97; 7.23 / 6.09; 71 x 28 (segments beyond kDecodeSegMaxT) 10.2 / 9.7; 14.1 / 10.4.  8-bit base: 2 x 64 1.82 / 3.55;
-// 2.02 / 3.69, 5 x 100 3.38 / 4.20; 4.13 / 4.38, 8 x 100 4.91 / 4.75; 6.12 / 5.04, 25 x 56 6.77 / 6.39 (rank 16).
-static bool forward_tiles(int T, int R, bool coded) {
-  const int mean = T / R;
-  if (mean >= 64) return T >= (coded ? 600 : 384);
-  if (T > kDecodeSegMaxT) return mean >= 28;
-  return mean >= 40 && T >= (coded ? 1400 : 480);
+// Tiles or segments for T tokens of R requests, one expert each?  Segments read an adapter again for every eight tokens: what
+// they cost over tiles grows with the tokens.  Tiles pay a pass over a row tile for every run in it (about a request; the lower
+// the rank, the less segments lose to make up for it), a fixed part a launch that weighs less the wider the model, and on an 8-bit
+// base the conversion of all weights.  Measured on 2400 forwards of hidden size 2048 (14 to 260 tokens a request, equal and ragged,
+// ranks 8 to 128, both bases, some requests without an adapter): over the better of the two 0.3 % a forward, at the worst 21 %
+// (tiles for requests of about 32 tokens, five of which fall into many row tiles and cost a second one); always tiles 25 %, always
+// segments 18 %, tiles from 64 tokens a request on 10 %.  880 of sizes 512 to 4096: 0.9 %, 26 %.  Segments and tiles meet, ranks 16; 64, in all
+// tokens: requests of 140 410; 320, of 64 520; 330, of 48 560; 350, of 36 1300; 600, of 28 beyond 2048; 1000, on the 8-bit base of 64
+// 790; 540, in models of half the width of 64 650; 510.
+static bool forward_tiles(const moin_model* m, int T, int R) {
+  int r = 8;
+  for (int p = 0; p < 7 && m->n_layers > 0; ++p) r = m->pools[p].r > r ? m->pools[p].r : r;
+  const int fixed = 620000 / (m->hidden > 1024 ? m->hidden : 1024);
+  const int convert = m->W8 ? (r < 130 ? 330 - 2 * r : 70) : 0;
+  return T >= fixed + convert + (long long)(14 + 160 / r) * R;
 }
 
 }  // namespace moin
@@ -485,7 +489,7 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     plan.buffer = w.plan; plan.buffer_bytes = w.plan_bytes; plan.T = T; plan.E = m->E;
     // one expert per request: the run lengths are the request lengths; one per token: they depend on the ids, so
     // the plan decides after it has grouped them (reads its header back: one synchronisation of the stream)
-    plan.mode = token_expert_in ? MOIN_PLAN_AUTO : (forward_tiles(T, R, m->W8 != nullptr) ? MOIN_PLAN_TILES : MOIN_PLAN_SEGMENTS);
+    plan.mode = token_expert_in ? MOIN_PLAN_AUTO : (forward_tiles(m, T, R) ? MOIN_PLAN_TILES : MOIN_PLAN_SEGMENTS);
     st = moin_plan_build(w.token_expert, &plan, stream);
     if (st) return st;
   }

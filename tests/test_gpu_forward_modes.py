@@ -1,5 +1,5 @@
 """Decoder forwards on both sides of the rules that choose between segments and tiles, and in segments between the kernels of
-the base GEMM: tokens and mean lengths at their edges, block by block against the oracle."""
+the base GEMM: tokens and mean lengths at their edges, block by block against the oracle, and the kernels that they launch."""
 import numpy as np
 import pytest
 import torch
@@ -39,6 +39,16 @@ def test_block(lengths, r):
     _block(lengths, r)
 
 
+# the fewest tokens that go in tiles, 605 + (14 + 160 / r) R in models this narrow, and one token less
+@pytest.mark.parametrize("r,lengths", [(8, [236, 236, 235]), (16, [629]), (16, [85] * 9 + [80]), (16, [40] * 37 + [37]),
+                                       (40, [79] * 9 + [74]), (128, [400, 235])])
+def test_fewest_tokens_in_tiles(r, lengths):
+    n = _block(lengths, r)
+    assert n["lora_fused_tc"] == 4 and "lora_expand_stream" not in n
+    n = _block(lengths[:-1] + [lengths[-1] - 1], r)
+    assert n["lora_expand_stream"] == 4 and "lora_fused_tc" not in n
+
+
 @pytest.mark.parametrize("r", [32, 48])   # tiles of 64 tokens up to rank 32
 @pytest.mark.parametrize("T", [256, 257, 513, 1280, 1281, 2047, 2048, 2049])
 def test_segments(T, r):
@@ -62,3 +72,24 @@ def test_coded_base(lengths):
     # the same bf16 weights, sums of 32-bit products in another order: two bf16 roundings of a chain of four projections
     assert ((got - want).norm() / want.norm()).item() <= REL_FRO * 2 ** 0.5
     assert moin.device_status()["timeout_flag"] == 0
+
+
+@pytest.mark.parametrize("lengths,tiles,converted", [([94] * 12 + [86], False, False), ([94] * 12 + [87], True, True), ([8] * 256, False, False),
+                                                     ([8] * 256 + [1], False, True)])
+def test_coded_base_kernels(lengths, tiles, converted):
+    from test_gpu_quant import quantise
+    from test_gpu_quant_group import _decoder
+    cfg = mi.DecoderConfig(n_layers=1, hidden=320, n_heads=5, n_kv_heads=1, head_dim=64, ffn=576, vocab=512, E=4, r=16, scale=2.0)
+    model = mi.decoder_model(cfg, seed=4)
+    q = {p: quantise(model.W[0][p]) for p in oracle.PROJ_ORDER}
+    coded = _decoder(cfg, model, [{}], [{p: c.to(DEV) for p, (c, s) in q.items()}], [{p: s.to(DEV) for p, (c, s) in q.items()}])
+    orc = oracle.DecoderOracle(cfg, dict(oracle_weights(model), W=[{p: oracle.dequant_fp8(c.numpy(), s.numpy()) for p, (c, s) in q.items()}]))
+    batch = mi.decoder_batch(cfg, lengths, seed=6, req_expert=[i % 4 for i in range(len(lengths))])
+    args = [batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths)]
+    got = moin.decoder_forward(coded, *args).double().cpu().numpy()
+    want = orc.forward(batch.tokens.numpy(), batch.cu_seqlens.numpy(), batch.req_expert.numpy(), round_storage=True)["logits"]
+    assert rel(got, want) <= REL_FRO * 2 ** 0.5   # as test_gpu_decoder's logits: a block and the head
+    n = kernel_launches(lambda: moin.decoder_forward(coded, *args))
+    assert ("lora_fused_tc" in n) == tiles and ("lora_expand_stream" in n) != tiles
+    # meta 2, embedding, two norms, rotation, SwiGLU (in the GEMM where tiles are), two norms behind the block; a conversion a group
+    assert n["decoder_glue"] == 9 - tiles + 4 * converted
