@@ -492,6 +492,9 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     plan.mode = token_expert_in ? MOIN_PLAN_AUTO : (forward_tiles(m, T, R) ? MOIN_PLAN_TILES : MOIN_PLAN_SEGMENTS);
     st = moin_plan_build(w.token_expert, &plan, stream);
     if (st) return st;
+    // Ids that change no more often than the requests do (as many tiles as R runs have at the most): the rule of one expert per
+    // request, so that the same batch takes the same kernels however it is given.  Else the plan's own choice.
+    if (token_expert_in && plan.n_tiles <= R + T / kTileRows) plan.mode = forward_tiles(m, T, R) ? MOIN_PLAN_TILES : MOIN_PLAN_SEGMENTS;
   }
   if (from_hidden) {
     cudaError_t e = cudaMemcpyAsync(w.res, taps->hidden_in, (size_t)T * H * 4, cudaMemcpyDeviceToDevice, s);
