@@ -164,10 +164,12 @@ __device__ __forceinline__ float key_to_float(uint32_t u) {   // upper half of a
 // on once the kernels before it are complete and their writes visible (no-ops in an ordinary launch).  The kernels of a
 // call are launched this way, so that a kernel's launch latency and set-up lie under the tail of the one before it
 // (about 2 us each).  Rule: a kernel waits before it touches global memory and lets the next one start only after that
-// - then everything before a running kernel is complete but the kernel right before it.  Three kernels differ, and say
+// - then everything before a running kernel is complete but the kernel right before it.  Four kernels differ, and say
 // beside their code how the order is kept: the adapter shrink beside the decode GEMM, which does not wait at its start
 // (its last CTA waits at its end); the expand behind it, which reads the plan and starts on the adapters before it waits,
-// and lets the next kernel start at once; and route_parts_kernel, which reads the queries before it waits.
+// and lets the next kernel start at once; route_parts_kernel, which reads the queries before it waits; and the decode GEMM
+// of a forward (w_early), which reads weights before it waits, and so must not stand behind a kernel that lets it start
+// before waiting itself: never right behind the shrink or the expand.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -523,7 +523,8 @@ static moin_status decoder_forward_impl(const moin_model* m, const int32_t* toke
     }
     return dq.n ? launch_dequant(dq, d_in, s) : MOIN_OK;
   };
-  // projections of a block that read the same input and do not depend on one another go out as one group
+  // projections of a block that read the same input and do not depend on one another go out as one group, right behind a norm,
+  // the attention or the SwiGLU, which wait before they let it start: its GEMM may read the caller's weights at once (w_early)
   auto proj_group = [&](int layer, int p0, int n, const void* in, int d_in, const int* d_out, void* const* outs) -> moin_status {
     // few tokens in short segments: the GEMM converts the codes itself (gemm_decode.cu has both sides' times)
     bool coded = m->W8 && decode_fp8_supported(hs, T, lora) && (!lora || plan.mode == MOIN_PLAN_SEGMENTS);

@@ -90,8 +90,9 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
     mbar_init(done, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // Weights older than the kernel before this one (the caller knows): the first stages' are on their way while that one ends.
-    // Forward of 112 tokens on the 8-bit base 1829 -> 1777 us, on the bf16 base 1751 -> 1744, of 14 tokens 1465 -> 1451.
+    // Weights that the kernel before this one leaves alone (see w_early): the first stages' are on their way while that one
+    // ends.  Forwards of 16 / 112 / 260 / 1000 tokens, rank 16: bf16 base 1334 -> 1289, 1763 -> 1745, 2495 -> 2479, 5722 -> 5694
+    // us; 8-bit base 1326 -> 1303, 1834 -> 1790, 2550 -> 2525, 5956 -> 5926.
     for (int s = 0; s < n_early; ++s) {
       mbar_expect_tx(full0 + 8 * s, stage_bytes);
       tma_load_2d(ring + s * stage_bytes, &maps.w[job], full0 + 8 * s, (kb0 + s) * kDgK, f0);
