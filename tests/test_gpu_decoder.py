@@ -9,7 +9,7 @@ import torch
 import moin_inputs as mi
 import oracle
 import paper_2410_09687_b200 as moin
-from gpu_util import DEV, REL_FRO
+from gpu_util import DEV, REL_FRO, kernel_launches
 
 pytestmark = pytest.mark.gpu
 
@@ -49,10 +49,10 @@ def setup():
     return model, gpu_model(model), oracle.DecoderOracle(CFG, oracle_weights(model))
 
 
-@pytest.mark.parametrize("lengths,experts", [([70, 1, 129, 33, 64], [0, 2, 3, -1, 5]),      # short requests: segments
-                                             ([200, 130, 257], [1, 1, 4]),                  # long runs: tiles
-                                             ([3, 530, 260], [5, 2, 0])])     # attention items beyond 256 keys
-def test_decoder_end_to_end_and_block_by_block(setup, lengths, experts):
+@pytest.mark.parametrize("lengths,experts,tiles", [([70, 1, 129, 33, 64], [0, 2, 3, -1, 5], False), ([200, 130, 257], [1, 1, 4], False),
+                                                   ([400, 260, 514], [1, 1, 4], True),
+                                                   ([3, 530, 260], [5, 2, 0], True)])     # attention items beyond 256 keys
+def test_decoder_end_to_end_and_block_by_block(setup, lengths, experts, tiles):
     model, gm, orc = setup
     batch = mi.decoder_batch(CFG, lengths, seed=4, req_expert=experts)
     tok, cu, re_ = batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV)
@@ -78,6 +78,7 @@ def test_decoder_end_to_end_and_block_by_block(setup, lengths, experts):
     # distance to the pure fp64 oracle is printed.
     logits = moin.decoder_forward(gm, tok, cu, re_, max(lengths), hidden_out=hid)
     torch.cuda.synchronize()
+    assert ("lora_fused_tc" in kernel_launches(lambda: moin.decoder_forward(gm, tok, cu, re_, max(lengths)))) == tiles
     got = logits.to(torch.float64).cpu().numpy()
     assert np.isfinite(got).all()
     exact = orc.forward(*args)["logits"]
@@ -153,9 +154,9 @@ def test_decoder_per_token_experts(setup):
     assert moin.device_status()["timeout_flag"] == 0
 
 
-@pytest.mark.parametrize("lengths,experts", [([130, 1, 64, 70], [3, -1, 9, 3]),            # long runs -> tile mode
-                                             ([5, 9, 1, 12, 7, 3, 8, 2], [1, 2, 3, 4, 5, 6, 7, 1])])  # decode-like
-def test_decoder_full_width_blocks(lengths, experts):
+@pytest.mark.parametrize("lengths,experts,tiles", [([130, 1, 64, 70], [3, -1, 9, 3], False), ([215, 1, 137], [3, -1, 9], True),
+                                                   ([5, 9, 1, 12, 7, 3, 8, 2], [1, 2, 3, 4, 5, 6, 7, 1], False)])  # decode-like
+def test_decoder_full_width_blocks(lengths, experts, tiles):
     """TinyLlama-width blocks (hidden 2048, 32/4 heads, SwiGLU 5632, vocab 32000, rank 64): every block is
     checked with the oracle's own block input, and the logits of the last block's output too."""
     cfg = mi.DecoderConfig(n_layers=2, E=16, r=64)
@@ -197,6 +198,7 @@ def test_decoder_full_width_blocks(lengths, experts):
             print(f"full-width logits after the last block: {e_log:.2e}")
             assert e_log <= 1.5 * REL_FRO
         h_in = ref["hidden"]
+    assert ("lora_fused_tc" in kernel_launches(lambda: moin.decoder_forward(gm, tok, cu, re_, max(lengths)))) == tiles
     assert moin.device_status()["timeout_flag"] == 0
 
 

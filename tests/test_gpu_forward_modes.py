@@ -93,3 +93,27 @@ def test_coded_base_kernels(lengths, tiles, converted):
     assert ("lora_fused_tc" in n) == tiles and ("lora_expand_stream" in n) != tiles
     # meta 2, embedding, two norms, rotation, SwiGLU (in the GEMM where tiles are), two norms behind the block; a conversion a group
     assert n["decoder_glue"] == 9 - tiles + 4 * converted
+
+
+@pytest.mark.parametrize("coded", [False, True])
+@pytest.mark.parametrize("lengths", [[9] * 8, [70, 41, 30]])
+def test_wide_block(lengths, coded):
+    """A block of full width in segments: reductions of more k-blocks than a CTA has stages, so that what was requested before the
+    wait and what follows it share the ring."""
+    from test_gpu_quant import quantise
+    from test_gpu_quant_group import _decoder
+    cfg = mi.DecoderConfig(n_layers=1, vocab=512, E=4, r=16, scale=2.0)
+    model = mi.decoder_model(cfg, seed=7)
+    q = {p: quantise(model.W[0][p]) for p in oracle.PROJ_ORDER}
+    W = {p: oracle.dequant_fp8(c.numpy(), s.numpy()) for p, (c, s) in q.items()}
+    if coded:
+        gm = _decoder(cfg, model, [{}], [{p: c.to(DEV) for p, (c, s) in q.items()}], [{p: s.to(DEV) for p, (c, s) in q.items()}])
+    else:
+        gm = _decoder(cfg, model, [{p: torch.from_numpy(w.view(np.int16)).view(torch.bfloat16).to(DEV) for p, w in W.items()}])
+    batch = mi.decoder_batch(cfg, lengths, seed=6, req_expert=[i % 4 for i in range(len(lengths))])
+    run = lambda: moin.decoder_forward(gm, batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths))
+    orc = oracle.DecoderOracle(cfg, dict(oracle_weights(model), W=[W]))
+    want = orc.forward(batch.tokens.numpy(), batch.cu_seqlens.numpy(), batch.req_expert.numpy(), round_storage=True)["logits"]
+    assert rel(run().double().cpu().numpy(), want) <= REL_FRO * 2 ** 0.5 * 1.5   # as test_gpu_decoder's blocks of this width, and the head
+    assert "lora_expand_stream" in kernel_launches(run)
+    assert moin.device_status()["timeout_flag"] == 0

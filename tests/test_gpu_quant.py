@@ -7,7 +7,7 @@ import torch
 import moin_inputs as mi
 import oracle
 import paper_2410_09687_b200 as moin
-from gpu_util import DEV, REL_FRO
+from gpu_util import DEV, REL_FRO, kernel_launches
 
 pytestmark = pytest.mark.gpu
 
@@ -61,7 +61,7 @@ def test_decoder_on_a_quantised_base():
         "W": Wdq, "A": [{p: mi.bf16_bits(model.pools[l][p].A) for p in order} for l in range(cfg.n_layers)],
         "B": [{p: mi.bf16_bits(model.pools[l][p].B) for p in order} for l in range(cfg.n_layers)],
         "slot_of_expert": model.pools[0]["q"].slot_of_expert.numpy()})
-    for lengths, experts in (([70, 1, 129, 33], [0, 2, 3, -1]), ([200, 130], [1, 4])):   # short segments / long runs
+    for lengths, experts, tiles in (([70, 1, 129, 33], [0, 2, 3, -1], False), ([200, 130], [1, 4], False), ([603, 390], [1, 4], True)):
         batch = mi.decoder_batch(cfg, lengths, seed=9, req_expert=experts)
         logits = moin.decoder_forward(gm, batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths))
         torch.cuda.synchronize()
@@ -72,5 +72,7 @@ def test_decoder_on_a_quantised_base():
         e_r = np.linalg.norm(got - rounded) / np.linalg.norm(rounded)
         e_x = np.linalg.norm(got - exact) / np.linalg.norm(exact)
         print(f"quantised base, lengths {lengths}: logits vs storage-rounded oracle {e_r:.2e}, vs fp64 oracle {e_x:.2e}")
+        args = [batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths)]
+        assert ("lora_fused_tc" in kernel_launches(lambda: moin.decoder_forward(gm, *args))) == tiles
         assert e_r <= REL_FRO * np.sqrt(cfg.n_layers + 1) and e_x <= 2 * REL_FRO * np.sqrt(cfg.n_layers + 1)
     assert moin.device_status()["timeout_flag"] == 0

@@ -33,7 +33,7 @@ def test_some_projections_coded(coded):
     mixed = _decoder(cfg, model, [{p: plain[p] for p in plain if p not in coded}], [{p: q[p][0].to(DEV) for p in coded}],
                      [{p: q[p][1].to(DEV) for p in coded}])
     ref = _decoder(cfg, model, [same])
-    for lengths in ([130, 77], [600, 9]):
+    for lengths in ([130, 77], [600, 9], [700, 403]):   # segments; tiles on either base
         batch = mi.decoder_batch(cfg, lengths, seed=5, req_expert=[0, 2])
         args = (batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths))
         # the same bf16 weights through the same kernels

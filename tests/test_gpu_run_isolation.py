@@ -7,7 +7,7 @@ import torch
 import moin_inputs as mi
 import oracle
 import paper_2410_09687_b200 as moin
-from gpu_util import DEV, assert_layer_close, gpu_pool, oracle_layer
+from gpu_util import DEV, assert_layer_close, gpu_pool, kernel_launches, oracle_layer
 from test_gpu_decoder import oracle_weights
 
 pytestmark = pytest.mark.gpu
@@ -41,10 +41,11 @@ def test_layer(lengths, experts, r, where):
         assert not torch.isfinite(y[torch.from_numpy(np.nonzero(te == 1)[0]).to(DEV)]).all(dim=1).any()
 
 
-def test_block_with_fused_product():
+@pytest.mark.parametrize("lengths,fused", [([290, 330, 275], True), ([90, 130, 75], False)])   # tiles / segments
+def test_block_with_fused_product(lengths, fused):
     cfg = mi.DecoderConfig(n_layers=1, hidden=256, n_heads=4, n_kv_heads=2, head_dim=64, ffn=576, vocab=512, E=3, r=16, scale=2.0)
     model = mi.decoder_model(cfg, seed=18)
-    lengths, experts = [90, 130, 75], [0, 1, 2]
+    experts = [0, 1, 2]
     batch = mi.decoder_batch(cfg, lengths, seed=18, req_expert=experts)
     args = (batch.tokens.numpy(), batch.cu_seqlens.numpy(), batch.req_expert.numpy())
     orc = oracle.DecoderOracle(cfg, oracle_weights(model))
@@ -58,8 +59,9 @@ def test_block_with_fused_product():
                            [{p: model.W[0][p].to(DEV) for p in oracle.PROJ_ORDER}], pools, cfg.E, cfg.scale)
     hin = torch.from_numpy(h_in).to(torch.float32).to(DEV)
     hid = torch.empty(batch.T, cfg.hidden, dtype=torch.float32, device=DEV)
-    moin.decoder_forward(gm, batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV), max(lengths),
-                         logits_mode=moin.LOGITS_NONE, hidden_in=hin, hidden_out=hid)
+    n = kernel_launches(lambda: moin.decoder_forward(gm, batch.tokens.to(DEV), batch.cu_seqlens.to(DEV), batch.req_expert.to(DEV),
+                                                     max(lengths), logits_mode=moin.LOGITS_NONE, hidden_in=hin, hidden_out=hid))
+    assert ("lora_fused_tc" in n) == fused
     d, ref = hid.double().cpu().numpy() - hin.double().cpu().numpy(), want - h_in
     own = slice(lengths[0], lengths[0] + lengths[1])
     others = np.r_[0:lengths[0], lengths[0] + lengths[1]:batch.T]
