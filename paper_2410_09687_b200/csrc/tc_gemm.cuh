@@ -23,7 +23,8 @@ bool tc_fused_supported(int r);
 
 // y = x W^T (bf16) and optionally y0 = x W^T (fp32) for few tokens, up to kMaxStreamJobs projections in one launch
 // (gemm_decode.cu).
-// w_scale != nullptr: W is 8-bit float codes with a scale per row (all jobs of a launch alike), T <= kDecodeFp8MaxT.
+// w_scale != nullptr: W is 8-bit float codes with a scale per row (all jobs of a launch alike), T <= kDecodeFp8MaxT without
+// adapters, kDecodeSegMaxT beside those of short segments.
 struct DecodeGemmJob { const __nv_bfloat16* x; const void* W; __nv_bfloat16* y; float* y0; int d_in, d_out; const float* w_scale; };
 constexpr int kDecodeGemmMaxT = 512, kDecodeFp8MaxT = 512;
 // Beside the adapters of short segments it takes more tokens: one launch for a group and the shrink under it, where CTA pairs take

@@ -35,9 +35,9 @@ struct TsParams {
 };
 
 // Where a projection's h goes for the tile in hand.
-struct TsOut { int job, slot, r_use; __nv_bfloat16* hb; };
+struct TsOut { int slot, r_use; __nv_bfloat16* hb; };
 __device__ __forceinline__ TsOut ts_out(const TsParams& p, const int (&slot)[kTcMaxShrinkJobs], int job) {
-  TsOut o = {job, slot[0], p.r, p.hb[0]};
+  TsOut o = {slot[0], p.r, p.hb[0]};
   const int* ranks = p.slot_rank[0];
 #pragma unroll
   for (int j = 1; j < kTcMaxShrinkJobs; ++j)
@@ -99,7 +99,7 @@ tc_shrink_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__ Ts
   const uint32_t tmem = *tmem_slot;
   pdl_begin();   // (the set-up above overlaps the tail of the kernel before)
 
-  // the first tile's entries together with the number of tiles (in bounds: no more clusters than tokens)
+  // the first tile's entries together with the number of tiles (one round trip less; in bounds: no more clusters than tokens)
   int4 nxt = make_int4(__ldg(p.tile_row0 + cluster), __ldg(p.tile_rows + cluster), __ldg(p.tile_expert + cluster), 0);
   const int total = __ldg(p.header + PH_NTILES), N = p.N, pitch = N + 4;
   const int nkb = p.K / kTsK, kb0 = nkb * rank / p.ks, kb1 = nkb * (rank + 1) / p.ks;
