@@ -265,7 +265,7 @@ cudaError_t launch_route_finish(const unsigned long long* keys, const __nv_bfloa
 // that device current.  The status block's address and the kernels' shared-memory opt-ins belong to one device, so
 // nothing here is shared between devices.
 constexpr int kMaxDevices = 64;
-constexpr int kOptinSlots = 18;
+constexpr int kOptinSlots = 19;
 struct HostState {
   DeviceStatus* status = nullptr;  // device address of the status block
   int device = -1;
@@ -280,7 +280,7 @@ moin_status record_cuda(cudaError_t e);       // MOIN_OK or MOIN_ERR_CUDA (remem
 // that attribute per device, so the "already done" note is kept per device too (slot = one id per kernel).
 enum {
   OPTIN_ROUTE_CLUSTER = 0, /* .. 7 */ OPTIN_ROUTE_SIMPLE = 8, OPTIN_ATTENTION = 9, OPTIN_DECODE_GEMM = 10,
-  OPTIN_DECODE_GEMM_FP8 = 11, OPTIN_TC_SHRINK = 12, OPTIN_TC_PAIR = 13 /* .. 17 */
+  OPTIN_DECODE_GEMM_FP8 = 11, OPTIN_TC_SHRINK = 12, OPTIN_TC_PAIR = 13, /* .. 17 */ OPTIN_DECODE_GEMM_EARLY = 18
 };
 template <class Fn>
 inline cudaError_t ensure_smem_optin(int slot, Fn* fn, size_t bytes) {

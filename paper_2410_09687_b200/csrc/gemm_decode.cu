@@ -31,7 +31,7 @@ constexpr int kDgFp8MaxN = 128, kDgFp8Cols = 256, kDgFp8Smem = 104 * 1024;
 
 struct DgMaps { CUtensorMap w[kMaxStreamJobs], x[kMaxStreamJobs]; };
 struct DgParams {
-  int n_jobs, T, nt, n_chunks, stages, tmem_cols, cluster, w_early;   // nt tokens per tile, n_chunks tiles over the tokens
+  int n_jobs, T, nt, n_chunks, stages, tmem_cols, cluster;   // nt tokens per tile, n_chunks tiles over the tokens
   int cta_end[kMaxStreamJobs];   // CTAs of jobs 0 .. j (each job's padded to whole clusters)
   int ks[kMaxStreamJobs], tiles[kMaxStreamJobs], K[kMaxStreamJobs], d_out[kMaxStreamJobs];
   __nv_bfloat16* y[kMaxStreamJobs];
@@ -40,7 +40,7 @@ struct DgParams {
   DeviceStatus* status;
 };
 
-template <bool FP8>
+template <bool FP8, bool EARLY>
 __global__ void __launch_bounds__(kDgThreads)
 decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -79,7 +79,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
   const bool on = tile < n_tiles;                                      // (the last cluster of a job may be padded)
   const int tok0 = (item - tile * p.n_chunks) * p.nt, f0 = tile * kDgM;
   const int nkb = on ? K / kDgK : 0, kb0 = nkb * rank / ks, kb1 = nkb * (rank + 1) / ks;
-  const int n_early = p.w_early ? min(S, kb1 - kb0) : 0;   // k-blocks whose weights do not wait for the kernel before
+  const int n_early = EARLY ? min(S, kb1 - kb0) : 0;   // k-blocks whose weights do not wait for the kernel before
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -120,7 +120,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
         if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 51)) break;
         const uint32_t sa = ring + s * stage_bytes, full = full0 + 8 * s;
         if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
-        if (kb - kb0 >= n_early) {
+        if (!EARLY || kb - kb0 >= n_early) {
           mbar_expect_tx(full, stage_bytes);
           tma_load_2d(sa, mw, full, kb * kDgK, f0);
         }
@@ -250,7 +250,7 @@ decode_gemm_kernel(const __grid_constant__ DgMaps maps, const DgParams p) {
 moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, bool small_tiles, bool w_early, cudaStream_t stream) {
   DgMaps maps;
   DgParams p = {};
-  p.n_jobs = n_jobs; p.T = T; p.status = hs->status; p.w_early = w_early;
+  p.n_jobs = n_jobs; p.T = T; p.status = hs->status;
   // Split a projection's reduction until its own CTAs fill their share of the SM slots or a CTA is down to four 64-wide
   // blocks (its own, whatever else is in the group).  Beside many tokens' adapters the share is half of the
   // SMs (decode step of 256 tokens with half / all / a quarter: 237 / 264 / 248 us); up to 64 tokens two CTAs fit an SM
@@ -314,11 +314,13 @@ moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_j
   const size_t out = (size_t)p.nt * kDgM * sizeof(float);
   while ((size_t)p.stages * stage < out) ++p.stages;
   size_t smem = (size_t)p.stages * stage + 1024 /*align*/ + 256 /*barriers*/;
-  auto* kernel = fp8 ? decode_gemm_kernel<true> : decode_gemm_kernel<false>;
+  // (codes come from forwards only, whose neighbours are known.  A kernel of its own for layer calls: with the early loads under a
+  // run-time flag they took 0.2 to 0.4 us a launch longer.)
+  auto* kernel = fp8 ? decode_gemm_kernel<true, true> : w_early ? decode_gemm_kernel<false, true> : decode_gemm_kernel<false, false>;
   // Half of the tensor memory for less than half of the shared memory would let a third CTA in, which then waits in the
   // allocation for CTAs that may wait for its own cluster: two at most.
   if (fp8 && smem < kDgFp8Smem) smem = kDgFp8Smem;
-  cudaError_t e = ensure_smem_optin(fp8 ? OPTIN_DECODE_GEMM_FP8 : OPTIN_DECODE_GEMM, kernel, 160 * 1024);
+  cudaError_t e = ensure_smem_optin(fp8 ? OPTIN_DECODE_GEMM_FP8 : w_early ? OPTIN_DECODE_GEMM_EARLY : OPTIN_DECODE_GEMM, kernel, 160 * 1024);
   if (e != cudaSuccess) return record_cuda(e);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ctas);

@@ -37,10 +37,10 @@ constexpr int kDecodeGemmMaxT = 512, kDecodeFp8MaxT = 512;
 // have an adapter, and loses (1024 tokens in runs of 12, pairs / this kernel, us: 2048 -> 2048 of rank 16 25.9 / 31.2, of rank 64
 // with an adapter for a tenth of the tokens 20.7 / 26.8; 704 -> 760 14.5 / 18.6).
 constexpr int kDecodeSegMaxT = 2048;
-// small_tiles: the rule for narrow adapters (see there).  w_early: W may be read before this kernel waits.  Only where the
-// kernel right before in the stream writes no weights and waits before it lets this one start, so that all older ones (a copy or
-// a conversion of W) are complete by then: behind a norm, an attention or a SwiGLU of this library, not behind the adapter
-// shrink or expand, which let the next kernel start first, and not in a call whose neighbours are not known.
+// small_tiles: the rule for narrow adapters (see there).  w_early: W may be read before this kernel waits (8-bit codes always are).
+// Only where the kernel right before in the stream writes no weights and waits before it lets this one start, so that all older
+// ones (a copy or a conversion of W) are complete by then: behind a norm, an attention or a SwiGLU of this library, not behind the
+// adapter shrink or expand, which let the next kernel start first, and not in a call whose neighbours are not known.
 moin_status launch_decode_gemm(HostState* hs, const DecodeGemmJob* jobs, int n_jobs, int T, bool small_tiles, bool w_early, cudaStream_t stream);
 // moin_lora_linear_group, and what a decoder forward says beside it (nullptr: a layer call).  w_scale != nullptr: a base of 8-bit
 // codes, jobs[j].W points to them and w_scale[j] to their row scales; short segments and few tokens only.
